@@ -3,17 +3,17 @@
 // the d_k x d_v state held on chip while a CTA walks over a segment of consecutive tiles.
 //
 // A sequence of N tiles is cut into segments of G tiles; one CTA sweeps one segment.
-//   forward : sweep_local  per segment, from a zero state: the state it leaves and its total decay
-//             seg_scan     per sequence, over the few segment ends: the state entering each segment
-//             sweep_fwd    per segment, from its true entry state: out = tril(Qc Kc^T) V + Qc Sc per tile
-//   backward: sweep_local  (backward flavour) also stores, per (sub-)chunk, the zero-start state in
-//                          fp16 and the decay since the segment start, and accumulates the segment's
-//                          contribution to the state gradient
-//             seg_scan     forward over the states, backward over the state gradients, gate-gradient carry
-//             sweep_bwd    per segment in reverse: dq, dk, dv, dgate with the state gradient on chip
-// With at least as many sequences as CTAs stay resident the sequences are not cut (one segment each):
-// the forward pass is then sweep_fwd alone, started from the start state, and the backward pass runs a
-// local sweep that only stores the per-chunk states.
+//   forward : sweep_local_fwd  per segment, from a zero state: the state it leaves and its total decay
+//             seg_scan         per sequence, over the few segment ends: the state entering each segment
+//             sweep_fwd        per segment, from its true entry state: out = tril(Qc Kc^T) V + Qc Sc per tile
+//   backward: sweep_local_bwd  per segment, from a zero state: per (sub-)chunk the state entering it in fp16
+//                              and the decay since the segment start; the segment's contribution to the
+//                              state gradient
+//             seg_scan         forward over the states, backward over the state gradients, gate-gradient carry
+//             sweep_bwd        per segment in reverse: dq, dk, dv, dgate with the state gradient on chip
+// Where the sequences are not cut (one segment each) the forward pass is sweep_fwd alone, started from the
+// start state, and the backward pass without state arguments needs no scan: its local sweep only stores
+// the per-chunk states, and the entry state, incoming gradient and carry of every segment are zero.
 // Per (sub-)chunk, with Lam the cumulative gate inside it, c = Lam_end / 2 per channel,
 //   Qc = q exp(Lam - c), Kc = k exp(c - Lam), Sc = diag(exp(c)) S_in, Dc = diag(exp(c)) D_out:
 //   P   = tril(Qc Kc^T)                         dP = tril(dO V^T)
@@ -24,11 +24,12 @@
 // In the backward sweep S_in = S_local + diag(G) S_segment, G the decay since the segment start, so
 // dO Sc^T = dO Sc_local^T + (dO S_segment^T) diag(exp(c) G): two products and one fused multiply-add.
 //
-// Every product is a tcgen05.mma (kind::f16, fp16 operands, fp32 accumulators in tensor memory)
-// issued by lane 0 of the last warp, which otherwise works like the others: all threads build operand tiles, mask
-// the scores and post-process accumulators, phase by phase.  Token rows of the next tile are
-// prefetched into registers; at d = 64 two CTAs of 256 threads share an SM, so one builds while the
+// Every product is a tcgen05.mma (kind::f16, fp16 operands, fp32 accumulators in tensor memory) issued by
+// lane 0 of the last warp, which otherwise works like the others: all threads build operand tiles, mask the
+// scores and post-process accumulators, phase by phase (columns.cuh holds the work split).  Rows of the
+// next tile are prefetched into registers; two CTAs of 256 threads share an SM, so one builds while the
 // other's products are in the tensor pipe.
+#include "columns.cuh"
 #include "sweep.cuh"
 
 namespace dig {
@@ -48,6 +49,7 @@ struct SweepArgs {
     float *s_out;           // ... and where the final state goes (may be null)
     int *status;
     int accumulate;
+    int scanned;            // backward pass: a segment scan ran (else every segment's entry state, gradient and carry are zero)
     Geom g;
     Plan plan;
 };
@@ -74,125 +76,65 @@ __device__ __forceinline__ void cta_teardown(Ctl *ctl, uint32_t tmem_cols)
     if (threadIdx.x < 32) tmem_dealloc(ctl->tmem_base, tmem_cols);
 }
 
-// Operand tiles of rows [lo, hi) of the prefetched tile (the other rows are zero):
-//   tK <- k 2^(off - Lam), tV <- v, and where present tQ <- q 2^(Lam - off), tG <- dO.
-__device__ __forceinline__ uint4 keep4(const uint4 &u, uint32_t m) { return make_uint4(u.x & m, u.y & m, u.z & m, u.w & m); }
-template <int D, int NT, bool HQ, bool HD>
-__device__ __forceinline__ void build_tiles(const Raw<Lay<D, NT>::NIT, HQ, HD> &r, char *tQ, char *tK, char *tV, char *tG,
-                                            const float *table, const float *off, const int *row_off, int lo, int hi)
+// Bounded wait whose verdict (with the thread's earlier ones) is uniform over the warp: tcgen05.ld must never
+// run under a lane-divergent condition.
+__device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, int *status, bool ok)
 {
-    using C = Cfg<D>;
-#pragma unroll
-    for (int i = 0; i < Lay<D, NT>::NIT; ++i) {
-        const int it = (int)threadIdx.x + NT * i;
-        if (item_exists<D, NT>(it)) {
-            const int row = it / C::NCH, j = it - row * C::NCH;
-            const int o = j * C::CHT + row * 16;
-            // rows outside the sub-chunk or past the end of the sequence become zeros: no branch, a mask on the
-            // packed result (which also discards whatever an out-of-range exponent produced there)
-            const uint32_t m = (row >= lo && row < hi && row_off[row] >= 0) ? 0xffffffffu : 0u;
-            float lam[8], of[8], x[8], y[8];
-            ld8(table + row * C::LAMP + 8 * j, lam);
-            ld8(off + 8 * j, of);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) lam[e] -= of[e];
-            unpack_b8(r.k[i], x);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) y[e] = x[e] * ex2(-lam[e]);
-            *reinterpret_cast<uint4 *>(tK + o) = keep4(pack_h8(y), m);
-            unpack_b8(r.v[i], x);
-            *reinterpret_cast<uint4 *>(tV + o) = keep4(pack_h8(x), m);
-            if (HQ) {
-                unpack_b8(r.q[i], x);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) y[e] = x[e] * ex2(lam[e]);
-                *reinterpret_cast<uint4 *>(tQ + o) = keep4(pack_h8(y), m);
-            }
-            if (HD) {
-                unpack_b8(r.d[i], x);
-                *reinterpret_cast<uint4 *>(tG + o) = keep4(pack_h8(x), m);
-            }
-        }
-    }
-}
-
-// State product with channels along M: acc <- A^T B, A and B token tiles read down their rows
-// (contraction over the 64 tokens).  Small heads: two value-column halves into the two lane halves.
-template <int D>
-__device__ __forceinline__ void issue_state_product(uint32_t tmem_acc, const char *tA, const char *tB)
-{
-    using C = Cfg<D>;
-    const uint32_t a = smem_u32(tA), b = smem_u32(tB);
-    if constexpr (C::BIGM) {
-        issue<128, C::NACC, true, true, T / 16, C::CHT, C::CHT>(tmem_acc, a, b, false);
-    } else {
-        constexpr int HCH = C::NCH / 2;
-        issue<64, D / 2, true, true, T / 16, C::CHT, C::CHT>(tmem_acc, a, b, false);
-        issue<64, D / 2, true, true, T / 16, C::CHT, C::CHT>(tmem_acc + (16u << 16), a, b + HCH * C::CHT, false);
-    }
-}
-
-// Bounded wait whose verdict is uniform over the warp (tcgen05.ld must never run under a
-// lane-divergent condition).
-__device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, int *status)
-{
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, status)) != 0;
+    const bool done = mbar_wait(bar, parity, status);
+    return __all_sync(0xffffffffu, done && ok) != 0;
 }
 
 #define SYNC_OR_DIE()                               \
     do {                                            \
-        if (!__syncthreads_and(ok)) goto die;       \
+        if (!__syncthreads_and(ok)) {               \
+            ok = false;                             \
+            goto die;                               \
+        }                                           \
     } while (0)
 
 // =================================================================================================
-// sweep_local: a segment from a zero state.
+// sweep_local_fwd: the state a segment leaves from a zero start, sum over its tokens of k 2^(gates after
+// the token) v^T, and its total decay.  The tiles are walked from the segment's end: every decay factor is
+// then a power of two below 1 that needs no centring (no sub-chunks, whatever the gates), and the products
+// of all tiles add up in tensor memory, so the state is read once per segment.  One barrier per tile: behind
+// it lie the group sums of this tile and the operand rows of the one before, whose product is issued there;
+// operand tiles and sums have two buffers, and the rows of the next tile are loaded a whole tile ahead.
+// Bound by the latency of its phases (IPC 1.4); 48 sequences of 4096 tokens, d = 64: 40.3 us with the state in
+// registers, decayed once per tile in scan order, 30.2 us now; 16 of 16384, d = 72: 79 -> 48.5 us.
 // =================================================================================================
-template <int D, int NT, bool BWD>
-struct LocalSmem {
+template <int D>
+struct LocalFwdSmem {
     using C = Cfg<D>;
-    using L = Lay<D, NT>;
-    static constexpr int kTiles = (BWD ? 4 : 2) * C::TILE_T;
-    // an M = 128 operand read down the rows of tQ / tK covers 16 chunks (more than the tile has): the
-    // bytes behind it belong to the next tile, which is mapped and holds finite fp16 values
-    static constexpr int kTilesPad = kTiles;
-    static_assert(!C::BIGM || 16 * C::CHT <= 2 * C::TILE_T, "an M = 128 operand must stay inside the tile area");
-    static constexpr int kFloats = T * C::LAMP + L::NSEG * D + 8 * D;
-    static constexpr size_t bytes = kTilesPad + kFloats * 4 + 4 * T * 4 + sizeof(Ctl);
-    static constexpr uint32_t tmem_cols = C::BIGM ? (BWD ? 256 : 128) : (BWD ? 64 : 32);
+    using L = Col<D>;
+    static constexpr int kBuf = 2 * C::TILE_T;                                // tK tV
+    static constexpr int kPad = L::X ? 16 * C::CHT - C::TILE_T : 0;           // the corner's operand reads past its tile
+    static constexpr size_t bytes = 2 * kBuf + kPad + 2 * 8 * D * 4 + 4 * T * 4 + sizeof(Ctl);
+    static constexpr uint32_t tmem_cols = L::ACCS <= 32 ? 32 : 64;
 };
 
-// SLOTS: also store, per (sub-)chunk, the zero-start state and the decay since the segment start (what the
-// backward sweep reads).  The backward flavour (BWD) always does and adds the segment's contribution to the
-// state gradient; a backward pass over uncut sequences needs only the stored states (BWD = false, SLOTS = true).
-template <int D, int NT, bool BWD, int OCC, bool SLOTS = BWD>
-__global__ void __launch_bounds__(NT, OCC)
-sweep_local(const SweepArgs a)
+template <int D>
+__global__ void __launch_bounds__(Col<D>::NT, 2)
+sweep_local_fwd(const SweepArgs a)
 {
-    static_assert(SLOTS || !BWD, "the backward flavour stores the per-chunk states");
     using C = Cfg<D>;
-    using L = Lay<D, NT>;
-    using SM = LocalSmem<D, NT, BWD>;
+    using L = Col<D>;
+    using SM = LocalFwdSmem<D>;
+    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs
     extern __shared__ __align__(128) char smem[];
-    char *tQ = smem, *tK = BWD ? tQ + C::TILE_T : smem, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T;
-    float *table = reinterpret_cast<float *>(smem + SM::kTilesPad);
-    float *sTot = table + T * C::LAMP, *vecb = sTot + L::NSEG * D;
-    int *rowOff = reinterpret_cast<int *>(vecb + 8 * D);
+    float *sTot = reinterpret_cast<float *>(smem + 2 * SM::kBuf + SM::kPad);
+    int *rowOff = reinterpret_cast<int *>(sTot + 2 * 8 * D);          // ring of four tiles
     Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 4 * T);
-    constexpr uint32_t aU = 0, aW = C::BIGM ? C::NACC : D / 2;
 
     const int tid = threadIdx.x;
-    constexpr int kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs (warps 0 and 1 carry the per-channel work)
-    cta_setup(ctl, 1, SM::tmem_cols, smem, SM::kTilesPad);
-    const uint32_t tmem = ctl->tmem_base, lane_base = (uint32_t)(32 * ((tid >> 5) & 3)) << 16;
+    cta_setup(ctl, 2, SM::tmem_cols, smem, 2 * SM::kBuf + SM::kPad);
+    const Who<D> w;
+    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     const Geom &g = a.g;
     const Plan &pl = a.plan;
-    const StateMap<D, NT> sm;
-    float S[L::NPS][8], Wl[L::NPS][8];
-    Raw<L::NIT, BWD, BWD> raw;
-    float gcum = 0.f;
-    uint32_t par = 0;
+    Cols<D, false, false> raw;
+    Cols<D, false, false> nxt;                          // rows and gates of the next tile, a whole tile ahead of their use
     bool ok = true;
-    int cur = 0, iter = 0;
+    uint32_t it = 0;                                    // tiles worked so far: buffer it & 1, its barrier's phase (it >> 1) & 1
     const int total = g.B * g.H * pl.nseg;
 
     pdl_wait();
@@ -200,110 +142,233 @@ sweep_local(const SweepArgs a)
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
-        load_state<D, NT>(nullptr, sm, S);
-        if (BWD) load_state<D, NT>(nullptr, sm, Wl);
-        gcum = 0.f;
-        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, b, h, D, t0, tid);
+        float2 after = make_float2(0.f, 0.f), xafter = after;          // gates of the tiles behind (log2), the thread's channels
+        if (tid < 3 * T && t1 - 1 - (tid >> 6) >= t0) {
+            const int tile = t1 - 1 - (tid >> 6);
+            rowOff[(tile & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, tile, tid & 63);
+        }
         __syncthreads();
-        load_raw<D, NT, BWD, BWD>(raw, a.q, a.k, a.v, a.d_out, a.gate, rowOff + cur * T);
+        {
+            uint32_t off[9];
+            row_offsets<D>(rowOff + ((t1 - 1) & 3) * T, w, off);
+            load_gates(raw.g, a.gate, off);
+            load_rows(raw, a.q, a.k, a.v, a.d_out, off);
+            if (t1 - 2 >= t0) {
+                row_offsets<D>(rowOff + ((t1 - 2) & 3) * T, w, off);
+                load_gates(nxt.g, a.gate, off);
+            }
+            const int nrow = g.L - (t1 - 1) * T;
+            if (nrow < T) { clear_tail_rows(raw, w, nrow); clear_tail_gates(raw, w, nrow); }
+            group_prefix<D>(raw, raw.g, w, sTot + (it & 1) * 8 * D);
+        }
+        for (int tile = t1 - 1; tile >= t0; --tile, ++it) {
+            tc_fence_before_sync();
+            SYNC_OR_DIE();
+            if (tid == kIssuer && tile < t1 - 1) {                    // the tile before is built
+                char *tK = smem + ((it + 1) & 1) * SM::kBuf;
+                tc_fence_after_sync();
+                issue_state<D>(tmem, tK, tK + C::TILE_T, tile < t1 - 2);
+                mma_commit(&ctl->bar[(it + 1) & 1]);
+            }
+            if (tid < T && tile - 3 >= t0) rowOff[((tile - 3) & 3) * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 3, tid);
+            if (tile > t0) {
+                uint32_t ro[9];
+                row_offsets<D>(rowOff + ((tile - 1) & 3) * T, w, ro);
+                load_rows(nxt, a.q, a.k, a.v, a.d_out, ro);
+            }
+            const Tot tt = tile_totals<D>(sTot + (it & 1) * 8 * D, w);
+            if (it >= 2) ok = wait_all(&ctl->bar[it & 1], ((it - 2) >> 1) & 1, a.status, ok);       // the buffer is free again
+            const float2 off = add2(after, sub2(tt.all, tt.before)), xoff = add2(xafter, sub2(tt.xall, tt.xbefore));
+            char *tK = smem + (it & 1) * SM::kBuf;
+            build_suffix_rows<D>(raw, w, off, xoff, tK, tK + C::TILE_T);
+            fence_async_smem();
+            after = add2(after, tt.all);
+            xafter = add2(xafter, tt.xall);
+            if (tile > t0) {
+                group_prefix<D>(raw, nxt.g, w, sTot + ((it + 1) & 1) * 8 * D);       // only the last tile of a sequence has a tail
+                if (tile - 2 >= t0) {
+                    uint32_t ro[9];
+                    row_offsets<D>(rowOff + ((tile - 2) & 3) * T, w, ro);
+                    load_gates(nxt.g, a.gate, ro);
+                    prefetch_rows<D, false, false>(a.q, a.k, a.v, a.d_out, rowOff + ((tile - 2) & 3) * T, w);
+                }
+#pragma unroll
+                for (int j = 0; j < raw.N; ++j) {
+                    raw.k[j] = nxt.k[j];
+                    raw.v[j] = nxt.v[j];
+                }
+            }
+        }
+        tc_fence_before_sync();
+        SYNC_OR_DIE();
+        if (tid == kIssuer) {
+            char *tK = smem + ((it + 1) & 1) * SM::kBuf;
+            tc_fence_after_sync();
+            issue_state<D>(tmem, tK, tK + C::TILE_T, t1 - t0 > 1);
+            mma_commit(&ctl->bar[(it + 1) & 1]);
+        }
+        ok = wait_all(&ctl->bar[(it + 1) & 1], ((it - 1) >> 1) & 1, a.status, ok);
+        tc_fence_after_sync();
+        if (ok) acc_to_global<D>(tl, StateOf<D>(w), a.seg_state + (size_t)sid * D * D);
+        if (w.grp == 0) {
+            *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.c2) = after;
+            if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.xc2) = xafter;
+        }
+    }
+die:
+    cta_teardown(ctl, SM::tmem_cols);
+}
+
+// =================================================================================================
+// sweep_local_bwd: what the backward sweep needs of a segment from a zero state.  In scan order, the state
+// in registers: per (sub-)chunk the state entering it (scaled to its centre, fp16) and the decay since the
+// segment start.  GRAD: also the segment's contribution to the gradient of the state entering it, the sum of
+// 2^(gates since the segment start) q dO^T; those factors are below 1, so these products simply add up in
+// tensor memory and are read once per segment.  A backward pass over uncut sequences needs only the states.
+// Pipelined over the (sub-)chunks: the products of one run while the next one's operand tiles are built (two
+// buffers of tiles and accumulators), and are folded into the state one step later.  48 sequences of 4096
+// tokens, d = 64: 66.6 us before (both sums in registers, no pipelining), 52.3 us now; 16 of 16384, d = 72: 122 -> 116 us.
+// =================================================================================================
+template <int D, bool GRAD>
+struct LocalBwdSmem {
+    using C = Cfg<D>;
+    using L = Col<D>;
+    static constexpr int kBuf = (GRAD ? 4 : 2) * C::TILE_T;                   // (tQ) tK tV (tG)
+    static constexpr int kPad = L::X ? 16 * C::CHT - C::TILE_T : 0;           // the corner's operand reads past its tile
+    static constexpr size_t bytes = 2 * kBuf + kPad + 2 * 8 * D * 4 + 4 * T * 4 + sizeof(Ctl);
+    static constexpr uint32_t aW = 2 * L::ACCS;                               // accumulator columns: two of the state, one of the gradient
+    static constexpr uint32_t cols = (GRAD ? 3 : 2) * L::ACCS;
+    static constexpr uint32_t tmem_cols = cols <= 64 ? 64 : cols <= 128 ? 128 : 256;
+};
+
+template <int D, bool GRAD>
+__global__ void __launch_bounds__(Col<D>::NT, 2)
+sweep_local_bwd(const SweepArgs a)
+{
+    using C = Cfg<D>;
+    using L = Col<D>;
+    using SM = LocalBwdSmem<D, GRAD>;
+    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs
+    extern __shared__ __align__(128) char smem[];
+    float *sTot = reinterpret_cast<float *>(smem + 2 * SM::kBuf + SM::kPad);
+    int *rowOff = reinterpret_cast<int *>(sTot + 2 * 8 * D);          // ring of four tiles
+    Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 4 * T);
+
+    const int tid = threadIdx.x;
+    cta_setup(ctl, 2, SM::tmem_cols, smem, 2 * SM::kBuf + SM::kPad);
+    const Who<D> w;
+    const StateOf<D> sm(w);
+    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
+    const Geom &g = a.g;
+    const Plan &pl = a.plan;
+    float S[L::NPS][8];
+    Cols<D, GRAD, GRAD> raw;
+    bool ok = true;
+    uint32_t it = 0;                                    // (sub-)chunks worked so far: buffer it & 1, its barrier's phase (it >> 1) & 1
+    const int total = g.B * g.H * pl.nseg;
+
+    auto load_tile = [&](int tile) {
+        uint32_t off[9];
+        row_offsets<D>(rowOff + (tile & 3) * T, w, off);
+        load_gates(raw.g, a.gate, off);
+        load_rows(raw, a.q, a.k, a.v, a.d_out, off);
+    };
+    // S <- 2^2c S + 2^c (Kc^T V), the product of step i
+    Decay dec;
+    auto fold = [&](uint32_t i) {
+        ok = wait_all(&ctl->bar[i & 1], (i >> 1) & 1, a.status, ok);
+        tc_fence_after_sync();
+        if (ok) fold_state<D>(tl + (i & 1) * L::ACCS, sm, S, dec);
+        tc_fence_before_sync();
+    };
+
+    pdl_wait();
+    pdl_launch_dependents();
+    for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
+        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
+        const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
+        get_state<D>(nullptr, sm, S);
+        float2 gsum = make_float2(0.f, 0.f), gxsum = gsum;             // gates since the segment start (log2), the thread's channels
+        bool pending = false;
+        if (tid < 2 * T) rowOff[((t0 + (tid >> 6)) & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, t0 + (tid >> 6), tid & 63);
+        __syncthreads();
+        load_tile(t0);
+        {
+            const int nrow = g.L - t0 * T;
+            if (nrow < T) { clear_tail_rows(raw, w, nrow); clear_tail_gates(raw, w, nrow); }
+            group_prefix<D>(raw, raw.g, w, sTot + (t0 & 1) * 8 * D);
+        }
         for (int tile = t0; tile < t1; ++tile) {
-            const int nrow = min(T, g.L - tile * T), nxt = (cur + 1) & 3;
-            if (tid < T) {
-                rowOff[nxt * T + tid] = tile + 1 < t1 ? tile_row_offset(g, b, h, D, tile + 1, tid) : -1;
-                // this kernel's tiles are short: the register prefetch alone does not cover the memory latency
-                if (tile + 2 < t1) prefetch_row<D, BWD, BWD>(a.q, a.k, a.v, a.d_out, a.gate, tile_row_offset(g, b, h, D, tile + 2, tid));
+            const int nrow = min(T, g.L - tile * T);
+            const bool more = tile + 1 < t1;
+            float *tot = sTot + (tile & 1) * 8 * D;
+            SYNC_OR_DIE();                                             // group totals are there
+            if (tid < T && tile + 2 < t1) rowOff[((tile + 2) & 3) * T + tid] = tile_row_offset(g, pl, b, h, D, tile + 2, tid);
+            const Tot whole = tile_totals<D>(tot, w);
+            Tot tt = whole;
+            int s = T;
+            if (pl.sub_max < T || beyond<D>(tt)) {
+                s = choose_window<D>(tot, w, min(pl.sub_max, T / 2), a.status);
+                const int w0 = 8 * w.grp / s * (s / 8);
+                tt = window_totals<D>(tot, w, w0, w0 + s / 8);
             }
-            write_gates<D, NT, BWD, BWD>(raw, table, rowOff + cur * T);
-            __syncthreads();
-            // the vectors of an undivided tile are written inside the prefix pass (no barrier of their own)
-            const bool whole_ok = pl.sub_max == T;
-            const Vec v0 = vec_of<D>(vecb, iter & 1);
-            float tot_c = 0.f;
-            const bool need = gate_prefix<D, NT>(table, sTot, tot_c, [&](int c, float t) {
-                if (whole_ok) {
-                    const float cv = 0.5f * t;
-                    v0.off[c] = cv;
-                    v0.ec[c] = ex2(cv);
-                    v0.e2c[c] = ex2(t);
-                    if (BWD) v0.aux[c] = ex2(gcum + cv);
-                }
-            });
-            const bool whole = whole_ok && !need;
-            int s = pl.sub_max;
-            if (need || s < T) {
-                bool bad;
-                s = choose_sub<D>(table, need ? min(s, T / 2) : s, &bad);
-                if (bad && tid == 0) atomicOr(a.status, kStatusRange);
-            }
+            const float2 off = centred(tt.before, tt.all), xoff = centred(tt.xbefore, tt.xall);
             const int nsub = (nrow + s - 1) / s;
-            for (int u = 0; u < nsub; ++u, ++iter) {
-                const int lo = u * s, hi = min(lo + s, T);
-                const Vec vc = vec_of<D>(vecb, iter & 1);
-                if (tid < D) {
-                    float t = tot_c;
-                    if (!whole) {
-                        const float base = lo ? table[(lo - 1) * C::LAMP + tid] : 0.f;
-                        t = table[(hi - 1) * C::LAMP + tid] - base;
-                        const float cv = 0.5f * t;
-                        vc.off[tid] = base + cv;
-                        vc.ec[tid] = ex2(cv);
-                        vc.e2c[tid] = ex2(t);
-                        if (BWD) vc.aux[tid] = ex2(gcum + cv);  // decay from the segment start to the sub-chunk's centre
-                    }
-                    if (SLOTS) {
-                        const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
-                        a.slot_g[slot * D + tid] = gcum;
-                    }
-                    gcum += t;
+            for (int u = 0; u < nsub; ++u, ++it) {
+                const int lo = u * s, hi = lo + s;
+                const bool last = u == nsub - 1, on = 8 * w.grp >= lo && 8 * w.grp < hi;
+                char *buf = smem + (it & 1) * SM::kBuf;
+                char *tQ = buf, *tK = GRAD ? tQ + C::TILE_T : buf, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T;
+                build_kv_rows<D>(raw, w, off, xoff, tK, tV, on);
+                if (GRAD) build_qd_rows<D>(raw, w, add2(gsum, whole.before), add2(gxsum, whole.xbefore), tQ, tG, on);
+                Tot tu = whole;
+                float2 gs = gsum, gxs = gxsum;                         // decay before the sub-chunk
+                if (s < T) {
+                    tu = window_totals<D>(tot, w, 0, lo / 8);
+                    gs = add2(gs, tu.all);
+                    gxs = add2(gxs, tu.xall);
+                    tu = window_totals<D>(tot, w, lo / 8, hi / 8);
                 }
-                if (!whole) __syncthreads();
-                {
-                    build_tiles<D, NT, BWD, BWD>(raw, tQ, tK, tV, tG, table, vc.off, rowOff + cur * T, lo, min(hi, nrow));
-                    if (SLOTS) {
-                        const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
-                        write_state_slot<D, NT>(a.slot_s + slot * (D * D), sm, S, vc.ec);
-                    }
-                    fence_async_smem();
+                const Decay now = decay_of<D>(sm, tu.all, tu.xall);
+                const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
+                if (w.grp == 0) {
+                    *reinterpret_cast<float2 *>(a.slot_g + slot * D + w.c2) = gs;
+                    if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.slot_g + slot * D + w.xc2) = gxs;
                 }
+                if (last && more) load_tile(tile + 1);
+                fence_async_smem();
                 tc_fence_before_sync();
-                SYNC_OR_DIE();
+                __syncthreads();
                 if (tid == kIssuer) {
                     tc_fence_after_sync();
-                    issue_state_product<D>(tmem + aU, tK, tV);                   // Kc^T V
-                    if (BWD) issue_state_product<D>(tmem + aW, tQ, tG);         // Qc^T dO
-                    mma_commit(&ctl->bar[0]);
+                    issue_state<D>(tmem + (it & 1) * L::ACCS, tK, tV);                             // Kc^T V
+                    if (GRAD) issue_state<D>(tmem + SM::aW, tQ, tG, pending);                      // + (q decayed)^T dO
+                    mma_commit(&ctl->bar[it & 1]);
                 }
-                {
-                    if (u == nsub - 1 && tile + 1 < t1)
-                        load_raw<D, NT, BWD, BWD>(raw, a.q, a.k, a.v, a.d_out, a.gate, rowOff + nxt * T);
-                    ok = wait_all(&ctl->bar[0], par, a.status);
-                    if (ok) {
-                        tc_fence_after_sync();
-                        update_state<D, NT>(lane_base, tmem + aU, sm, S, vc.e2c, vc.ec);
-                        if (BWD) {
-                            // W_segment += (decay since the segment start) * exp(c) * (Qc^T dO)
-                            const float fs = sm.valid ? vc.aux[sm.c] : 0.f;
-#pragma unroll
-                            for (int i = 0; i < L::NPS; ++i)
-                                if (sm.has(i)) {
-                                    float w[8];
-                                    tmem_ld8(lane_base + tmem + aW + sm.tcol(i), w);
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e) Wl[i][e] += fs * w[e];
-                                }
-                        }
-                    }
-                    tc_fence_before_sync();
-                }
-                par ^= 1;
+                // the register prefetch alone does not cover the memory latency of tiles this short
+                if (last && tile + 2 < t1) prefetch_rows<D, GRAD, GRAD>(a.q, a.k, a.v, a.d_out, rowOff + ((tile + 2) & 3) * T, w);
+                if (last && tile + 2 < t1) prefetch_gates<D>(a.gate, rowOff + ((tile + 2) & 3) * T, w);
+                if (pending) fold(it - 1);
+                dec = now;
+                put_state<D, D * 16>(reinterpret_cast<char *>(a.slot_s + slot * (D * D)), sm, S, dec);
+                pending = true;
             }
-            cur = nxt;
+            gsum = add2(gsum, whole.all);
+            gxsum = add2(gxsum, whole.xall);
+            if (more) {                                                // the next tile's gate sums while the products run
+                const int nr = g.L - (tile + 1) * T;
+                if (nr < T) { clear_tail_rows(raw, w, nr); clear_tail_gates(raw, w, nr); }
+                group_prefix<D>(raw, raw.g, w, sTot + ((tile + 1) & 1) * 8 * D);
+            }
         }
-        {
-            store_state<D, NT>(a.seg_state + (size_t)sid * D * D, sm, S);
-            if (BWD) store_state<D, NT>(a.seg_dstate + (size_t)sid * D * D, sm, Wl);
-            if (tid < D) a.seg_gamma[(size_t)sid * D + tid] = gcum;
+        fold(it - 1);
+        save_state<D>(a.seg_state + (size_t)sid * D * D, sm, S);
+        if (GRAD && ok) acc_to_global<D>(tl + SM::aW, sm, a.seg_dstate + (size_t)sid * D * D);
+        if (w.grp == 0) {
+            *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.c2) = gsum;
+            if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.xc2) = gxsum;
         }
+        tc_fence_before_sync();
     }
 die:
     cta_teardown(ctl, SM::tmem_cols);
@@ -439,183 +504,172 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
 
 // =================================================================================================
 // sweep_fwd: a segment from its entry state; writes out.
+// Bound by the latency of its phases (three barriers and two waits for products per tile; IPC 1.5, two CTAs per
+// SM).  16 sequences of 16384 tokens, d = 72: 114 us with the row-chunk work split, 84 us now; 768 of 256, d = 64
+// (uncut): 60 -> 52 us.  Three CTAs per SM on 80 registers: 72 us against 59 us on 48 sequences of 4096 tokens, d = 64.
 // =================================================================================================
-template <int D, int NT>
+template <int D>
 struct FwdSmem {
     using C = Cfg<D>;
-    using L = Lay<D, NT>;
+    using L = Col<D>;
     static constexpr int kTiles = 3 * C::TILE_T + C::TILE_S + C::TILE_P;      // tQ tK tV tS tP
-    static constexpr int kFloats = T * C::LAMP + L::NSEG * D + 8 * D;
-    static constexpr size_t bytes = kTiles + kFloats * 4 + 4 * T * 4 + sizeof(Ctl);
-    static constexpr uint32_t tmem_cols = C::BIGM ? 256 : 128;
+    static constexpr size_t bytes = kTiles + 8 * D * 4 + 2 * T * 4 + sizeof(Ctl);
+    static constexpr uint32_t aP = 0, aO = 32, aU = aO + L::HW;               // accumulator columns
+    static constexpr uint32_t tmem_cols = 128;
+    static_assert(aU + L::ACCS <= tmem_cols, "tensor memory");
 };
 
-template <int D, int NT, typename TO, int OCC>
-__global__ void __launch_bounds__(NT, OCC)
+template <int D, typename TO>
+__global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_fwd(const SweepArgs a)
 {
     using C = Cfg<D>;
-    using L = Lay<D, NT>;
-    using SM = FwdSmem<D, NT>;
+    using L = Col<D>;
+    using SM = FwdSmem<D>;
+    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs
     extern __shared__ __align__(128) char smem[];
     char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tS = tV + C::TILE_T, *tP = tS + C::TILE_S;
-    float *table = reinterpret_cast<float *>(smem + SM::kTiles);
-    float *sTot = table + T * C::LAMP, *vecb = sTot + L::NSEG * D;
-    int *rowOff = reinterpret_cast<int *>(vecb + 8 * D);
-    Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 4 * T);
-    // the state product is issued after the scores have been read and reuses their columns
-    constexpr uint32_t aP = 0, aO = C::BIGM ? C::NACC : 64, aU = aP;
-    static_assert(aO + C::NACC <= SM::tmem_cols, "tensor memory");
+    float *sTot = reinterpret_cast<float *>(smem + SM::kTiles);
+    int *rowOff = reinterpret_cast<int *>(sTot + 8 * D);
+    Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 2 * T);
 
-    const int tid = threadIdx.x, lane = tid & 31, q4 = (tid >> 5) & 3, cg = tid >> 7, hf = lane >> 4;
-    constexpr int kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs (warps 0 and 1 carry the per-channel work)
-    const int r16 = 16 * q4 + (lane & 15);
+    const int tid = threadIdx.x;
     cta_setup(ctl, 1, SM::tmem_cols, smem, SM::kTiles);
-    const uint32_t tmem = ctl->tmem_base, lane_base = (uint32_t)(32 * q4) << 16;
+    const Who<D> w;
+    const StateOf<D> sm(w);
+    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     const Geom &g = a.g;
     const Plan &pl = a.plan;
-    const StateMap<D, NT> sm;
     float S[L::NPS][8];
-    Raw<L::NIT, true, false> raw;
-    uint32_t par = 0;
+    Cols<D, true, false> raw;
     bool ok = true;
-    int cur = 0, iter = 0;
+    int cur = 0;
     const int total = g.B * g.H * pl.nseg;
     TO *out = reinterpret_cast<TO *>(a.out);
 
+    auto load_tile = [&](int slot) {
+        uint32_t off[9];
+        row_offsets<D>(rowOff + slot * T, w, off);
+        load_gates(raw.g, a.gate, off);
+        load_rows(raw, a.q, a.k, a.v, nullptr, off);
+    };
     // The first tile's rows are inputs of the call: their loads need not wait for the scan kernel (whose own
     // wait covered whatever produced them).  Uncut sequences have no kernel in front that has waited: wait first.
+    auto prime = [&](int sid) {
+        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
+        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, pl, b, h, D, sg * pl.G, tid);
+        __syncthreads();
+        load_tile(cur);
+    };
     if (pl.nseg == 1) pdl_wait();
-    {
-        const int sid = blockIdx.x;
-        if (sid < total) {
-            const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
-            if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, b, h, D, sg * pl.G, tid);
-            __syncthreads();
-            load_raw<D, NT, true, false>(raw, a.q, a.k, a.v, nullptr, a.gate, rowOff + cur * T);
-        }
-    }
+    if ((int)blockIdx.x < total) prime(blockIdx.x);
     pdl_wait();
     pdl_launch_dependents();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
-        if (pl.nseg == 1) load_state<D, NT>(a.s_in ? a.s_in + (size_t)sid * D * D : nullptr, sm, S);      // uncut: no scan ran
-        else load_state<D, NT>(a.seg_state + (size_t)sid * D * D, sm, S);
-        if (sid != (int)blockIdx.x) {
-            if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, b, h, D, t0, tid);
-            __syncthreads();
-            load_raw<D, NT, true, false>(raw, a.q, a.k, a.v, nullptr, a.gate, rowOff + cur * T);
+        if (pl.nseg == 1) get_state<D>(a.s_in ? a.s_in + (size_t)sid * D * D : nullptr, sm, S);      // uncut: no scan ran
+        else get_state<D>(a.seg_state + (size_t)sid * D * D, sm, S);
+        if (sid != (int)blockIdx.x) prime(sid);
+        {
+            const int nrow = g.L - t0 * T;
+            if (nrow < T) { clear_tail_rows(raw, w, nrow); clear_tail_gates(raw, w, nrow); }
+            group_prefix<D>(raw, raw.g, w, sTot);
         }
         for (int tile = t0; tile < t1; ++tile) {
-            const int nrow = min(T, g.L - tile * T), nxt = (cur + 1) & 3;
-            if (tid < T) rowOff[nxt * T + tid] = tile + 1 < t1 ? tile_row_offset(g, b, h, D, tile + 1, tid) : -1;
-            write_gates<D, NT, true, false>(raw, table, rowOff + cur * T);
-            __syncthreads();
-            const int my_off = rowOff[cur * T + r16];
-            // the vectors of an undivided tile are written inside the prefix pass (no barrier of their own)
-            const bool whole_ok = pl.sub_max == T;
-            const Vec v0 = vec_of<D>(vecb, iter & 1);
-            float tot_c = 0.f;
-            const bool need = gate_prefix<D, NT>(table, sTot, tot_c, [&](int c, float t) {
-                if (whole_ok) {
-                    const float cv = 0.5f * t;
-                    v0.off[c] = cv;
-                    v0.ec[c] = ex2(cv);
-                    v0.e2c[c] = ex2(t);
-                }
-            });
-            const bool whole = whole_ok && !need;
-            int s = pl.sub_max;
-            if (need || s < T) {
-                bool bad;
-                s = choose_sub<D>(table, need ? min(s, T / 2) : s, &bad);
-                if (bad && tid == 0) atomicOr(a.status, kStatusRange);
+            const int nrow = min(T, g.L - tile * T), nxt = cur ^ 1;
+            const bool more = tile + 1 < t1;
+            tc_fence_before_sync();
+            SYNC_OR_DIE();                                       // group totals are there, the previous tile's products are done
+            const int my_off = rowOff[cur * T + w.r16];
+            if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile + 1, tid);
+            // Where some channel's gates sum to too much for one centring (or shorter chunks were asked for) the tile
+            // is worked in sub-chunks: the other rows of the operand tiles are zero, each has its own centring.
+            const Tot whole = tile_totals<D>(sTot, w);
+            Tot tt = whole;
+            int s = T;
+            if (pl.sub_max < T || beyond<D>(tt)) {
+                s = choose_window<D>(sTot, w, min(pl.sub_max, T / 2), a.status);
+                const int w0 = 8 * w.grp / s * (s / 8);
+                tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
             }
+            const float2 off = centred(tt.before, tt.all), xoff = centred(tt.xbefore, tt.xall);
             const int nsub = (nrow + s - 1) / s;
-            for (int u = 0; u < nsub; ++u, ++iter) {
-                const int lo = u * s, hi = min(lo + s, T);
-                const Vec vc = vec_of<D>(vecb, iter & 1);
-                if (!whole) {
-                    if (tid < D) {
-                        const float base = lo ? table[(lo - 1) * C::LAMP + tid] : 0.f;
-                        const float t = table[(hi - 1) * C::LAMP + tid] - base, cv = 0.5f * t;
-                        vc.off[tid] = base + cv;
-                        vc.ec[tid] = ex2(cv);
-                        vc.e2c[tid] = ex2(t);
-                    }
-                    __syncthreads();
-                }
-                {
-                    build_tiles<D, NT, true, false>(raw, tQ, tK, tV, nullptr, table, vc.off, rowOff + cur * T, lo, min(hi, nrow));
-                    write_state_tile<D, NT>(tS, sm, S, vc.ec);                       // Sc = diag(2^c) S
-                    fence_async_smem();
-                }
+            for (int u = 0; u < nsub; ++u) {
+                const int lo = u * s, hi = lo + s;
+                const bool last = u == nsub - 1;
+                build_rows<D>(raw, w, off, xoff, tQ, tK, tV, nullptr, 8 * w.grp >= lo && 8 * w.grp < hi);
+                Tot tu = whole;
+                if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
+                const Decay dec = decay_of<D>(sm, tu.all, tu.xall);
+                put_state<D, C::CHS>(tS, sm, S, dec);            // Sc = diag(2^c) S
+                fence_async_smem();
                 tc_fence_before_sync();
-                SYNC_OR_DIE();
+                __syncthreads();
                 if (tid == kIssuer) {
                     tc_fence_after_sync();
-                    issue<64, 64, false, false, C::KS, C::CHT, C::CHT>(tmem + aP, smem_u32(tQ), smem_u32(tK), false);   // Qc Kc^T
+                    issue_scores<D>(tmem + SM::aP, tQ, tK);                                       // Qc Kc^T
                     mma_commit(&ctl->bar[0]);
-                    issue<64, D, false, true, C::KS, C::CHT, C::CHS>(tmem + aO, smem_u32(tQ), smem_u32(tS), false);     // Qc Sc
+                    issue_split<D, C::KS, C::CHS>(tmem + SM::aO, tQ, tS, false);                  // Qc Sc
+                    issue_state<D>(tmem + SM::aU, tK, tV);                                        // Kc^T V
                 }
-                {
-                    if (u == nsub - 1 && tile + 1 < t1)
-                        load_raw<D, NT, true, false>(raw, a.q, a.k, a.v, nullptr, a.gate, rowOff + nxt * T);
-                    ok = wait_all(&ctl->bar[0], 0, a.status);          // completes twice per iteration: parities 0, 1
-                    if (ok) {
-                        tc_fence_after_sync();
-                        // scores of row r16 (lanes 0-15 hold accumulator rows): keep s <= t, the diagonal has weight 1.
-                        // Column chunks entirely above the diagonal for all 16 rows of the warp are never written (the
-                        // tile starts out zero), chunks entirely below it need no selects.
+                if (last && more) load_tile(nxt);
+                ok = wait_all(&ctl->bar[0], 0, a.status, ok);          // completes twice per iteration: parities 0, 1
+                tc_fence_after_sync();
+                // Scores of row r16: lanes 0-15 hold the even 8-token chunks, lanes 16-31 the odd ones.  Keep s <= t, the
+                // diagonal has weight 1.  Chunks above the diagonal of all 16 rows of the warp are never written (the tile
+                // starts out zero), pairs below it need no selects.
 #pragma unroll
-                        for (int i = 0; i < L::NPT; ++i) {
-                            const int sc = cg + L::NCG * i;
-                            if (sc < T / 8 && 8 * sc <= 16 * q4 + 15) {           // uniform over the warp
-                                float p[8];
-                                tmem_ld8(lane_base + tmem + aP + 8 * sc, p);
-                                if (8 * sc + 7 > 16 * q4) {
+                for (int i = 0; i < 2; ++i) {
+                    const int pr = w.cg + 2 * i;
+                    if (ok && pr <= w.q4) {                // uniform over the warp
+                        float p[8];
+                        tmem_ld8(tl + SM::aP + 8 * pr, p);
+                        const int sc = 2 * pr + w.hf;
+                        if (pr == w.q4) {
 #pragma unroll
-                                    for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= r16) ? p[e] : 0.f;
-                                }
-                                if (hf == 0) *reinterpret_cast<uint4 *>(tP + sc * C::CHT + r16 * 16) = pack_h8(p);
-                            }
+                            for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= w.r16) ? p[e] : 0.f;
                         }
+                        *reinterpret_cast<uint4 *>(tP + sc * C::CHT + w.r16 * 16) = pack_h8(p);
                     }
-                    fence_async_smem();
                 }
+                fence_async_smem();
                 tc_fence_before_sync();
-                SYNC_OR_DIE();
+                __syncthreads();
                 if (tid == kIssuer) {
                     tc_fence_after_sync();
-                    issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + aO, smem_u32(tP), smem_u32(tV), true);     // + P V
-                    issue_state_product<D>(tmem + aU, tK, tV);                                                         // Kc^T V
+                    issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);                  // + P V
                     mma_commit(&ctl->bar[0]);
                 }
-                {
-                    ok = wait_all(&ctl->bar[0], 1, a.status);
-                    if (ok) {
-                        tc_fence_after_sync();
-                        update_state<D, NT>(lane_base, tmem + aU, sm, S, vc.e2c, vc.ec);
-                        const bool inrow = hf == 0 && r16 >= lo && r16 < hi && my_off >= 0;
-                        const size_t ro = (size_t)(my_off < 0 ? 0 : my_off);
+                if (last && more) {                                // the next tile's gate sums while the products run
+                    const int nr = g.L - (tile + 1) * T;
+                    if (nr < T) { clear_tail_rows(raw, w, nr); clear_tail_gates(raw, w, nr); }
+                    group_prefix<D>(raw, raw.g, w, sTot);
+                }
+                ok = wait_all(&ctl->bar[0], 1, a.status, ok);
+                tc_fence_after_sync();
+                if (ok) {
+                    const bool inrow = w.r16 >= lo && w.r16 < min(hi, nrow);
 #pragma unroll
-                        for (int i = 0; i < L::NPC; ++i) {
-                            const int jc = cg + L::NCG * i;
-                            if (jc < C::NCH) {
-                                float o[8];
-                                tmem_ld8(lane_base + tmem + aO + 8 * jc, o);
-                                if (inrow) store_out8(out + ro + 8 * jc, o, a.accumulate != 0);
-                            }
+                    for (int i = 0; i < L::NPO; ++i) {
+                        const int jc = w.cg + 2 * i;
+                        if (jc < L::NV0) {                        // uniform over the warp
+                            float o[8];
+                            tmem_ld8(tl + SM::aO + 8 * jc, o);
+                            if (inrow && jc < (w.hf ? L::NV1 : L::NV0))
+                                store_out8(out + (uint32_t)my_off + 8 * ((w.hf ? L::NV0 : 0) + jc), o, a.accumulate != 0);
                         }
                     }
+                    fold_state<D>(tl + SM::aU, sm, S, dec);
+                }
+                if (!last) {                              // the operand tiles and the accumulators are free again
                     tc_fence_before_sync();
+                    SYNC_OR_DIE();
                 }
-                par ^= 1;
             }
             cur = nxt;
         }
-        if (pl.nseg == 1 && a.s_out) store_state<D, NT>(a.s_out + (size_t)sid * D * D, sm, S);
+        if (pl.nseg == 1 && a.s_out) save_state<D>(a.s_out + (size_t)sid * D * D, sm, S);
     }
 die:
     cta_teardown(ctl, SM::tmem_cols);
@@ -623,60 +677,84 @@ die:
 
 // =================================================================================================
 // sweep_bwd: a segment in reverse scan order with the state gradient on chip.
+// After the second group of products the dq and dk accumulators go through shared memory (over the
+// operand tiles that are spent by then) to the column threads, which still hold the decay exponents of
+// their rows: they scale and store dq and dk, form q dq - k dk and sum it down their rows.
+// Bound by latency like the forward sweep.  48 sequences of 4096 tokens, d = 64: 140 us with the row-chunk work
+// split, 106 us now; 16 of 16384, d = 72: 252 -> 186 us (217 us before the L2 was asked for the next tile's rows early).
 // =================================================================================================
-template <int D, int NT>
+template <int D>
 struct BwdSmem {
     using C = Cfg<D>;
-    using L = Lay<D, NT>;
-    static constexpr int kTiles = 4 * C::TILE_T + 3 * C::TILE_S + 2 * C::TILE_P;      // tQ tK tV tG | tS tI tD | tP tdP
-    static constexpr int kFloats = T * C::LAMP + L::NSEG * D + 8 * D + 2 * D;
-    static constexpr size_t bytes = kTiles + kFloats * 4 + 4 * T * 4 + sizeof(Ctl);
+    using L = Col<D>;
+    static constexpr int LDP = D + 4;                                          // floats per row of an accumulator buffer
+    static constexpr int kBuf = T * LDP * 4;
+    static constexpr int kOver = 2 * C::TILE_T + C::TILE_S;                    // tV tG tD: spent when the accumulators are complete
+    static constexpr int kRegion = 2 * kBuf > kOver ? 2 * kBuf : kOver;
+    static constexpr int kTiles = 2 * C::TILE_T + kRegion + 2 * C::TILE_P + 2 * C::TILE_S;      // tQ tK | tV tG tD .. | tP tdP | tS tI
+    static constexpr size_t bytes = kTiles + (2 * 8 * D + D) * 4 + 2 * T * 4 + sizeof(Ctl);
+    static constexpr uint32_t aP = 0, aQK = 64, aV = aQK + D, aW = aV + D;     // accumulator columns
     static constexpr uint32_t tmem_cols = 256;
+    static_assert(aW + L::ACCS <= tmem_cols, "tensor memory");
 };
 
-template <int D, int NT, typename TO, int OCC>
-__global__ void __launch_bounds__(NT, OCC)
+__device__ __forceinline__ void store_pair(float *p, float x, float y, bool add)
+{
+    if (add) {
+        const float2 o = *reinterpret_cast<const float2 *>(p);
+        x += o.x;
+        y += o.y;
+    }
+    *reinterpret_cast<float2 *>(p) = make_float2(x, y);
+}
+__device__ __forceinline__ void store_pair(bf16 *p, float x, float y, bool) { *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(x, y); }
+
+template <int D, typename TO>
+__global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_bwd(const SweepArgs a)
 {
     using C = Cfg<D>;
-    using L = Lay<D, NT>;
-    using SM = BwdSmem<D, NT>;
+    using L = Col<D>;
+    using SM = BwdSmem<D>;
+    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs and the bulk copies
     extern __shared__ __align__(128) char smem[];
-    char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T;
-    char *tS = tG + C::TILE_T, *tI = tS + C::TILE_S, *tD = tI + C::TILE_S;
-    char *tP = tD + C::TILE_S, *tdP = tP + C::TILE_P;
-    float *table = reinterpret_cast<float *>(smem + SM::kTiles);
-    float *sTot = table + T * C::LAMP, *vecb = sTot + L::NSEG * D, *sCarry = vecb + 8 * D;
-    int *rowOff = reinterpret_cast<int *>(sCarry + 2 * D);
-    Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 4 * T);
-    constexpr uint32_t W0 = C::BIGM ? C::NACC : 64;
-    constexpr uint32_t aP = 0, aQK = W0, aV = W0 + C::NACC, kHi = 16u << 16;
-    static_assert(aV + C::NACC <= SM::tmem_cols, "tensor memory");
+    char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T, *tD = tG + C::TILE_T;
+    char *tP = tV + SM::kRegion, *tdP = tP + C::TILE_P, *tS = tdP + C::TILE_P, *tI = tS + C::TILE_S;
+    float *bufQ = reinterpret_cast<float *>(tV), *bufK = bufQ + T * SM::LDP;
+    float *sTot = reinterpret_cast<float *>(smem + SM::kTiles), *sX = sTot + 8 * D, *sAux = sX + 8 * D;
+    int *rowOff = reinterpret_cast<int *>(sAux + D);
+    Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 2 * T);
 
-    const int tid = threadIdx.x, lane = tid & 31, q4 = (tid >> 5) & 3, cg = tid >> 7, hf = lane >> 4;
-    constexpr int kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs (warps 0 and 1 carry the per-channel work)
-    const int r16 = 16 * q4 + (lane & 15);
+    const int tid = threadIdx.x;
     cta_setup(ctl, 2, SM::tmem_cols, smem, SM::kTiles);
-    const uint32_t tmem = ctl->tmem_base, lane_base = (uint32_t)(32 * q4) << 16;
+    const Who<D> w;
+    const StateOf<D> sm(w);
+    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     uint64_t *barG1 = &ctl->bar[0], *barS = &ctl->bar[1];
     const Geom &g = a.g;
     const Plan &pl = a.plan;
-    const StateMap<D, NT> sm;
     float Dst[L::NPS][8];
-    Raw<L::NIT, true, true> raw;
+    Cols<D, true, true> raw;
     uint32_t par = 0;
     bool ok = true;
-    int cur = 0, iter = 0, cpar = 0;
+    int cur = 0;
     const int total = g.B * g.H * pl.nseg;
     TO *dq = reinterpret_cast<TO *>(a.dq), *dk = reinterpret_cast<TO *>(a.dk), *dv = reinterpret_cast<TO *>(a.dv);
+    const bool acc_out = a.accumulate != 0, entry = a.scanned != 0;
 
+    auto load_all = [&](int slot) {
+        uint32_t off[9];
+        row_offsets<D>(rowOff + slot * T, w, off);
+        load_gates(raw.g, a.gate, off);
+        load_rows(raw, a.q, a.k, a.v, a.d_out, off);
+    };
     // the first tile's rows are inputs of the call: their loads need not wait for the scan kernel
     auto prime = [&](int sid) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t1 = min(sg * pl.G + pl.G, pl.ntile);
-        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, b, h, D, t1 - 1, tid);
+        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, pl, b, h, D, t1 - 1, tid);
         __syncthreads();
-        load_raw<D, NT, true, true>(raw, a.q, a.k, a.v, a.d_out, a.gate, rowOff + cur * T);
+        load_all(cur);
     };
     if ((int)blockIdx.x < total) prime(blockIdx.x);
     pdl_wait();
@@ -684,8 +762,13 @@ sweep_bwd(const SweepArgs a)
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
-        load_state<D, NT>(a.seg_dstate + (size_t)sid * D * D, sm, Dst);
-        if (tid < D) sCarry[cpar * D + tid] = a.seg_carry[(size_t)sid * D + tid];
+        // without a scan (uncut sequences, no state arguments) the entry state, the incoming state gradient and the carry are zero
+        get_state<D>(entry ? a.seg_dstate + (size_t)sid * D * D : nullptr, sm, Dst);
+        float2 carry = make_float2(0.f, 0.f), xcarry = carry;            // gate gradient carried in from later tiles
+        if (entry) {
+            carry = *reinterpret_cast<const float2 *>(a.seg_carry + (size_t)sid * D + w.c2);
+            if (L::X) xcarry = *reinterpret_cast<const float2 *>(a.seg_carry + (size_t)sid * D + w.xc2);
+        }
         if (sid != (int)blockIdx.x) prime(sid);
         if (tid == kIssuer) {
             // the zero-start state of the sub-chunk worked first (always slot 0 of its tile) and, once per
@@ -693,207 +776,207 @@ sweep_bwd(const SweepArgs a)
             // products of the one before are done
             const char *src = reinterpret_cast<const char *>(a.slot_s + ((size_t)bh * pl.ntile + (t1 - 1)) * (D * D));
             const char *seg16 = reinterpret_cast<const char *>(a.seg_state16 + (size_t)sid * D * D);
-            mbar_arrive_expect_tx(barS, 2u * C::NCH * D * 16u);
+            mbar_arrive_expect_tx(barS, (entry ? 2u : 1u) * C::NCH * D * 16u);
             for (int j = 0; j < C::NCH; ++j) {
                 bulk_g2s(tS + j * C::CHS, src + j * D * 16, D * 16, barS);
-                bulk_g2s(tI + j * C::CHS, seg16 + j * D * 16, D * 16, barS);
+                if (entry) bulk_g2s(tI + j * C::CHS, seg16 + j * D * 16, D * 16, barS);
             }
         }
+        {
+            const int nrow = g.L - (t1 - 1) * T;
+            if (nrow < T) { clear_tail_rows(raw, w, nrow); clear_tail_gates(raw, w, nrow); }
+            group_prefix<D>(raw, raw.g, w, sTot);
+        }
         for (int tile = t1 - 1; tile >= t0; --tile) {
-            const int nrow = min(T, g.L - tile * T), nxt = (cur + 1) & 3;
-            if (tid < T) rowOff[nxt * T + tid] = tile > t0 ? tile_row_offset(g, b, h, D, tile - 1, tid) : -1;
-            write_gates<D, NT, true, true>(raw, table, rowOff + cur * T);
-            __syncthreads();
-            const int my_off = rowOff[cur * T + r16];
-            // decay since the segment start of the sub-chunk worked first (always slot 0): fetched ahead of its use
-            const float g_first = tid < D ? a.slot_g[((size_t)bh * pl.ntile + tile) * D + tid] : 0.f;
-            // the vectors of an undivided tile are written inside the prefix pass (no barrier of their own)
-            const bool whole_ok = pl.sub_max == T;
-            const Vec v0 = vec_of<D>(vecb, iter & 1);
-            float tot_c = 0.f;
-            const bool need = gate_prefix<D, NT>(table, sTot, tot_c, [&](int c, float t) {
-                if (whole_ok) {
-                    const float cv = 0.5f * t;
-                    v0.off[c] = cv;
-                    v0.ec[c] = ex2(cv);
-                    v0.e2c[c] = ex2(t);
-                    v0.aux[c] = ex2(cv + g_first);
-                }
-            });
-            const bool whole = whole_ok && !need;
-            int s = pl.sub_max;
-            if (need || s < T) {
-                bool bad;
-                s = choose_sub<D>(table, need ? min(s, T / 2) : s, &bad);
-                if (bad && tid == 0) atomicOr(a.status, kStatusRange);
+            const int nrow = min(T, g.L - tile * T), nxt = cur ^ 1;
+            const bool more = tile > t0;
+            SYNC_OR_DIE();                                       // group totals are there, the accumulator buffers are free
+            const int my_off = rowOff[cur * T + w.r16];
+            if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 1, tid);
+            const Tot whole = tile_totals<D>(sTot, w);
+            Tot tt = whole;
+            int s = T;
+            if (pl.sub_max < T || beyond<D>(tt)) {
+                s = choose_window<D>(sTot, w, min(pl.sub_max, T / 2), a.status);
+                const int w0 = 8 * w.grp / s * (s / 8);
+                tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
             }
+            const float2 off = centred(tt.before, tt.all), xoff = centred(tt.xbefore, tt.xall);
             const int nsub = (nrow + s - 1) / s;
-            for (int u = nsub - 1; u >= 0; --u, ++iter) {
-                const int lo = u * s, hi = min(lo + s, T), hiv = min(hi, nrow);
+            float2 tot = make_float2(0.f, 0.f), xtot = tot;      // sums of q dq - k dk over the group
+            for (int u = nsub - 1; u >= 0; --u) {
+                const int lo = u * s, hi = lo + s;
+                const bool mine = 8 * w.grp >= lo && 8 * w.grp < hi;
                 const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
-                const Vec vc = vec_of<D>(vecb, iter & 1);
-                if (!whole) {
-                    if (tid < D) {
-                        const float base = lo ? table[(lo - 1) * C::LAMP + tid] : 0.f;
-                        const float t = table[(hi - 1) * C::LAMP + tid] - base, cv = 0.5f * t;
-                        vc.off[tid] = base + cv;
-                        vc.ec[tid] = ex2(cv);
-                        vc.e2c[tid] = ex2(t);
-                        vc.aux[tid] = ex2(cv + (u == nsub - 1 ? g_first : a.slot_g[slot * D + tid]));   // exp(c) * decay since the segment start
-                    }
-                    __syncthreads();
-                }
-                {
-                    build_tiles<D, NT, true, true>(raw, tQ, tK, tV, tG, table, vc.off, rowOff + cur * T, lo, hiv);
-                    write_state_tile<D, NT>(tD, sm, Dst, vc.ec);                    // Dc = diag(2^c) D
-                    fence_async_smem();
-                }
+                build_rows<D>(raw, w, off, xoff, tQ, tK, tV, tG, mine);
+                Tot tu = whole;
+                if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
+                const Decay dec = decay_of<D>(sm, tu.all, tu.xall);
+                put_state<D, C::CHS>(tD, sm, Dst, dec);          // Dc = diag(2^c) D
+                if (L::X) clear_pads<D>(tV, tG, tD);
+                fence_async_smem();
                 tc_fence_before_sync();
-                SYNC_OR_DIE();
+                __syncthreads();
                 if (tid == kIssuer) {
-                    ok = mbar_wait(barS, par, a.status);          // both state tiles have landed
+                    ok = mbar_wait(barS, par, a.status) && ok;         // the state tiles have landed
                     tc_fence_after_sync();
                     const uint32_t sQ = smem_u32(tQ), sK = smem_u32(tK), sV = smem_u32(tV), sG = smem_u32(tG);
                     const uint32_t sS = smem_u32(tS), sI = smem_u32(tI), sD = smem_u32(tD);
-                    issue<64, 64, false, false, C::KS, C::CHT, C::CHT>(tmem + aP, sQ, sK, false);             // Qc Kc^T
-                    issue<64, 64, false, false, C::KS, C::CHT, C::CHT>(tmem + aP + kHi, sG, sV, false);       // dO V^T
+                    issue<64, 64, false, false, C::KS, C::CHT, C::CHT>(tmem + SM::aP, sQ, sK, false);                   // Qc Kc^T
+                    issue<64, 64, false, false, C::KS, C::CHT, C::CHT>(tmem + SM::aP + kHiLanes, sG, sV, false);        // dO V^T
                     mma_commit(barG1);
-                    issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + aQK, sG, sS, false);             // dO Sc_local^T
-                    issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + aV, sG, sI, false);              // dO S_segment^T
-                    issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + aQK + kHi, sV, sD, false);       // V Dc^T
-                    issue<64, D, false, true, C::KS, C::CHT, C::CHS>(tmem + aV + kHi, sK, sD, false);         // Kc Dc
+                    issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + SM::aQK, sG, sS, false);                   // dO Sc_local^T
+                    if (entry) issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + SM::aV, sG, sI, false);         // dO S_segment^T
+                    issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + SM::aQK + kHiLanes, sV, sD, false);        // V Dc^T
+                    issue<64, D, false, true, C::KS, C::CHT, C::CHS>(tmem + SM::aV + kHiLanes, sK, sD, false);          // Kc Dc
+                    issue_state<D>(tmem + SM::aW, tQ, tG);                                                              // Qc^T dO
                 }
-                {
-                    // the raw rows are spent: the next tile's gates (needed first) start now, its q, k, v, dO rows
-                    // after the epilogue, which needs the registers
-                    if (u == 0 && tile > t0)
-                        load_raw<D, NT, true, true, true, false>(raw, a.q, a.k, a.v, a.d_out, a.gate, rowOff + nxt * T);
-                    ok = wait_all(barG1, 0, a.status);                 // completes twice per iteration: parities 0, 1
-                    if (ok) {
-                        tc_fence_after_sync();
-                        // lanes 0-15: scores, lanes 16-31: dO V^T; keep s <= t, the diagonal has weight 1.  Column
-                        // chunks entirely above the diagonal for all rows of the warp are never written (the tiles
-                        // start out zero), chunks entirely below it need no selects.
+                if (entry && w.grp == 0) {                       // decay from the segment start to the sub-chunk's centre
+                    const float2 G = *reinterpret_cast<const float2 *>(a.slot_g + slot * D + w.c2);
+                    *reinterpret_cast<float2 *>(sAux + w.c2) = make_float2(ex2(0.5f * tu.all.x + G.x), ex2(0.5f * tu.all.y + G.y));
+                    if (L::X && w.xrow == 0) {
+                        const float2 X = *reinterpret_cast<const float2 *>(a.slot_g + slot * D + w.xc2);
+                        *reinterpret_cast<float2 *>(sAux + w.xc2) = make_float2(ex2(0.5f * tu.xall.x + X.x), ex2(0.5f * tu.xall.y + X.y));
+                    }
+                }
+                if (u == 0 && more) {
+                    prefetch_gates<D>(a.gate, rowOff + nxt * T, w);
+                    if (!kRowsEarly<D>) prefetch_rows<D, true, true>(a.q, a.k, a.v, a.d_out, rowOff + nxt * T, w);
+                }
+                if (kRowsEarly<D> && u == 0 && more) {
+                    uint32_t ro[9];
+                    row_offsets<D>(rowOff + nxt * T, w, ro);
+                    load_rows(raw, a.q, a.k, a.v, a.d_out, ro);
+                }
+                ok = wait_all(barG1, 0, a.status, ok);         // completes twice per iteration: parities 0, 1
+                tc_fence_after_sync();
+                // lanes 0-15: scores, lanes 16-31: dO V^T; keep s <= t, the diagonal has weight 1.  Column chunks
+                // entirely above the diagonal for all rows of the warp are never written (the tiles start out zero),
+                // chunks entirely below it need no selects.
+                if (ok) {
 #pragma unroll
-                        for (int i = 0; i < L::NPT; ++i) {
-                            const int sc = cg + L::NCG * i;
-                            if (sc < T / 8 && 8 * sc <= 16 * q4 + 15) {           // uniform over the warp
-                                float p[8];
-                                tmem_ld8(lane_base + tmem + aP + 8 * sc, p);
-                                if (8 * sc + 7 > 16 * q4) {
+                    for (int i = 0; i < 4; ++i) {
+                        const int sc = w.cg + 2 * i;
+                        if (i <= w.q4) {                         // uniform over the warp: sc <= 2 q4 + 1
+                            float p[8];
+                            tmem_ld8(tl + SM::aP + 8 * sc, p);
+                            if (i == w.q4) {
 #pragma unroll
-                                    for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= r16) ? p[e] : 0.f;
-                                }
-                                *reinterpret_cast<uint4 *>((hf ? tdP : tP) + sc * C::CHT + r16 * 16) = pack_h8(p);
+                                for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= w.r16) ? p[e] : 0.f;
                             }
+                            *reinterpret_cast<uint4 *>((w.hf ? tdP : tP) + sc * C::CHT + w.r16 * 16) = pack_h8(p);
                         }
                     }
-                    fence_async_smem();
                 }
+                fence_async_smem();
                 tc_fence_before_sync();
-                SYNC_OR_DIE();
+                __syncthreads();
                 if (tid == kIssuer) {
                     tc_fence_after_sync();
                     const uint32_t sQ = smem_u32(tQ), sK = smem_u32(tK), sG = smem_u32(tG);
                     const uint32_t sP = smem_u32(tP), sdP = smem_u32(tdP);
-                    issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + aQK, sdP, sK, true);             // + dP Kc
-                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + aQK + kHi, sdP, sQ, true);        // + dP^T Qc
-                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + aV + kHi, sP, sG, true);          // + P^T dO
-                    issue_state_product<D>(tmem + aP, tQ, tG);                                                // Qc^T dO
+                    issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK, sdP, sK, true);                   // + dP Kc
+                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK + kHiLanes, sdP, sQ, true);         // + dP^T Qc
+                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aV + kHiLanes, sP, sG, true);           // + P^T dO
                     mma_commit(barG1);
                 }
-                {
-                    ok = wait_all(barG1, 1, a.status);
-                    if (ok) {
-                        tc_fence_after_sync();
-                        if (tid == kIssuer && (u > 0 || tile > t0)) {
-                            // every product has completed: fetch the next sub-chunk's zero-start state
-                            const size_t nslot = u > 0 ? slot + (size_t)g.B * g.H * pl.ntile : (size_t)bh * pl.ntile + (tile - 1);
-                            const char *src = reinterpret_cast<const char *>(a.slot_s + nslot * (D * D));
-                            mbar_arrive_expect_tx(barS, (uint32_t)C::NCH * D * 16u);
-                            for (int j = 0; j < C::NCH; ++j) bulk_g2s(tS + j * C::CHS, src + j * D * 16, D * 16, barS);
-                        }
-                        const bool inrow = r16 >= lo && r16 < hiv;
-                        const size_t ro = (size_t)(my_off < 0 ? 0 : my_off);
-#pragma unroll
-                        for (int i = 0; i < L::NPC; ++i) {
-                            const int jc = cg + L::NCG * i;
-                            if (jc < C::NCH) {          // uniform over the warp
-                                float a1[8], a2[8], x[8];
-                                // lanes 0-15: dq accumulator and dO S_segment^T; lanes 16-31: dk and dv accumulators
-                                tmem_ld8_pair(lane_base + tmem + aQK + 8 * jc, lane_base + tmem + aV + 8 * jc, a1, a2);
-                                if (hf == 0) {
-                                    float hh[8];
-                                    ld8(vc.aux + 8 * jc, hh);
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e) a1[e] = fmaf(hh[e], a2[e], a1[e]);
-                                } else if (inrow) {
-                                    store_out8(dv + ro + 8 * jc, a2, a.accumulate != 0);
-                                }
-                                {
-                                    // q*dq = Qc * (dq accumulator), k*dk = Kc * (dk accumulator): the decay factors cancel
-                                    float t8[8];
-                                    unpack_h8(*reinterpret_cast<const uint4 *>((hf ? tK : tQ) + jc * C::CHT + r16 * 16), t8);
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e) x[e] = t8[e] * a1[e];
-                                }
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) x[e] -= __shfl_xor_sync(0xffffffffu, x[e], 16);
-                                {
-                                    float lam[8], of[8];
-                                    ld8(table + r16 * C::LAMP + 8 * jc, lam);
-                                    ld8(vc.off + 8 * jc, of);
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e) a1[e] *= ex2(hf ? of[e] - lam[e] : lam[e] - of[e]);
-                                }
-                                __syncwarp();           // both halves have read their gates before the table is overwritten
-                                if (inrow) {
-                                    if (hf == 0) st8(table + r16 * C::LAMP + 8 * jc, x);        // q*dq - k*dk
-                                    store_out8((hf ? dk : dq) + ro + 8 * jc, a1, a.accumulate != 0);
-                                }
-                            }
-                        }
-                        // D <- 2^(2c) D + 2^c (Qc^T dO)
-                        update_state<D, NT>(lane_base, tmem + aP, sm, Dst, vc.e2c, vc.ec);
-                        if (u == 0 && tile > t0)
-                            load_raw<D, NT, true, true, false, true>(raw, a.q, a.k, a.v, a.d_out, a.gate, rowOff + nxt * T);
+                ok = wait_all(barG1, 1, a.status, ok);
+                tc_fence_after_sync();
+                if (ok) {
+                    if (tid == kIssuer && (u > 0 || more)) {
+                        // every product has completed: fetch the next sub-chunk's zero-start state
+                        const size_t nslot = u > 0 ? slot + (size_t)g.B * g.H * pl.ntile : (size_t)bh * pl.ntile + (tile - 1);
+                        const char *src = reinterpret_cast<const char *>(a.slot_s + nslot * (D * D));
+                        mbar_arrive_expect_tx(barS, (uint32_t)C::NCH * D * 16u);
+                        for (int j = 0; j < C::NCH; ++j) bulk_g2s(tS + j * C::CHS, src + j * D * 16, D * 16, barS);
                     }
-                    tc_fence_before_sync();
+                    const bool inrow = w.r16 >= lo && w.r16 < min(hi, nrow);
+                    float *buf = (w.hf ? bufK : bufQ) + w.r16 * SM::LDP;
+#pragma unroll
+                    for (int i = 0; i < (C::NCH + 1) / 2; ++i) {
+                        const int jc = w.cg + 2 * i;
+                        if (jc < C::NCH) {                       // uniform over the warp
+                            // lanes 0-15: dq accumulator and dO S_segment^T; lanes 16-31: dk and dv accumulators
+                            float x0[8], x1[8];
+                            tmem_ld8_pair(tl + SM::aQK + 8 * jc, tl + SM::aV + 8 * jc, x0, x1);
+                            if (w.hf) {
+                                if (inrow) store_out8(dv + (uint32_t)my_off + 8 * jc, x1, acc_out);
+                            } else if (entry) {
+                                float hh[8];
+                                ld8(sAux + 8 * jc, hh);
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) x0[e] = fmaf(hh[e], x1[e], x0[e]);
+                            }
+                            st8(buf + 8 * jc, x0);
+                        }
+                    }
+                    fold_state<D>(tl + SM::aW, sm, Dst, dec);    // D <- 2^(2c) D + 2^c (Qc^T dO)
                 }
+                if (!kRowsEarly<D> && u == 0 && more) {
+                    uint32_t ro[9];
+                    row_offsets<D>(rowOff + nxt * T, w, ro);
+                    load_rows(raw, a.q, a.k, a.v, a.d_out, ro);
+                }
+                tc_fence_before_sync();
+                __syncthreads();
+                if (mine) {                                      // uniform over the warp
+                    // q dq = Qc (dq accumulator), k dk = Kc (dk accumulator): the decay factors cancel.  raw.g becomes
+                    // the suffix sums of the group's rows.
+                    const int *ro = rowOff + cur * T;
+#pragma unroll
+                    for (int j = raw.N - 1; j >= 0; --j) {
+                        const int row = item_row(w, j), c2 = j < 8 ? w.c2 : w.xc2, o = pair_offset<D>(row, c2);
+                        const float2 aq = *reinterpret_cast<const float2 *>(bufQ + row * SM::LDP + c2);
+                        const float2 ak = *reinterpret_cast<const float2 *>(bufK + row * SM::LDP + c2);
+                        const float2 q2 = __half22float2(*reinterpret_cast<const __half2 *>(tQ + o));
+                        const float2 k2 = __half22float2(*reinterpret_cast<const __half2 *>(tK + o));
+                        const float ex = raw.g[j].x + (j < 8 ? off.x : xoff.x), ey = raw.g[j].y + (j < 8 ? off.y : xoff.y);
+                        const int r = ro[row];
+                        if (row < nrow) {
+                            store_pair(dq + (uint32_t)(r + c2), aq.x * ex2(ex), aq.y * ex2(ey), acc_out);
+                            store_pair(dk + (uint32_t)(r + c2), ak.x * ex2(-ex), ak.y * ex2(-ey), acc_out);
+                        }
+                        const float x = q2.x * aq.x - k2.x * ak.x, y = q2.y * aq.y - k2.y * ak.y;
+                        if (j < 8) {
+                            tot.x += x;
+                            tot.y += y;
+                            raw.g[j] = tot;
+                        } else {
+                            xtot = make_float2(x, y);
+#pragma unroll
+                            for (int k = 1; k < 8; k <<= 1) {
+                                const float px = __shfl_down_sync(0xffffffffu, xtot.x, 4 * k), py = __shfl_down_sync(0xffffffffu, xtot.y, 4 * k);
+                                if (w.xrow + k < 8) { xtot.x += px; xtot.y += py; }
+                            }
+                            raw.g[j] = xtot;
+                        }
+                    }
+                }
+                if (u > 0) __syncthreads();                      // the accumulator buffers become operand tiles again
                 par ^= 1;
             }
-            // gate gradient of the tile: suffix sums of q*dq - k*dk down the rows plus what later tiles carry in
-            SYNC_OR_DIE();
+            // gate gradient of the tile: suffix sums of q dq - k dk down the rows plus what later tiles carry in
+            *reinterpret_cast<float2 *>(sX + w.grp * D + w.c2) = tot;
+            if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(sX + w.grp * D + w.xc2) = xtot;
+            __syncthreads();
             {
-                const bool active = tid < L::NSEG * D;
-                const int seg = tid / D, c = tid - seg * D, r0 = seg * L::RPS;
-                float sfx[L::RPS];
-                if (active) {
-                    float run = 0.f;
+                const Tot after = later_totals<D>(sX, w);
+                const float2 add = make_float2(carry.x + after.before.x, carry.y + after.before.y);
+                const float2 xadd = make_float2(xcarry.x + after.xbefore.x, xcarry.y + after.xbefore.y);
+                carry.x += after.all.x; carry.y += after.all.y;
+                xcarry.x += after.xall.x; xcarry.y += after.xall.y;
+                const int *ro = rowOff + cur * T;
 #pragma unroll
-                    for (int j = L::RPS - 1; j >= 0; --j) {
-                        if (r0 + j < nrow) run += table[(r0 + j) * C::LAMP + c];
-                        sfx[j] = run;
-                    }
-                    sTot[seg * D + c] = run;
+                for (int j = 0; j < raw.N; ++j) {
+                    const int r = ro[item_row(w, j)], c2 = j < 8 ? w.c2 : w.xc2;
+                    if (item_row(w, j) < nrow) store_pair(a.dgate + (uint32_t)(r + c2), raw.g[j].x + (j < 8 ? add.x : xadd.x), raw.g[j].y + (j < 8 ? add.y : xadd.y), acc_out);
                 }
-                __syncthreads();
-                if (active) {
-                    float add = sCarry[cpar * D + c], all = 0.f;
-#pragma unroll
-                    for (int sgm = 0; sgm < L::NSEG; ++sgm) {
-                        const float t = sTot[sgm * D + c];
-                        if (sgm > seg) add += t;
-                        all += t;
-                    }
-                    if (seg == 0) sCarry[(cpar ^ 1) * D + c] = sCarry[cpar * D + c] + all;
-#pragma unroll
-                    for (int j = 0; j < L::RPS; ++j) {
-                        const int ro = r0 + j < nrow ? rowOff[cur * T + r0 + j] : -1;
-                        if (ro >= 0) a.dgate[(size_t)ro + c] = (a.accumulate ? a.dgate[(size_t)ro + c] : 0.f) + (sfx[j] + add);
-                    }
-                }
-                cpar ^= 1;
+            }
+            if (more) {
+                uint32_t ro[9];
+                row_offsets<D>(rowOff + nxt * T, w, ro);
+                load_gates(raw.g, a.gate, ro);
+                group_prefix<D>(raw, raw.g, w, sTot);                   // only the last tile of a sequence has a tail, and it comes first
             }
             cur = nxt;
         }
@@ -906,25 +989,18 @@ die:
 #undef SYNC_OR_DIE
 
 // ---- host side ----------------------------------------------------------------------------------
-// Launch shapes per head size: worker threads per CTA and CTAs per SM of each kernel (the light
-// kernels run more CTAs per SM on fewer registers, which hides the latency of their short tiles).
-template <int D>
-struct Shape {          // d = 64: two CTAs of 256 threads per SM
-    static constexpr int NT_LOCAL_F = 256, NT_LOCAL_B = 256, NT_FWD = 256, NT_BWD = 256, OCC = 2;
-};
-template <>
-struct Shape<72> {
-    static constexpr int NT_LOCAL_F = 640, NT_LOCAL_B = 640, NT_FWD = 640, NT_BWD = 640, OCC = 1;
-};
+constexpr int kPerSm = 2;       // CTAs of 256 threads that share an SM, for every kernel of the family
 
-// A forward pass whose sequences are not cut (one segment each) runs the forward sweep alone, from the
-// start state: no local sweep, no scan.  Cut sequences pay for the local sweep as well, about 0.7 of a
-// forward sweep; the backward pass needs the local sweep (the per-tile states) in either case.
+// Segment length.  A pass costs (tiles of a segment + one of fill and drain) per round of resident CTAs.
+// Uncut sequences (one segment each) run the forward sweep alone; cut ones also run the local sweep, about
+// half of a forward sweep per tile, and the scan, and these two launches take about as long as three tiles
+// of a forward sweep when the machine is not full.  The backward pass needs the local sweep in either case.
 Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
 {
     Plan p;
     p.ntile = (g.L + T - 1) / T;
     p.sub_max = g.C < T ? g.C : T;
+    p.gh_inv = g.gh > 1 ? (uint32_t)((1ull << 32) / (unsigned)g.gh) : 0xffffffffu;
     const long long slots = (long long)sms * per_sm, bh = (long long)g.B * g.H;
     long long best = -1;
     p.G = p.ntile;
@@ -932,7 +1008,7 @@ Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
         const int nseg = (p.ntile + G - 1) / G;
         const long long rounds = (bh * nseg + slots - 1) / slots;
         long long cost = rounds * (G + 1) * 10;             // a segment costs about one tile of fill and drain
-        if (!backward && nseg > 1) cost += cost * 7 / 10;
+        if (nseg > 1) cost += backward ? 15 : cost / 2 + 30;
         if (best < 0 || cost < best) {
             best = cost;
             p.G = G;
@@ -967,13 +1043,6 @@ SweepWs carve(char *base, const Geom &g, const Plan &pl, bool backward)
     return w;
 }
 
-// CTAs per SM of the heaviest kernel of a pass: segments are sized for that many slots
-int sweep_per_sm(int d, bool backward)
-{
-    (void)backward;
-    return d == 64 ? Shape<64>::OCC : Shape<72>::OCC;
-}
-
 template <typename K>
 dig_status set_smem(K kern, size_t bytes)
 {
@@ -983,14 +1052,11 @@ dig_status set_smem(K kern, size_t bytes)
 template <int D, bool BWD>
 dig_status run(const GlaArgs &ga)
 {
-    using SH = Shape<D>;
-    constexpr int NT_L = BWD ? SH::NT_LOCAL_B : SH::NT_LOCAL_F, NT_M = BWD ? SH::NT_BWD : SH::NT_FWD;
-    constexpr int OCC_L = SH::OCC, OCC_M = SH::OCC;
     const Geom &g = ga.g;
     const int sms = device_sm_count();
     int *status = device_status_ptr();
     if (!status || sms <= 0) return DIG_ERR_CUDA;
-    const Plan pl = make_plan(g, sms, OCC_M, BWD);
+    const Plan pl = make_plan(g, sms, kPerSm, BWD);
     const SweepWs w = carve(reinterpret_cast<char *>(ga.ws), g, pl, BWD);
     const long long total = (long long)g.B * g.H * pl.nseg;
     if (total > (1ll << 30) || (long long)g.B * g.L * g.H * D >= (1ll << 31)) return DIG_ERR_UNSUPPORTED;     // 31-bit row offsets
@@ -1004,8 +1070,7 @@ dig_status run(const GlaArgs &ga)
     a.accumulate = ga.accumulate;
     a.g = g;
     a.plan = pl;
-    const int grid_l = (int)(total < (long long)sms * OCC_L ? total : (long long)sms * OCC_L);
-    const int grid_m = (int)(total < (long long)sms * OCC_M ? total : (long long)sms * OCC_M);
+    const dim3 grid((unsigned)(total < (long long)sms * kPerSm ? total : (long long)sms * kPerSm)), block(Col<D>::NT);
     a.s_in = ga.sio.s_in;
     a.s_out = ga.sio.s_out;
     const bool sweep_only = !BWD && pl.nseg == 1;      // uncut sequences: the forward sweep starts from the start state itself
@@ -1013,22 +1078,25 @@ dig_status run(const GlaArgs &ga)
     // backward pass over uncut sequences whose start-state gradient is not asked for: the segment's own
     // contribution to the state gradient is never used, the local sweep only has to store the states
     const bool states_only = BWD && pl.nseg == 1 && ga.sio.ds_in == nullptr;
-    if (states_only) {
-        auto kern = sweep_local<D, SH::NT_LOCAL_F, false, OCC_L, true>;
-        constexpr size_t smem = LocalSmem<D, SH::NT_LOCAL_F, false>::bytes;
+    // ... and without state arguments there is nothing to scan: entry state, incoming gradient and carry are zero
+    const bool scan = !sweep_only && !(states_only && ga.sio.s_in == nullptr && ga.sio.ds_out == nullptr);
+    a.scanned = scan;
+    if (!sweep_only) {
+        void (*kern)(SweepArgs) = nullptr;
+        size_t smem = 0;
+        if constexpr (BWD) {
+            kern = states_only ? sweep_local_bwd<D, false> : sweep_local_bwd<D, true>;
+            smem = states_only ? LocalBwdSmem<D, false>::bytes : LocalBwdSmem<D, true>::bytes;
+        } else {
+            kern = sweep_local_fwd<D>;
+            smem = LocalFwdSmem<D>::bytes;
+        }
         if ((st = set_smem(kern, smem)) != DIG_OK) return st;
         KernelTimer t(KID_SW_LOCAL, ga.stream);
-        launch_pdl(kern, dim3(grid_l), dim3(SH::NT_LOCAL_F), smem, ga.stream, a);
-        if ((st = cuda_ok(cudaGetLastError())) != DIG_OK) return st;
-    } else if (!sweep_only) {
-        auto kern = sweep_local<D, NT_L, BWD, OCC_L>;
-        constexpr size_t smem = LocalSmem<D, NT_L, BWD>::bytes;
-        if ((st = set_smem(kern, smem)) != DIG_OK) return st;
-        KernelTimer t(KID_SW_LOCAL, ga.stream);
-        launch_pdl(kern, dim3(grid_l), dim3(NT_L), smem, ga.stream, a);
+        launch_pdl(kern, grid, block, smem, ga.stream, a);
         if ((st = cuda_ok(cudaGetLastError())) != DIG_OK) return st;
     }
-    if (!sweep_only) {
+    if (scan) {
         auto kern = seg_scan<D, BWD>;
         KernelTimer t(KID_SW_SCAN, ga.stream);
         launch_pdl(kern, dim3(g.B * g.H, D / 8), dim3(64), 0, ga.stream, w.seg_state, (const float *)w.seg_gamma, w.seg_dstate,
@@ -1037,19 +1105,19 @@ dig_status run(const GlaArgs &ga)
     }
     const bool f32 = ga.dtype == DIG_BF16_F32OUT;
     if constexpr (!BWD) {
-        constexpr size_t smem = FwdSmem<D, NT_M>::bytes;
-        auto k16 = sweep_fwd<D, NT_M, bf16, OCC_M>;
-        auto k32 = sweep_fwd<D, NT_M, float, OCC_M>;
+        constexpr size_t smem = FwdSmem<D>::bytes;
+        auto k16 = sweep_fwd<D, bf16>;
+        auto k32 = sweep_fwd<D, float>;
         if ((st = set_smem(k16, smem)) != DIG_OK || (st = set_smem(k32, smem)) != DIG_OK) return st;
         KernelTimer t(KID_SW_FWD, ga.stream);
-        launch_pdl(f32 ? k32 : k16, dim3(grid_m), dim3(NT_M), smem, ga.stream, a);
+        launch_pdl(f32 ? k32 : k16, grid, block, smem, ga.stream, a);
     } else {
-        constexpr size_t smem = BwdSmem<D, NT_M>::bytes;
-        auto k16 = sweep_bwd<D, NT_M, bf16, OCC_M>;
-        auto k32 = sweep_bwd<D, NT_M, float, OCC_M>;
+        constexpr size_t smem = BwdSmem<D>::bytes;
+        auto k16 = sweep_bwd<D, bf16>;
+        auto k32 = sweep_bwd<D, float>;
         if ((st = set_smem(k16, smem)) != DIG_OK || (st = set_smem(k32, smem)) != DIG_OK) return st;
         KernelTimer t(KID_SW_BWD, ga.stream);
-        launch_pdl(f32 ? k32 : k16, dim3(grid_m), dim3(NT_M), smem, ga.stream, a);
+        launch_pdl(f32 ? k32 : k16, grid, block, smem, ga.stream, a);
     }
     return cuda_ok(cudaGetLastError());
 }
@@ -1067,7 +1135,7 @@ size_t sweep_workspace_bytes(const Geom &g, bool backward)
 {
     int sms = device_sm_count();
     if (sms <= 0) sms = 148;
-    const Plan pl = make_plan(g, sms, sweep_per_sm(g.dk, backward), backward);
+    const Plan pl = make_plan(g, sms, kPerSm, backward);
     return carve(nullptr, g, pl, backward).bytes;
 }
 

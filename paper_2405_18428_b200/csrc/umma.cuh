@@ -1,5 +1,5 @@
 // Thin wrappers over the sm_100a tensor-core path used by the GLA kernels: tensor-memory
-// allocation, shared-memory matrix descriptors, tcgen05.mma (kind::tf32), completion barriers and
+// allocation, shared-memory matrix descriptors, tcgen05.mma (kind::f16), completion barriers and
 // tensor-memory loads.  Every wait is bounded by wall-clock time and reports through a status word.
 #pragma once
 
@@ -14,37 +14,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// ---- shared-memory operand tiles ----------------------------------------------------------
-// Operand tiles hold fp32 words (values already rounded to tf32), row-major in column blocks of
-// 32 words: block b holds columns [32b, 32b+32) of all ROWS rows, 128 bytes per row.  Two
-// swizzle patterns exist because kind::tf32 reads the two operand orientations differently:
-//   K-format  (contraction along the tile's columns, "K-major"): 16-byte chunks of a row XOR-ed
-//             with (row & 7)  -- the 128-byte swizzle, descriptor layout type 2;
-//   M-format  (contraction along the tile's rows, "MN-major"): 32-byte chunks of a row XOR-ed
-//             with (row & 3)  -- the 128-byte swizzle with 32-byte base, layout type 1, the only
-//             MN-major layout tf32 operands may use.
-// A tile that is read in both orientations is stored twice.  Tile bases are 1024-byte aligned.
-template <int ROWS>
-__device__ __forceinline__ uint32_t tile_offset(int row, int col)       // K-format
-{
-    return (uint32_t)((col >> 5) * (ROWS * 128) + row * 128 + ((((col & 31) >> 2) ^ (row & 7)) << 4) +
-                      ((col & 3) << 2));
-}
-template <int ROWS>
-__device__ __forceinline__ uint32_t tile_offset_m(int row, int col)     // M-format
-{
-    return (uint32_t)((col >> 5) * (ROWS * 128) + row * 128 + ((((col & 31) >> 3) ^ (row & 3)) << 5) +
-                      ((col & 7) << 2));
-}
-
-// Round to tf32 (10 explicit mantissa bits), nearest with ties away from zero: what
-// cvt.rna.tf32.f32 computes for finite values, done with two integer operations because the
-// conversion instruction runs at a quarter of their rate.
-__device__ __forceinline__ float to_tf32(float x)
-{
-    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
-}
-
 // 64-bit matrix descriptor: start address, leading / stride byte offsets (all >> 4), descriptor
 // version 1, layout type in the top three bits.
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes,
@@ -57,42 +26,6 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)layout_type << 61;
     return d;
-}
-
-// K-major view of a K-format tile (rows = M or N index, columns = contraction index), starting at
-// (row0, k0), row0 a multiple of 8: 8-row groups are 1024 bytes apart; a step of 8 along K stays
-// inside one 128-byte row (32 bytes per step) or moves to the next column block.
-template <int ROWS>
-__device__ __forceinline__ uint64_t desc_kmajor(uint32_t tile_saddr, int row0, int k0)
-{
-    const uint32_t a = tile_saddr + (k0 >> 5) * (ROWS * 128) + row0 * 128 + ((k0 & 31) << 2);
-    return make_desc(a, 16, 1024, 2);
-}
-// MN-major view of an M-format tile (rows = contraction index, columns = M or N index), starting
-// at (k0, col0) with k0 a multiple of 4 and col0 a multiple of 32: column blocks are ROWS*128 bytes
-// apart (leading offset), 4-row groups along K 512 bytes apart (stride offset).
-template <int ROWS>
-__device__ __forceinline__ uint64_t desc_mnmajor(uint32_t tile_saddr, int k0, int col0)
-{
-    const uint32_t a = tile_saddr + (col0 >> 5) * (ROWS * 128) + k0 * 128;
-    return make_desc(a, ROWS * 128, 512, 1);
-}
-
-// Instruction descriptor for kind::tf32 with fp32 accumulation.
-__host__ __device__ constexpr uint32_t idesc_tf32(int M, int N, bool a_mn_major, bool b_mn_major)
-{
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((a_mn_major ? 1u : 0u) << 15) |
-           ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// D[tmem] (+)= A[smem] * B[smem]; one thread issues.
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         bool accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
 }
 
 // Instruction descriptor for kind::f16 with fp16 operands and fp32 accumulation, and the instruction.
@@ -150,9 +83,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *s
         uint32_t ok;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok) : "r"(addr), "r"(parity), "r"(20000u) : "memory");      // may sleep up to 20 us per try
+            : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
         if (ok) return true;
         if ((it & 7) == 7) {
             const uint64_t now = global_ns();
@@ -173,19 +106,6 @@ __device__ __forceinline__ void bulk_g2s(void *smem_dst, const void *gsrc, uint3
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  :: "r"(smem_u32(smem_dst)), "l"(gsrc), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
-// Shared -> global bulk copy, tracked by the issuing thread's bulk-copy groups.
-__device__ __forceinline__ void bulk_s2g(void *gdst, const void *smem_src, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                 :: "l"(gdst), "r"(smem_u32(smem_src)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// Waits until this thread's committed bulk stores have finished reading shared memory / have completed.
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// Barrier over the first `threads` threads of the CTA only (hardware barrier 1).
-__device__ __forceinline__ void sync_group(int threads) { asm volatile("bar.sync 1, %0;" :: "r"(threads) : "memory"); }
-
 // One arrival that also announces `bytes` of pending bulk-copy traffic.
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
 {
@@ -205,38 +125,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(taddr), "r"(cols) : "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's tensor-memory lane (lane = 32*(warp%4) + laneid).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
-{
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// 16 consecutive fp32 columns of this thread's tensor-memory lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 // 8 consecutive fp32 columns of this thread's tensor-memory lane.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8])
 {
@@ -263,8 +151,6 @@ __device__ __forceinline__ void tmem_ld8_pair(uint32_t ta, uint32_t tb, float (&
 #pragma unroll
     for (int i = 0; i < 8; ++i) { a[i] = __uint_as_float(r[i]); b[i] = __uint_as_float(r[8 + i]); }
 }
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[32]) { tmem_ld32(taddr, v); }
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[16]) { tmem_ld16(taddr, v); }
 
 }  // namespace umma
 }  // namespace dig
