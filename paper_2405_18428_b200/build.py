@@ -1,9 +1,12 @@
-"""Builds the C-ABI CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds the C-ABI CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU) and the CPython
+module that calls it with torch tensors."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -11,6 +14,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(os.path.dirname(PKG), "include")
 OBJDIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdig_gla.so")
+BINDING_SRC = os.path.join(CSRC, "binding.cpp")
+BINDING = os.path.join(PKG, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -24,6 +29,16 @@ def _deps_mtime():
     hdrs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     hdrs += [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE)]
     return max(os.path.getmtime(h) for h in hdrs)
+
+
+def _binding_cmd(out):
+    torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"], INCLUDE]
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", *[a for d in inc for a in ("-isystem", d)], BINDING_SRC, "-o", out,
+            LIB, "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu",
+            "-lc10_cuda", "-lc10"]
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
@@ -54,6 +69,10 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         tmp = LIB + f".tmp{os.getpid()}"
         run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp, *objs])
         os.replace(tmp, LIB)
+    if force or not os.path.exists(BINDING) or os.path.getmtime(BINDING) < max(os.path.getmtime(BINDING_SRC), hdr_m):
+        tmp = BINDING + f".tmp{os.getpid()}"
+        run(_binding_cmd(tmp))
+        os.replace(tmp, BINDING)
     return LIB
 
 

@@ -131,8 +131,14 @@ __global__ void wait_that_expires(int *status, unsigned long long limit_ns)
 
 int *device_status_ptr()
 {
-    int *p = nullptr;
-    if (cudaGetSymbolAddress(reinterpret_cast<void **>(&p), g_device_status) != cudaSuccess) return nullptr;
+    static std::atomic<int *> cached[64];           // the address is fixed per device
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    int *p = cached[dev].load();
+    if (p == nullptr) {
+        if (cudaGetSymbolAddress(reinterpret_cast<void **>(&p), g_device_status) != cudaSuccess) return nullptr;
+        cached[dev].store(p);
+    }
     return p;
 }
 

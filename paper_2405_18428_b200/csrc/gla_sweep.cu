@@ -1004,8 +1004,8 @@ Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
     const long long slots = (long long)sms * per_sm, bh = (long long)g.B * g.H;
     long long best = -1;
     p.G = p.ntile;
-    for (int G = p.ntile; G >= 1; --G) {
-        const int nseg = (p.ntile + G - 1) / G;
+    // the shortest G of every number of segments that occurs (about 2 sqrt(ntile) of them)
+    for (int nseg = 1, G = p.ntile;; nseg = (p.ntile + G - 2) / (G - 1), G = (p.ntile + nseg - 1) / nseg) {
         const long long rounds = (bh * nseg + slots - 1) / slots;
         long long cost = rounds * (G + 1) * 10;             // a segment costs about one tile of fill and drain
         if (nseg > 1) cost += backward ? 15 : cost / 2 + 30;
@@ -1013,6 +1013,7 @@ Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
             best = cost;
             p.G = G;
         }
+        if (G == 1) break;
     }
     p.nseg = (p.ntile + p.G - 1) / p.G;
     return p;
