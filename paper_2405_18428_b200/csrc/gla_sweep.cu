@@ -375,42 +375,49 @@ die:
 }
 
 // =================================================================================================
-// seg_scan: the recurrence over segment ends, one sequence per blockIdx.x, 8 state rows per block,
-// 8 lanes per row.  Forward: seg_state[s] (state a segment leaves from a zero start) becomes the
-// state entering segment s.  Backward flavour: seg_dstate[s] (the segment's own contribution)
-// becomes the gradient with respect to the state leaving segment s, seg_carry the gate-gradient
-// carried into the segment from later ones, seg_state16 an fp16 copy of the entry states in the
-// dense chunk-major order the backward sweep bulk-copies.
+// seg_scan: the recurrence over segment ends, 16 lanes per (sequence, state row), a lane four neighbouring
+// value channels (and four more at d = 72, lanes 0 and 1).  Forward: seg_state[s] (state a segment
+// leaves from a zero start) becomes the state entering segment s.  Backward flavour: seg_dstate[s] (the
+// segment's own contribution) becomes the gradient with respect to the state leaving segment s, seg_carry
+// the gate-gradient carried into the segment from later ones, seg_state16 an fp16 copy of the entry states
+// in the dense chunk-major order the backward sweep bulk-copies.
+// Bound by the latency of its loads, which do not depend on the recurrence: NB segments are in flight
+// together.  49 segments x 6 sequences, d = 64: 8.0 us with 8 lanes per row and fewer loads in flight, 6.1 us now;
+// backward flavour, 18 x 16, d = 72: 14.6 -> 10.1 us.  A whole warp per row: 12.9 us (five shuffles per row, half of
+// the lanes idle in the second piece).
 // =================================================================================================
+constexpr int kScanRows = 8;                          // state rows per block
 template <int D, bool BWD>
-__global__ void __launch_bounds__(64)
+__global__ void __launch_bounds__(16 * kScanRows)
 seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg_carry, __half *seg_state16,
          const float *s_in, float *s_out, const float *ds_out, float *ds_in, int nseg)
 {
-    constexpr int NV = (D / 4 + 7) / 8;               // float4 pieces per lane
-    constexpr int NB = NV <= 2 ? 8 : 4;               // segments whose loads are in flight together
-    const int bh = blockIdx.x, c = blockIdx.y * 8 + (threadIdx.x >> 3), l8 = threadIdx.x & 7;
+    constexpr int NV = (D / 4 + 15) / 16;             // float4 pieces per lane
+    constexpr int NB = NV == 1 ? (BWD ? 8 : 16) : (BWD ? 6 : 12);         // segments whose loads are in flight together
+    const int bh = blockIdx.x, c = blockIdx.y * kScanRows + (threadIdx.x >> 4), lane = threadIdx.x & 15;
+    static_assert(D % kScanRows == 0, "whole blocks of rows");
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const size_t dd = (size_t)D * D, io = bh * dd + (size_t)c * D + 4 * lane, st0 = (size_t)bh * nseg * dd + (size_t)c * D + 4 * lane;
+    const float *gam0 = seg_gamma + (size_t)bh * nseg * D + c;
+    auto has = [&](int i) { return i == 0 || lane < D / 4 - 16; };
+    auto ld = [&](const float *p, int i) { return has(i) ? *reinterpret_cast<const float4 *>(p + 64 * i) : zero; };
+    auto st = [&](float *p, int i, float4 v) { if (has(i)) *reinterpret_cast<float4 *>(p + 64 * i) = v; };
+    auto step = [](float g, float4 x, float4 t) { return make_float4(g * x.x + t.x, g * x.y + t.y, g * x.z + t.z, g * x.w + t.w); };
     pdl_wait();
     pdl_launch_dependents();
     float4 s[NV];
-    const size_t row = (size_t)c * D;
-    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int e = 4 * (l8 + 8 * i);
-        s[i] = (s_in && e < D) ? *reinterpret_cast<const float4 *>(s_in + (size_t)bh * D * D + row + e) : zero4;
-    }
+    for (int i = 0; i < NV; ++i) s[i] = s_in ? ld(s_in + io, i) : zero;
     for (int sg0 = 0; sg0 < nseg; sg0 += NB) {
         float4 t[NB][NV];
         float gam[NB];
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
-            const int sg = min(sg0 + j, nseg - 1);
-            gam[j] = seg_gamma[((size_t)bh * nseg + sg) * D + c];
+            const int sg = sg0 + j;
+            if (sg < nseg) {
+                gam[j] = gam0[(size_t)sg * D];
 #pragma unroll
-            for (int i = 0; i < NV; ++i) {
-                const int e = 4 * (l8 + 8 * i);
-                t[j][i] = e < D ? *reinterpret_cast<const float4 *>(seg_state + ((size_t)bh * nseg + sg) * D * D + row + e) : zero4;
+                for (int i = 0; i < NV; ++i) t[j][i] = ld(seg_state + st0 + sg * dd, i);
             }
         }
 #pragma unroll
@@ -420,38 +427,26 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
                 const float gm = exp2f(gam[j]);
 #pragma unroll
                 for (int i = 0; i < NV; ++i) {
-                    const int e = 4 * (l8 + 8 * i);
-                    if (e < D) {
-                        *reinterpret_cast<float4 *>(seg_state + ((size_t)bh * nseg + sg) * D * D + row + e) = s[i];
-                        if (BWD) {
-                            __half2 lo = __floats2half2_rn(s[i].x, s[i].y), hi = __floats2half2_rn(s[i].z, s[i].w);
-                            uint2 pk;
-                            pk.x = *reinterpret_cast<uint32_t *>(&lo);
-                            pk.y = *reinterpret_cast<uint32_t *>(&hi);
-                            char *dst = reinterpret_cast<char *>(seg_state16 + ((size_t)bh * nseg + sg) * D * D);
-                            *reinterpret_cast<uint2 *>(dst + ((e >> 3) * D + c) * 16 + (e & 7) * 2) = pk;
-                        }
-                        s[i] = make_float4(gm * s[i].x + t[j][i].x, gm * s[i].y + t[j][i].y, gm * s[i].z + t[j][i].z,
-                                           gm * s[i].w + t[j][i].w);
+                    st(seg_state + st0 + sg * dd, i, s[i]);
+                    if (BWD && has(i)) {
+                        const int e = 4 * lane + 64 * i;
+                        const __half2 h[2] = {__floats2half2_rn(s[i].x, s[i].y), __floats2half2_rn(s[i].z, s[i].w)};
+                        char *dst = reinterpret_cast<char *>(seg_state16 + ((size_t)bh * nseg + sg) * dd);
+                        *reinterpret_cast<uint2 *>(dst + ((e >> 3) * D + c) * 16 + (e & 7) * 2) = *reinterpret_cast<const uint2 *>(h);
                     }
+                    s[i] = step(gm, s[i], t[j][i]);
                 }
             }
         }
     }
     if (s_out) {
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int e = 4 * (l8 + 8 * i);
-            if (e < D) *reinterpret_cast<float4 *>(s_out + (size_t)bh * D * D + row + e) = s[i];
-        }
+        for (int i = 0; i < NV; ++i) st(s_out + io, i, s[i]);
     }
     if (BWD) {
         float4 d[NV];
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int e = 4 * (l8 + 8 * i);
-            d[i] = (ds_out && e < D) ? *reinterpret_cast<const float4 *>(ds_out + (size_t)bh * D * D + row + e) : zero4;
-        }
+        for (int i = 0; i < NV; ++i) d[i] = ds_out ? ld(ds_out + io, i) : zero;
         // s holds the state leaving the last segment; walking back, it is replaced by the entry state of
         // the segment just handled, which is the state leaving the one before it
         for (int sg0 = nseg - 1; sg0 >= 0; sg0 -= NB) {
@@ -459,45 +454,43 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
             float gam[NB];
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
-                const int sg = max(sg0 - j, 0);
-                gam[j] = seg_gamma[((size_t)bh * nseg + sg) * D + c];
+                const int sg = sg0 - j;
+                if (sg >= 0) {
+                    gam[j] = gam0[(size_t)sg * D];
 #pragma unroll
-                for (int i = 0; i < NV; ++i) {
-                    const int e = 4 * (l8 + 8 * i);
-                    t[j][i] = e < D ? *reinterpret_cast<const float4 *>(seg_dstate + ((size_t)bh * nseg + sg) * D * D + row + e) : zero4;
-                    sp[j][i] = e < D ? *reinterpret_cast<const float4 *>(seg_state + ((size_t)bh * nseg + sg) * D * D + row + e) : zero4;
+                    for (int i = 0; i < NV; ++i) {
+                        t[j][i] = ld(seg_dstate + st0 + sg * dd, i);
+                        sp[j][i] = ld(seg_state + st0 + sg * dd, i);
+                    }
                 }
             }
+            float dot[NB];
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
                 const int sg = sg0 - j;
+                dot[j] = 0.f;
                 if (sg >= 0) {
                     const float gm = exp2f(gam[j]);
-                    float dot = 0.f;
 #pragma unroll
                     for (int i = 0; i < NV; ++i) {
-                        const int e = 4 * (l8 + 8 * i);
-                        if (e < D) {
-                            *reinterpret_cast<float4 *>(seg_dstate + ((size_t)bh * nseg + sg) * D * D + row + e) = d[i];
-                            dot += s[i].x * d[i].x + s[i].y * d[i].y + s[i].z * d[i].z + s[i].w * d[i].w;
-                            d[i] = make_float4(gm * d[i].x + t[j][i].x, gm * d[i].y + t[j][i].y, gm * d[i].z + t[j][i].z,
-                                               gm * d[i].w + t[j][i].w);
-                            s[i] = sp[j][i];
-                        }
+                        st(seg_dstate + st0 + sg * dd, i, d[i]);
+                        dot[j] += s[i].x * d[i].x + s[i].y * d[i].y + s[i].z * d[i].z + s[i].w * d[i].w;
+                        d[i] = step(gm, d[i], t[j][i]);
+                        s[i] = sp[j][i];
                     }
-                    dot += __shfl_xor_sync(0xffffffffu, dot, 4);
-                    dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-                    dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-                    if (l8 == 0) seg_carry[((size_t)bh * nseg + sg) * D + c] = dot;
                 }
             }
+#pragma unroll
+            for (int m = 8; m >= 1; m >>= 1)
+#pragma unroll
+                for (int j = 0; j < NB; ++j) dot[j] += __shfl_xor_sync(0xffffffffu, dot[j], m);
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+                if (lane == j && sg0 - j >= 0) seg_carry[((size_t)bh * nseg + sg0 - j) * D + c] = dot[j];
         }
         if (ds_in) {
 #pragma unroll
-            for (int i = 0; i < NV; ++i) {
-                const int e = 4 * (l8 + 8 * i);
-                if (e < D) *reinterpret_cast<float4 *>(ds_in + (size_t)bh * D * D + row + e) = d[i];
-            }
+            for (int i = 0; i < NV; ++i) st(ds_in + io, i, d[i]);
         }
     }
 }
@@ -1100,7 +1093,7 @@ dig_status run(const GlaArgs &ga)
     if (scan) {
         auto kern = seg_scan<D, BWD>;
         KernelTimer t(KID_SW_SCAN, ga.stream);
-        launch_pdl(kern, dim3(g.B * g.H, D / 8), dim3(64), 0, ga.stream, w.seg_state, (const float *)w.seg_gamma, w.seg_dstate,
+        launch_pdl(kern, dim3(g.B * g.H, D / kScanRows), dim3(16 * kScanRows), 0, ga.stream, w.seg_state, (const float *)w.seg_gamma, w.seg_dstate,
                    w.seg_carry, w.seg_state16, ga.sio.s_in, ga.sio.s_out, ga.sio.ds_out, ga.sio.ds_in, pl.nseg);
         if ((st = cuda_ok(cudaGetLastError())) != DIG_OK) return st;
     }
