@@ -693,12 +693,8 @@ struct BwdSmem {
 
 __device__ __forceinline__ void store_pair(float *p, float x, float y, bool add)
 {
-    if (add) {
-        const float2 o = *reinterpret_cast<const float2 *>(p);
-        x += o.x;
-        y += o.y;
-    }
-    *reinterpret_cast<float2 *>(p) = make_float2(x, y);
+    if (add) asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" :: "l"(p), "f"(x), "f"(y) : "memory");
+    else *reinterpret_cast<float2 *>(p) = make_float2(x, y);
 }
 __device__ __forceinline__ void store_pair(bf16 *p, float x, float y, bool) { *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(x, y); }
 
@@ -1135,21 +1131,25 @@ size_t sweep_workspace_bytes(const Geom &g, bool backward)
 
 namespace {
 
-// fp32 sums -> bf16 results (round to nearest even), 8 elements per thread.
-__global__ void __launch_bounds__(256) round_to_bf16(const float *__restrict__ src, bf16 *__restrict__ dst, size_t n8)
+// fp32 sums -> bf16 results (round to nearest even), 8 elements per thread; blockIdx.y selects the tensor.
+struct RoundArgs {
+    const float *src[3];
+    bf16 *dst[3];
+};
+__global__ void __launch_bounds__(256) round_to_bf16(const RoundArgs a, size_t n8)
 {
     pdl_wait();
     pdl_launch_dependents();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n8) return;
     float f[8];
-    ld8(src + 8 * i, f);
-    store_out8(dst + 8 * i, f);
+    ld8(a.src[blockIdx.y] + 8 * i, f);
+    store_out8(a.dst[blockIdx.y] + 8 * i, f);
 }
-dig_status launch_round(const float *src, void *dst, size_t n, cudaStream_t s)
+dig_status launch_round(const RoundArgs &a, int tensors, size_t n, cudaStream_t s)
 {
     const size_t n8 = n / 8;
-    launch_pdl(round_to_bf16, dim3((unsigned)((n8 + 255) / 256)), dim3(256), 0, s, src, (bf16 *)dst, n8);
+    launch_pdl(round_to_bf16, dim3((unsigned)((n8 + 255) / 256), tensors), dim3(256), 0, s, a, n8);
     return cuda_ok(cudaGetLastError());
 }
 
@@ -1184,7 +1184,8 @@ dig_status sweep_gla_fwd_multi(const GlaArgs &a0, unsigned mask)
         const dig_status st = sweep_gla_fwd(a);
         if (st != DIG_OK) return st;
     }
-    return narrow ? launch_round(reinterpret_cast<const float *>(extra), a0.out, tok * a.g.dv, a.stream) : DIG_OK;
+    if (!narrow) return DIG_OK;
+    return launch_round(RoundArgs{{reinterpret_cast<const float *>(extra)}, {(bf16 *)a0.out}}, 1, tok * a.g.dv, a.stream);
 }
 
 dig_status sweep_gla_bwd_multi(const GlaArgs &a0, unsigned mask)
@@ -1207,10 +1208,7 @@ dig_status sweep_gla_bwd_multi(const GlaArgs &a0, unsigned mask)
         if (st != DIG_OK) return st;
     }
     if (!narrow) return DIG_OK;
-    dig_status st;
-    if ((st = launch_round(sq, a0.dq, tok * a.g.dk, a.stream)) != DIG_OK) return st;
-    if ((st = launch_round(sk, a0.dk, tok * a.g.dk, a.stream)) != DIG_OK) return st;
-    return launch_round(sv, a0.dv, tok * a.g.dv, a.stream);
+    return launch_round(RoundArgs{{sq, sk, sv}, {(bf16 *)a0.dq, (bf16 *)a0.dk, (bf16 *)a0.dv}}, 3, tok * a.g.dk, a.stream);      // d_k = d_v
 }
 
 dig_status sweep_gla_fwd(const GlaArgs &a)

@@ -87,16 +87,15 @@ __device__ __forceinline__ void st8(float *p, const float (&f)[8])
     *reinterpret_cast<float4 *>(p) = make_float4(f[0], f[1], f[2], f[3]);
     *reinterpret_cast<float4 *>(p + 4) = make_float4(f[4], f[5], f[6], f[7]);
 }
-// 8 results to global memory in the output storage type.  `add`: on top of what is there (fp32
-// outputs only; used when several scan orders are summed into one buffer).
+// 8 results to global memory in the output storage type.  `add`: on top of what is there (fp32 outputs only;
+// used when several scan orders are summed into one buffer).  The addition is left to the L2 (a vector
+// reduction): every element gets one addition per scan order and the orders follow one another on the
+// stream, so the sum does not depend on scheduling, and nothing waits for the old values.
 __device__ __forceinline__ void store_out8(float *p, const float (&f)[8], bool add = false)
 {
     if (add) {
-        float o[8];
-        ld8(p, o);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] += f[e];
-        st8(p, o);
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(p), "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]) : "memory");
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(p + 4), "f"(f[4]), "f"(f[5]), "f"(f[6]), "f"(f[7]) : "memory");
     } else {
         st8(p, f);
     }
