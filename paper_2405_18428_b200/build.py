@@ -37,7 +37,7 @@ def _binding_cmd(out):
     inc = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
            os.path.join(cuda, "include"), sysconfig.get_paths()["include"], INCLUDE]
     return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", *[a for d in inc for a in ("-isystem", d)], BINDING_SRC, "-o", out,
-            LIB, "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu",
+            "-L" + PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu",
             "-lc10_cuda", "-lc10"]
 
 
