@@ -43,32 +43,6 @@ struct Col {
     static_assert(D == 64 || D == 72, "32 channel pairs, or 36 of which 4 are extra items");
 };
 
-__device__ __forceinline__ float lo_f(uint32_t b) { return __uint_as_float(b << 16); }
-__device__ __forceinline__ float hi_f(uint32_t b) { return __uint_as_float(b & 0xffff0000u); }
-
-// Packed fp32 pairs: one instruction for two additions, products or fused multiply-adds (same rounding as two).
-__device__ __forceinline__ unsigned long long as_u64(float2 a) { return ((unsigned long long)__float_as_uint(a.y) << 32) | __float_as_uint(a.x); }
-__device__ __forceinline__ float2 as_f2(unsigned long long u) { return make_float2(__uint_as_float((uint32_t)u), __uint_as_float((uint32_t)(u >> 32))); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b)
-{
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
-    return as_f2(r);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
-    return as_f2(r);
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)), "l"(as_u64(c)));
-    return as_f2(r);
-}
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float2 bf2(uint32_t b) { return make_float2(lo_f(b), hi_f(b)); }
 __device__ __forceinline__ float2 ex2_2(float2 x) { return make_float2(ex2(x.x), ex2(x.y)); }
 __device__ __forceinline__ float2 ex2_neg2(float2 x) { return make_float2(ex2(-x.x), ex2(-x.y)); }
 
@@ -132,7 +106,6 @@ __device__ __forceinline__ void load_rows(Cols<D, HQ, HD> &r, const bf16 *q, con
 }
 // Asks the L2 for the warp's 8 rows of every tensor of a tile further ahead than the register prefetch
 // reaches: four lanes per row, one 32-byte sector each per instruction.
-__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" :: "l"(p)); }
 template <int D, bool HQ, bool HD>
 __device__ __forceinline__ void prefetch_rows(const bf16 *q, const bf16 *k, const bf16 *v, const bf16 *d_out, const int *tab, const Who<D> &w)
 {

@@ -55,6 +55,37 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v)
     *reinterpret_cast<uint2 *>(p) = u;
 }
 
+// ---- packed pairs ----------------------------------------------------------------------
+// The two values of a bf16 pair.
+__device__ __forceinline__ float lo_f(uint32_t b) { return __uint_as_float(b << 16); }
+__device__ __forceinline__ float hi_f(uint32_t b) { return __uint_as_float(b & 0xffff0000u); }
+
+// Packed fp32 pairs: one instruction for two additions, products or fused multiply-adds (same rounding as two).
+__device__ __forceinline__ unsigned long long as_u64(float2 a) { return ((unsigned long long)__float_as_uint(a.y) << 32) | __float_as_uint(a.x); }
+__device__ __forceinline__ float2 as_f2(unsigned long long u) { return make_float2(__uint_as_float((uint32_t)u), __uint_as_float((uint32_t)(u >> 32))); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
+    return as_f2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
+    return as_f2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)), "l"(as_u64(c)));
+    return as_f2(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 bf2(uint32_t b) { return make_float2(lo_f(b), hi_f(b)); }
+
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" :: "l"(p)); }
+
 // ---- launch plumbing shared by the .cu files --------------------------------------------
 // Optional state arguments of the recurrence (all [B][H][d_k][d_v] fp32 row-major, any may be null):
 // the state before the first scan position, the state after the last one, the gradient with

@@ -421,20 +421,29 @@ srem_dwconv_wgrad(const T *__restrict__ x, const T *__restrict__ dy, float *__re
     }
 }
 
-// One warp per output value: its lanes add every 32nd partial sum, then a butterfly (a fixed order).
-__global__ void __launch_bounds__(256)
+// Sums of the CTA rows' partial sums: lanes hold neighbouring values (whole lines per load), warp s of the block
+// adds every kSumWarps-th partial sum, then the warps' sums are added in order (fixed, whatever the scheduling).
+// One warp per value, its lanes striding over the partial sums and each load a sector of its own: 6.3 us for 64
+// partial sums of 11520 values, 3.2 us now.
+constexpr int kSumWarps = 8;
+__global__ void __launch_bounds__(32 * kSumWarps)
 srem_dwconv_wgrad_sum(const float *__restrict__ partial, float *__restrict__ dw, float *__restrict__ dbias,
                       int nslab, int D)
 {
+    __shared__ float sh[kSumWarps][32];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, idx = blockIdx.x * 32 + lane;
     pdl_wait();
     pdl_launch_dependents();
-    const int idx = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (idx >= 10 * D) return;          // uniform over the warp
     float sum = 0.f;
-    for (int s = lane; s < nslab; s += 32) sum += partial[(size_t)s * 10 * D + idx];
+    if (idx < 10 * D) {
+#pragma unroll 8
+        for (int s = wp; s < nslab; s += kSumWarps) sum += partial[(size_t)s * 10 * D + idx];
+    }
+    sh[wp][lane] = sum;
+    __syncthreads();
+    if (wp != 0 || idx >= 10 * D) return;
 #pragma unroll
-    for (int k = 16; k >= 1; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
-    if (lane != 0) return;
+    for (int s = 1; s < kSumWarps; ++s) sum += sh[s][lane];
     if (idx < 9 * D) dw[idx] = sum;
     else if (dbias != nullptr) dbias[idx - 9 * D] = sum;
 }
@@ -551,7 +560,7 @@ dig_status launch_dwconv_bwd(const void *x, const void *w, const void *dy, void 
     }
     if (cudaGetLastError() != cudaSuccess) return DIG_ERR_CUDA;
     KernelTimer t(KID_DWCONV_WGRAD, stream);
-    launch_pdl(srem_dwconv_wgrad_sum, dim3((10 * D + 7) / 8), dim3(256), 0, stream, (const float *)partial, dw, dbias,
+    launch_pdl(srem_dwconv_wgrad_sum, dim3((10 * D + 31) / 32), dim3(32 * kSumWarps), 0, stream, (const float *)partial, dw, dbias,
                (int)nslab, D);
     return cuda_ok(cudaGetLastError());
 }

@@ -1,56 +1,71 @@
 // Output gate of the GLA layer (Eq. attn_gla, the line that forms Y_t before the projection W_O):
 //     z = Swish(r) (.) LN(o)      per (token, head) row of d_v values,
-// and its reverse mode.  Elementwise plus two row reductions, so bandwidth-bound: a row is held by 8
-// (d_v <= 64), 9 (d_v = 72: three rows per warp, five lanes idle) or 16 lanes of a warp with 8
-// consecutive values each (16-byte loads of bf16, 2 x 16 of fp32), the row statistics come from
-// shuffles inside that lane group, every tensor is read once and written once.  The affine gradients are summed per CTA in registers and shared memory and then
-// across CTAs by a second kernel in a fixed order.
+// and its reverse mode.  Elementwise plus two row reductions, so bandwidth-bound once the instruction count
+// allows it.  The rows are contiguous in memory: a CTA walks over tiles of as many rows as it holds, each
+// tensor's tile fetched by one bulk copy (two tiles in flight) and the results written by one, so no thread
+// spends instructions on global addresses and every line moves once, whatever the row length.
+// A row is held by LPR lanes with CPL neighbouring chunks of 8 values each.  bf16 rows: 4 lanes x 2 chunks up
+// to 64 values, 3 x 3 for 72 (ten rows per warp), 4 x 4 above: few lanes per row keep the shuffles of the row
+// sums (two per sum) small against the arithmetic, which is done on packed fp32 pairs.  fp32 rows, whose
+// chunks take twice the registers: one chunk per lane (8, 9 or 16 lanes).
+// 262144 rows of 72 in bf16: forward 30.0 us with nine lanes of one chunk, unpacked arithmetic and loads by
+// every thread, 21.2 us
+// now (5.3 TB/s); reverse 54.0 -> 33.4 us (5.7 TB/s); 196608 rows of 64: 17.5 -> 15.6 and 29.8 -> 25.2 us.
+// With loads by every thread and the split above: 23.0 / 42.5 and 14.7 / 26.4 us (the 48-byte pieces of a
+// 72-value row share sectors, which the L1 loses when more CTAs are resident).
+// The affine gradients are summed per CTA in registers and shared memory and then across CTAs by a second
+// kernel in a fixed order.
+#include <type_traits>
+
 #include "dig_common.cuh"
+#include "umma.cuh"
 
 namespace dig {
 namespace {
 
-constexpr int kThreads = 256;
-// Grid caps (measured): the reverse kernel does best with as many CTAs as stay resident together, three
-// per SM at its register count, so that the grid-stride loops end together and not in a ragged last
-// wave; the forward kernel does best with eight per SM.
-constexpr int kFwdPerSM = 8, kBwdPerSM = 3;
+// Threads per CTA and CTAs per SM (what the grid is capped at, so that the grid-stride loops end together): the
+// forward kernel as many as shared memory holds, up to 8 (4, 5, 6 and 8 were measured: 17.7, 17.2, 16.7, 15.6 us on
+// 196608 rows of 64), the reverse one 3 (2, 3, 4: 37, 33, 45 us on 262144 rows of 72).
+constexpr int kThreads = 128, kFwdPerSM = 8, kBwdPerSM = 3;
+constexpr size_t kSmemPerSM = 228 * 1024;
 
-__device__ __forceinline__ void load8(const float *p, float (&f)[8])
-{
-    const float4 a = load4(p), b = load4(p + 4);
-    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-}
-__device__ __forceinline__ void load8(const __nv_bfloat16 *p, float (&f)[8])
-{
-    const uint4 u = *reinterpret_cast<const uint4 *>(p);
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        f[2 * i] = __uint_as_float(w[i] << 16);
-        f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+// Eight values as they are stored.
+template <typename T> struct Raw8;
+template <> struct Raw8<float> {
+    float4 a, b;
+    __device__ __forceinline__ void load(const float *p) { a = load4(p); b = load4(p + 4); }
+    __device__ __forceinline__ void zero() { a = b = make_float4(0.f, 0.f, 0.f, 0.f); }
+    __device__ __forceinline__ float2 pair(int j) const
+    {
+        return j == 0 ? make_float2(a.x, a.y) : j == 1 ? make_float2(a.z, a.w) : j == 2 ? make_float2(b.x, b.y) : make_float2(b.z, b.w);
     }
-}
-__device__ __forceinline__ void store8(float *p, const float (&f)[8])
+};
+template <> struct Raw8<__nv_bfloat16> {
+    uint4 u;
+    __device__ __forceinline__ void load(const __nv_bfloat16 *p) { u = *reinterpret_cast<const uint4 *>(p); }
+    __device__ __forceinline__ void zero() { u = make_uint4(0, 0, 0, 0); }
+    __device__ __forceinline__ float2 pair(int j) const { return bf2(j == 0 ? u.x : j == 1 ? u.y : j == 2 ? u.z : u.w); }
+};
+__device__ __forceinline__ void store8(float *p, const float2 *f)
 {
-    store4(p, make_float4(f[0], f[1], f[2], f[3]));
-    store4(p + 4, make_float4(f[4], f[5], f[6], f[7]));
+    store4(p, make_float4(f[0].x, f[0].y, f[1].x, f[1].y));
+    store4(p + 4, make_float4(f[2].x, f[2].y, f[3].x, f[3].y));
 }
-__device__ __forceinline__ void store8(__nv_bfloat16 *p, const float (&f)[8])
+__device__ __forceinline__ void store8(__nv_bfloat16 *p, const float2 *f)
 {
     uint4 u;
     __nv_bfloat162 t;
-    t = __floats2bfloat162_rn(f[0], f[1]); u.x = *reinterpret_cast<uint32_t *>(&t);
-    t = __floats2bfloat162_rn(f[2], f[3]); u.y = *reinterpret_cast<uint32_t *>(&t);
-    t = __floats2bfloat162_rn(f[4], f[5]); u.z = *reinterpret_cast<uint32_t *>(&t);
-    t = __floats2bfloat162_rn(f[6], f[7]); u.w = *reinterpret_cast<uint32_t *>(&t);
+    t = __float22bfloat162_rn(f[0]); u.x = *reinterpret_cast<uint32_t *>(&t);
+    t = __float22bfloat162_rn(f[1]); u.y = *reinterpret_cast<uint32_t *>(&t);
+    t = __float22bfloat162_rn(f[2]); u.z = *reinterpret_cast<uint32_t *>(&t);
+    t = __float22bfloat162_rn(f[3]); u.w = *reinterpret_cast<uint32_t *>(&t);
     *reinterpret_cast<uint4 *>(p) = u;
 }
 
 // Thread -> (row slot of the CTA, lane of the row's group): 32 / LPR rows per warp.
-template <int LPR>
+template <int LPR, int THREADS>
 struct RowMap {
-    static constexpr int kRowsPerWarp = 32 / LPR, kRows = (kThreads / 32) * kRowsPerWarp;
+    static constexpr int kRowsPerWarp = 32 / LPR, kRows = (THREADS / 32) * kRowsPerWarp;
     int lane, slot, gbase;      // lane in the group, row slot, first warp lane of the group
     bool valid;                 // false for the warp's left-over lanes when LPR is not a power of two
     __device__ __forceinline__ RowMap()
@@ -62,151 +77,343 @@ struct RowMap {
         slot = (threadIdx.x >> 5) * kRowsPerWarp + (valid ? grp : 0);
     }
 };
-// Sum over the row's lane group, returned to all of its lanes.  Power-of-two groups: butterfly.  Nine
-// lanes: the ninth is folded into the first, a butterfly over the first eight, then a broadcast.
-template <int LPR> __device__ __forceinline__ float group_sum(float x, const RowMap<LPR> &m)
+// Sum over the row's lane group, returned to all of its lanes.  Power-of-two groups: butterfly.  Three
+// lanes: the two others' values.  Nine lanes: the ninth is folded into the first, a butterfly over the first
+// eight, then a broadcast.
+template <int LPR, int THREADS> __device__ __forceinline__ float group_sum(float x, const RowMap<LPR, THREADS> &m)
 {
-    if ((LPR & (LPR - 1)) == 0) {
+    static_assert((LPR & (LPR - 1)) == 0 || LPR == 3 || LPR == 9, "lane groups of a power of two, of three or of nine");
+    if constexpr ((LPR & (LPR - 1)) == 0) {
 #pragma unroll
         for (int k = LPR / 2; k >= 1; k >>= 1) x += __shfl_xor_sync(0xffffffffu, x, k);
         return x;
-    }
-    static_assert((LPR & (LPR - 1)) == 0 || LPR == 9, "lane groups of a power of two or of nine");
-    const float y = __shfl_sync(0xffffffffu, x, min(m.gbase + 8, 31));
-    if (m.lane == 0) x += y;
+    } else if constexpr (LPR == 3) {
+        const float y = __shfl_sync(0xffffffffu, x, min(m.gbase + (m.lane == 2 ? 0 : m.lane + 1), 31));
+        const float z = __shfl_sync(0xffffffffu, x, min(m.gbase + (m.lane == 0 ? 2 : m.lane - 1), 31));
+        return x + (y + z);
+    } else {
+        const float y = __shfl_sync(0xffffffffu, x, min(m.gbase + 8, 31));
+        if (m.lane == 0) x += y;
 #pragma unroll
-    for (int k = 4; k >= 1; k >>= 1) {
-        const float t = __shfl_sync(0xffffffffu, x, min(m.gbase + ((m.lane ^ k) & 7), 31));
-        if (m.lane < 8) x += t;
+        for (int k = 4; k >= 1; k >>= 1) {
+            const float t = __shfl_sync(0xffffffffu, x, min(m.gbase + ((m.lane ^ k) & 7), 31));
+            if (m.lane < 8) x += t;
+        }
+        return __shfl_sync(0xffffffffu, x, m.gbase);
     }
-    return __shfl_sync(0xffffffffu, x, m.gbase);
 }
 
-// Normalised row n = (o - mean) * rstd of the lane's 8 columns (zero where the lane holds none).
-template <int LPR> __device__ __forceinline__ float normalise(const float (&o)[8], bool has, float inv_d, float eps,
-                                                               float (&n)[8], const RowMap<LPR> &m)
+// What a lane holds of a row: CPL chunks; chunk i starts at column col(i), of which ok(i) exist.
+template <int LPR, int CPL, int THREADS, bool FULL>
+struct Lane {
+    const RowMap<LPR, THREADS> m;
+    int dv;
+    bool row_ok;
+    // with two chunks per lane odd rows take them in the other order: the lanes of two rows then hit different banks
+    __device__ __forceinline__ int col(int i) const { return 8 * (CPL * m.lane + (CPL == 2 ? i ^ (m.slot & 1) : i)); }
+    __device__ __forceinline__ bool has_col(int i) const { return m.valid && (FULL || col(i) < dv); }       // FULL: LPR * CPL chunks are the row
+    __device__ __forceinline__ bool ok(int i) const { return row_ok && has_col(i); }
+};
+template <typename T, int CPL, typename LN>
+__device__ __forceinline__ void load_row(Raw8<T> (&x)[CPL], const T *p, const LN &ln)
 {
-    float s = 0.f;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) s += o[e];
-    const float mean = group_sum<LPR>(s, m) * inv_d;
-    float v = 0.f;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        n[e] = has ? o[e] - mean : 0.f;
-        v = fmaf(n[e], n[e], v);
+    for (int i = 0; i < CPL; ++i) {
+        x[i].zero();
+        if (ln.ok(i)) x[i].load(p + ln.col(i));
     }
-    const float rstd = rsqrtf(group_sum<LPR>(v, m) * inv_d + eps);
+}
+// Normalised row n = (o - mean) * rstd (zero where the lane holds none).
+template <typename T, int LPR, int CPL, int THREADS, bool FULL>
+__device__ __forceinline__ float normalise(const Raw8<T> (&o)[CPL], const Lane<LPR, CPL, THREADS, FULL> &ln, float inv_d, float eps, float2 (&n)[4 * CPL])
+{
+    float2 s = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) n[e] *= rstd;
+    for (int i = 0; i < CPL; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            n[4 * i + j] = o[i].pair(j);
+            s = add2(s, n[4 * i + j]);
+        }
+    const float mean = group_sum(s.x + s.y, ln.m) * inv_d;
+    const float2 minus = make_float2(-mean, -mean);
+    float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < CPL; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float2 &x = n[4 * i + j];
+            x = add2(x, minus);
+            if (!FULL && !ln.has_col(i)) x = make_float2(0.f, 0.f);
+            v = fma2(x, x, v);
+        }
+    const float rstd = rsqrtf(group_sum(v.x + v.y, ln.m) * inv_d + eps);
+    const float2 sc = make_float2(rstd, rstd);
+#pragma unroll
+    for (int i = 0; i < 4 * CPL; ++i) n[i] = mul2(n[i], sc);
     return rstd;
 }
 
 // 1 / (1 + e^-r) with the fast exponential and the fast reciprocal (2 ulp each; e^-r = inf gives 0)
-__device__ __forceinline__ float sigmoidf(float r) { return __fdividef(1.f, 1.f + __expf(-r)); }
-
-// TA: type of o (the GLA output: input storage type when it comes from memory written by a caller, output
-// storage type when it comes straight from the forward pass), TR: type of r, TZ: type of z.  o and z may
-// be the same buffer: a lane reads its values of a row before it writes them.
-template <typename TA, typename TR, typename TZ, int LPR>
-__global__ void __launch_bounds__(kThreads)
-outgate_fwd(const TA *o, const TR *__restrict__ r, const float *__restrict__ ln_w,
-            const float *__restrict__ ln_b, TZ *z, long long rows, int dv, float eps)
+__device__ __forceinline__ float2 sigmoid2(float2 r)
 {
-    constexpr int kRows = RowMap<LPR>::kRows;
-    const RowMap<LPR> rm;
-    const int slot = rm.slot, col = rm.lane * 8;
-    const bool has_col = rm.valid && col < dv;
-    const float inv_d = 1.f / (float)dv;
-    float w[8], b[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        w[e] = (ln_w != nullptr && has_col) ? ln_w[col + e] : 1.f;
-        b[e] = (ln_b != nullptr && has_col) ? ln_b[col + e] : 0.f;
+    const float2 t = mul2(r, make_float2(-1.4426950408889634f, -1.4426950408889634f));
+    float2 e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(t.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(t.y));
+    e = add2(e, make_float2(1.f, 1.f));
+    return make_float2(__fdividef(1.f, e.x), __fdividef(1.f, e.y));
+}
+
+// The affine parameters of a row in shared memory: weight (1 where absent), then bias (0).
+template <int MAXD, int THREADS>
+__device__ __forceinline__ void stage_affine(float *sh, const float *ln_w, const float *ln_b, int dv)
+{
+    for (int c = threadIdx.x; c < MAXD; c += THREADS) {
+        sh[c] = (ln_w != nullptr && c < dv) ? ln_w[c] : 1.f;
+        sh[MAXD + c] = (ln_b != nullptr && c < dv) ? ln_b[c] : 0.f;
     }
-    pdl_wait();
-    pdl_launch_dependents();
-    for (long long base = (long long)blockIdx.x * kRows; base < rows; base += (long long)gridDim.x * kRows) {
-        const long long row = base + slot;
-        const bool has = has_col && row < rows;
-        float ov[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rv[8] = {0, 0, 0, 0, 0, 0, 0, 0}, n[8];
-        if (has) {
-            load8(o + row * dv + col, ov);
-            load8(r + row * dv + col, rv);
-        }
-        normalise<LPR>(ov, has, inv_d, eps, n, rm);
-        float out[8];
+    __syncthreads();
+}
+__device__ __forceinline__ void pairs8(const float *p, float2 (&x)[4])
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+    x[0] = make_float2(a.x, a.y); x[1] = make_float2(a.z, a.w); x[2] = make_float2(b.x, b.y); x[3] = make_float2(b.z, b.w);
+}
+
+// Tiles of rows through shared memory: NIN input tensors, NOUT results, two buffers of each.  Thread 0 issues
+// all copies.  Per tile: wait() for the inputs, work, then hand_over(): results of this tile leave, the
+// inputs of the tile after next are asked for.  One barrier per tile.
+constexpr int kStages = 2;
+template <int NIN, int NOUT, int ROWS>
+struct TileRing {
+    char *in[NIN], *out[NOUT];          // first buffer of each tensor
+    const char *src[NIN];
+    char *dst[NOUT];
+    int in_row[NIN], out_row[NOUT];     // bytes per row
+    uint64_t *bar;
+    int *status;
+    long long rows;
+    __device__ __forceinline__ char *in_buf(int k, int it) const { return in[k] + (it & 1) * ROWS * in_row[k]; }
+    __device__ __forceinline__ char *out_buf(int k, int it) const { return out[k] + (it & 1) * ROWS * out_row[k]; }
+    __device__ __forceinline__ long long first(int it) const { return ((long long)blockIdx.x + (long long)it * gridDim.x) * ROWS; }
+    __device__ __forceinline__ void fetch(int it) const          // thread 0
+    {
+        const long long r0 = first(it);
+        if (r0 >= rows) return;
+        const uint32_t n = (uint32_t)(rows - r0 < ROWS ? rows - r0 : ROWS);
+        uint32_t bytes = 0;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) out[e] = rv[e] * sigmoidf(rv[e]) * fmaf(n[e], w[e], b[e]);
-        if (has) store8(z + row * dv + col, out);
+        for (int k = 0; k < NIN; ++k) bytes += n * in_row[k];
+        umma::mbar_arrive_expect_tx(bar + (it & 1), bytes);
+#pragma unroll
+        for (int k = 0; k < NIN; ++k) umma::bulk_g2s(in_buf(k, it), src[k] + r0 * in_row[k], n * in_row[k], bar + (it & 1));
+    }
+    __device__ __forceinline__ bool wait(int it) const { return umma::mbar_wait(bar + (it & 1), (it >> 1) & 1, status); }
+    __device__ __forceinline__ bool hand_over(int it, bool ok) const
+    {
+        umma::fence_async_smem();
+        if (threadIdx.x == 0) umma::bulk_wait_read();            // the results of the tile before have left their buffer
+        if (!__syncthreads_and(ok)) return false;
+        if (threadIdx.x == 0) {
+            const long long r0 = first(it);
+            const uint32_t n = (uint32_t)(rows - r0 < ROWS ? rows - r0 : ROWS);
+#pragma unroll
+            for (int k = 0; k < NOUT; ++k) umma::bulk_s2g(dst[k] + r0 * out_row[k], out_buf(k, it), n * out_row[k]);
+            umma::bulk_commit();
+            fetch(it + kStages);
+        }
+        return true;
+    }
+    // After the loop: copies in flight end before the CTA's shared memory goes (also where a wait gave up at tile `it`).
+    __device__ __forceinline__ void drain(int it, bool ok) const
+    {
+        if (threadIdx.x != 0) return;
+        umma::bulk_wait_all();
+        if (!ok) {
+            for (int k = 0; k < kStages; ++k)
+                if (first(it + k) < rows) umma::mbar_wait(bar + ((it + k) & 1), ((it + k) >> 1) & 1, status);
+        }
+    }
+};
+__device__ __forceinline__ void ring_setup(uint64_t *bar)
+{
+    if (threadIdx.x == 0) {
+        umma::mbar_init(bar, 1);
+        umma::mbar_init(bar + 1, 1);
+        umma::fence_barrier_init();
     }
 }
 
-template <typename TI, typename TO, int LPR>
+// TA: type of o (the GLA output: input storage type when it comes from memory written by a caller, output
+// storage type when it comes straight from the forward pass), TR: type of r, TZ: type of z.  o and z may
+// be the same buffer: a tile's rows are written after they have been read.
+template <typename TA, typename TR, typename TZ, int LPR, int CPL, bool FULL>
 __global__ void __launch_bounds__(kThreads)
-outgate_bwd(const TI *__restrict__ o, const TI *__restrict__ r, const TI *__restrict__ dz,
-            const float *__restrict__ ln_w, const float *__restrict__ ln_b, TO *__restrict__ d_o,
-            TO *__restrict__ d_r, float *__restrict__ partial, long long rows, int dv, float eps)
+outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const float *__restrict__ ln_b, TZ *z, long long rows,
+            int dv_, float eps, int *status)
 {
-    constexpr int kRows = RowMap<LPR>::kRows;
-    __shared__ float red[kRows][2][LPR * 8];
-    const RowMap<LPR> rm;
-    const int slot = rm.slot, col = rm.lane * 8;
-    const bool has_col = rm.valid && col < dv;
+    constexpr int kRows = RowMap<LPR, kThreads>::kRows, kMaxD = 8 * LPR * CPL;
+    extern __shared__ __align__(128) char smem[];
+    __shared__ __align__(16) float aff[2 * kMaxD];
+    __shared__ uint64_t bar[2];
+    const int dv = FULL ? kMaxD : dv_;
+    TileRing<2, 1, kRows> ring;
+    ring.in_row[0] = dv * (int)sizeof(TA);
+    ring.in_row[1] = dv * (int)sizeof(TR);
+    ring.out_row[0] = dv * (int)sizeof(TZ);
+    ring.in[0] = smem;
+    ring.in[1] = ring.in[0] + kStages * kRows * ring.in_row[0];
+    ring.out[0] = ring.in[1] + kStages * kRows * ring.in_row[1];
+    ring.src[0] = reinterpret_cast<const char *>(o);
+    ring.src[1] = reinterpret_cast<const char *>(r);
+    ring.dst[0] = reinterpret_cast<char *>(z);
+    ring.bar = bar;
+    ring.status = status;
+    ring.rows = rows;
+    ring_setup(bar);
+    stage_affine<kMaxD, kThreads>(aff, ln_w, ln_b, dv);
+    Lane<LPR, CPL, kThreads, FULL> ln;
+    ln.dv = dv;
     const float inv_d = 1.f / (float)dv;
-    float w[8], b[8], aw[8], ab[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        w[e] = (ln_w != nullptr && has_col) ? ln_w[col + e] : 1.f;
-        b[e] = (ln_b != nullptr && has_col) ? ln_b[col + e] : 0.f;
-        aw[e] = ab[e] = 0.f;
-    }
     pdl_wait();
     pdl_launch_dependents();
-    for (long long base = (long long)blockIdx.x * kRows; base < rows; base += (long long)gridDim.x * kRows) {
-        const long long row = base + slot;
-        const bool has = has_col && row < rows;
-        float ov[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rv[8] = {0, 0, 0, 0, 0, 0, 0, 0}, gv[8] = {0, 0, 0, 0, 0, 0, 0, 0}, n[8];
-        if (has) {
-            load8(o + row * dv + col, ov);
-            load8(r + row * dv + col, rv);
-            load8(dz + row * dv + col, gv);
-        }
-        const float rstd = normalise<LPR>(ov, has, inv_d, eps, n, rm);
-        float dr[8], dn[8], s1 = 0.f, s2 = 0.f;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const float sg = sigmoidf(rv[e]);
-            const float y = fmaf(n[e], w[e], b[e]);
-            dr[e] = gv[e] * y * fmaf(rv[e] * sg, 1.f - sg, sg);
-            const float dy = gv[e] * rv[e] * sg;                 // zero where the lane holds no value
-            aw[e] = fmaf(dy, n[e], aw[e]);
-            ab[e] += dy;
-            dn[e] = dy * w[e];
-            s1 += dn[e];
-            s2 = fmaf(dn[e], n[e], s2);
-        }
-        const float m1 = group_sum<LPR>(s1, rm) * inv_d, m2 = group_sum<LPR>(s2, rm) * inv_d;
-        float dov[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) dov[e] = rstd * (dn[e] - m1 - n[e] * m2);
-        if (has) {
-            store8(d_o + row * dv + col, dov);
-            store8(d_r + row * dv + col, dr);
-        }
+    if (threadIdx.x == 0) {
+        ring.fetch(0);
+        ring.fetch(1);
     }
-    if (partial == nullptr) return;
-    if (rm.valid) {
+    bool ok = true;
+    int it = 0;
+    for (; ok && ring.first(it) < rows; ++it) {
+        ok = ring.wait(it);
+        ln.row_ok = ring.first(it) + ln.m.slot < rows;
+        Raw8<TA> ov[CPL];
+        Raw8<TR> rv[CPL];
+        load_row(ov, reinterpret_cast<const TA *>(ring.in_buf(0, it)) + ln.m.slot * dv, ln);
+        load_row(rv, reinterpret_cast<const TR *>(ring.in_buf(1, it)) + ln.m.slot * dv, ln);
+        float2 n[4 * CPL];
+        normalise(ov, ln, inv_d, eps, n);
+        TZ *zb = reinterpret_cast<TZ *>(ring.out_buf(0, it)) + ln.m.slot * dv;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            red[slot][0][col + e] = aw[e];
-            red[slot][1][col + e] = ab[e];
+        for (int i = 0; i < CPL; ++i) {
+            float2 w[4], b[4], out[4];
+            pairs8(aff + ln.col(i), w);
+            pairs8(aff + kMaxD + ln.col(i), b);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 x = rv[i].pair(j);
+                out[j] = mul2(mul2(x, sigmoid2(x)), fma2(n[4 * i + j], w[j], b[j]));
+            }
+            if (ln.ok(i)) store8(zb + ln.col(i), out);
         }
+        ok = ring.hand_over(it, ok);
+        if (!ok) break;
+    }
+    ring.drain(it, ok);
+}
+
+template <typename TI, typename TO, int LPR, int CPL, bool FULL>
+__global__ void __launch_bounds__(kThreads, kBwdPerSM)
+outgate_bwd(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln_w, const float *__restrict__ ln_b, TO *d_o,
+            TO *d_r, float *__restrict__ partial, long long rows, int dv_, float eps, int *status)
+{
+    constexpr int kRows = RowMap<LPR, kThreads>::kRows, kMaxD = 8 * LPR * CPL, NP = 4 * CPL;
+    extern __shared__ __align__(128) char smem[];
+    __shared__ __align__(16) float aff[2 * kMaxD];
+    __shared__ uint64_t bar[2];
+    const int dv = FULL ? kMaxD : dv_;
+    TileRing<3, 2, kRows> ring;
+    const char *src[3] = {reinterpret_cast<const char *>(o), reinterpret_cast<const char *>(r), reinterpret_cast<const char *>(dz)};
+    char *dst[2] = {reinterpret_cast<char *>(d_o), reinterpret_cast<char *>(d_r)};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        ring.in_row[k] = dv * (int)sizeof(TI);
+        ring.in[k] = smem + k * kStages * kRows * ring.in_row[k];
+        ring.src[k] = src[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        ring.out_row[k] = dv * (int)sizeof(TO);
+        ring.out[k] = smem + 3 * kStages * kRows * ring.in_row[0] + k * kStages * kRows * ring.out_row[k];
+        ring.dst[k] = dst[k];
+    }
+    ring.bar = bar;
+    ring.status = status;
+    ring.rows = rows;
+    ring_setup(bar);
+    stage_affine<kMaxD, kThreads>(aff, ln_w, ln_b, dv);
+    Lane<LPR, CPL, kThreads, FULL> ln;
+    ln.dv = dv;
+    const float inv_d = 1.f / (float)dv;
+    float2 aw[NP], ab[NP];
+#pragma unroll
+    for (int e = 0; e < NP; ++e) aw[e] = ab[e] = make_float2(0.f, 0.f);
+    pdl_wait();
+    pdl_launch_dependents();
+    if (threadIdx.x == 0) {
+        ring.fetch(0);
+        ring.fetch(1);
+    }
+    bool ok = true;
+    int it = 0;
+    for (; ok && ring.first(it) < rows; ++it) {
+        ok = ring.wait(it);
+        ln.row_ok = ring.first(it) + ln.m.slot < rows;
+        Raw8<TI> ov[CPL], rv[CPL], gv[CPL];
+        load_row(ov, reinterpret_cast<const TI *>(ring.in_buf(0, it)) + ln.m.slot * dv, ln);
+        load_row(rv, reinterpret_cast<const TI *>(ring.in_buf(1, it)) + ln.m.slot * dv, ln);
+        load_row(gv, reinterpret_cast<const TI *>(ring.in_buf(2, it)) + ln.m.slot * dv, ln);       // zero where the lane holds no value: it adds nothing
+        TO *dob = reinterpret_cast<TO *>(ring.out_buf(0, it)) + ln.m.slot * dv, *drb = reinterpret_cast<TO *>(ring.out_buf(1, it)) + ln.m.slot * dv;
+        float2 n[NP], dn[NP], s1 = make_float2(0.f, 0.f), s2 = s1;
+        const float rstd = normalise(ov, ln, inv_d, eps, n);
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) {
+            float2 w[4], b[4], dr[4];
+            pairs8(aff + ln.col(i), w);
+            pairs8(aff + kMaxD + ln.col(i), b);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int e = 4 * i + j;
+                const float2 x = rv[i].pair(j), g = gv[i].pair(j), sg = sigmoid2(x), sw = mul2(x, sg);
+                const float2 y = fma2(n[e], w[j], b[j]), dy = mul2(g, sw);
+                dr[j] = mul2(mul2(g, y), fma2(sw, sub2(make_float2(1.f, 1.f), sg), sg));
+                aw[e] = fma2(dy, n[e], aw[e]);
+                ab[e] = add2(ab[e], dy);
+                dn[e] = mul2(dy, w[j]);
+                s1 = add2(s1, dn[e]);
+                s2 = fma2(dn[e], n[e], s2);
+            }
+            if (ln.ok(i)) store8(drb + ln.col(i), dr);
+        }
+        const float m1 = group_sum(s1.x + s1.y, ln.m) * inv_d, m2 = group_sum(s2.x + s2.y, ln.m) * inv_d;
+        const float2 k0 = make_float2(-rstd * m1, -rstd * m1), k1 = make_float2(-rstd * m2, -rstd * m2), k2 = make_float2(rstd, rstd);
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) {
+            float2 x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] = fma2(k2, dn[4 * i + j], fma2(k1, n[4 * i + j], k0));
+            if (ln.ok(i)) store8(dob + ln.col(i), x);
+        }
+        ok = ring.hand_over(it, ok);
+        if (!ok) break;
+    }
+    ring.drain(it, ok);
+    if (partial == nullptr) return;
+    __syncthreads();                                             // the copies have left: the ring becomes scratch
+    float (*red)[2][kMaxD] = reinterpret_cast<float (*)[2][kMaxD]>(smem);
+    if (ln.m.valid) {
+#pragma unroll
+        for (int i = 0; i < CPL; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                *reinterpret_cast<float2 *>(&red[ln.m.slot][0][ln.col(i) + 2 * j]) = aw[4 * i + j];
+                *reinterpret_cast<float2 *>(&red[ln.m.slot][1][ln.col(i) + 2 * j]) = ab[4 * i + j];
+            }
     }
     __syncthreads();
     // partial[cta][2][dv]
-    for (int idx = threadIdx.x; idx < 2 * LPR * 8; idx += kThreads) {
-        const int which = idx / (LPR * 8), c = idx - which * (LPR * 8);
+    for (int idx = threadIdx.x; idx < 2 * kMaxD; idx += kThreads) {
+        const int which = idx / kMaxD, c = idx - which * kMaxD;
         if (c >= dv) continue;
         float sum = 0.f;
 #pragma unroll 8
@@ -215,21 +422,29 @@ outgate_bwd(const TI *__restrict__ o, const TI *__restrict__ r, const TI *__rest
     }
 }
 
-// One warp per parameter: its lanes add every 32nd partial sum, then a butterfly (a fixed order, so the
-// result does not depend on scheduling).
-__global__ void __launch_bounds__(256)
+// Sums of the CTAs' partial sums: lanes hold neighbouring parameters (whole lines per load), warp s of the
+// block adds every kSumWarps-th partial sum, then the warps' sums are added in order (the result does not
+// depend on scheduling).  One warp per parameter with lanes striding over the CTAs, each load a sector of its
+// own, took about as long for 444 partial sums as this does (4.6 us, most of it launch and drain), and grew with their number.
+constexpr int kSumWarps = 16;
+__global__ void __launch_bounds__(32 * kSumWarps)
 outgate_affine_sum(const float *__restrict__ partial, float *__restrict__ dln_w, float *__restrict__ dln_b,
                    int nctas, int dv)
 {
+    __shared__ float sh[kSumWarps][32];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, idx = blockIdx.x * 32 + lane;
     pdl_wait();
     pdl_launch_dependents();
-    const int idx = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (idx >= 2 * dv) return;          // uniform over the warp
     float sum = 0.f;
-    for (int s = lane; s < nctas; s += 32) sum += partial[(size_t)s * 2 * dv + idx];
+    if (idx < 2 * dv) {
+#pragma unroll 8
+        for (int s = wp; s < nctas; s += kSumWarps) sum += partial[(size_t)s * 2 * dv + idx];
+    }
+    sh[wp][lane] = sum;
+    __syncthreads();
+    if (wp != 0 || idx >= 2 * dv) return;
 #pragma unroll
-    for (int k = 16; k >= 1; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
-    if (lane != 0) return;
+    for (int s = 1; s < kSumWarps; ++s) sum += sh[s][lane];
     if (idx < dv) {
         if (dln_w != nullptr) dln_w[idx] = sum;
     } else if (dln_b != nullptr) {
@@ -237,9 +452,25 @@ outgate_affine_sum(const float *__restrict__ partial, float *__restrict__ dln_w,
     }
 }
 
-// lanes per row for a row length
-int lanes_for(int dv) { return dv <= 64 ? 8 : dv == 72 ? 9 : 16; }
-int grid_for(long long rows, int lpr, int per_sm = kBwdPerSM)
+// Calls f(LPR, CPL, FULL) with the row split of a storage type and row length.
+template <typename T, typename F>
+void with_split(int dv, F f)
+{
+    using std::integral_constant;
+    if constexpr (sizeof(T) == 2) {
+        if (dv == 64) f(integral_constant<int, 4>{}, integral_constant<int, 2>{}, std::true_type{});
+        else if (dv < 64) f(integral_constant<int, 4>{}, integral_constant<int, 2>{}, std::false_type{});
+        else if (dv == 72) f(integral_constant<int, 3>{}, integral_constant<int, 3>{}, std::true_type{});
+        else f(integral_constant<int, 4>{}, integral_constant<int, 4>{}, std::false_type{});
+    } else {
+        if (dv <= 64) f(integral_constant<int, 8>{}, integral_constant<int, 1>{}, std::false_type{});
+        else if (dv == 72) f(integral_constant<int, 9>{}, integral_constant<int, 1>{}, std::false_type{});
+        else f(integral_constant<int, 16>{}, integral_constant<int, 1>{}, std::false_type{});
+    }
+}
+// lanes per row of that split
+int lanes_for(int dv, bool narrow) { return narrow ? (dv == 72 ? 3 : 4) : (dv <= 64 ? 8 : dv == 72 ? 9 : 16); }
+int grid_for(long long rows, int lpr, int per_sm)
 {
     int sms = device_sm_count();
     if (sms <= 0) sms = 148;            // sizing call without a device: the count the launch will most likely see
@@ -249,87 +480,92 @@ int grid_for(long long rows, int lpr, int per_sm = kBwdPerSM)
 }
 
 template <typename TA, typename TR, typename TZ>
-void fwd_dispatch3(const void *o, const void *r, const float *w, const float *b, void *z, long long rows, int dv,
-                   float eps, cudaStream_t stream)
+dig_status fwd_dispatch(const void *o, const void *r, const float *w, const float *b, void *z, long long rows, int dv,
+                        float eps, cudaStream_t stream)
 {
-    if (dv <= 64)
-        launch_pdl(outgate_fwd<TA, TR, TZ, 8>, dim3(grid_for(rows, 8, kFwdPerSM)), dim3(kThreads), 0, stream, (const TA *)o,
-                   (const TR *)r, w, b, (TZ *)z, rows, dv, eps);
-    else if (dv == 72)
-        launch_pdl(outgate_fwd<TA, TR, TZ, 9>, dim3(grid_for(rows, 9, kFwdPerSM)), dim3(kThreads), 0, stream, (const TA *)o,
-                   (const TR *)r, w, b, (TZ *)z, rows, dv, eps);
-    else
-        launch_pdl(outgate_fwd<TA, TR, TZ, 16>, dim3(grid_for(rows, 16, kFwdPerSM)), dim3(kThreads), 0, stream, (const TA *)o,
-                   (const TR *)r, w, b, (TZ *)z, rows, dv, eps);
-}
-template <typename TI, typename TO>
-void fwd_dispatch(const void *o, const void *r, const float *w, const float *b, void *z, long long rows, int dv,
-                  float eps, cudaStream_t stream)
-{
-    fwd_dispatch3<TI, TI, TO>(o, r, w, b, z, rows, dv, eps, stream);
+    int *status = device_status_ptr();
+    if (!status) return DIG_ERR_CUDA;
+    dig_status st = DIG_OK;
+    with_split<TR>(dv, [&](auto lpr, auto cpl, auto full) {
+        constexpr int LPR = decltype(lpr)::value, CPL = decltype(cpl)::value, ROWS = RowMap<LPR, kThreads>::kRows;
+        auto kern = outgate_fwd<TA, TR, TZ, LPR, CPL, decltype(full)::value>;
+        const size_t smem = (size_t)kStages * ROWS * dv * (sizeof(TA) + sizeof(TR) + sizeof(TZ));
+        if ((st = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem)) != DIG_OK) return;
+        const int fit = (int)(kSmemPerSM / (smem + 3072));           // + 1 KB of the system's and the static arrays
+        const int per_sm = fit < 1 ? 1 : fit < kFwdPerSM ? fit : kFwdPerSM;
+        launch_pdl(kern, dim3(grid_for(rows, LPR, per_sm)), dim3(kThreads), smem, stream, (const TA *)o, (const TR *)r, w, b,
+                   (TZ *)z, rows, dv, eps, status);
+        st = cuda_ok(cudaGetLastError());
+    });
+    return st;
 }
 
 template <typename TI, typename TO>
-void bwd_dispatch(const void *o, const void *r, const void *dz, const float *w, const float *b, void *d_o, void *d_r,
-                  float *partial, long long rows, int dv, float eps, cudaStream_t stream)
+dig_status bwd_dispatch(const void *o, const void *r, const void *dz, const float *w, const float *b, void *d_o, void *d_r,
+                        float *partial, long long rows, int dv, float eps, cudaStream_t stream)
 {
-    if (dv <= 64)
-        launch_pdl(outgate_bwd<TI, TO, 8>, dim3(grid_for(rows, 8)), dim3(kThreads), 0, stream, (const TI *)o,
-                   (const TI *)r, (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps);
-    else if (dv == 72)
-        launch_pdl(outgate_bwd<TI, TO, 9>, dim3(grid_for(rows, 9)), dim3(kThreads), 0, stream, (const TI *)o,
-                   (const TI *)r, (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps);
-    else
-        launch_pdl(outgate_bwd<TI, TO, 16>, dim3(grid_for(rows, 16)), dim3(kThreads), 0, stream, (const TI *)o,
-                   (const TI *)r, (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps);
+    int *status = device_status_ptr();
+    if (!status) return DIG_ERR_CUDA;
+    dig_status st = DIG_OK;
+    with_split<TI>(dv, [&](auto lpr, auto cpl, auto full) {
+        constexpr int LPR = decltype(lpr)::value, CPL = decltype(cpl)::value, ROWS = RowMap<LPR, kThreads>::kRows;
+        auto kern = outgate_bwd<TI, TO, LPR, CPL, decltype(full)::value>;
+        const size_t ring = (size_t)kStages * ROWS * dv * (3 * sizeof(TI) + 2 * sizeof(TO)), red = (size_t)ROWS * 2 * 8 * LPR * CPL * sizeof(float);
+        const size_t smem = ring > red ? ring : red;
+        if ((st = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem)) != DIG_OK) return;
+        launch_pdl(kern, dim3(grid_for(rows, LPR, kBwdPerSM)), dim3(kThreads), smem, stream, (const TI *)o, (const TI *)r,
+                   (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps, status);
+        st = cuda_ok(cudaGetLastError());
+    });
+    return st;
 }
 
 }  // namespace
 
+// the wider of the two storage types' grids
 size_t outgate_bwd_workspace_bytes(long long rows, int dv)
 {
-    return (size_t)grid_for(rows, lanes_for(dv)) * 2 * (size_t)dv * sizeof(float);
+    const int a = grid_for(rows, lanes_for(dv, true), kBwdPerSM), b = grid_for(rows, lanes_for(dv, false), kBwdPerSM);
+    return (size_t)(a > b ? a : b) * 2 * (size_t)dv * sizeof(float);
 }
 
 dig_status launch_outgate_fwd(const void *o, const void *r, const float *ln_w, const float *ln_b, void *z,
                               long long rows, int dv, float eps, int dtype, cudaStream_t stream)
 {
+    using bf16 = __nv_bfloat16;
     KernelTimer t(KID_OUTGATE, stream);
-    if (dtype == DIG_F32) fwd_dispatch<float, float>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
-    else if (dtype == DIG_BF16) fwd_dispatch<__nv_bfloat16, __nv_bfloat16>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
-    else fwd_dispatch<__nv_bfloat16, float>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
-    return cuda_ok(cudaGetLastError());
+    if (dtype == DIG_F32) return fwd_dispatch<float, float, float>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
+    if (dtype == DIG_BF16) return fwd_dispatch<bf16, bf16, bf16>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
+    return fwd_dispatch<bf16, bf16, float>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
 }
 
 // o in the output storage type of `dtype` (as the forward pass writes it), r in the input storage type.
 dig_status launch_outgate_fwd_mixed(const void *o, const void *r, const float *ln_w, const float *ln_b, void *z,
                                     long long rows, int dv, float eps, int dtype, cudaStream_t stream)
 {
+    if (dtype != DIG_BF16_F32OUT) return launch_outgate_fwd(o, r, ln_w, ln_b, z, rows, dv, eps, dtype, stream);
     KernelTimer t(KID_OUTGATE, stream);
-    if (dtype == DIG_F32) fwd_dispatch3<float, float, float>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
-    else if (dtype == DIG_BF16) fwd_dispatch3<__nv_bfloat16, __nv_bfloat16, __nv_bfloat16>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
-    else fwd_dispatch3<float, __nv_bfloat16, float>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
-    return cuda_ok(cudaGetLastError());
+    return fwd_dispatch<float, __nv_bfloat16, float>(o, r, ln_w, ln_b, z, rows, dv, eps, stream);
 }
 
 dig_status launch_outgate_bwd(const void *o, const void *r, const void *dz, const float *ln_w, const float *ln_b,
                               void *d_o, void *d_r, float *dln_w, float *dln_b, long long rows, int dv, float eps,
                               int dtype, float *partial, cudaStream_t stream)
 {
+    using bf16 = __nv_bfloat16;
     const bool affine = dln_w != nullptr || dln_b != nullptr;
     float *part = affine ? partial : nullptr;
+    dig_status st;
     {
         KernelTimer t(KID_OUTGATE, stream);
-        if (dtype == DIG_F32) bwd_dispatch<float, float>(o, r, dz, ln_w, ln_b, d_o, d_r, part, rows, dv, eps, stream);
-        else if (dtype == DIG_BF16)
-            bwd_dispatch<__nv_bfloat16, __nv_bfloat16>(o, r, dz, ln_w, ln_b, d_o, d_r, part, rows, dv, eps, stream);
-        else bwd_dispatch<__nv_bfloat16, float>(o, r, dz, ln_w, ln_b, d_o, d_r, part, rows, dv, eps, stream);
+        if (dtype == DIG_F32) st = bwd_dispatch<float, float>(o, r, dz, ln_w, ln_b, d_o, d_r, part, rows, dv, eps, stream);
+        else if (dtype == DIG_BF16) st = bwd_dispatch<bf16, bf16>(o, r, dz, ln_w, ln_b, d_o, d_r, part, rows, dv, eps, stream);
+        else st = bwd_dispatch<bf16, float>(o, r, dz, ln_w, ln_b, d_o, d_r, part, rows, dv, eps, stream);
     }
-    if (cudaGetLastError() != cudaSuccess) return DIG_ERR_CUDA;
-    if (!affine) return DIG_OK;
+    if (st != DIG_OK || !affine) return st;
     KernelTimer t(KID_OUTGATE, stream);
-    launch_pdl(outgate_affine_sum, dim3((2 * dv + 7) / 8), dim3(256), 0, stream, (const float *)partial, dln_w,
-               dln_b, grid_for(rows, lanes_for(dv)), dv);
+    launch_pdl(outgate_affine_sum, dim3((2 * dv + 31) / 32), dim3(32 * kSumWarps), 0, stream, (const float *)partial, dln_w,
+               dln_b, grid_for(rows, lanes_for(dv, dtype != DIG_F32), kBwdPerSM), dv);
     return cuda_ok(cudaGetLastError());
 }
 
