@@ -60,10 +60,12 @@ struct Who {
     int grp, c2;            // row group (warp), first channel of the pair
     int xrow, xc2;          // extra item: row inside the group, first channel
     int q4, cg, hf, r16;    // tensor-memory lane quarter, warp of the quarter (0 / 1), lane half, accumulator row (M = 64)
+    // The last warp issues the MMAs and the bulk copies (under elect_one()).
+    __device__ __forceinline__ bool issuer() const { return grp == Col<D>::NT / 32 - 1; }
     __device__ __forceinline__ Who()
     {
         const int lane = threadIdx.x & 31;
-        grp = threadIdx.x >> 5;
+        grp = (int)warp_uniform(threadIdx.x >> 5);
         c2 = 2 * lane;
         xrow = lane >> 2;
         xc2 = 64 + 2 * (lane & 3);

@@ -25,7 +25,7 @@
 // dO Sc^T = dO Sc_local^T + (dO S_segment^T) diag(exp(c) G): two products and one fused multiply-add.
 //
 // Every product is a tcgen05.mma (kind::f16, fp16 operands, fp32 accumulators in tensor memory) issued by
-// lane 0 of the last warp, which otherwise works like the others: all threads build operand tiles, mask the
+// one thread of the last warp, which otherwise works like the others: all threads build operand tiles, mask the
 // scores and post-process accumulators, phase by phase (columns.cuh holds the work split).  Rows of the
 // next tile are prefetched into registers; two CTAs of 256 threads share an SM, so one builds while the
 // other's products are in the tensor pipe.
@@ -119,7 +119,6 @@ sweep_local_fwd(const SweepArgs a)
     using C = Cfg<D>;
     using L = Col<D>;
     using SM = LocalFwdSmem<D>;
-    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs
     extern __shared__ __align__(128) char smem[];
     float *sTot = reinterpret_cast<float *>(smem + 2 * SM::kBuf + SM::kPad);
     int *rowOff = reinterpret_cast<int *>(sTot + 2 * 8 * D);          // ring of four tiles
@@ -128,7 +127,7 @@ sweep_local_fwd(const SweepArgs a)
     const int tid = threadIdx.x;
     cta_setup(ctl, 2, SM::tmem_cols, smem, 2 * SM::kBuf + SM::kPad);
     const Who<D> w;
-    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
+    const uint32_t tmem = warp_uniform(ctl->tmem_base), tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     const Geom &g = a.g;
     const Plan &pl = a.plan;
     Cols<D, false, false> raw;
@@ -164,7 +163,7 @@ sweep_local_fwd(const SweepArgs a)
         for (int tile = t1 - 1; tile >= t0; --tile, ++it) {
             tc_fence_before_sync();
             SYNC_OR_DIE();
-            if (tid == kIssuer && tile < t1 - 1) {                    // the tile before is built
+            if (w.issuer() && tile < t1 - 1 && elect_one()) {                    // the tile before is built
                 char *tK = smem + ((it + 1) & 1) * SM::kBuf;
                 tc_fence_after_sync();
                 issue_state<D>(tmem, tK, tK + C::TILE_T, tile < t1 - 2);
@@ -201,7 +200,7 @@ sweep_local_fwd(const SweepArgs a)
         }
         tc_fence_before_sync();
         SYNC_OR_DIE();
-        if (tid == kIssuer) {
+        if (w.issuer() && elect_one()) {
             char *tK = smem + ((it + 1) & 1) * SM::kBuf;
             tc_fence_after_sync();
             issue_state<D>(tmem, tK, tK + C::TILE_T, t1 - t0 > 1);
@@ -248,7 +247,6 @@ sweep_local_bwd(const SweepArgs a)
     using C = Cfg<D>;
     using L = Col<D>;
     using SM = LocalBwdSmem<D, GRAD>;
-    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs
     extern __shared__ __align__(128) char smem[];
     float *sTot = reinterpret_cast<float *>(smem + 2 * SM::kBuf + SM::kPad);
     int *rowOff = reinterpret_cast<int *>(sTot + 2 * 8 * D);          // ring of four tiles
@@ -258,7 +256,7 @@ sweep_local_bwd(const SweepArgs a)
     cta_setup(ctl, 2, SM::tmem_cols, smem, 2 * SM::kBuf + SM::kPad);
     const Who<D> w;
     const StateOf<D> sm(w);
-    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
+    const uint32_t tmem = warp_uniform(ctl->tmem_base), tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     const Geom &g = a.g;
     const Plan &pl = a.plan;
     float S[L::NPS][8];
@@ -339,7 +337,7 @@ sweep_local_bwd(const SweepArgs a)
                 fence_async_smem();
                 tc_fence_before_sync();
                 __syncthreads();
-                if (tid == kIssuer) {
+                if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
                     issue_state<D>(tmem + (it & 1) * L::ACCS, tK, tV);                             // Kc^T V
                     if (GRAD) issue_state<D>(tmem + SM::aW, tQ, tG, pending);                      // + (q decayed)^T dO
@@ -519,7 +517,6 @@ sweep_fwd(const SweepArgs a)
     using C = Cfg<D>;
     using L = Col<D>;
     using SM = FwdSmem<D>;
-    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs
     extern __shared__ __align__(128) char smem[];
     char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tS = tV + C::TILE_T, *tP = tS + C::TILE_S;
     float *sTot = reinterpret_cast<float *>(smem + SM::kTiles);
@@ -530,7 +527,7 @@ sweep_fwd(const SweepArgs a)
     cta_setup(ctl, 1, SM::tmem_cols, smem, SM::kTiles);
     const Who<D> w;
     const StateOf<D> sm(w);
-    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
+    const uint32_t tmem = warp_uniform(ctl->tmem_base), tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     const Geom &g = a.g;
     const Plan &pl = a.plan;
     float S[L::NPS][8];
@@ -599,7 +596,7 @@ sweep_fwd(const SweepArgs a)
                 fence_async_smem();
                 tc_fence_before_sync();
                 __syncthreads();
-                if (tid == kIssuer) {
+                if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
                     issue_scores<D>(tmem + SM::aP, tQ, tK);                                       // Qc Kc^T
                     mma_commit(&ctl->bar[0]);
@@ -629,7 +626,7 @@ sweep_fwd(const SweepArgs a)
                 fence_async_smem();
                 tc_fence_before_sync();
                 __syncthreads();
-                if (tid == kIssuer) {
+                if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
                     issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);                  // + P V
                     mma_commit(&ctl->bar[0]);
@@ -705,7 +702,6 @@ sweep_bwd(const SweepArgs a)
     using C = Cfg<D>;
     using L = Col<D>;
     using SM = BwdSmem<D>;
-    constexpr int NT = L::NT, kIssuer = NT - 32;        // lane 0 of the last warp issues the MMAs and the bulk copies
     extern __shared__ __align__(128) char smem[];
     char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T, *tD = tG + C::TILE_T;
     char *tP = tV + SM::kRegion, *tdP = tP + C::TILE_P, *tS = tdP + C::TILE_P, *tI = tS + C::TILE_S;
@@ -718,7 +714,7 @@ sweep_bwd(const SweepArgs a)
     cta_setup(ctl, 2, SM::tmem_cols, smem, SM::kTiles);
     const Who<D> w;
     const StateOf<D> sm(w);
-    const uint32_t tmem = ctl->tmem_base, tl = tmem + ((uint32_t)(32 * w.q4) << 16);
+    const uint32_t tmem = warp_uniform(ctl->tmem_base), tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     uint64_t *barG1 = &ctl->bar[0], *barS = &ctl->bar[1];
     const Geom &g = a.g;
     const Plan &pl = a.plan;
@@ -759,7 +755,7 @@ sweep_bwd(const SweepArgs a)
             if (L::X) xcarry = *reinterpret_cast<const float2 *>(a.seg_carry + (size_t)sid * D + w.xc2);
         }
         if (sid != (int)blockIdx.x) prime(sid);
-        if (tid == kIssuer) {
+        if (w.issuer() && elect_one()) {
             // the zero-start state of the sub-chunk worked first (always slot 0 of its tile) and, once per
             // segment, the state entering the segment; later sub-chunks' states are fetched as soon as the
             // products of the one before are done
@@ -806,7 +802,7 @@ sweep_bwd(const SweepArgs a)
                 fence_async_smem();
                 tc_fence_before_sync();
                 __syncthreads();
-                if (tid == kIssuer) {
+                if (w.issuer() && elect_one()) {
                     ok = mbar_wait(barS, par, a.status) && ok;         // the state tiles have landed
                     tc_fence_after_sync();
                     const uint32_t sQ = smem_u32(tQ), sK = smem_u32(tK), sV = smem_u32(tV), sG = smem_u32(tG);
@@ -860,7 +856,7 @@ sweep_bwd(const SweepArgs a)
                 fence_async_smem();
                 tc_fence_before_sync();
                 __syncthreads();
-                if (tid == kIssuer) {
+                if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
                     const uint32_t sQ = smem_u32(tQ), sK = smem_u32(tK), sG = smem_u32(tG);
                     const uint32_t sP = smem_u32(tP), sdP = smem_u32(tdP);
@@ -872,7 +868,7 @@ sweep_bwd(const SweepArgs a)
                 ok = wait_all(barG1, 1, a.status, ok);
                 tc_fence_after_sync();
                 if (ok) {
-                    if (tid == kIssuer && (u > 0 || more)) {
+                    if (w.issuer() && (u > 0 || more) && elect_one()) {
                         // every product has completed: fetch the next sub-chunk's zero-start state
                         const size_t nslot = u > 0 ? slot + (size_t)g.B * g.H * pl.ntile : (size_t)bh * pl.ntile + (tile - 1);
                         const char *src = reinterpret_cast<const char *>(a.slot_s + nslot * (D * D));
@@ -971,7 +967,7 @@ sweep_bwd(const SweepArgs a)
         }
     }
 die:
-    if (!ok && tid == kIssuer) mbar_wait(barS, par, a.status);      // let bulk copies in flight land
+    if (!ok && w.issuer() && elect_one()) mbar_wait(barS, par, a.status);      // let bulk copies in flight land
     cta_teardown(ctl, SM::tmem_cols);
 }
 

@@ -14,6 +14,18 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The value of lane 0, known to the compiler to be the same in the whole warp.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+// True in one thread of a converged warp, the same one every time.  Inside a branch on warp-uniform values
+// and this, tcgen05 operands stay in uniform registers: a 64 x 32 x 16 MMA then issues every 26 cycles
+// (64 x 64: 33); under `threadIdx.x == k` the compiler moves every operand over lane by lane, 52 cycles each.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // 64-bit matrix descriptor: start address, leading / stride byte offsets (all >> 4), descriptor
 // version 1, layout type in the top three bits.
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes,
