@@ -499,12 +499,12 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
 // SM).  16 sequences of 16384 tokens, d = 72: 114 us with the row-chunk work split, 84 us now; 768 of 256, d = 64
 // (uncut): 60 -> 52 us.  Three CTAs per SM on 80 registers: 72 us against 59 us on 48 sequences of 4096 tokens, d = 64.
 // =================================================================================================
-template <int D>
+template <int D, typename TO>
 struct FwdSmem {
     using C = Cfg<D>;
     using L = Col<D>;
     static constexpr int kTiles = 3 * C::TILE_T + C::TILE_S + C::TILE_P;      // tQ tK tV tS tP
-    static constexpr size_t bytes = kTiles + 8 * D * 4 + 2 * T * 4 + sizeof(Ctl);
+    static constexpr size_t bytes = kTiles + Staging<D, TO>::kBytes + 8 * D * 4 + 4 * T * 4 + sizeof(Ctl);
     static constexpr uint32_t aP = 0, aO = 32, aU = aO + L::HW;               // accumulator columns
     static constexpr uint32_t tmem_cols = 128;
     static_assert(aU + L::ACCS <= tmem_cols, "tensor memory");
@@ -516,12 +516,13 @@ sweep_fwd(const SweepArgs a)
 {
     using C = Cfg<D>;
     using L = Col<D>;
-    using SM = FwdSmem<D>;
+    using SM = FwdSmem<D, TO>;
     extern __shared__ __align__(128) char smem[];
     char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tS = tV + C::TILE_T, *tP = tS + C::TILE_S;
-    float *sTot = reinterpret_cast<float *>(smem + SM::kTiles);
-    int *rowOff = reinterpret_cast<int *>(sTot + 8 * D);
-    Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 2 * T);
+    char *stage = smem + SM::kTiles;
+    float *sTot = reinterpret_cast<float *>(stage + Staging<D, TO>::kBytes);
+    int *rowOff = reinterpret_cast<int *>(sTot + 8 * D);               // ring of four tiles: the one before, this one, the next
+    Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 4 * T);
 
     const int tid = threadIdx.x;
     cta_setup(ctl, 1, SM::tmem_cols, smem, SM::kTiles);
@@ -533,7 +534,7 @@ sweep_fwd(const SweepArgs a)
     float S[L::NPS][8];
     Cols<D, true, false> raw;
     bool ok = true;
-    int cur = 0;
+    int cur = 0, staged = 0;                            // rows of the tile before that wait in the staging buffer
     const int total = g.B * g.H * pl.nseg;
     TO *out = reinterpret_cast<TO *>(a.out);
 
@@ -567,11 +568,10 @@ sweep_fwd(const SweepArgs a)
             group_prefix<D>(raw, raw.g, w, sTot);
         }
         for (int tile = t0; tile < t1; ++tile) {
-            const int nrow = min(T, g.L - tile * T), nxt = cur ^ 1;
+            const int nrow = min(T, g.L - tile * T), nxt = (cur + 1) & 3, prv = (cur + 3) & 3;
             const bool more = tile + 1 < t1;
             tc_fence_before_sync();
             SYNC_OR_DIE();                                       // group totals are there, the previous tile's products are done
-            const int my_off = rowOff[cur * T + w.r16];
             if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile + 1, tid);
             // Where some channel's gates sum to too much for one centring (or shorter chunks were asked for) the tile
             // is worked in sub-chunks: the other rows of the operand tiles are zero, each has its own centring.
@@ -583,12 +583,12 @@ sweep_fwd(const SweepArgs a)
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
             }
-            const float2 off = centred(tt.before, tt.all), xoff = centred(tt.xbefore, tt.xall);
+            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
             const int nsub = (nrow + s - 1) / s;
             for (int u = 0; u < nsub; ++u) {
                 const int lo = u * s, hi = lo + s;
                 const bool last = u == nsub - 1;
-                build_rows<D>(raw, w, off, xoff, tQ, tK, tV, nullptr, 8 * w.grp >= lo && 8 * w.grp < hi);
+                build_rows<D>(raw, w, tQ, tK, tV, nullptr, 8 * w.grp >= lo && 8 * w.grp < hi);
                 Tot tu = whole;
                 if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
                 const Decay dec = decay_of<D>(sm, tu.all, tu.xall);
@@ -603,6 +603,8 @@ sweep_fwd(const SweepArgs a)
                     issue_split<D, C::KS, C::CHS>(tmem + SM::aO, tQ, tS, false);                  // Qc Sc
                     issue_state<D>(tmem + SM::aU, tK, tV);                                        // Kc^T V
                 }
+                if (staged) flush_rows<D>(out, stage, rowOff + prv * T, w, staged, a.accumulate != 0);
+                staged = 0;
                 if (last && more) load_tile(nxt);
                 ok = wait_all(&ctl->bar[0], 0, a.status, ok);          // completes twice per iteration: parities 0, 1
                 tc_fence_after_sync();
@@ -646,8 +648,7 @@ sweep_fwd(const SweepArgs a)
                         if (jc < L::NV0) {                        // uniform over the warp
                             float o[8];
                             tmem_ld8(tl + SM::aO + 8 * jc, o);
-                            if (inrow && jc < (w.hf ? L::NV1 : L::NV0))
-                                store_out8(out + (uint32_t)my_off + 8 * ((w.hf ? L::NV0 : 0) + jc), o, a.accumulate != 0);
+                            if (inrow && jc < (w.hf ? L::NV1 : L::NV0)) stage_row<D, TO>(stage, w.r16, (w.hf ? L::NV0 : 0) + jc, o);
                         }
                     }
                     fold_state<D>(tl + SM::aU, sm, S, dec);
@@ -657,8 +658,12 @@ sweep_fwd(const SweepArgs a)
                     SYNC_OR_DIE();
                 }
             }
+            staged = nrow;
             cur = nxt;
         }
+        SYNC_OR_DIE();
+        flush_rows<D>(out, stage, rowOff + ((cur + 3) & 3) * T, w, staged, a.accumulate != 0);
+        staged = 0;
         if (pl.nseg == 1 && a.s_out) save_state<D>(a.s_out + (size_t)sid * D * D, sm, S);
     }
 die:
@@ -673,7 +678,7 @@ die:
 // Bound by latency like the forward sweep.  48 sequences of 4096 tokens, d = 64: 140 us with the row-chunk work
 // split, 106 us now; 16 of 16384, d = 72: 252 -> 186 us (217 us before the L2 was asked for the next tile's rows early).
 // =================================================================================================
-template <int D>
+template <int D, typename TO>
 struct BwdSmem {
     using C = Cfg<D>;
     using L = Col<D>;
@@ -682,7 +687,13 @@ struct BwdSmem {
     static constexpr int kOver = 2 * C::TILE_T + C::TILE_S;                    // tV tG tD: spent when the accumulators are complete
     static constexpr int kRegion = 2 * kBuf > kOver ? 2 * kBuf : kOver;
     static constexpr int kTiles = 2 * C::TILE_T + kRegion + 2 * C::TILE_P + 2 * C::TILE_S;      // tQ tK | tV tG tD .. | tP tdP | tS tI
-    static constexpr size_t bytes = kTiles + (2 * 8 * D + D) * 4 + 2 * T * 4 + sizeof(Ctl);
+    // dv leaves through a staging buffer (see Staging): one of its own at d = 64; at d = 72, where two CTAs leave no
+    // room for it, the zero-start state's tile, whose refill then waits for the copy; fp32 results do not fit there
+    // and are stored directly
+    static constexpr bool kStage = D == 64 || sizeof(TO) == 2, kOwnStage = D == 64;
+    static constexpr int kStageBytes = kOwnStage ? Staging<D, TO>::kBytes : 0;
+    static_assert(!kStage || kOwnStage || Staging<D, TO>::kBytes <= C::NCH * C::CHS, "the state tile's zero chunk stays clean");
+    static constexpr size_t bytes = kTiles + kStageBytes + (2 * 8 * D + D) * 4 + 2 * T * 4 + sizeof(Ctl);
     static constexpr uint32_t aP = 0, aQK = 64, aV = aQK + D, aW = aV + D;     // accumulator columns
     static constexpr uint32_t tmem_cols = 256;
     static_assert(aW + L::ACCS <= tmem_cols, "tensor memory");
@@ -701,12 +712,13 @@ sweep_bwd(const SweepArgs a)
 {
     using C = Cfg<D>;
     using L = Col<D>;
-    using SM = BwdSmem<D>;
+    using SM = BwdSmem<D, TO>;
     extern __shared__ __align__(128) char smem[];
     char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T, *tD = tG + C::TILE_T;
     char *tP = tV + SM::kRegion, *tdP = tP + C::TILE_P, *tS = tdP + C::TILE_P, *tI = tS + C::TILE_S;
     float *bufQ = reinterpret_cast<float *>(tV), *bufK = bufQ + T * SM::LDP;
-    float *sTot = reinterpret_cast<float *>(smem + SM::kTiles), *sX = sTot + 8 * D, *sAux = sX + 8 * D;
+    char *stage = SM::kOwnStage ? smem + SM::kTiles : tS;
+    float *sTot = reinterpret_cast<float *>(smem + SM::kTiles + SM::kStageBytes), *sX = sTot + 8 * D, *sAux = sX + 8 * D;
     int *rowOff = reinterpret_cast<int *>(sAux + D);
     Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 2 * T);
 
@@ -732,6 +744,16 @@ sweep_bwd(const SweepArgs a)
         row_offsets<D>(rowOff + slot * T, w, off);
         load_gates(raw.g, a.gate, off);
         load_rows(raw, a.q, a.k, a.v, a.d_out, off);
+    };
+    // The zero-start state of the (sub-)chunk worked after sub-chunk u of `tile` (whose slot is given): the issuing
+    // thread asks for it once the tile of the one before is free.
+    auto fetch_next = [&](int bh, size_t slot, int u, int tile, bool more) {
+        if (w.issuer() && (u > 0 || more) && elect_one()) {
+            const size_t nslot = u > 0 ? slot + (size_t)g.B * g.H * pl.ntile : (size_t)bh * pl.ntile + (tile - 1);
+            const char *src = reinterpret_cast<const char *>(a.slot_s + nslot * (D * D));
+            mbar_arrive_expect_tx(barS, (uint32_t)C::NCH * D * 16u);
+            for (int j = 0; j < C::NCH; ++j) bulk_g2s(tS + j * C::CHS, src + j * D * 16, D * 16, barS);
+        }
     };
     // the first tile's rows are inputs of the call: their loads need not wait for the scan kernel
     auto prime = [&](int sid) {
@@ -776,7 +798,6 @@ sweep_bwd(const SweepArgs a)
             const int nrow = min(T, g.L - tile * T), nxt = cur ^ 1;
             const bool more = tile > t0;
             SYNC_OR_DIE();                                       // group totals are there, the accumulator buffers are free
-            const int my_off = rowOff[cur * T + w.r16];
             if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 1, tid);
             const Tot whole = tile_totals<D>(sTot, w);
             Tot tt = whole;
@@ -786,14 +807,14 @@ sweep_bwd(const SweepArgs a)
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
             }
-            const float2 off = centred(tt.before, tt.all), xoff = centred(tt.xbefore, tt.xall);
+            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
             const int nsub = (nrow + s - 1) / s;
             float2 tot = make_float2(0.f, 0.f), xtot = tot;      // sums of q dq - k dk over the group
             for (int u = nsub - 1; u >= 0; --u) {
                 const int lo = u * s, hi = lo + s;
                 const bool mine = 8 * w.grp >= lo && 8 * w.grp < hi;
                 const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
-                build_rows<D>(raw, w, off, xoff, tQ, tK, tV, tG, mine);
+                build_rows<D>(raw, w, tQ, tK, tV, tG, mine);
                 Tot tu = whole;
                 if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
                 const Decay dec = decay_of<D>(sm, tu.all, tu.xall);
@@ -868,13 +889,7 @@ sweep_bwd(const SweepArgs a)
                 ok = wait_all(barG1, 1, a.status, ok);
                 tc_fence_after_sync();
                 if (ok) {
-                    if (w.issuer() && (u > 0 || more) && elect_one()) {
-                        // every product has completed: fetch the next sub-chunk's zero-start state
-                        const size_t nslot = u > 0 ? slot + (size_t)g.B * g.H * pl.ntile : (size_t)bh * pl.ntile + (tile - 1);
-                        const char *src = reinterpret_cast<const char *>(a.slot_s + nslot * (D * D));
-                        mbar_arrive_expect_tx(barS, (uint32_t)C::NCH * D * 16u);
-                        for (int j = 0; j < C::NCH; ++j) bulk_g2s(tS + j * C::CHS, src + j * D * 16, D * 16, barS);
-                    }
+                    if (SM::kOwnStage || !SM::kStage) fetch_next(bh, slot, u, tile, more);           // every product has completed
                     const bool inrow = w.r16 >= lo && w.r16 < min(hi, nrow);
                     float *buf = (w.hf ? bufK : bufQ) + w.r16 * SM::LDP;
 #pragma unroll
@@ -885,7 +900,10 @@ sweep_bwd(const SweepArgs a)
                             float x0[8], x1[8];
                             tmem_ld8_pair(tl + SM::aQK + 8 * jc, tl + SM::aV + 8 * jc, x0, x1);
                             if (w.hf) {
-                                if (inrow) store_out8(dv + (uint32_t)my_off + 8 * jc, x1, acc_out);
+                                if (inrow) {
+                                    if constexpr (SM::kStage) stage_row<D, TO>(stage, w.r16, jc, x1);
+                                    else store_out8(dv + (uint32_t)rowOff[cur * T + w.r16] + 8 * jc, x1, acc_out);
+                                }
                             } else if (entry) {
                                 float hh[8];
                                 ld8(sAux + 8 * jc, hh);
@@ -915,7 +933,7 @@ sweep_bwd(const SweepArgs a)
                         const float2 ak = *reinterpret_cast<const float2 *>(bufK + row * SM::LDP + c2);
                         const float2 q2 = __half22float2(*reinterpret_cast<const __half2 *>(tQ + o));
                         const float2 k2 = __half22float2(*reinterpret_cast<const __half2 *>(tK + o));
-                        const float ex = raw.g[j].x + (j < 8 ? off.x : xoff.x), ey = raw.g[j].y + (j < 8 ? off.y : xoff.y);
+                        const float ex = raw.g[j].x, ey = raw.g[j].y;
                         const int r = ro[row];
                         if (row < nrow) {
                             store_pair(dq + (uint32_t)(r + c2), aq.x * ex2(ex), aq.y * ex2(ey), acc_out);
@@ -937,13 +955,21 @@ sweep_bwd(const SweepArgs a)
                         }
                     }
                 }
-                if (u > 0) __syncthreads();                      // the accumulator buffers become operand tiles again
+                // the state tile as staging holds this sub-chunk's rows only
+                if (SM::kStage && (!SM::kOwnStage || u == 0)) flush_rows<D>(dv, stage, rowOff + cur * T, w, SM::kOwnStage || mine ? nrow : 0, acc_out);
+                if (u > 0) {
+                    fence_async_smem();
+                    __syncthreads();                             // the accumulator buffers become operand tiles again
+                    if (SM::kStage && !SM::kOwnStage) fetch_next(bh, slot, u, tile, more);
+                }
                 par ^= 1;
             }
             // gate gradient of the tile: suffix sums of q dq - k dk down the rows plus what later tiles carry in
             *reinterpret_cast<float2 *>(sX + w.grp * D + w.c2) = tot;
             if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(sX + w.grp * D + w.xc2) = xtot;
+            if (SM::kStage && !SM::kOwnStage) fence_async_smem();
             __syncthreads();
+            if (SM::kStage && !SM::kOwnStage) fetch_next(bh, 0, 0, tile, more);
             {
                 const Tot after = later_totals<D>(sX, w);
                 const float2 add = make_float2(carry.x + after.before.x, carry.y + after.before.y);
@@ -1091,19 +1117,19 @@ dig_status run(const GlaArgs &ga)
     }
     const bool f32 = ga.dtype == DIG_BF16_F32OUT;
     if constexpr (!BWD) {
-        constexpr size_t smem = FwdSmem<D>::bytes;
+        constexpr size_t smem16 = FwdSmem<D, bf16>::bytes, smem32 = FwdSmem<D, float>::bytes;
         auto k16 = sweep_fwd<D, bf16>;
         auto k32 = sweep_fwd<D, float>;
-        if ((st = set_smem(k16, smem)) != DIG_OK || (st = set_smem(k32, smem)) != DIG_OK) return st;
+        if ((st = set_smem(k16, smem16)) != DIG_OK || (st = set_smem(k32, smem32)) != DIG_OK) return st;
         KernelTimer t(KID_SW_FWD, ga.stream);
-        launch_pdl(f32 ? k32 : k16, grid, block, smem, ga.stream, a);
+        launch_pdl(f32 ? k32 : k16, grid, block, f32 ? smem32 : smem16, ga.stream, a);
     } else {
-        constexpr size_t smem = BwdSmem<D>::bytes;
+        constexpr size_t smem16 = BwdSmem<D, bf16>::bytes, smem32 = BwdSmem<D, float>::bytes;
         auto k16 = sweep_bwd<D, bf16>;
         auto k32 = sweep_bwd<D, float>;
-        if ((st = set_smem(k16, smem)) != DIG_OK || (st = set_smem(k32, smem)) != DIG_OK) return st;
+        if ((st = set_smem(k16, smem16)) != DIG_OK || (st = set_smem(k32, smem32)) != DIG_OK) return st;
         KernelTimer t(KID_SW_BWD, ga.stream);
-        launch_pdl(f32 ? k32 : k16, grid, block, smem, ga.stream, a);
+        launch_pdl(f32 ? k32 : k16, grid, block, f32 ? smem32 : smem16, ga.stream, a);
     }
     return cuda_ok(cudaGetLastError());
 }
