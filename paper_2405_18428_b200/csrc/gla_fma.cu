@@ -1,8 +1,15 @@
 // fp32-FMA kernel family for chunkwise gated linear attention (Eq. attn_gla, evaluated chunk
 // by chunk as Section 3.5 describes).  Serves DIG_F32 (products must be fp32-accurate, which a
 // single tf32 tensor-core pass is not) and any bf16 request the tensor-core family does not
-// cover.  One CTA per (chunk, batch*head); every contraction is a register-blocked 4x4 FMA loop
-// over shared-memory tiles.
+// cover.  One CTA per (chunk, batch*head); every contraction is a register-blocked FMA loop over
+// shared-memory tiles: 4x4 blocks in the state and output kernels, 8x4 in the gradient kernel.
+//
+// What bounds it: latency.  A CTA holds a whole chunk (C = d = 64 in fp32: 80 to 160 KB) and 192 chunks fill 148 SMs
+// once or twice, so a kernel's time is one or two CTAs' serial chain of load, prefix, scores, products.  Hence all
+// tiles of a kernel are asked for at once, prefix sums run in segments on all threads, loops are unrolled so that
+// several shared loads are in flight, and rounds and waits in front of the states' arrival are filled by the
+// programmatic launch.  B = 2, H = 6, L = 1024, d = C = 64 (us, before -> now): state 18 -> 11.2, with gradients
+// 26 -> 16.9, outputs 29 -> 21.2, gradients 100 -> 58; one 256-token sequence of 6 heads: 14.7 -> 8.5, 21.4 -> 15.6.
 //
 // Notation per chunk (rows j = 0..C-1 in scan order, zero rows past the end of the sequence):
 //   Lam_j = inclusive prefix sum of the gates, gamma = exp(Lam_{C-1}),
@@ -13,30 +20,35 @@
 namespace dig {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;        // state and output kernels
+constexpr int kBwdThreads = 512;     // gradient kernel
 
 // ---- 4x4 register-blocked contractions over shared memory --------------------------------
-// acc[i][j] += sum_k A[(r0+i)*lda + k] * Bm[(c0 + j*cstep)*ldb + k]
+// acc[i][j] += sum_k A[(r0+i)*lda + k] * Bm[(c0 + j*cstep)*ldb + k], columns j < jn only (jn uniform enough over a
+// warp to skip whole pieces of a causal product)
 __device__ __forceinline__ void mm_nt(float (&acc)[4][4], const float *A, int lda, int r0,
-                                      const float *Bm, int ldb, int c0, int cstep, int K)
+                                      const float *Bm, int ldb, int c0, int cstep, int K, int jn)
 {
+#pragma unroll 2
     for (int k = 0; k < K; k += 4) {
-        float4 a[4], b[4];
+        float4 a[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4 *>(A + (r0 + i) * lda + k);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4 *>(Bm + (c0 + j * cstep) * ldb + k);
+        for (int j = 0; j < 4; ++j)
+            if (j < jn) {
+                const float4 b = *reinterpret_cast<const float4 *>(Bm + (c0 + j * cstep) * ldb + k);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                acc[i][j] += a[i].x * b[j].x + a[i].y * b[j].y + a[i].z * b[j].z + a[i].w * b[j].w;
+                for (int i = 0; i < 4; ++i)
+                    acc[i][j] += a[i].x * b.x + a[i].y * b.y + a[i].z * b.z + a[i].w * b.w;
+            }
     }
 }
 // acc[i][j] += sum_{k<K} A[(r0+i)*lda + k] * Bm[k*ldb + c0 + j]
 __device__ __forceinline__ void mm_nn(float (&acc)[4][4], const float *A, int lda, int r0,
                                       const float *Bm, int ldb, int c0, int K)
 {
+#pragma unroll 4
     for (int k = 0; k < K; k += 4) {
         float4 a[4], b[4];
 #pragma unroll
@@ -56,6 +68,7 @@ __device__ __forceinline__ void mm_nn(float (&acc)[4][4], const float *A, int ld
 __device__ __forceinline__ void mm_tn(float (&acc)[4][4], const float *A, int lda, int r0,
                                       const float *Bm, int ldb, int c0, int K)
 {
+#pragma unroll 8
     for (int k = 0; k < K; ++k) {
         const float4 a = *reinterpret_cast<const float4 *>(A + k * lda + r0);
         const float4 b = *reinterpret_cast<const float4 *>(Bm + k * ldb + c0);
@@ -75,37 +88,150 @@ __device__ __forceinline__ void zero(float (&acc)[4][4])
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 }
 
-// ---- tile loaders ----------------------------------------------------------------------------
-// Copies the chunk's rows of a [B][L][H][d] tensor into shared memory (row stride ld floats),
-// rows past the end of the sequence become zero.
-template <typename T>
-__device__ __forceinline__ void load_tile(float *dst, int ld, const T *src, const Geom &g, int b,
-                                          int h, int chunk, int d)
+// ---- 8x4 blocks of the gradient kernel -------------------------------------------------------------
+// Eight rows from r0, four columns cb, cb + cs, cb + 2 cs, cb + 3 cs: neighbouring lanes read neighbouring rows
+// (nt: an odd number of 16-byte words apart) or columns of B, so no access conflicts, and 12 loads feed 128
+// multiply-adds (4x4 blocks on neighbouring columns: 8 feed 64, and the nt products hit two banks eight times).
+struct Acc8 {
+    float v[8][4];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] = 0.f;
+    }
+};
+// += sum_k A[(r0+i)*lda + k] * B[(cb + j*cs)*ldb + k]
+__device__ __forceinline__ void mm8_nt(Acc8 &acc, const float *A, int lda, int r0, const float *B, int ldb, int cb, int cs, int K)
 {
-    const int per_row = d >> 2;
-    for (int idx = threadIdx.x; idx < g.C * per_row; idx += kThreads) {
-        const int j = idx / per_row, c = (idx - j * per_row) << 2;
-        const int p = chunk * g.C + j;
-        float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (p < g.L) {
-            const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-            val = load4(src + tok_offset(g, b, t, h, d) + c);
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float4 b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4 *>(B + (cb + j * cs) * ldb + k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 a = *reinterpret_cast<const float4 *>(A + (r0 + i) * lda + k);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc.v[i][j] += a.x * b[j].x + a.y * b[j].y + a.z * b[j].z + a.w * b[j].w;
         }
-        *reinterpret_cast<float4 *>(dst + j * ld + c) = val;
+    }
+}
+// += sum_{k<K} A[(r0+i)*lda + k] * scale[k] * B[k*ldb + cb + j*cs]   (SCALED: with the factor)
+template <bool SCALED>
+__device__ __forceinline__ void mm8_nn(Acc8 &acc, const float *A, int lda, int r0, const float *B, int ldb, int cb, int cs, int K, const float *scale)
+{
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float b[4][4];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[kk][j] = B[(k + kk) * ldb + cb + j * cs];
+        float4 sc = make_float4(1.f, 1.f, 1.f, 1.f);
+        if (SCALED) sc = *reinterpret_cast<const float4 *>(scale + k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float4 a = *reinterpret_cast<const float4 *>(A + (r0 + i) * lda + k);
+            if (SCALED) a = make_float4(a.x * sc.x, a.y * sc.y, a.z * sc.z, a.w * sc.w);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc.v[i][j] += a.x * b[0][j] + a.y * b[1][j] + a.z * b[2][j] + a.w * b[3][j];
+        }
+    }
+}
+// += sum_{k0<=k<K} A[k*lda + r0 + i] * B[k*ldb + cb + j*cs]
+__device__ __forceinline__ void mm8_tn(Acc8 &acc, const float *A, int lda, int r0, const float *B, int ldb, int cb, int cs, int k0, int K)
+{
+#pragma unroll 4
+    for (int k = k0; k < K; ++k) {
+        const float4 a0 = *reinterpret_cast<const float4 *>(A + k * lda + r0), a1 = *reinterpret_cast<const float4 *>(A + k * lda + r0 + 4);
+        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float b = B[k * ldb + cb + j * cs];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc.v[i][j] = fmaf(a[i], b, acc.v[i][j]);
+        }
     }
 }
 
-// In place: gates -> inclusive prefix sums along the rows of the chunk, one thread per channel.
-__device__ __forceinline__ void prefix_gates(float *lam, int ld, int C, int dk)
+// ---- tile loaders ----------------------------------------------------------------------------
+// Row table: (token, head) row of the chunk's row j in a [B][L][H][.] tensor, -1 past the end of the sequence.  It
+// lies in the padding behind the rows of a tile.
+struct Rows {
+    int *p;
+    int ld;
+    __device__ __forceinline__ Rows(float *tile, int ld_, int d) : p(reinterpret_cast<int *>(tile + d)), ld(ld_) {}
+    __device__ __forceinline__ int operator[](int j) const { return p[j * ld]; }
+};
+__device__ __forceinline__ void fill_rows(const Rows &rows, const Geom &g, int b, int h, int chunk)
 {
-    for (int c = threadIdx.x; c < dk; c += kThreads) {
+    for (int j = threadIdx.x; j < g.C; j += blockDim.x) {
+        const int p = chunk * g.C + j;
+        rows.p[j * rows.ld] = p < g.L ? (b * g.L + scan_token(p, g.dir, g.gh, g.gw, g.L)) * g.H + h : -1;
+    }
+}
+// Copies the chunk's rows of a [B][L][H][d] tensor into shared memory (row stride ld floats), rows past the end
+// of the sequence become zero.  fp32 travels by cp.async, so that all tiles of a kernel are in flight together and
+// a CTA pays the latency of global memory once; loads_done() before the barrier that publishes them.
+__device__ __forceinline__ void cp_async16(float *dst, const float *src, bool on)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void loads_done() { asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void load_tile(float *dst, int ld, const float *src, const Rows &sRow, int C, int d)
+{
+    const int per_row = d >> 2, n = C * per_row;
+    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
+        const int j = idx / per_row, c = (idx - j * per_row) << 2, row = sRow[j];
+        cp_async16(dst + j * ld + c, src + (size_t)max(row, 0) * d + c, row >= 0);
+    }
+}
+__device__ __forceinline__ void load_tile(float *dst, int ld, const __nv_bfloat16 *src, const Rows &sRow, int C, int d)
+{
+    const int per_row = d >> 2, n = C * per_row;
+    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
+        const int j = idx / per_row, c = (idx - j * per_row) << 2, row = sRow[j];
+        *reinterpret_cast<float4 *>(dst + j * ld + c) = row >= 0 ? load4(src + (size_t)row * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+// A [dk][dv] state of the workspace -> [dk][ld] tile.
+__device__ __forceinline__ void load_state(float *dst, int ld, const float *src, int dk, int dv)
+{
+    const int per_row = dv >> 2, n = dk * per_row;
+    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
+        const int r = idx / per_row, c = (idx - r * per_row) << 2;
+        cp_async16(dst + r * ld + c, src + 4 * (size_t)idx, true);
+    }
+}
+
+// In place: gates -> inclusive prefix sums down the rows; the rows are cut in as many segments as there are
+// threads per channel, whose totals go through sSeg ([segments][dk] floats).  Contains two barriers, the last at the end.
+__device__ __forceinline__ void prefix_gates(float *lam, int ld, int C, int dk, float *sSeg)
+{
+    const int nseg = min((int)blockDim.x / dk, 8), rows = (C + nseg - 1) / nseg;
+    const int seg = threadIdx.x / dk, c = threadIdx.x - seg * dk, j0 = seg * rows, j1 = min(j0 + rows, C);
+    if (seg < nseg) {
         float run = 0.f;
-        for (int j = 0; j < C; ++j) {
+#pragma unroll 8
+        for (int j = j0; j < j1; ++j) {
             run += lam[j * ld + c];
             lam[j * ld + c] = run;
         }
+        sSeg[seg * dk + c] = run;
     }
+    __syncthreads();
+    if (seg < nseg && seg > 0) {
+        float add = 0.f;
+        for (int s = 0; s < seg; ++s) add += sSeg[s * dk + c];
+#pragma unroll 8
+        for (int j = j0; j < j1; ++j) lam[j * ld + c] += add;
+    }
+    __syncthreads();
 }
+__device__ __forceinline__ float4 exp4(float4 x) { return make_float4(expf(x.x), expf(x.y), expf(x.z), expf(x.w)); }
+__device__ __forceinline__ float4 mul4(float4 a, float4 b) { return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w); }
 
 // ---- kernel 1: chunk-local state contributions ------------------------------------------------
 // U = Kh^T V  (and, for the backward pass, W = Qt^T dO); gamma = exp(Lam_{C-1}).
@@ -119,53 +245,39 @@ fma_chunk_state(const T *__restrict__ q, const T *__restrict__ k, const T *__res
     extern __shared__ __align__(16) float smem[];
     const int chunk = blockIdx.x, bh = blockIdx.y, b = bh / g.H, h = bh - b * g.H;
     const int ldk = g.dk + 4, ldv = g.dv + 4;
-    float *sX = smem;                       // gates -> Lam -> Kh
+    float *sLam = smem;                     // gates -> Lam
+    float *sX = sLam + g.C * ldk;           // k -> Kh
     float *sV = sX + g.C * ldk;
-    float *sQ = sV + g.C * ldv;             // BWD: Qt
+    float *sSeg = sV + g.C * ldv;           // [8][dk]
+    float *sQ = sSeg + 8 * g.dk;            // BWD: Qt
     float *sG = sQ + (BWD ? g.C * ldk : 0); // BWD: dO
 
-    load_tile(sX, ldk, gate, g, b, h, chunk, g.dk);
-    load_tile(sV, ldv, v, g, b, h, chunk, g.dv);
-    if (BWD) load_tile(sG, ldv, d_out, g, b, h, chunk, g.dv);
+    const Rows sRow(sV, ldv, g.dv);
+    fill_rows(sRow, g, b, h, chunk);
+    pdl_wait();
+    pdl_launch_dependents();
     __syncthreads();
-    prefix_gates(sX, ldk, g.C, g.dk);
+    load_tile(sLam, ldk, gate, sRow, g.C, g.dk);
+    load_tile(sX, ldk, k, sRow, g.C, g.dk);
+    load_tile(sV, ldv, v, sRow, g.C, g.dv);
+    if (BWD) {
+        load_tile(sQ, ldk, q, sRow, g.C, g.dk);
+        load_tile(sG, ldv, d_out, sRow, g.C, g.dv);
+    }
+    loads_done();
     __syncthreads();
+    prefix_gates(sLam, ldk, g.C, g.dk, sSeg);
     const size_t chunk_id = (size_t)bh * g.N + chunk;
-    for (int c = threadIdx.x; c < g.dk; c += kThreads)
-        gamma[chunk_id * g.dk + c] = expf(sX[(g.C - 1) * ldk + c]);
+    const float *sLast = sLam + (g.C - 1) * ldk;
+    for (int c = threadIdx.x; c < g.dk; c += kThreads) gamma[chunk_id * g.dk + c] = expf(sLast[c]);
     {
         const int per_row = g.dk >> 2;
         for (int idx = threadIdx.x; idx < g.C * per_row; idx += kThreads) {
-            const int j = idx / per_row, c = (idx - j * per_row) << 2;
-            const int p = chunk * g.C + j;
-            float4 kk = make_float4(0.f, 0.f, 0.f, 0.f), qq = kk;
-            if (p < g.L) {
-                const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-                kk = load4(k + tok_offset(g, b, t, h, g.dk) + c);
-                if (BWD) qq = load4(q + tok_offset(g, b, t, h, g.dk) + c);
-            }
-            const float4 lam = *reinterpret_cast<const float4 *>(sX + j * ldk + c);
-            const float4 last = *reinterpret_cast<const float4 *>(sX + (g.C - 1) * ldk + c);
-            if (BWD) {
-                *reinterpret_cast<float4 *>(sQ + j * ldk + c) =
-                    make_float4(qq.x * expf(lam.x), qq.y * expf(lam.y), qq.z * expf(lam.z), qq.w * expf(lam.w));
-            }
-            // the last row is read by other threads as `last`: defer its overwrite
-            if (j != g.C - 1)
-                *reinterpret_cast<float4 *>(sX + j * ldk + c) =
-                    make_float4(kk.x * expf(last.x - lam.x), kk.y * expf(last.y - lam.y),
-                                kk.z * expf(last.z - lam.z), kk.w * expf(last.w - lam.w));
-        }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < per_row; idx += kThreads) {   // last row: Kh = k
-            const int j = g.C - 1, c = idx << 2;
-            const int p = chunk * g.C + j;
-            float4 kk = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p < g.L) {
-                const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-                kk = load4(k + tok_offset(g, b, t, h, g.dk) + c);
-            }
-            *reinterpret_cast<float4 *>(sX + j * ldk + c) = kk;
+            const int j = idx / per_row, o = j * ldk + ((idx - j * per_row) << 2);
+            const float4 lam = *reinterpret_cast<const float4 *>(sLam + o), last = *reinterpret_cast<const float4 *>(sLast + o - j * ldk);
+            const float4 e = exp4(make_float4(last.x - lam.x, last.y - lam.y, last.z - lam.z, last.w - lam.w));
+            *reinterpret_cast<float4 *>(sX + o) = mul4(*reinterpret_cast<const float4 *>(sX + o), e);
+            if (BWD) *reinterpret_cast<float4 *>(sQ + o) = mul4(*reinterpret_cast<const float4 *>(sQ + o), exp4(lam));
         }
     }
     __syncthreads();
@@ -190,50 +302,34 @@ fma_chunk_state(const T *__restrict__ q, const T *__restrict__ k, const T *__res
     }
 }
 
-// Fills sQ = Qt, sK = Kt from the prefix sums held in sLam (sLam is kept).
-template <typename T>
-__device__ __forceinline__ void make_qt_kt(float *sQ, float *sK, const float *sLam, int ldk,
-                                           const T *q, const T *k, const Geom &g, int b, int h,
-                                           int chunk)
+// In place: q -> Qt = q exp(Lam), k -> Kt = k exp(-Lam), Lam -> exp(Lam).
+__device__ __forceinline__ void make_qt_kt(float *sQ, float *sK, float *sLam, int ldk, int C, int dk)
 {
-    const int per_row = g.dk >> 2;
-    for (int idx = threadIdx.x; idx < g.C * per_row; idx += kThreads) {
-        const int j = idx / per_row, c = (idx - j * per_row) << 2;
-        const int p = chunk * g.C + j;
-        float4 kk = make_float4(0.f, 0.f, 0.f, 0.f), qq = kk;
-        if (p < g.L) {
-            const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-            const size_t off = tok_offset(g, b, t, h, g.dk) + c;
-            kk = load4(k + off);
-            qq = load4(q + off);
-        }
-        const float4 lam = *reinterpret_cast<const float4 *>(sLam + j * ldk + c);
-        *reinterpret_cast<float4 *>(sQ + j * ldk + c) =
-            make_float4(qq.x * expf(lam.x), qq.y * expf(lam.y), qq.z * expf(lam.z), qq.w * expf(lam.w));
-        *reinterpret_cast<float4 *>(sK + j * ldk + c) =
-            make_float4(kk.x * expf(-lam.x), kk.y * expf(-lam.y), kk.z * expf(-lam.z), kk.w * expf(-lam.w));
+    const int per_row = dk >> 2;
+    for (int idx = threadIdx.x; idx < C * per_row; idx += blockDim.x) {
+        const int j = idx / per_row, o = j * ldk + ((idx - j * per_row) << 2);
+        const float4 lam = *reinterpret_cast<const float4 *>(sLam + o), e = exp4(lam);
+        *reinterpret_cast<float4 *>(sLam + o) = e;
+        *reinterpret_cast<float4 *>(sQ + o) = mul4(*reinterpret_cast<const float4 *>(sQ + o), e);
+        *reinterpret_cast<float4 *>(sK + o) = mul4(*reinterpret_cast<const float4 *>(sK + o), exp4(make_float4(-lam.x, -lam.y, -lam.z, -lam.w)));
     }
 }
 
-// P[t][s] = Qt_t . Kt_s for s <= t, 0 above the diagonal (the token's own k^T v enters undecayed,
-// so the diagonal weight is exactly q_t . k_t).
-__device__ __forceinline__ void make_masked_scores(float *sP, int ldp, const float *sA, int lda,
-                                                   const float *sB, int ldb, int C, int K)
+// One 4x4 block (rows r0.., columns cb, cb+nb, ..) of P[t][s] = A_t . B_s for s <= t, 0 above the diagonal (the
+// token's own k^T v enters undecayed, so the diagonal weight is exactly q_t . k_t).
+__device__ __forceinline__ void score_block(float *sP, int ldp, const float *sA, int lda, const float *sB, int ldb, int C, int K, int blk)
 {
-    const int nb = C >> 2;
-    for (int blk = threadIdx.x; blk < nb * nb; blk += kThreads) {
-        const int r0 = (blk / nb) << 2, cb = blk % nb;       // columns cb, cb+nb, cb+2nb, cb+3nb
-        float acc[4][4];
-        zero(acc);
-        if (cb <= r0 + 3) mm_nt(acc, sA, lda, r0, sB, ldb, cb, nb, K);
+    const int nb = C >> 2, r0 = (blk / nb) << 2, cb = blk % nb;
+    float acc[4][4];
+    zero(acc);
+    mm_nt(acc, sA, lda, r0, sB, ldb, cb, nb, K, (r0 + 3) / nb + 1);       // columns from j * nb > r0 + 3 on lie above the diagonal
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int s = cb + j * nb;
-                sP[(r0 + i) * ldp + s] = (s <= r0 + i) ? acc[i][j] : 0.f;
-            }
-    }
+        for (int j = 0; j < 4; ++j) {
+            const int s = cb + j * nb;
+            sP[(r0 + i) * ldp + s] = (s <= r0 + i) ? acc[i][j] : 0.f;
+        }
 }
 
 // ---- kernel 3: outputs ---------------------------------------------------------------------------
@@ -252,26 +348,30 @@ fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     float *sK = sQ + g.C * ldk;
     float *sV = sK + g.C * ldk;
     float *sS = sV + g.C * ldv;             // [dk][ldv]
+    float *sSeg = sS;                       // [8][dk], before the state arrives
     float *sP = sLam;                       // scores reuse the gate buffer once Qt, Kt exist
     // (sP needs C*(C+4) <= C*(dk+4) floats only when C <= dk; otherwise it gets its own space)
     if (g.C > g.dk) sP = sS + g.dk * ldv;
 
-    load_tile(sLam, ldk, gate, g, b, h, chunk, g.dk);
-    load_tile(sV, ldv, v, g, b, h, chunk, g.dv);
-    {
-        const float *S = states + ((size_t)bh * g.N + chunk) * g.dk * g.dv;
-        const int per_row = g.dv >> 2;
-        for (int idx = threadIdx.x; idx < g.dk * per_row; idx += kThreads) {
-            const int r = idx / per_row, c = (idx - r * per_row) << 2;
-            *reinterpret_cast<float4 *>(sS + r * ldv + c) = *reinterpret_cast<const float4 *>(S + r * g.dv + c);
-        }
-    }
+    const Rows sRow(sV, ldv, g.dv);
+    fill_rows(sRow, g, b, h, chunk);
     __syncthreads();
-    prefix_gates(sLam, ldk, g.C, g.dk);
+    // the inputs of the call: whatever produced them has completed before the kernels in front of this one started
+    load_tile(sLam, ldk, gate, sRow, g.C, g.dk);
+    load_tile(sV, ldv, v, sRow, g.C, g.dv);
+    load_tile(sQ, ldk, q, sRow, g.C, g.dk);
+    load_tile(sK, ldk, k, sRow, g.C, g.dk);
+    loads_done();
     __syncthreads();
-    make_qt_kt(sQ, sK, sLam, ldk, q, k, g, b, h, chunk);
+    prefix_gates(sLam, ldk, g.C, g.dk, sSeg);
+    make_qt_kt(sQ, sK, sLam, ldk, g.C, g.dk);
     __syncthreads();
-    make_masked_scores(sP, ldp, sQ, ldk, sK, ldk, g.C, g.dk);
+    pdl_wait();                             // the states come from the scan in front
+    pdl_launch_dependents();
+    load_state(sS, ldv, states + ((size_t)bh * g.N + chunk) * g.dk * g.dv, g.dk, g.dv);
+    const int nb = g.C >> 2;
+    for (int blk = threadIdx.x; blk < nb * nb; blk += kThreads) score_block(sP, ldp, sQ, ldk, sK, ldk, g.C, g.dk, blk);
+    loads_done();
     __syncthreads();
     const int nrb = g.C >> 2, ncb = g.dv >> 2;
     for (int blk = threadIdx.x; blk < nrb * ncb; blk += kThreads) {
@@ -282,11 +382,8 @@ fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
         mm_nn(acc, sQ, ldk, r0, sS, ldv, c0, g.dk);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int p = chunk * g.C + r0 + i;
-            if (p < g.L) {
-                const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-                store4(out + tok_offset(g, b, t, h, g.dv) + c0, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
-            }
+            const int row = sRow[r0 + i];
+            if (row >= 0) store4(out + (size_t)row * g.dv + c0, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
         }
     }
 }
@@ -297,8 +394,17 @@ fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
 //   dk = (dP^T Qt) * exp(-Lam) + (V D^T) * exp(Lam_{C-1}-Lam)
 //   dv = P^T dO + Kh D
 //   dgate_j = carry + sum_{r >= j in chunk} (q*dq - k*dk)_r
+// After the scores, three groups of whole warps compute the blocks of dq, dk and dv side by side in registers: one
+// CTA of 512 threads per SM, 128 registers each (256 threads with 4x4 blocks took 87 us where this takes 58).  With
+// s = dP^T Qt + gamma (V D^T), dk = s / exp(Lam), q*dq = Qt (dq accumulator) and k*dk = Kt s.
+__host__ __device__ inline int grad_blocks(int C, int d) { return ((C / 8) * (d / 4) + 31) & ~31; }
+// The tile of q*dq - k*dk lies over the score tiles where it fits and one round of blocks is all there is.
+__host__ __device__ inline bool x_over_scores(int C, int dk, int dv)
+{
+    return dk + 4 <= 2 * (C + 4) && 2 * grad_blocks(C, dk) + grad_blocks(C, dv) <= kBwdThreads;
+}
 template <typename T, typename TO>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kBwdThreads)
 fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v,
               const float *__restrict__ gate, const T *__restrict__ d_out,
               const float *__restrict__ states, const float *__restrict__ dstates,
@@ -308,6 +414,7 @@ fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     extern __shared__ __align__(16) float smem[];
     const int chunk = blockIdx.x, bh = blockIdx.y, b = bh / g.H, h = bh - b * g.H;
     const int ldk = g.dk + 4, ldv = g.dv + 4, ldp = g.C + 4;
+    const bool over = x_over_scores(g.C, g.dk, g.dv);
     float *sLam = smem;
     float *sQ = sLam + g.C * ldk;
     float *sK = sQ + g.C * ldk;
@@ -317,110 +424,121 @@ fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     float *sD = sS + g.dk * ldv;            // [dk][ldv]
     float *sP = sD + g.dk * ldv;            // [C][ldp]
     float *sdP = sP + g.C * ldp;            // [C][ldp]
-    float *sX = sdP + g.C * ldp;            // [C][ldk]  q*dq - k*dk
+    float *sSeg = sS;                       // [8][dk], before the states arrive and after they are spent
+    float *sX = over ? sP : sdP + g.C * ldp;              // [C][ldk]  q*dq - k*dk
+    const float *sGam = sLam + (g.C - 1) * ldk;           // exp(Lam_{C-1}) once Lam has become exp(Lam)
+    const size_t chunk_id = (size_t)bh * g.N + chunk;
 
-    load_tile(sLam, ldk, gate, g, b, h, chunk, g.dk);
-    load_tile(sV, ldv, v, g, b, h, chunk, g.dv);
-    load_tile(sG, ldv, d_out, g, b, h, chunk, g.dv);
-    {
-        const size_t off = ((size_t)bh * g.N + chunk) * g.dk * g.dv;
-        const int per_row = g.dv >> 2;
-        for (int idx = threadIdx.x; idx < g.dk * per_row; idx += kThreads) {
-            const int r = idx / per_row, c = (idx - r * per_row) << 2;
-            *reinterpret_cast<float4 *>(sS + r * ldv + c) = *reinterpret_cast<const float4 *>(states + off + r * g.dv + c);
-            *reinterpret_cast<float4 *>(sD + r * ldv + c) = *reinterpret_cast<const float4 *>(dstates + off + r * g.dv + c);
-        }
+    const Rows sRow(sV, ldv, g.dv);
+    fill_rows(sRow, g, b, h, chunk);
+    __syncthreads();
+    // the inputs of the call: whatever produced them has completed before the kernels in front of this one started
+    load_tile(sLam, ldk, gate, sRow, g.C, g.dk);
+    load_tile(sV, ldv, v, sRow, g.C, g.dv);
+    load_tile(sG, ldv, d_out, sRow, g.C, g.dv);
+    load_tile(sQ, ldk, q, sRow, g.C, g.dk);
+    load_tile(sK, ldk, k, sRow, g.C, g.dk);
+    loads_done();
+    __syncthreads();
+    prefix_gates(sLam, ldk, g.C, g.dk, sSeg);
+    make_qt_kt(sQ, sK, sLam, ldk, g.C, g.dk);
+    __syncthreads();
+    pdl_wait();                             // the states come from the scans in front
+    pdl_launch_dependents();
+    load_state(sS, ldv, states + chunk_id * g.dk * g.dv, g.dk, g.dv);
+    load_state(sD, ldv, dstates + chunk_id * g.dk * g.dv, g.dk, g.dv);
+    const int nb = g.C >> 2, nsc = nb * nb;
+    for (int blk = threadIdx.x; blk < 2 * nsc; blk += kBwdThreads) {
+        const bool p = blk < nsc;           // scores, then dO V^T
+        score_block(p ? sP : sdP, ldp, p ? sQ : sG, p ? ldk : ldv, p ? sK : sV, p ? ldk : ldv, g.C, p ? g.dk : g.dv, p ? blk : blk - nsc);
     }
-    __syncthreads();
-    prefix_gates(sLam, ldk, g.C, g.dk);
-    __syncthreads();
-    make_qt_kt(sQ, sK, sLam, ldk, q, k, g, b, h, chunk);
-    __syncthreads();
-    make_masked_scores(sP, ldp, sQ, ldk, sK, ldk, g.C, g.dk);
-    make_masked_scores(sdP, ldp, sG, ldv, sV, ldv, g.C, g.dv);
+    loads_done();
     __syncthreads();
 
-    // dv = P^T dO + (Kt*gamma) D
-    {
-        const int nrb = g.C >> 2, ncb = g.dv >> 2;
-        for (int blk = threadIdx.x; blk < nrb * ncb; blk += kThreads) {
-            const int r0 = (blk / ncb) << 2, c0 = (blk % ncb) << 2;
-            float acc[4][4], acc2[4][4];
-            zero(acc);
-            zero(acc2);
-            // P^T: rows t >= s only; start at the 4-aligned row r0
-            mm_tn(acc, sP + r0 * ldp, ldp, r0, sG + r0 * ldv, ldv, c0, g.C - r0);
-            // Kh D = sum_c Kt[s][c] gamma[c] D[c][e]
-            for (int c = 0; c < g.dk; ++c) {
-                const float gm = expf(sLam[(g.C - 1) * ldk + c]);
-                const float4 d4 = *reinterpret_cast<const float4 *>(sD + c * ldv + c0);
+    const int nk = grad_blocks(g.C, g.dk), nv = grad_blocks(g.C, g.dv), total = 2 * nk + nv;
+    for (int base = 0; base < total; base += kBwdThreads) {
+        const int t = base + threadIdx.x, kind = t < nk ? 0 : t < 2 * nk ? 1 : t < total ? 2 : 3;      // uniform over a warp
+        const int blk = t - kind * nk, d = kind == 2 ? g.dv : g.dk, cs = d >> 2, r0 = 8 * (blk / cs), cb = blk % cs;
+        const bool on = kind < 3 && r0 < g.C;
+        Acc8 a1;
+        a1.zero();
+        if (on) {
+            if (kind == 0) {
+                mm8_nn<false>(a1, sdP, ldp, r0, sK, ldk, cb, cs, r0 + 8, nullptr);        // dP Kt
+                mm8_nt(a1, sG, ldv, r0, sS, ldv, cb, cs, g.dv);                           // dO S^T
+            } else if (kind == 1) {
+                mm8_nt(a1, sV, ldv, r0, sD, ldv, cb, cs, g.dv);                           // V D^T
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float kh = sK[(r0 + i) * ldk + c] * gm;
-                    acc2[i][0] += kh * d4.x; acc2[i][1] += kh * d4.y; acc2[i][2] += kh * d4.z; acc2[i][3] += kh * d4.w;
-                }
-            }
+                for (int j = 0; j < 4; ++j) {
+                    const float gm = sGam[cb + j * cs];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int p = chunk * g.C + r0 + i;
-                if (p < g.L) {
-                    const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-                    store4(dv + tok_offset(g, b, t, h, g.dv) + c0,
-                           make_float4(acc[i][0] + acc2[i][0], acc[i][1] + acc2[i][1],
-                                       acc[i][2] + acc2[i][2], acc[i][3] + acc2[i][3]));
+                    for (int i = 0; i < 8; ++i) a1.v[i][j] *= gm;
                 }
+                mm8_tn(a1, sdP, ldp, r0, sQ, ldk, cb, cs, r0, g.C);                       // + dP^T Qt
+            } else {
+                mm8_tn(a1, sP, ldp, r0, sG, ldv, cb, cs, r0, g.C);                        // P^T dO
+                mm8_nn<true>(a1, sK, ldk, r0, sD, ldv, cb, cs, g.dk, sGam);               // Kh D
             }
         }
-    }
-
-    // dq, dk for the same (row, channel) block; x = q*dq - k*dk goes to sX for the gate gradient
-    {
-        const int nrb = g.C >> 2, ncb = g.dk >> 2;
-        for (int blk = threadIdx.x; blk < nrb * ncb; blk += kThreads) {
-            const int r0 = (blk / ncb) << 2, c0 = (blk % ncb) << 2;
-            float aq[4][4], ak[4][4], ak2[4][4];
-            zero(aq); zero(ak); zero(ak2);
-            mm_nn(aq, sdP, ldp, r0, sK, ldk, c0, r0 + 4);                          // dP Kt
-            mm_nt(aq, sG, ldv, r0, sS, ldv, c0, 1, g.dv);                          // dO S^T
-            mm_tn(ak, sdP + r0 * ldp, ldp, r0, sQ + r0 * ldk, ldk, c0, g.C - r0);  // dP^T Qt
-            mm_nt(ak2, sV, ldv, r0, sD, ldv, c0, 1, g.dv);                         // V D^T
-            const float4 last = *reinterpret_cast<const float4 *>(sLam + (g.C - 1) * ldk + c0);
-            const float lc[4] = {last.x, last.y, last.z, last.w};
+        if (over) __syncthreads();          // the score tiles are spent: they become the tile of q*dq - k*dk
+        if (on) {
+            TO *dst = kind == 0 ? dq : kind == 1 ? dk : dv;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int p = chunk * g.C + r0 + i;
-                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (p < g.L) {
-                    const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-                    const size_t off = tok_offset(g, b, t, h, g.dk) + c0;
-                    const float4 lam = *reinterpret_cast<const float4 *>(sLam + (r0 + i) * ldk + c0);
-                    const float lv[4] = {lam.x, lam.y, lam.z, lam.w};
-                    float dqv[4], dkv[4];
+            for (int i = 0; i < 8; ++i) {
+                const int row = sRow[r0 + i], o = (r0 + i) * ldk + cb;
+                float r[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        dqv[j] = aq[i][j] * expf(lv[j]);
-                        dkv[j] = ak[i][j] * expf(-lv[j]) + ak2[i][j] * expf(lc[j] - lv[j]);
+                for (int j = 0; j < 4; ++j) {
+                    r[j] = a1.v[i][j];
+                    if (kind == 0) {
+                        sX[o + j * cs] = sQ[o + j * cs] * r[j];
+                        r[j] *= sLam[o + j * cs];
+                    } else if (kind == 1) {
+                        r[j] /= sLam[o + j * cs];
                     }
-                    store4(dq + off, make_float4(dqv[0], dqv[1], dqv[2], dqv[3]));
-                    store4(dk + off, make_float4(dkv[0], dkv[1], dkv[2], dkv[3]));
-                    const float4 qq = load4(q + off), kk = load4(k + off);
-                    x = make_float4(qq.x * dqv[0] - kk.x * dkv[0], qq.y * dqv[1] - kk.y * dkv[1],
-                                    qq.z * dqv[2] - kk.z * dkv[2], qq.w * dqv[3] - kk.w * dkv[3]);
                 }
-                *reinterpret_cast<float4 *>(sX + (r0 + i) * ldk + c0) = x;
+                if (row >= 0) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) dst[(size_t)row * d + cb + j * cs] = TO(r[j]);
+                }
             }
+        }
+        __syncthreads();                    // every block of dq comes before the same block of dk
+        if (on && kind == 1) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int o = (r0 + i) * ldk + cb + j * cs;
+                    sX[o] -= sK[o] * a1.v[i][j];
+                }
         }
     }
     __syncthreads();
-    // gate gradient: suffix sum of x down the chunk plus what later chunks carry in
-    for (int c = threadIdx.x; c < g.dk; c += kThreads) {
-        float run = carry[((size_t)bh * g.N + chunk) * g.dk + c];
-        for (int j = g.C - 1; j >= 0; --j) {
-            const int p = chunk * g.C + j;
-            if (p >= g.L) continue;
-            run += sX[j * ldk + c];
-            const int t = scan_token(p, g.dir, g.gh, g.gw, g.L);
-            dgate[tok_offset(g, b, t, h, g.dk) + c] = run;
+    // gate gradient: suffix sums of x down the chunk plus what later chunks carry in, the rows cut in segments
+    {
+        const int nseg = min(kBwdThreads / g.dk, 8), rows = (g.C + nseg - 1) / nseg;
+        const int seg = threadIdx.x / g.dk, c = threadIdx.x - seg * g.dk, j0 = seg * rows, j1 = min(j0 + rows, g.C);
+        if (seg < nseg) {
+            float run = 0.f;
+#pragma unroll 8
+            for (int j = j1 - 1; j >= j0; --j) {
+                run += sX[j * ldk + c];
+                sX[j * ldk + c] = run;
+            }
+            sSeg[seg * g.dk + c] = run;
+        }
+        __syncthreads();
+        if (seg < nseg) {
+            float add = carry[chunk_id * g.dk + c];
+            for (int s = seg + 1; s < nseg; ++s) add += sSeg[s * g.dk + c];
+            float *dst = dgate + c;
+#pragma unroll 8
+            for (int j = j0; j < j1; ++j) {
+                const int row = sRow[j];
+                const float x = sX[j * ldk + c] + add;
+                if (row >= 0) dst[(size_t)row * g.dk] = x;
+            }
         }
     }
 }
@@ -428,7 +546,7 @@ fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
 size_t smem_state(const Geom &g, bool bwd)
 {
     const size_t ldk = g.dk + 4, ldv = g.dv + 4;
-    return sizeof(float) * (size_t)g.C * (ldk + ldv) * (bwd ? 2 : 1);
+    return sizeof(float) * ((size_t)g.C * ((bwd ? 3 : 2) * ldk + (bwd ? 2 : 1) * ldv) + 8 * (size_t)g.dk);
 }
 size_t smem_out(const Geom &g)
 {
@@ -440,7 +558,9 @@ size_t smem_out(const Geom &g)
 size_t smem_bwd(const Geom &g)
 {
     const size_t ldk = g.dk + 4, ldv = g.dv + 4, ldp = g.C + 4;
-    return sizeof(float) * ((size_t)g.C * (4 * ldk + 2 * ldv + 2 * ldp) + 2 * (size_t)g.dk * ldv);
+    size_t n = (size_t)g.C * (3 * ldk + 2 * ldv + 2 * ldp) + 2 * (size_t)g.dk * ldv;
+    if (!x_over_scores(g.C, g.dk, g.dv)) n += (size_t)g.C * ldk;
+    return sizeof(float) * n;
 }
 constexpr size_t kMaxSmem = 227 * 1024;
 
@@ -461,14 +581,14 @@ dig_status fwd_typed(const GlaArgs &a)
     auto k1 = fma_chunk_state<T, false>;
     if ((st = set_smem(k1, smem_state(g, false))) != DIG_OK) return st;
     { KernelTimer t(KID_FMA_STATE, a.stream);
-    k1<<<grid, kThreads, smem_state(g, false), a.stream>>>(
-        (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate, nullptr, w.states, w.gamma, nullptr, g); }
+    launch_pdl(k1, grid, dim3(kThreads), smem_state(g, false), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+               (const T *)nullptr, w.states, w.gamma, (float *)nullptr, g); }
     if ((st = launch_state_scan_fwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
     auto k3 = fma_chunk_out<T, TO>;
     if ((st = set_smem(k3, smem_out(g))) != DIG_OK) return st;
     KernelTimer t(KID_FMA_OUT, a.stream);
-    k3<<<grid, kThreads, smem_out(g), a.stream>>>((const T *)a.q, (const T *)a.k, (const T *)a.v,
-                                                  a.gate, w.states, (TO *)a.out, g);
+    launch_pdl(k3, grid, dim3(kThreads), smem_out(g), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+               (const float *)w.states, (TO *)a.out, g);
     return cuda_ok(cudaGetLastError());
 }
 
@@ -484,15 +604,14 @@ dig_status bwd_typed(const GlaArgs &a)
     auto k4 = fma_chunk_bwd<T, TO>;
     if ((st = set_smem(k4, smem_bwd(g))) != DIG_OK) return st;
     { KernelTimer t(KID_FMA_STATE, a.stream);
-    k1<<<grid, kThreads, smem_state(g, true), a.stream>>>(
-        (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate, (const T *)a.d_out, w.states, w.gamma,
-        w.dstates, g); }
+    launch_pdl(k1, grid, dim3(kThreads), smem_state(g, true), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+               (const T *)a.d_out, w.states, w.gamma, w.dstates, g); }
     if ((st = launch_state_scan_fwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
     if ((st = launch_state_scan_bwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
     KernelTimer t(KID_FMA_BWD, a.stream);
-    k4<<<grid, kThreads, smem_bwd(g), a.stream>>>(
-        (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate, (const T *)a.d_out, w.states, w.dstates,
-        w.carry, (TO *)a.dq, (TO *)a.dk, (TO *)a.dv, a.dgate, g);
+    launch_pdl(k4, grid, dim3(kBwdThreads), smem_bwd(g), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+               (const T *)a.d_out, (const float *)w.states, (const float *)w.dstates, (const float *)w.carry, (TO *)a.dq,
+               (TO *)a.dk, (TO *)a.dv, a.dgate, g);
     return cuda_ok(cudaGetLastError());
 }
 

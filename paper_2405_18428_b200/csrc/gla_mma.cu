@@ -359,6 +359,8 @@ mma_chunk_state(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__
     float *sSegV = sMlast + dvp;            // [4][dvp]
 
     fill_rows(sRow, g, C, b, h, chunk);
+    pdl_wait();
+    pdl_launch_dependents();
     __syncthreads();
     if (BETA) load_gates(sM, ldv, bd.bgate, sRow, C, dv, dvp);
     load_gates(sLam, ldk, gate, sRow, C, dk, dkp);
@@ -434,12 +436,15 @@ mma_chunk_out(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
 
     fill_rows(sRow, g, C, b, h, chunk);
     __syncthreads();
+    // the inputs of the call: whatever produced them has completed before the kernels in front of this one started
     if (BETA) load_gates(sM, ldv, bd.bgate, sRow, C, dv, dv);
     load_gates(sLam, ldk, gate, sRow, C, dk, dk);
-    load_state(sS, ldv, states + ((size_t)bh * g.N + chunk) * dk * dv, dk, dv);
     load_rows(sV, ldv, v, sRow, C, dv, dv);
     load_rows(sQ, ldk, q, sRow, C, dk, dk);
     load_rows(sK, ldk, k, sRow, C, dk, dk);
+    pdl_wait();                             // the states come from the scan in front
+    pdl_launch_dependents();
+    load_state(sS, ldv, states + ((size_t)bh * g.N + chunk) * dk * dv, dk, dv);
     cp_async_wait_all();
     __syncthreads();
     prefix_gates(sLam, ldk, C, dkp, sLast, sSeg);
@@ -515,14 +520,17 @@ mma_chunk_bwd(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
 
     fill_rows(sRow, g, C, b, h, chunk);
     __syncthreads();
+    // the inputs of the call: whatever produced them has completed before the kernels in front of this one started
     if (BETA) load_gates(sM, ldv, bd.bgate, sRow, C, dv, dv);
     load_gates(sLam, ldk, gate, sRow, C, dk, dk);
-    load_state(sS, ldv, states + chunk_id * dk * dv, dk, dv);
-    load_state(sD, ldv, dstates + chunk_id * dk * dv, dk, dv);
     load_rows(sV, ldv, v, sRow, C, dv, dv);
     load_rows(sG, ldv, d_out, sRow, C, dv, dv);
     load_rows(sQ, ldk, q, sRow, C, dk, dk);
     load_rows(sK, ldk, k, sRow, C, dk, dk);
+    pdl_wait();                             // the states come from the scans in front
+    pdl_launch_dependents();
+    load_state(sS, ldv, states + chunk_id * dk * dv, dk, dv);
+    load_state(sD, ldv, dstates + chunk_id * dk * dv, dk, dv);
     cp_async_wait_all();
     __syncthreads();
     prefix_gates(sLam, ldk, C, dkp, sLast, sSeg);
@@ -743,15 +751,15 @@ dig_status fwd_dims(const GlaArgs &a)
     if ((st = set_smem(k3, smem_out(g, BETA))) != DIG_OK) return st;
     {
         KernelTimer t(KID_MMA_STATE, a.stream);
-        k1<<<grid, kThreads, smem_state(g, false, BETA), a.stream>>>((const TI *)a.q, (const TI *)a.k, (const TI *)a.v,
-                                                                    a.gate, nullptr, w.states, w.gamma, nullptr, bd, g);
+        launch_pdl(k1, grid, dim3(kThreads), smem_state(g, false, BETA), a.stream, (const TI *)a.q, (const TI *)a.k, (const TI *)a.v,
+                   a.gate, (const TI *)nullptr, w.states, w.gamma, (float *)nullptr, bd, g);
     }
     if (BETA) st = launch_state_scan_fwd_beta(w, bd.gamma_v, g, a.stream, kRound);
     else st = launch_state_scan_fwd(w, g, a.stream, a.sio, kRound);
     if (st != DIG_OK) return st;
     KernelTimer t(KID_MMA_OUT, a.stream);
-    k3<<<grid, kThreads, smem_out(g, BETA), a.stream>>>((const TI *)a.q, (const TI *)a.k, (const TI *)a.v, a.gate,
-                                                        w.states, (TO *)a.out, bd, g);
+    launch_pdl(k3, grid, dim3(kThreads), smem_out(g, BETA), a.stream, (const TI *)a.q, (const TI *)a.k, (const TI *)a.v, a.gate,
+               (const float *)w.states, (TO *)a.out, bd, g);
     return cuda_ok(cudaGetLastError());
 }
 
@@ -770,9 +778,8 @@ dig_status bwd_dims(const GlaArgs &a)
     if ((st = set_smem(k4, smem_bwd(g, BETA))) != DIG_OK) return st;
     {
         KernelTimer t(KID_MMA_STATE, a.stream);
-        k1<<<grid, kThreads, smem_state(g, true, BETA), a.stream>>>((const TI *)a.q, (const TI *)a.k, (const TI *)a.v,
-                                                                   a.gate, (const TI *)a.d_out, w.states, w.gamma, w.dstates,
-                                                                   bd, g);
+        launch_pdl(k1, grid, dim3(kThreads), smem_state(g, true, BETA), a.stream, (const TI *)a.q, (const TI *)a.k, (const TI *)a.v,
+                   a.gate, (const TI *)a.d_out, w.states, w.gamma, w.dstates, bd, g);
     }
     if (BETA) {
         if ((st = launch_state_scan_fwd_beta(w, bd.gamma_v, g, a.stream, kRound)) != DIG_OK) return st;
@@ -783,9 +790,9 @@ dig_status bwd_dims(const GlaArgs &a)
     }
     {
         KernelTimer t(KID_MMA_BWD, a.stream);
-        k4<<<grid, kThreads, smem_bwd(g, BETA), a.stream>>>((const TI *)a.q, (const TI *)a.k, (const TI *)a.v, a.gate,
-                                                            (const TI *)a.d_out, w.states, w.dstates, w.carry, (TO *)a.dq,
-                                                            (TO *)a.dk, (TO *)a.dv, a.dgate, bd, g);
+        launch_pdl(k4, grid, dim3(kThreads), smem_bwd(g, BETA), a.stream, (const TI *)a.q, (const TI *)a.k, (const TI *)a.v, a.gate,
+                   (const TI *)a.d_out, (const float *)w.states, (const float *)w.dstates, (const float *)w.carry, (TO *)a.dq,
+                   (TO *)a.dk, (TO *)a.dv, a.dgate, bd, g);
     }
     if (cudaGetLastError() != cudaSuccess) return DIG_ERR_CUDA;
     if (BETA) return launch_beta_carry(bd.dbgate, bd.xtot, g, a.stream);

@@ -132,6 +132,8 @@ state_scan_bwd(const float *__restrict__ states, float *__restrict__ dstates,
                const float *__restrict__ gamma, float *__restrict__ carry, const float *__restrict__ s_final,
                const float *__restrict__ ds_out, float *__restrict__ ds_in, int N, int dk, int dv)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * kRowsPerBlock + (threadIdx.x >> 5);
     if (c >= dk) return;
@@ -203,6 +205,8 @@ __global__ void __launch_bounds__(kScanThreads)
 state_scan_fwd_beta(float *__restrict__ states, const float *__restrict__ gamma, const float *__restrict__ gamma_v,
                     float *__restrict__ s_final, int N, int dk, int dv, bool tf32)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     const int e4 = blockIdx.x * kScanThreads + threadIdx.x;
     if (e4 * 4 >= dk * dv) return;
     const int row = (e4 * 4) / dv, col = (e4 * 4) - row * dv;
@@ -240,6 +244,8 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock)
 state_scan_bwd_beta(const float *__restrict__ states, float *__restrict__ dstates, const float *__restrict__ gamma,
                     const float *__restrict__ gamma_v, float *__restrict__ carry, int N, int dk, int dv, bool tf32)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * kRowsPerBlock + (threadIdx.x >> 5);
     if (c >= dk) return;
@@ -294,6 +300,8 @@ state_scan_bwd_beta(const float *__restrict__ states, float *__restrict__ dstate
 __global__ void __launch_bounds__(128)
 beta_suffix_totals(float *__restrict__ xtot, int N, int dv, int total)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     const int idx = blockIdx.x * 128 + threadIdx.x;
     if (idx >= total) return;
     const int bh = idx / dv, e = idx - bh * dv;
@@ -310,6 +318,8 @@ beta_suffix_totals(float *__restrict__ xtot, int N, int dv, int total)
 __global__ void __launch_bounds__(256)
 beta_add_carry(float *__restrict__ dbgate, const float *__restrict__ xtot, Geom g)
 {
+    pdl_wait();
+    pdl_launch_dependents();
     const int per_row = g.dv >> 2;
     const long long idx = (long long)blockIdx.x * 256 + threadIdx.x;
     const long long total = (long long)g.B * g.H * g.L * per_row;
@@ -338,15 +348,15 @@ dig_status launch_state_scan_fwd(const Workspace &w, const Geom &g, cudaStream_t
     if ((long long)grid.x * grid.y * kScanThreads < 16384) {       // few sequences: one element per thread
         const dim3 grid1((g.dk * g.dv + kScan1Threads - 1) / kScan1Threads, g.B * g.H);
         if (tf32)
-            state_scan_fwd1<true><<<grid1, kScan1Threads, 0, s>>>(w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
+            launch_pdl(state_scan_fwd1<true>, grid1, dim3(kScan1Threads), 0, s, w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
         else
-            state_scan_fwd1<false><<<grid1, kScan1Threads, 0, s>>>(w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
+            launch_pdl(state_scan_fwd1<false>, grid1, dim3(kScan1Threads), 0, s, w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
         return cuda_ok(cudaGetLastError());
     }
     if (tf32)
-        state_scan_fwd<true><<<grid, kScanThreads, 0, s>>>(w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
+        launch_pdl(state_scan_fwd<true>, grid, dim3(kScanThreads), 0, s, w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
     else
-        state_scan_fwd<false><<<grid, kScanThreads, 0, s>>>(w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
+        launch_pdl(state_scan_fwd<false>, grid, dim3(kScanThreads), 0, s, w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
     return cuda_ok(cudaGetLastError());
 }
 
@@ -356,10 +366,10 @@ dig_status launch_state_scan_bwd(const Workspace &w, const Geom &g, cudaStream_t
     const dim3 grid((g.dk + kRowsPerBlock - 1) / kRowsPerBlock, g.B * g.H);
     KernelTimer t(KID_SCAN_BWD, s);
     if (tf32)
-        state_scan_bwd<true><<<grid, 32 * kRowsPerBlock, 0, s>>>(w.states, w.dstates, w.gamma, w.carry, w.sfinal, sio.ds_out,
+        launch_pdl(state_scan_bwd<true>, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, w.carry, w.sfinal, sio.ds_out,
                                                                  sio.ds_in, g.N, g.dk, g.dv);
     else
-        state_scan_bwd<false><<<grid, 32 * kRowsPerBlock, 0, s>>>(w.states, w.dstates, w.gamma, w.carry, w.sfinal, sio.ds_out,
+        launch_pdl(state_scan_bwd<false>, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, w.carry, w.sfinal, sio.ds_out,
                                                                   sio.ds_in, g.N, g.dk, g.dv);
     return cuda_ok(cudaGetLastError());
 }
@@ -368,7 +378,7 @@ dig_status launch_state_scan_fwd_beta(const Workspace &w, const float *gamma_v, 
 {
     const dim3 grid((g.dk * g.dv / 4 + kScanThreads - 1) / kScanThreads, g.B * g.H);
     KernelTimer t(KID_SCAN_FWD, s);
-    state_scan_fwd_beta<<<grid, kScanThreads, 0, s>>>(w.states, w.gamma, gamma_v, w.sfinal, g.N, g.dk, g.dv, tf32);
+    launch_pdl(state_scan_fwd_beta, grid, dim3(kScanThreads), 0, s, w.states, w.gamma, gamma_v, w.sfinal, g.N, g.dk, g.dv, tf32);
     return cuda_ok(cudaGetLastError());
 }
 
@@ -376,7 +386,7 @@ dig_status launch_state_scan_bwd_beta(const Workspace &w, const float *gamma_v, 
 {
     const dim3 grid((g.dk + kRowsPerBlock - 1) / kRowsPerBlock, g.B * g.H);
     KernelTimer t(KID_SCAN_BWD, s);
-    state_scan_bwd_beta<<<grid, 32 * kRowsPerBlock, 0, s>>>(w.states, w.dstates, w.gamma, gamma_v, w.carry, g.N, g.dk, g.dv, tf32);
+    launch_pdl(state_scan_bwd_beta, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, gamma_v, w.carry, g.N, g.dk, g.dv, tf32);
     return cuda_ok(cudaGetLastError());
 }
 
@@ -384,10 +394,10 @@ dig_status launch_beta_carry(float *dbgate, float *xtot, const Geom &g, cudaStre
 {
     KernelTimer t(KID_SCAN_BWD, s);
     const int total = g.B * g.H * g.dv;
-    beta_suffix_totals<<<(total + 127) / 128, 128, 0, s>>>(xtot, g.N, g.dv, total);
+    launch_pdl(beta_suffix_totals, dim3((total + 127) / 128), dim3(128), 0, s, xtot, g.N, g.dv, total);
     if (cudaGetLastError() != cudaSuccess) return DIG_ERR_CUDA;
     const long long n = (long long)g.B * g.H * g.L * (g.dv >> 2);
-    beta_add_carry<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dbgate, xtot, g);
+    launch_pdl(beta_add_carry, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, dbgate, xtot, g);
     return cuda_ok(cudaGetLastError());
 }
 

@@ -48,6 +48,20 @@ def test_chunk128_forward_and_d72():
     check_workload(wl.scaled(d_k=72, d_v=72, chunk=64, backward=True), 1)
 
 
+@pytest.mark.parametrize("dk,dv,chunk,grid,dtype", [
+    (128, 8, 64, (5, 13), "f32"),       # one row past a chunk; two rounds of gradient blocks
+    (64, 64, 16, (3, 11), "f32"),       # the q*dq - k*dk tile does not fit over the scores
+    (8, 128, 32, (1, 31), "bf16"),      # one row short of a chunk
+    (8, 8, 128, (9, 29), "f32"),        # fewer channels than one warp's columns
+    (72, 72, 64, (2, 32), "bf16"),
+])
+def test_gradient_block_rounds_and_tile_edges(dk, dv, chunk, grid, dtype):
+    from parity import check_workload
+    wl = Workload("rounds", B=1, H=2, grid_h=grid[0], grid_w=grid[1], d_k=dk, d_v=dv, chunk=chunk, dtype=dtype,
+                  backward=True, tau=(16.0, 2.0), seed=8)
+    check_workload(wl, 2)
+
+
 def test_c2_bf16_storage_on_fma_family():
     from parity import check_workload
     errs = check_workload(CONFIGS["C2"], 2)
