@@ -120,6 +120,15 @@ def test_conv_bwd_tiny_grids():
         _conv_bwd_case(1, gh, gw, 8, "f32", 2, with_bias=True)
 
 
+@pytest.mark.parametrize("B,gh,gw,D,dtype,direction", [
+    (1, 37, 53, 136, "bf16", 1),        # strips cut into uneven row segments, one column in the last strip's second half
+    (3, 2, 33, 72, "bf16", 2),          # more strips than partial sums: a CTA walks several, the last one column wide
+    (2, 65, 12, 200, "f32", 3),         # a last channel block of 8 channels, segments of 8 rows and one of 1
+])
+def test_conv_bwd_strip_edges(B, gh, gw, D, dtype, direction):
+    _conv_bwd_case(B, gh, gw, D, dtype, direction, with_bias=True, seed=20 + direction)
+
+
 @pytest.mark.parametrize("cfg", ["C2", "C5"])
 def test_conv_bwd_benchmark_shapes(cfg):
     from paper_2405_18428_b200 import dig
