@@ -41,7 +41,6 @@ gate_logsigmoid(const T *__restrict__ g, float *__restrict__ gate, size_t n8, in
                 InvTau inv_tau)
 {
     pdl_wait();
-    pdl_launch_dependents();      // only once this kernel's own predecessor has completed
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += stride) {
         const size_t e = i * 8;
@@ -53,6 +52,7 @@ gate_logsigmoid(const T *__restrict__ g, float *__restrict__ gate, size_t n8, in
         store4(gate + e + 4, make_float4(log_sigmoid(b.x) * it, log_sigmoid(b.y) * it,
                                          log_sigmoid(b.z) * it, log_sigmoid(b.w) * it));
     }
+    pdl_launch_dependents();
 }
 
 }  // namespace

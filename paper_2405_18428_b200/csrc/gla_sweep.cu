@@ -137,7 +137,6 @@ sweep_local_fwd(const SweepArgs a)
     const int total = g.B * g.H * pl.nseg;
 
     pdl_wait();
-    pdl_launch_dependents();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
@@ -216,6 +215,7 @@ sweep_local_fwd(const SweepArgs a)
     }
 die:
     cta_teardown(ctl, SM::tmem_cols);
+    pdl_launch_dependents();
 }
 
 // =================================================================================================
@@ -281,7 +281,6 @@ sweep_local_bwd(const SweepArgs a)
     };
 
     pdl_wait();
-    pdl_launch_dependents();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
@@ -370,6 +369,7 @@ sweep_local_bwd(const SweepArgs a)
     }
 die:
     cta_teardown(ctl, SM::tmem_cols);
+    pdl_launch_dependents();
 }
 
 // =================================================================================================
@@ -555,7 +555,6 @@ sweep_fwd(const SweepArgs a)
     if (pl.nseg == 1) pdl_wait();
     if ((int)blockIdx.x < total) prime(blockIdx.x);
     pdl_wait();
-    pdl_launch_dependents();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
@@ -668,6 +667,7 @@ sweep_fwd(const SweepArgs a)
     }
 die:
     cta_teardown(ctl, SM::tmem_cols);
+    pdl_launch_dependents();
 }
 
 // =================================================================================================
@@ -765,7 +765,6 @@ sweep_bwd(const SweepArgs a)
     };
     if ((int)blockIdx.x < total) prime(blockIdx.x);
     pdl_wait();
-    pdl_launch_dependents();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
@@ -995,6 +994,7 @@ sweep_bwd(const SweepArgs a)
 die:
     if (!ok && w.issuer() && elect_one()) mbar_wait(barS, par, a.status);      // let bulk copies in flight land
     cta_teardown(ctl, SM::tmem_cols);
+    pdl_launch_dependents();
 }
 
 #undef SYNC_OR_DIE

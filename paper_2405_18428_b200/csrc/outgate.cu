@@ -277,7 +277,6 @@ outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const floa
     ln.dv = dv;
     const float inv_d = 1.f / (float)dv;
     pdl_wait();
-    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         ring.fetch(0);
         ring.fetch(1);
@@ -309,6 +308,7 @@ outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const floa
         ok = ring.hand_over(it, ok);
         if (!ok) break;
     }
+    pdl_launch_dependents();
     ring.drain(it, ok);
 }
 
@@ -349,7 +349,6 @@ outgate_bwd(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln
 #pragma unroll
     for (int e = 0; e < NP; ++e) aw[e] = ab[e] = make_float2(0.f, 0.f);
     pdl_wait();
-    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         ring.fetch(0);
         ring.fetch(1);
@@ -397,6 +396,7 @@ outgate_bwd(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln
         ok = ring.hand_over(it, ok);
         if (!ok) break;
     }
+    pdl_launch_dependents();
     ring.drain(it, ok);
     if (partial == nullptr) return;
     __syncthreads();                                             // the copies have left: the ring becomes scratch
