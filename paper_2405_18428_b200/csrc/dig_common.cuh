@@ -162,10 +162,9 @@ size_t mma_beta_workspace_bytes(const Geom &g, bool backward);
 // Chunk-state scans, shared by both families (plain fp32 FMA, bandwidth-bound).
 dig_status launch_state_scan_fwd(const Workspace &w, const Geom &g, cudaStream_t s, const StateIO &sio, bool tf32 = false);
 dig_status launch_state_scan_bwd(const Workspace &w, const Geom &g, cudaStream_t s, const StateIO &sio, bool tf32 = false);
-// Scans with the value-channel gate (row-major states, tf32-rounded results) and the cross-chunk part of its gradient.
+// Scans with the value-channel gate (row-major states, tf32-rounded results).
 dig_status launch_state_scan_fwd_beta(const Workspace &w, const float *gamma_v, const Geom &g, cudaStream_t s, bool tf32);
 dig_status launch_state_scan_bwd_beta(const Workspace &w, const float *gamma_v, const Geom &g, cudaStream_t s, bool tf32);
-dig_status launch_beta_carry(float *dbgate, float *xtot, const Geom &g, cudaStream_t s);
 
 // Device status word (bounded waits report here).
 int *device_status_ptr();

@@ -21,7 +21,9 @@ namespace dig {
 namespace {
 
 constexpr int kThreads = 256;        // state and output kernels
-constexpr int kBwdThreads = 512;     // gradient kernel
+constexpr int kBwdThreads = 512;     // gradient kernel, at most
+// Threads of the gradient kernel: 128 registers each fill an SM with one CTA of a 64-token chunk or two of a shorter one
+__host__ __device__ inline int bwd_threads(int C) { return C >= 64 ? kBwdThreads : kBwdThreads / 2; }
 
 // ---- 4x4 register-blocked contractions over shared memory --------------------------------
 // acc[i][j] += sum_k A[(r0+i)*lda + k] * Bm[(c0 + j*cstep)*ldb + k], columns j < jn only (jn uniform enough over a
@@ -401,7 +403,7 @@ __host__ __device__ inline int grad_blocks(int C, int d) { return ((C / 8) * (d 
 // The tile of q*dq - k*dk lies over the score tiles where it fits and one round of blocks is all there is.
 __host__ __device__ inline bool x_over_scores(int C, int dk, int dv)
 {
-    return dk + 4 <= 2 * (C + 4) && 2 * grad_blocks(C, dk) + grad_blocks(C, dv) <= kBwdThreads;
+    return dk + 4 <= 2 * (C + 4) && 2 * grad_blocks(C, dk) + grad_blocks(C, dv) <= bwd_threads(C);
 }
 template <typename T, typename TO>
 __global__ void __launch_bounds__(kBwdThreads)
@@ -414,6 +416,7 @@ fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     extern __shared__ __align__(16) float smem[];
     const int chunk = blockIdx.x, bh = blockIdx.y, b = bh / g.H, h = bh - b * g.H;
     const int ldk = g.dk + 4, ldv = g.dv + 4, ldp = g.C + 4;
+    const int threads = blockDim.x;
     const bool over = x_over_scores(g.C, g.dk, g.dv);
     float *sLam = smem;
     float *sQ = sLam + g.C * ldk;
@@ -448,7 +451,7 @@ fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     load_state(sS, ldv, states + chunk_id * g.dk * g.dv, g.dk, g.dv);
     load_state(sD, ldv, dstates + chunk_id * g.dk * g.dv, g.dk, g.dv);
     const int nb = g.C >> 2, nsc = nb * nb;
-    for (int blk = threadIdx.x; blk < 2 * nsc; blk += kBwdThreads) {
+    for (int blk = threadIdx.x; blk < 2 * nsc; blk += threads) {
         const bool p = blk < nsc;           // scores, then dO V^T
         score_block(p ? sP : sdP, ldp, p ? sQ : sG, p ? ldk : ldv, p ? sK : sV, p ? ldk : ldv, g.C, p ? g.dk : g.dv, p ? blk : blk - nsc);
     }
@@ -456,7 +459,7 @@ fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     __syncthreads();
 
     const int nk = grad_blocks(g.C, g.dk), nv = grad_blocks(g.C, g.dv), total = 2 * nk + nv;
-    for (int base = 0; base < total; base += kBwdThreads) {
+    for (int base = 0; base < total; base += threads) {
         const int t = base + threadIdx.x, kind = t < nk ? 0 : t < 2 * nk ? 1 : t < total ? 2 : 3;      // uniform over a warp
         const int blk = t - kind * nk, d = kind == 2 ? g.dv : g.dk, cs = d >> 2, r0 = 8 * (blk / cs), cb = blk % cs;
         const bool on = kind < 3 && r0 < g.C;
@@ -517,7 +520,7 @@ fma_chunk_bwd(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     __syncthreads();
     // gate gradient: suffix sums of x down the chunk plus what later chunks carry in, the rows cut in segments
     {
-        const int nseg = min(kBwdThreads / g.dk, 8), rows = (g.C + nseg - 1) / nseg;
+        const int nseg = min(threads / g.dk, 8), rows = (g.C + nseg - 1) / nseg;
         const int seg = threadIdx.x / g.dk, c = threadIdx.x - seg * g.dk, j0 = seg * rows, j1 = min(j0 + rows, g.C);
         if (seg < nseg) {
             float run = 0.f;
@@ -609,7 +612,7 @@ dig_status bwd_typed(const GlaArgs &a)
     if ((st = launch_state_scan_fwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
     if ((st = launch_state_scan_bwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
     KernelTimer t(KID_FMA_BWD, a.stream);
-    launch_pdl(k4, grid, dim3(kBwdThreads), smem_bwd(g), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+    launch_pdl(k4, grid, dim3(bwd_threads(g.C)), smem_bwd(g), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
                (const T *)a.d_out, (const float *)w.states, (const float *)w.dstates, (const float *)w.carry, (TO *)a.dq,
                (TO *)a.dk, (TO *)a.dv, a.dgate, g);
     return cuda_ok(cudaGetLastError());

@@ -12,6 +12,13 @@
 // x = hi + lo: three products hi*hi + lo*hi + hi*lo per fragment pair leave errors of order 2^-21,
 // the accuracy fp32 storage is held to.
 //
+// What bounds it: the words of shared memory a fragment costs, and latency, since the fp32 tiles of a 64-token chunk leave
+// room for one CTA of the gradient kernel per SM.  Hence all tiles of a kernel are loaded in one pass, the gradient
+// kernel works in 32-row warp tiles, and products whose operands both lie along their rows spread over all banks.
+// Full gate, 8 x 1024 tokens of 6 heads, d = C = 64 (us, before -> now): state 24 -> 20.4, with gradients 39 -> 30,
+// outputs 35.6 -> 33.4, gradients 108 -> 88, and 13.5 for the value gate's sums over later chunks -> none (the gradient
+// kernel takes them from the state leaving its chunk).
+//
 // Notation per chunk (rows j = 0..C-1 in scan order, zero rows past the end of the sequence):
 //   Lam_j = inclusive prefix sum of the gates, gamma = exp(Lam_{C-1}),
 //   Qt = q*exp(Lam), Kt = k*exp(-Lam), Kh = k*exp(Lam_{C-1}-Lam),
@@ -41,7 +48,7 @@ __host__ __device__ constexpr int tight(int d) { return d + 4; }
 template <int C_, int DK_, int DV_>
 struct FixedDims {
     static constexpr int kC = C_, kDK = DK_, kDV = DV_;      // 0 = not known at compile time
-    __device__ explicit FixedDims(const Geom &) {}
+    __host__ __device__ explicit FixedDims(const Geom &) {}
     __device__ constexpr int C() const { return C_; }
     __device__ constexpr int dk() const { return DK_; }
     __device__ constexpr int dv() const { return DV_; }
@@ -49,7 +56,7 @@ struct FixedDims {
 struct AnyDims {
     static constexpr int kC = 0, kDK = 0, kDV = 0;
     int c_, dk_, dv_;
-    __device__ explicit AnyDims(const Geom &g) : c_(g.C), dk_(g.dk), dv_(g.dv) {}
+    __host__ __device__ explicit AnyDims(const Geom &g) : c_(g.C), dk_(g.dk), dv_(g.dv) {}
     __device__ int C() const { return c_; }
     __device__ int dk() const { return dk_; }
     __device__ int dv() const { return dv_; }
@@ -60,7 +67,6 @@ struct BetaDev {
     const float *bgate;     // log(beta) [B][L][H][d_v]
     float *gamma_v;         // [B*H][N][d_v]  exp of the chunk totals of bgate
     float *dbgate;          // gradient with respect to bgate (backward pass)
-    float *xtot;            // [B*H][N][d_v]  chunk totals of o*do - v*dv (backward pass)
 };
 
 __device__ __forceinline__ float tf32r(float x)
@@ -87,44 +93,62 @@ __device__ __forceinline__ void mma8(float (&c)[4], const uint32_t (&a)[4], uint
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// One warp: acc[nb] += A(r0 .. r0+15, k) * B(k, c0 + 8 nb .. c0 + 8 nb + 7) for k in [k0, k1), nb < nbw.
+// One warp: acc[mb][nb] += A(r0 + 16 mb .. + 15, k) * B(k, c0 + 8 nb .. + 7) for k in [k0, k1), mb < mbw, nb < nbw.
 // A(m, k) = A[m*sam + k*sak], B(k, n) = Bm[k*sbk + n*sbn]; k0, k1 multiples of 8.
 // Fragment layout of m16n8k8: with g = lane / 4, t = lane % 4 a lane holds A(g | g+8, t | t+4),
-// B(t | t+4, g) and the results C(g | g+8, 2t | 2t+1).
-template <bool PR, int NB>
-__device__ __forceinline__ void warp_mma(float (&acc)[NB][4], const float *A, int sam, int sak, int r0,
-                                         const float *Bm, int sbk, int sbn, int c0, int nbw, int k0, int k1)
+// B(t | t+4, g) and the results C(g | g+8, 2t | 2t+1).  The four + four lanes of a contraction step may hold any of its
+// eight indices as long as A and B agree: where both operands lie with the contraction down their rows (strides
+// sak = sbk = a row) they take 2t and 2t+1 (ALONG), which spreads rows a multiple of four words apart over all banks
+// (t and t+4: two lanes to a bank).
+template <bool PR, bool ALONG, int MB, int NB>
+__device__ __forceinline__ void warp_mma(float (&acc)[MB][NB][4], const float *A, int sam, int sak, int r0,
+                                         const float *Bm, int sbk, int sbn, int c0, int mbw, int nbw, int k0, int k1)
 {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const float *pa = A + (r0 + g) * sam + (t + k0) * sak;
-    const float *pb = Bm + (t + k0) * sbk + (c0 + g) * sbn;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, t0 = ALONG ? 2 * t : t, dt = ALONG ? 1 : 4;
+    const float *pa = A + (r0 + g) * sam + (t0 + k0) * sak;
+    const float *pb = Bm + (t0 + k0) * sbk + (c0 + g) * sbn;
 #pragma unroll 2
     for (int k = k0; k < k1; k += 8) {
-        const float af[4] = {pa[0], pa[8 * sam], pa[4 * sak], pa[8 * sam + 4 * sak]};
-        uint32_t a[4], al[4];
+        uint32_t a[MB][4], al[MB][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (PR) split_tf32(af[i], a[i], al[i]);
-            else a[i] = __float_as_uint(af[i]);
-        }
+        for (int mb = 0; mb < MB; ++mb)
+            if (mb < mbw) {
+                const float *pm = pa + 16 * mb * sam;
+                const float af[4] = {pm[0], pm[8 * sam], pm[dt * sak], pm[8 * sam + dt * sak]};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (PR) split_tf32(af[i], a[mb][i], al[mb][i]);
+                    else a[mb][i] = __float_as_uint(af[i]);
+                }
+            }
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
             if (nb < nbw) {
-                const float bf0 = pb[8 * nb * sbn], bf1 = pb[4 * sbk + 8 * nb * sbn];
+                const float bf0 = pb[8 * nb * sbn], bf1 = pb[dt * sbk + 8 * nb * sbn];
+                uint32_t b0 = __float_as_uint(bf0), b1 = __float_as_uint(bf1), b0l, b1l;
                 if (PR) {
-                    uint32_t b0, b1, b0l, b1l;
                     split_tf32(bf0, b0, b0l);
                     split_tf32(bf1, b1, b1l);
-                    mma8(acc[nb], al, b0, b1);          // the small terms first
-                    mma8(acc[nb], a, b0l, b1l);
-                    mma8(acc[nb], a, b0, b1);
-                } else {
-                    mma8(acc[nb], a, __float_as_uint(bf0), __float_as_uint(bf1));
                 }
+#pragma unroll
+                for (int mb = 0; mb < MB; ++mb)
+                    if (mb < mbw) {
+                        if (PR) {
+                            mma8(acc[mb][nb], al[mb], b0, b1);          // the small terms first
+                            mma8(acc[mb][nb], a[mb], b0l, b1l);
+                        }
+                        mma8(acc[mb][nb], a[mb], b0, b1);
+                    }
             }
         pa += 8 * sak;
         pb += 8 * sbk;
     }
+}
+template <bool PR, bool ALONG, int NB>
+__device__ __forceinline__ void warp_mma(float (&acc)[NB][4], const float *A, int sam, int sak, int r0,
+                                         const float *Bm, int sbk, int sbn, int c0, int nbw, int k0, int k1)
+{
+    warp_mma<PR, ALONG>(reinterpret_cast<float (&)[1][NB][4]>(acc), A, sam, sak, r0, Bm, sbk, sbn, c0, 1, nbw, k0, k1);
 }
 
 template <int NB>
@@ -137,6 +161,12 @@ __device__ __forceinline__ void zero(float (&acc)[NB][4])
 }
 
 // Calls f(row, col, v0, v1) for every pair of adjacent result columns this lane holds (col even).
+template <int MB, int NB>
+__device__ __forceinline__ void zero(float (&acc)[MB][NB][4])
+{
+#pragma unroll
+    for (int mb = 0; mb < MB; ++mb) zero(acc[mb]);
+}
 template <int NB, typename F>
 __device__ __forceinline__ void for_pairs(const float (&acc)[NB][4], int r0, int c0, int nbw, F f)
 {
@@ -147,6 +177,14 @@ __device__ __forceinline__ void for_pairs(const float (&acc)[NB][4], int r0, int
             f(r0 + g, c0 + 8 * nb + 2 * t, acc[nb][0], acc[nb][1]);
             f(r0 + g + 8, c0 + 8 * nb + 2 * t, acc[nb][2], acc[nb][3]);
         }
+}
+
+template <int MB, int NB, typename F>
+__device__ __forceinline__ void for_pairs(const float (&acc)[MB][NB][4], int r0, int c0, int mbw, int nbw, F f)
+{
+#pragma unroll
+    for (int mb = 0; mb < MB; ++mb)
+        if (mb < mbw) for_pairs(acc[mb], r0 + 16 * mb, c0, nbw, f);
 }
 
 // The warp tiles of an M x N result (M a multiple of 16, N of 8): 16 rows by a group of 8-column
@@ -160,6 +198,15 @@ __host__ __device__ constexpr int tile_splits(int M, int N)
 __host__ __device__ constexpr int tile_frags(int M, int N) { return ((N >> 3) + tile_splits(M, N) - 1) / tile_splits(M, N); }
 // Fragments per warp tile as a compile-time bound: exact when both extents are known, else the maximum.
 __host__ __device__ constexpr int frag_bound(int M, int N) { return (M > 0 && N > 0) ? tile_frags(M, N) : kMaxNB; }
+// 8-column fragments of the gradient kernel's tiles of up to 32 rows: the columns are split until the tiles of one
+// result are eight (two results side by side fill the warps), and to `most` fragments (registers: two accumulators each).
+// 32 x 16 tiles read 16 words of shared memory a lane for four MMAs, 16 x 16 tiles 12 for two.
+__host__ __device__ constexpr int grad_frags(int C, int N, int most)
+{
+    const int want = C >= 32 && C <= 256 ? 8 / ((C + 31) / 32) : 8, nf = N > 0 ? N >> 3 : 64;
+    const int n = (nf + want - 1) / want;
+    return C <= 0 || N <= 0 || n > most ? most : n;
+}
 struct Tiling {
     int nrt, nfrag, nbw, ntiles;
     __device__ Tiling(int M, int N) : nrt(M >> 4), nfrag(N >> 3), nbw(tile_frags(M, N)), ntiles((M >> 4) * tile_splits(M, N)) {}
@@ -203,31 +250,30 @@ __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
-__device__ __forceinline__ void load_rows(float *dst, int ld, const __nv_bfloat16 *src, const int *sRow, int C, int d, int dp)
+// NT tiles with the same row length: all of a thread's loads of a pass are in flight together.
+template <int NT>
+__device__ __forceinline__ void load_tiles(float *const (&dst)[NT], int ld, const __nv_bfloat16 *const (&src)[NT], const int *sRow, int C, int d, int dp)
 {
-    constexpr int U = 4;
+    constexpr int U = NT == 1 ? 4 : 2;
     const int per_row = dp >> 2, n = C * per_row;      // dp: columns to fill (d, or d padded to 16)
     for (int base = threadIdx.x; base < n; base += U * kThreads) {
-        uint2 raw[U];
+        uint2 raw[U][NT];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int idx = base + u * kThreads;
-            raw[u] = make_uint2(0u, 0u);
-            if (idx < n) {
-                const int j = idx / per_row, c = (idx - j * per_row) << 2;
-                const int row = sRow[j];
-                if (row >= 0 && c < d) raw[u] = *reinterpret_cast<const uint2 *>(src + (size_t)row * d + c);
-            }
+            const int idx = base + u * kThreads, j = idx / per_row, c = (idx - j * per_row) << 2;
+            const int row = idx < n ? sRow[j] : -1;
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+                raw[u][i] = row >= 0 && c < d ? *reinterpret_cast<const uint2 *>(src[i] + (size_t)row * d + c) : make_uint2(0u, 0u);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int idx = base + u * kThreads;
-            if (idx < n) {
-                const int j = idx / per_row, c = (idx - j * per_row) << 2;
-                *reinterpret_cast<float4 *>(dst + j * ld + c) =
-                    make_float4(__uint_as_float(raw[u].x << 16), __uint_as_float(raw[u].x & 0xffff0000u),
-                                __uint_as_float(raw[u].y << 16), __uint_as_float(raw[u].y & 0xffff0000u));
-            }
+            const int idx = base + u * kThreads, j = idx / per_row, c = (idx - j * per_row) << 2;
+            if (idx < n)
+#pragma unroll
+                for (int i = 0; i < NT; ++i)
+                    *reinterpret_cast<float4 *>(dst[i] + j * ld + c) =
+                        make_float4(lo_f(raw[u][i].x), hi_f(raw[u][i].x), lo_f(raw[u][i].y), hi_f(raw[u][i].y));
         }
     }
 }
@@ -241,9 +287,11 @@ __device__ __forceinline__ void load_gates(float *dst, int ld, const float *gate
         else *reinterpret_cast<float4 *>(dst + j * ld + c) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
-__device__ __forceinline__ void load_rows(float *dst, int ld, const float *src, const int *sRow, int C, int d, int dp)
+template <int NT>
+__device__ __forceinline__ void load_tiles(float *const (&dst)[NT], int ld, const float *const (&src)[NT], const int *sRow, int C, int d, int dp)
 {
-    load_gates(dst, ld, src, sRow, C, d, dp);       // fp32 rows travel like the gates
+#pragma unroll
+    for (int i = 0; i < NT; ++i) load_gates(dst[i], ld, src[i], sRow, C, d, dp);       // fp32 rows travel like the gates
 }
 // A [dk][dv] state of the workspace (rounded to tf32 by the scan kernels) -> [dk][ld] tile.
 __device__ __forceinline__ void load_state(float *dst, int ld, const float *src, int dk, int dv)
@@ -255,32 +303,47 @@ __device__ __forceinline__ void load_state(float *dst, int ld, const float *src,
         else *reinterpret_cast<float4 *>(dst + r * ld + c) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
+// First of the threads that work on the value-channel gate: behind those of the key-channel gate (four per channel)
+// where the CTA has that many, else the same.
+__device__ __forceinline__ int value_thread(int dkp, int dvp) { return 4 * (dkp + dvp) <= kThreads ? (int)threadIdx.x - 4 * dkp : (int)threadIdx.x; }
+
 // In place: gates -> inclusive prefix sums down the rows of the chunk; sLast receives the last row.
 // Four threads per channel take a quarter of the rows each; sSeg ([4][dkp]) carries the quarter totals.
-// Contains two barriers.
-__device__ __forceinline__ void prefix_gates(float *lam, int ld, int C, int dkp, float *sLast, float *sSeg)
+// BETA: the same for the value-channel gate.  Contains two barriers.
+template <bool BETA>
+__device__ __forceinline__ void prefix_gates(float *lam, int ld, int C, int dkp, float *sLast, float *sSeg, float *lam_v, int ldv, int dvp, float *sLastV, float *sSegV)
 {
     const int rows = C >> 2;                    // C is a multiple of 16
-    const int c = threadIdx.x % dkp, seg = threadIdx.x / dkp;      // 4 * dkp <= kThreads
-    float run = 0.f;
-    if (seg < 4) {
+    auto sums = [&](float *x, int ldx, int dp, float *segs, int tid) -> float {
+        const int c = tid % dp, seg = tid / dp;      // 4 * dp <= kThreads
+        float run = 0.f;
+        if (tid >= 0 && seg < 4) {
 #pragma unroll 8
-        for (int j = seg * rows; j < (seg + 1) * rows; ++j) {
-            run += lam[j * ld + c];
-            lam[j * ld + c] = run;
+            for (int j = seg * rows; j < (seg + 1) * rows; ++j) {
+                run += x[j * ldx + c];
+                x[j * ldx + c] = run;
+            }
+            segs[seg * dp + c] = run;
         }
-        sSeg[seg * dkp + c] = run;
-    }
+        return run;
+    };
+    auto shift = [&](float *x, int ldx, int dp, const float *segs, float *last, int tid, float run) {
+        const int c = tid % dp, seg = tid / dp;
+        if (tid >= 0 && seg < 4) {
+            float add = 0.f;
+            for (int sg = 0; sg < seg; ++sg) add += segs[sg * dp + c];
+            if (seg > 0) {
+#pragma unroll 8
+                for (int j = seg * rows; j < (seg + 1) * rows; ++j) x[j * ldx + c] += add;
+            }
+            if (seg == 3) last[c] = run + add;
+        }
+    };
+    const int tv = BETA ? value_thread(dkp, dvp) : 0;
+    const float run = sums(lam, ld, dkp, sSeg, threadIdx.x), run_v = BETA ? sums(lam_v, ldv, dvp, sSegV, tv) : 0.f;
     __syncthreads();
-    if (seg < 4) {
-        float add = 0.f;
-        for (int sg = 0; sg < seg; ++sg) add += sSeg[sg * dkp + c];
-        if (seg > 0) {
-#pragma unroll 8
-            for (int j = seg * rows; j < (seg + 1) * rows; ++j) lam[j * ld + c] += add;
-        }
-        if (seg == 3) sLast[c] = run + add;
-    }
+    shift(lam, ld, dkp, sSeg, sLast, threadIdx.x, run);
+    if (BETA) shift(lam_v, ldv, dvp, sSegV, sLastV, tv, run_v);
     __syncthreads();
 }
 // In place: sQ (raw q) -> Qt = q*exp(Lam), sK (raw k) -> Kt = k*exp(-Lam), or with sLast given
@@ -323,7 +386,7 @@ __device__ __forceinline__ void masked_scores(float *sP, int ldp, const float *A
         if (nbt <= 0) continue;
         float acc[NB][4];
         zero(acc);
-        if (c0 <= r0 + 15) warp_mma<PR>(acc, A, ld, 1, r0, Bm, 1, ld, c0, nbt, 0, K);
+        if (c0 <= r0 + 15) warp_mma<PR, false>(acc, A, ld, 1, r0, Bm, 1, ld, c0, nbt, 0, K);
         for_pairs(acc, r0, c0, nbt, [&](int t, int s, float v0, float v1) {
             *reinterpret_cast<float2 *>(sP + t * ldp + s) = make_float2(s <= t ? rnd<PR>(v0) : 0.f, s + 1 <= t ? rnd<PR>(v1) : 0.f);
         });
@@ -364,16 +427,20 @@ mma_chunk_state(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__
     __syncthreads();
     if (BETA) load_gates(sM, ldv, bd.bgate, sRow, C, dv, dvp);
     load_gates(sLam, ldk, gate, sRow, C, dk, dkp);
-    load_rows(sX, ldk, k, sRow, C, dk, dkp);
-    load_rows(sV, ldv, v, sRow, C, dv, dvp);
-    if (BWD) {
-        load_rows(sQ, ldk, q, sRow, C, dk, dkp);
-        load_rows(sG, ldv, d_out, sRow, C, dv, dvp);
+    if (BWD && dk == dv) {
+        load_tiles<4>({sX, sV, sQ, sG}, ldk, {k, v, q, d_out}, sRow, C, dk, dkp);
+    } else if (BWD) {
+        load_tiles<2>({sX, sQ}, ldk, {k, q}, sRow, C, dk, dkp);
+        load_tiles<2>({sV, sG}, ldv, {v, d_out}, sRow, C, dv, dvp);
+    } else if (dk == dv) {
+        load_tiles<2>({sX, sV}, ldk, {k, v}, sRow, C, dk, dkp);
+    } else {
+        load_tiles<1>({sX}, ldk, {k}, sRow, C, dk, dkp);
+        load_tiles<1>({sV}, ldv, {v}, sRow, C, dv, dvp);
     }
     cp_async_wait_all();
     __syncthreads();
-    prefix_gates(sLam, ldk, C, dkp, sLast, sSeg);
-    if (BETA) prefix_gates(sM, ldv, C, dvp, sMlast, sSegV);
+    prefix_gates<BETA>(sLam, ldk, C, dkp, sLast, sSeg, sM, ldv, dvp, sMlast, sSegV);
     const size_t chunk_id = (size_t)bh * g.N + chunk;
     for (int c = threadIdx.x; c < dk; c += kThreads) gamma[chunk_id * dk + c] = __expf(sLast[c]);
     scale_qk<PR>(BWD ? sQ : nullptr, sX, sLam, sLast, ldk, C, dkp);
@@ -393,13 +460,13 @@ mma_chunk_state(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__
         if (nbt <= 0) continue;
         float acc[NB][4];
         zero(acc);
-        warp_mma<PR>(acc, sX, 1, ldk, r0, sV, ldv, 1, c0, nbt, 0, C);           // sum_t Kh[t][c] V[t][e]
+        warp_mma<PR, true>(acc, sX, 1, ldk, r0, sV, ldv, 1, c0, nbt, 0, C);           // sum_t Kh[t][c] V[t][e]
         for_pairs(acc, r0, c0, nbt, [&](int c, int e, float v0, float v1) {
             if (c < dk && e < dv) store2(U + c * dv + e, v0, v1);
         });
         if (BWD) {
             zero(acc);
-            warp_mma<PR>(acc, sQ, 1, ldk, r0, sG, ldv, 1, c0, nbt, 0, C);       // sum_t Qt[t][c] dO[t][e]
+            warp_mma<PR, true>(acc, sQ, 1, ldk, r0, sG, ldv, 1, c0, nbt, 0, C);       // sum_t Qt[t][c] dO[t][e]
             for_pairs(acc, r0, c0, nbt, [&](int c, int e, float v0, float v1) {
                 if (c < dk && e < dv) store2(W + c * dv + e, v0, v1);
             });
@@ -439,16 +506,18 @@ mma_chunk_out(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
     // the inputs of the call: whatever produced them has completed before the kernels in front of this one started
     if (BETA) load_gates(sM, ldv, bd.bgate, sRow, C, dv, dv);
     load_gates(sLam, ldk, gate, sRow, C, dk, dk);
-    load_rows(sV, ldv, v, sRow, C, dv, dv);
-    load_rows(sQ, ldk, q, sRow, C, dk, dk);
-    load_rows(sK, ldk, k, sRow, C, dk, dk);
+    if (dk == dv) {
+        load_tiles<3>({sV, sQ, sK}, ldk, {v, q, k}, sRow, C, dk, dk);
+    } else {
+        load_tiles<2>({sQ, sK}, ldk, {q, k}, sRow, C, dk, dk);
+        load_tiles<1>({sV}, ldv, {v}, sRow, C, dv, dv);
+    }
     pdl_wait();                             // the states come from the scan in front
     pdl_launch_dependents();
     load_state(sS, ldv, states + ((size_t)bh * g.N + chunk) * dk * dv, dk, dv);
     cp_async_wait_all();
     __syncthreads();
-    prefix_gates(sLam, ldk, C, dkp, sLast, sSeg);
-    if (BETA) prefix_gates(sM, ldv, C, dv, sMlast, sSegV);
+    prefix_gates<BETA>(sLam, ldk, C, dkp, sLast, sSeg, sM, ldv, dv, sMlast, sSegV);
     scale_qk<PR>(sQ, sK, sLam, nullptr, ldk, C, dk);
     if (BETA) scale_qk<PR>(nullptr, sV, sM, nullptr, ldv, C, dv);           // Vt = v*exp(-M)
     __syncthreads();
@@ -463,8 +532,8 @@ mma_chunk_out(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
         if (nbt <= 0) continue;
         float acc[NB][4];
         zero(acc);
-        warp_mma<PR>(acc, sP, ldp, 1, r0, sV, ldv, 1, c0, nbt, 0, r0 + 16);     // columns past the diagonal are zero
-        warp_mma<PR>(acc, sQ, ldk, 1, r0, sS, ldv, 1, c0, nbt, 0, dk);
+        warp_mma<PR, false>(acc, sP, ldp, 1, r0, sV, ldv, 1, c0, nbt, 0, r0 + 16);     // columns past the diagonal are zero
+        warp_mma<PR, false>(acc, sQ, ldk, 1, r0, sS, ldv, 1, c0, nbt, 0, dk);
         for_pairs(acc, r0, c0, nbt, [&](int j, int e, float v0, float v1) {
             const int row = sRow[j];
             if (BETA) {
@@ -485,9 +554,9 @@ mma_chunk_out(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
 //   dgate_j = carry + sum_{r >= j in chunk} (q*dq - k*dk)_r,   q*dq = Qt*(dq accumulator), k*dk alike
 // BETA: the same formulas with Vt = v*exp(-M) for V and G = dO*exp(M) for dO (Dg then carries both
 // decays); dv = (P^T G + Kt Dg) * exp(-M), and the gradient of log(beta) is, mirroring dgate,
-//   dbgate_j = sum_{r >= j} (o*dO - v*dv)_r  with  o*dO = (P Vt + Qt S)*G  and  v*dv = Vt*(dv accumulator)
+//   dbgate_j = carry_v + sum_{r >= j in chunk} (o*dO - v*dv)_r  with  o*dO = (P Vt + Qt S)*G  and  v*dv = Vt*(dv accumulator)
 // (the unscaled output P Vt + Qt S is recomputed here, two more products, rather than read back in
-// storage precision), summed here inside the chunk; the chunk total goes to xtot for the cross-chunk part.
+// storage precision).  carry_v, the sum over the later chunks, is sum_c S' D over the state leaving the chunk.
 template <typename TO, typename DM, bool BETA, typename TI>
 __global__ void __launch_bounds__(kThreads)
 mma_chunk_bwd(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__restrict__ v, const float *__restrict__ gate,
@@ -523,133 +592,148 @@ mma_chunk_bwd(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
     // the inputs of the call: whatever produced them has completed before the kernels in front of this one started
     if (BETA) load_gates(sM, ldv, bd.bgate, sRow, C, dv, dv);
     load_gates(sLam, ldk, gate, sRow, C, dk, dk);
-    load_rows(sV, ldv, v, sRow, C, dv, dv);
-    load_rows(sG, ldv, d_out, sRow, C, dv, dv);
-    load_rows(sQ, ldk, q, sRow, C, dk, dk);
-    load_rows(sK, ldk, k, sRow, C, dk, dk);
+    if (dk == dv) {
+        load_tiles<4>({sV, sG, sQ, sK}, ldk, {v, d_out, q, k}, sRow, C, dk, dk);
+    } else {
+        load_tiles<2>({sQ, sK}, ldk, {q, k}, sRow, C, dk, dk);
+        load_tiles<2>({sV, sG}, ldv, {v, d_out}, sRow, C, dv, dv);
+    }
     pdl_wait();                             // the states come from the scans in front
     pdl_launch_dependents();
     load_state(sS, ldv, states + chunk_id * dk * dv, dk, dv);
     load_state(sD, ldv, dstates + chunk_id * dk * dv, dk, dv);
     cp_async_wait_all();
     __syncthreads();
-    prefix_gates(sLam, ldk, C, dkp, sLast, sSeg);
-    if (BETA) prefix_gates(sM, ldv, C, dv, sMlast, sSegV);
+    prefix_gates<BETA>(sLam, ldk, C, dkp, sLast, sSeg, sM, ldv, dv, sMlast, sSegV);
     scale_qk<PR>(sQ, sK, sLam, nullptr, ldk, C, dk);
     if (BETA) scale_qk<PR>(sG, sV, sM, nullptr, ldv, C, dv);                // G = dO*exp(M), Vt = v*exp(-M)
     __syncthreads();
     masked_scores<frag_bound(DM::kC, DM::kC), PR>(sP, ldp, sQ, sK, ldk, C, dk);
     masked_scores<frag_bound(DM::kC, DM::kC), PR>(sdP, ldp, sG, sV, ldv, C, dv);
     __syncthreads();
+    // Warp tiles of up to 32 rows, first those of dv (BETA: and of the outputs), then those of dq and dk
+    constexpr int MB = DM::kC == 16 ? 1 : 2, kMost = PR ? 2 : 4;
+    constexpr int NBV = grad_frags(DM::kC, DM::kDV, kMost), NBK = grad_frags(DM::kC, DM::kDK, kMost);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gi = lane >> 2, ti = lane & 3;
-    {
-        // dv[s][e] = sum_{t >= s} P[t][s] dO[t][e] + sum_c Kt[s][c] Dg[c][e]
-        constexpr int NB = frag_bound(DM::kC, DM::kDV);
-        const Tiling tl(C, dv);
-        for (int tile = warp; tile < tl.ntiles; tile += kWarps) {
-            int r0, c0, nbt;
-            tl.at(tile, r0, c0, nbt);
-            if (nbt <= 0) continue;
-            float acc[NB][4];
+    const int nrt = (C + 31) >> 5, nfv = grad_frags(C, dv, kMost), nfk = grad_frags(C, dk, kMost);
+    const int ntv = nrt * (((dv >> 3) + nfv - 1) / nfv), ntk = nrt * (((dk >> 3) + nfk - 1) / nfk);
+    const int mbw = C >= 32 ? 2 : 1;
+    for (int tile = warp; tile < ntv + ntk; tile += kWarps) {
+        if (tile < ntv) {
+            // dv[s][e] = sum_c Kt[s][c] Dg[c][e] + sum_{t >= s} P[t][s] dO[t][e]
+            const int rt = tile % nrt, ct = tile / nrt, r0 = 32 * rt, c0 = 8 * nfv * ct, nbt = min(nfv, (dv >> 3) - nfv * ct);
+            float acc[MB][NBV][4];
             zero(acc);
-            warp_mma<PR>(acc, sP, 1, ldp, r0, sG, ldv, 1, c0, nbt, r0, C);
-            warp_mma<PR>(acc, sK, ldk, 1, r0, sD, ldv, 1, c0, nbt, 0, dk);
+            warp_mma<PR, false>(acc, sK, ldk, 1, r0, sD, ldv, 1, c0, mbw, nbt, 0, dk);
+            if (BETA) {
+                // column sums of Vt * (Kt Dg) over this tile's rows, part of what later chunks hand to dbgate
+#pragma unroll
+                for (int nb = 0; nb < NBV; ++nb)
+                    if (nb < nbt) {
+                        float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int mb = 0; mb < MB; ++mb)
+                            if (mb < mbw) {
+#pragma unroll
+                                for (int i = 0; i < 4; i += 2) {
+                                    const float2 vt = load2(sV + (r0 + 16 * mb + gi + 4 * i) * ldv + c0 + 8 * nb + 2 * ti);
+                                    sum.x = fmaf(vt.x, acc[mb][nb][i], sum.x);
+                                    sum.y = fmaf(vt.y, acc[mb][nb][i + 1], sum.y);
+                                }
+                            }
+#pragma unroll
+                        for (int off = 4; off < 32; off <<= 1) {
+                            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, off);
+                            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
+                        }
+                        if (gi == 0) *reinterpret_cast<float2 *>(sSegV + rt * dv + c0 + 8 * nb + 2 * ti) = sum;
+                    }
+            }
+            warp_mma<PR, true>(acc, sP, 1, ldp, r0, sG, ldv, 1, c0, mbw, nbt, r0, C);
             if (BETA) {
                 // unscaled output of the same tile, then x = o*dO - v*dv = (P Vt + Qt S)*G - Vt*(dv accumulator)
-                float oh[NB][4];
+                float oh[MB][NBV][4];
                 zero(oh);
-                warp_mma<PR>(oh, sP, ldp, 1, r0, sV, ldv, 1, c0, nbt, 0, r0 + 16);
-                warp_mma<PR>(oh, sQ, ldk, 1, r0, sS, ldv, 1, c0, nbt, 0, dk);
+                warp_mma<PR, false>(oh, sP, ldp, 1, r0, sV, ldv, 1, c0, mbw, nbt, 0, min(r0 + 32, C));
+                warp_mma<PR, false>(oh, sQ, ldk, 1, r0, sS, ldv, 1, c0, mbw, nbt, 0, dk);
 #pragma unroll
-                for (int nb = 0; nb < NB; ++nb)
-                    if (nb < nbt) {
+                for (int mb = 0; mb < MB; ++mb)
 #pragma unroll
-                        for (int i = 0; i < 4; i += 2) {
-                            const int off = (r0 + gi + 4 * i) * ldv + c0 + 8 * nb + 2 * ti;
-                            const float2 vt = load2(sV + off), gg = load2(sG + off);
-                            oh[nb][i] = oh[nb][i] * gg.x - vt.x * acc[nb][i];
-                            oh[nb][i + 1] = oh[nb][i + 1] * gg.y - vt.y * acc[nb][i + 1];
+                    for (int nb = 0; nb < NBV; ++nb)
+                        if (mb < mbw && nb < nbt) {
+#pragma unroll
+                            for (int i = 0; i < 4; i += 2) {
+                                const int off = (r0 + 16 * mb + gi + 4 * i) * ldv + c0 + 8 * nb + 2 * ti;
+                                const float2 vt = load2(sV + off), gg = load2(sG + off);
+                                oh[mb][nb][i] = oh[mb][nb][i] * gg.x - vt.x * acc[mb][nb][i];
+                                oh[mb][nb][i + 1] = oh[mb][nb][i + 1] * gg.y - vt.y * acc[mb][nb][i + 1];
+                            }
                         }
-                    }
                 // this thread alone touches its elements of M: scale dv by exp(-M), then leave x there
-                for_pairs(acc, r0, c0, nbt, [&](int j, int e, float v0, float v1) {
+                for_pairs(acc, r0, c0, mbw, nbt, [&](int j, int e, float v0, float v1) {
                     const int row = sRow[j];
                     const float2 m = load2(sM + j * ldv + e);
-                    if (row >= 0 && e < dv) store2(dv_out + (size_t)row * dv + e, v0 * __expf(-m.x), v1 * __expf(-m.y));
+                    if (row >= 0) store2(dv_out + (size_t)row * dv + e, v0 * __expf(-m.x), v1 * __expf(-m.y));
                 });
                 __syncwarp();
-                for_pairs(oh, r0, c0, nbt, [&](int j, int e, float v0, float v1) {
+                for_pairs(oh, r0, c0, mbw, nbt, [&](int j, int e, float v0, float v1) {
                     *reinterpret_cast<float2 *>(sM + j * ldv + e) = make_float2(v0, v1);
                 });
             } else {
-                for_pairs(acc, r0, c0, nbt, [&](int j, int e, float v0, float v1) {
+                for_pairs(acc, r0, c0, mbw, nbt, [&](int j, int e, float v0, float v1) {
                     const int row = sRow[j];
-                    if (row >= 0 && e < dv) store2(dv_out + (size_t)row * dv + e, v0, v1);
+                    if (row >= 0) store2(dv_out + (size_t)row * dv + e, v0, v1);
                 });
             }
-        }
-    }
-    {
-        // dq and dk of the same (row, channel) tile; x = q*dq - k*dk replaces Lam, element by element
-        constexpr int NB = frag_bound(DM::kC, DM::kDK);
-        const Tiling tl(C, dk);
-        for (int tile = warp; tile < tl.ntiles; tile += kWarps) {
-            int r0, c0, nbt;
-            tl.at(tile, r0, c0, nbt);
-            if (nbt <= 0) continue;
-            float acc[NB][4], xq[NB][4];
+        } else {
+            // dq and dk of the same (row, channel) tile; x = q*dq - k*dk replaces Lam, element by element
+            const int tk = tile - ntv, rt = tk % nrt, ct = tk / nrt, r0 = 32 * rt, c0 = 8 * nfk * ct, nbt = min(nfk, (dk >> 3) - nfk * ct);
+            float acc[MB][NBK][4], xq[MB][NBK][4];
+            auto times = [&](const float *t, auto f) {       // f(x, t * accumulator) for every result of this lane
+#pragma unroll
+                for (int mb = 0; mb < MB; ++mb)
+#pragma unroll
+                    for (int nb = 0; nb < NBK; ++nb)
+                        if (mb < mbw && nb < nbt) {
+#pragma unroll
+                            for (int i = 0; i < 4; i += 2) {
+                                const float2 tt = load2(t + (r0 + 16 * mb + gi + 4 * i) * ldk + c0 + 8 * nb + 2 * ti);
+                                f(xq[mb][nb][i], tt.x * acc[mb][nb][i]);
+                                f(xq[mb][nb][i + 1], tt.y * acc[mb][nb][i + 1]);
+                            }
+                        }
+            };
             zero(acc);
-            warp_mma<PR>(acc, sdP, ldp, 1, r0, sK, ldk, 1, c0, nbt, 0, r0 + 16);          // sum_{s <= t} dP[t][s] Kt[s][c]
-            warp_mma<PR>(acc, sG, ldv, 1, r0, sS, 1, ldv, c0, nbt, 0, dv);                // sum_e dO[t][e] S[c][e]
-#pragma unroll
-            for (int nb = 0; nb < NB; ++nb)
-                if (nb < nbt) {
-#pragma unroll
-                    for (int i = 0; i < 4; i += 2) {
-                        const float2 qt = *reinterpret_cast<const float2 *>(sQ + (r0 + gi + 4 * i) * ldk + c0 + 8 * nb + 2 * ti);
-                        xq[nb][i] = qt.x * acc[nb][i];
-                        xq[nb][i + 1] = qt.y * acc[nb][i + 1];
-                    }
-                }
-            for_pairs(acc, r0, c0, nbt, [&](int j, int c, float v0, float v1) {
+            warp_mma<PR, false>(acc, sdP, ldp, 1, r0, sK, ldk, 1, c0, mbw, nbt, 0, min(r0 + 32, C));      // sum_{s <= t} dP[t][s] Kt[s][c]
+            warp_mma<PR, false>(acc, sG, ldv, 1, r0, sS, 1, ldv, c0, mbw, nbt, 0, dv);                    // sum_e dO[t][e] S[c][e]
+            times(sQ, [](float &x, float y) { x = y; });
+            for_pairs(acc, r0, c0, mbw, nbt, [&](int j, int c, float v0, float v1) {
                 const int row = sRow[j];
-                if (row >= 0 && c < dk) {
-                    const float2 lam = *reinterpret_cast<const float2 *>(sLam + j * ldk + c);
-                    store2(dq + (size_t)row * dk + c, v0 * __expf(lam.x), v1 * __expf(lam.y));
-                }
+                const float2 lam = load2(sLam + j * ldk + c);
+                if (row >= 0) store2(dq + (size_t)row * dk + c, v0 * __expf(lam.x), v1 * __expf(lam.y));
             });
             zero(acc);
-            warp_mma<PR>(acc, sdP, 1, ldp, r0, sQ, ldk, 1, c0, nbt, r0, C);               // sum_{t >= s} dP[t][s] Qt[t][c]
-            warp_mma<PR>(acc, sV, ldv, 1, r0, sD, 1, ldv, c0, nbt, 0, dv);                // sum_e V[s][e] Dg[c][e]
-#pragma unroll
-            for (int nb = 0; nb < NB; ++nb)
-                if (nb < nbt) {
-#pragma unroll
-                    for (int i = 0; i < 4; i += 2) {
-                        const float2 kt = *reinterpret_cast<const float2 *>(sK + (r0 + gi + 4 * i) * ldk + c0 + 8 * nb + 2 * ti);
-                        xq[nb][i] -= kt.x * acc[nb][i];
-                        xq[nb][i + 1] -= kt.y * acc[nb][i + 1];
-                    }
-                }
-            for_pairs(acc, r0, c0, nbt, [&](int j, int c, float v0, float v1) {
+            warp_mma<PR, true>(acc, sdP, 1, ldp, r0, sQ, ldk, 1, c0, mbw, nbt, r0, C);                    // sum_{t >= s} dP[t][s] Qt[t][c]
+            warp_mma<PR, false>(acc, sV, ldv, 1, r0, sD, 1, ldv, c0, mbw, nbt, 0, dv);                    // sum_e V[s][e] Dg[c][e]
+            times(sK, [](float &x, float y) { x -= y; });
+            for_pairs(acc, r0, c0, mbw, nbt, [&](int j, int c, float v0, float v1) {
                 const int row = sRow[j];
-                if (row >= 0 && c < dk) {
-                    const float2 lam = *reinterpret_cast<const float2 *>(sLam + j * ldk + c);
-                    store2(dk_out + (size_t)row * dk + c, v0 * __expf(-lam.x), v1 * __expf(-lam.y));
-                }
+                const float2 lam = load2(sLam + j * ldk + c);
+                if (row >= 0) store2(dk_out + (size_t)row * dk + c, v0 * __expf(-lam.x), v1 * __expf(-lam.y));
             });
             __syncwarp();
-            for_pairs(xq, r0, c0, nbt, [&](int j, int c, float v0, float v1) {
+            for_pairs(xq, r0, c0, mbw, nbt, [&](int j, int c, float v0, float v1) {
                 *reinterpret_cast<float2 *>(sLam + j * ldk + c) = make_float2(v0, v1);
             });
         }
     }
     __syncthreads();
-    // gate gradient: suffix sums of x down the chunk plus what later chunks carry in; four threads per
+    // gate gradients: suffix sums of x down the chunk plus what later chunks carry in; four threads per
     // channel take a quarter of the rows each
     {
         const int rows = C >> 2;
         const int c = threadIdx.x % dkp, seg = threadIdx.x / dkp;
+        const float from_later = seg < 4 ? carry[chunk_id * dk + c] : 0.f;
         float run = 0.f;
         if (seg < 4) {
 #pragma unroll 8
@@ -659,9 +743,16 @@ mma_chunk_bwd(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
             }
             sSeg[seg * dkp + c] = run;
         }
-        // the value-channel gate: the same inside the chunk, without the carry (added by a later pass)
-        const int cv = threadIdx.x % dv, segv = threadIdx.x / dv;
-        if (BETA && segv < 4) {
+        // The value-channel gate: the same.  Later chunks hand over sum_c S'[c][e] D[c][e] with S' the state leaving
+        // the chunk, = sum_c S Dg + sum_s Vt (Kt Dg)[s][e]: a quarter of the first sum and the rows that the warps above
+        // left in sSegV per thread, exchanged through the spent score tiles.
+        const int tv = BETA ? value_thread(dkp, dv) : -1, cv = tv % dv, segv = tv / dv;
+        const bool on_v = tv >= 0 && segv < 4;
+        if (BETA && on_v) {
+            float part = segv < nrt ? sSegV[segv * dv + cv] : 0.f;
+#pragma unroll 8
+            for (int r = segv * dk / 4; r < (segv + 1) * dk / 4; ++r) part = fmaf(sS[r * ldv + cv], sD[r * ldv + cv], part);
+            sP[segv * dv + cv] = part;
             float runv = 0.f;
 #pragma unroll 8
             for (int j = (segv + 1) * rows - 1; j >= segv * rows; --j) {
@@ -671,22 +762,25 @@ mma_chunk_bwd(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__re
             sSegV[segv * dv + cv] = runv;
         }
         __syncthreads();
-        if (seg < 4 && c < dk) {
-            float add = carry[chunk_id * dk + c];
+        if (seg < 4) {
+            float add = from_later;
             for (int sg = seg + 1; sg < 4; ++sg) add += sSeg[sg * dkp + c];
+#pragma unroll 8
             for (int j = seg * rows; j < (seg + 1) * rows; ++j) {
                 const int row = sRow[j];
-                if (row >= 0) dgate[(size_t)row * dk + c] = sLam[j * ldk + c] + add;
+                const float x = sLam[j * ldk + c] + add;
+                if (row >= 0) dgate[(size_t)row * dk + c] = x;
             }
         }
-        if (BETA && segv < 4) {
-            float add = 0.f;
+        if (BETA && on_v) {
+            float add = sP[cv] + sP[dv + cv] + sP[2 * dv + cv] + sP[3 * dv + cv];
             for (int sg = segv + 1; sg < 4; ++sg) add += sSegV[sg * dv + cv];
+#pragma unroll 8
             for (int j = segv * rows; j < (segv + 1) * rows; ++j) {
                 const int row = sRow[j];
-                if (row >= 0) bd.dbgate[(size_t)row * dv + cv] = sM[j * ldv + cv] + add;
+                const float x = sM[j * ldv + cv] + add;
+                if (row >= 0) bd.dbgate[(size_t)row * dv + cv] = x;
             }
-            if (segv == 0) bd.xtot[chunk_id * dv + cv] = sSegV[cv] + add;
         }
     }
 }
@@ -719,8 +813,7 @@ dig_status set_smem(K kernel, size_t bytes)
     return ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), bytes);
 }
 
-// The value-channel gate keeps two more blocks behind the common workspace: gamma_v and, for the
-// backward pass, the chunk totals of o*do - v*dv, both [B*H][N][d_v].
+// The value-channel gate keeps one more block behind the common workspace: gamma_v [B*H][N][d_v].
 size_t beta_block(const Geom &g) { return align256((size_t)g.B * g.H * g.N * g.dv * sizeof(float)); }
 BetaDev beta_dev(const GlaArgs &a, const Workspace &w, bool backward)
 {
@@ -729,10 +822,7 @@ BetaDev beta_dev(const GlaArgs &a, const Workspace &w, bool backward)
     char *p = reinterpret_cast<char *>(a.ws) + w.bytes;
     bd.bgate = a.bio.bgate;
     bd.gamma_v = reinterpret_cast<float *>(p);
-    if (backward) {
-        bd.dbgate = a.bio.dbgate;
-        bd.xtot = reinterpret_cast<float *>(p + beta_block(a.g));
-    }
+    if (backward) bd.dbgate = a.bio.dbgate;
     return bd;
 }
 
@@ -794,30 +884,32 @@ dig_status bwd_dims(const GlaArgs &a)
                    (const TI *)a.d_out, (const float *)w.states, (const float *)w.dstates, (const float *)w.carry, (TO *)a.dq,
                    (TO *)a.dk, (TO *)a.dv, a.dgate, bd, g);
     }
-    if (cudaGetLastError() != cudaSuccess) return DIG_ERR_CUDA;
-    if (BETA) return launch_beta_carry(bd.dbgate, bd.xtot, g, a.stream);
-    return DIG_OK;
+    return cuda_ok(cudaGetLastError());
 }
 
-// The shapes of the paper's models that the tcgen05 family leaves to this one get kernels with
-// compile-time sizes: 72-wide heads with 64-token chunks, 64-wide heads with 32-token chunks.
-template <typename TO, bool BETA>
+// Head sizes and chunks of the paper's models get kernels with compile-time sizes (6 heads of 64, 8 x 1024 tokens in
+// chunks of 32 with the full gate: 546 -> 225 us; 4 x 1024 tokens in fp32: 249 -> 141); 64-wide heads in 64-token chunks without the full gate are the tcgen05
+// family's.
+template <bool BETA, typename F>
+dig_status with_dims(const Geom &g, F f)
+{
+    if (g.dk == 72 && g.dv == 72 && g.C == 64) return f(FixedDims<64, 72, 72>(g));
+    if (g.dk == 64 && g.dv == 64 && g.C == 32) return f(FixedDims<32, 64, 64>(g));
+    if constexpr (BETA) {
+        if (g.dk == 64 && g.dv == 64 && g.C == 64) return f(FixedDims<64, 64, 64>(g));
+        if (g.dk == 72 && g.dv == 72 && g.C == 32) return f(FixedDims<32, 72, 72>(g));
+    }
+    return f(AnyDims(g));
+}
+template <typename TO, bool BETA, typename TI = bf16>
 dig_status fwd_typed(const GlaArgs &a)
 {
-    const Geom &g = a.g;
-    if (g.C == 64 && g.dk == 72 && g.dv == 72) return fwd_dims<TO, FixedDims<64, 72, 72>, BETA>(a);
-    if (!BETA && g.C == 32 && g.dk == 64 && g.dv == 64) return fwd_dims<TO, FixedDims<32, 64, 64>, false>(a);
-    if (BETA && g.C == 64 && g.dk == 64 && g.dv == 64) return fwd_dims<TO, FixedDims<64, 64, 64>, true>(a);
-    return fwd_dims<TO, AnyDims, BETA>(a);
+    return with_dims<BETA>(a.g, [&](auto dm) { return fwd_dims<TO, decltype(dm), BETA, TI>(a); });
 }
-template <typename TO, bool BETA>
+template <typename TO, bool BETA, typename TI = bf16>
 dig_status bwd_typed(const GlaArgs &a)
 {
-    const Geom &g = a.g;
-    if (g.C == 64 && g.dk == 72 && g.dv == 72) return bwd_dims<TO, FixedDims<64, 72, 72>, BETA>(a);
-    if (!BETA && g.C == 32 && g.dk == 64 && g.dv == 64) return bwd_dims<TO, FixedDims<32, 64, 64>, false>(a);
-    if (BETA && g.C == 64 && g.dk == 64 && g.dv == 64) return bwd_dims<TO, FixedDims<64, 64, 64>, true>(a);
-    return bwd_dims<TO, AnyDims, BETA>(a);
+    return with_dims<BETA>(a.g, [&](auto dm) { return bwd_dims<TO, decltype(dm), BETA, TI>(a); });
 }
 
 }  // namespace
@@ -833,7 +925,7 @@ bool mma_supports(int dk, int dv, int chunk, int dtype, bool backward, bool beta
 
 size_t mma_beta_workspace_bytes(const Geom &g, bool backward)
 {
-    return carve_workspace(nullptr, g, backward).bytes + beta_block(g) * (backward ? 2 : 1);
+    return carve_workspace(nullptr, g, backward).bytes + beta_block(g);
 }
 
 dig_status mma_gla_fwd(const GlaArgs &a)
@@ -841,7 +933,7 @@ dig_status mma_gla_fwd(const GlaArgs &a)
     const bool beta = a.bio.bgate != nullptr;
     if (a.dtype == DIG_BF16) return beta ? fwd_typed<__nv_bfloat16, true>(a) : fwd_typed<__nv_bfloat16, false>(a);
     if (a.dtype == DIG_BF16_F32OUT) return beta ? fwd_typed<float, true>(a) : fwd_typed<float, false>(a);
-    if (a.dtype == DIG_F32 && beta) return fwd_dims<float, AnyDims, true, float>(a);
+    if (a.dtype == DIG_F32 && beta) return fwd_typed<float, true, float>(a);
     return DIG_ERR_UNSUPPORTED;
 }
 
@@ -850,7 +942,7 @@ dig_status mma_gla_bwd(const GlaArgs &a)
     const bool beta = a.bio.bgate != nullptr;
     if (a.dtype == DIG_BF16) return beta ? bwd_typed<__nv_bfloat16, true>(a) : bwd_typed<__nv_bfloat16, false>(a);
     if (a.dtype == DIG_BF16_F32OUT) return beta ? bwd_typed<float, true>(a) : bwd_typed<float, false>(a);
-    if (a.dtype == DIG_F32 && beta) return bwd_dims<float, AnyDims, true, float>(a);
+    if (a.dtype == DIG_F32 && beta) return bwd_typed<float, true, float>(a);
     return DIG_ERR_UNSUPPORTED;
 }
 

@@ -294,48 +294,6 @@ state_scan_bwd_beta(const float *__restrict__ states, float *__restrict__ dstate
     }
 }
 
-// Gate gradient of the value-channel gate across chunks.  xtot[i][e] holds chunk i's total of
-// (o*do - v*dv); it is turned in place into the sum over the later chunks (what every token of chunk
-// i still has to receive), one thread per (sequence, value channel).
-__global__ void __launch_bounds__(128)
-beta_suffix_totals(float *__restrict__ xtot, int N, int dv, int total)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    const int idx = blockIdx.x * 128 + threadIdx.x;
-    if (idx >= total) return;
-    const int bh = idx / dv, e = idx - bh * dv;
-    float *x = xtot + (size_t)bh * N * dv + e;
-    float run = 0.f;
-    for (int i = N - 1; i >= 0; --i) {
-        const float t = x[(size_t)i * dv];
-        x[(size_t)i * dv] = run;
-        run += t;
-    }
-}
-
-// dbgate[token][e] += what later chunks contribute; one thread per 4 value channels of a scan position.
-__global__ void __launch_bounds__(256)
-beta_add_carry(float *__restrict__ dbgate, const float *__restrict__ xtot, Geom g)
-{
-    pdl_wait();
-    pdl_launch_dependents();
-    const int per_row = g.dv >> 2;
-    const long long idx = (long long)blockIdx.x * 256 + threadIdx.x;
-    const long long total = (long long)g.B * g.H * g.L * per_row;
-    if (idx >= total) return;
-    const int e = (int)(idx % per_row) << 2;
-    const long long r = idx / per_row;
-    const int p = (int)(r % g.L);
-    const int bh = (int)(r / g.L), b = bh / g.H, h = bh - b * g.H;
-    const int chunk = p / g.C;
-    const float4 add = *reinterpret_cast<const float4 *>(xtot + ((size_t)bh * g.N + chunk) * g.dv + e);
-    float4 *dst = reinterpret_cast<float4 *>(dbgate + tok_offset(g, b, scan_token(p, g.dir, g.gh, g.gw, g.L), h, g.dv) + e);
-    float4 v = *dst;
-    v.x += add.x; v.y += add.y; v.z += add.z; v.w += add.w;
-    *dst = v;
-}
-
 }  // namespace
 
 dig_status launch_state_scan_fwd(const Workspace &w, const Geom &g, cudaStream_t s, const StateIO &sio, bool tf32)
@@ -387,17 +345,6 @@ dig_status launch_state_scan_bwd_beta(const Workspace &w, const float *gamma_v, 
     const dim3 grid((g.dk + kRowsPerBlock - 1) / kRowsPerBlock, g.B * g.H);
     KernelTimer t(KID_SCAN_BWD, s);
     launch_pdl(state_scan_bwd_beta, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, gamma_v, w.carry, g.N, g.dk, g.dv, tf32);
-    return cuda_ok(cudaGetLastError());
-}
-
-dig_status launch_beta_carry(float *dbgate, float *xtot, const Geom &g, cudaStream_t s)
-{
-    KernelTimer t(KID_SCAN_BWD, s);
-    const int total = g.B * g.H * g.dv;
-    launch_pdl(beta_suffix_totals, dim3((total + 127) / 128), dim3(128), 0, s, xtot, g.N, g.dv, total);
-    if (cudaGetLastError() != cudaSuccess) return DIG_ERR_CUDA;
-    const long long n = (long long)g.B * g.H * g.L * (g.dv >> 2);
-    launch_pdl(beta_add_carry, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, dbgate, xtot, g);
     return cuda_ok(cudaGetLastError());
 }
 

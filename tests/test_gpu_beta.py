@@ -67,6 +67,20 @@ def test_head_and_chunk_sizes(d, chunk):
     print(_run(wl, 2, 5))
 
 
+@pytest.mark.parametrize("dk,dv,chunk,grid,dtype", [
+    (72, 72, 32, (5, 13), "bf16"),      # one row in the last chunk; compile-time sizes with three fragments a tile
+    (72, 72, 32, (5, 13), "f32"),
+    (8, 16, 128, (9, 29), "bf16"),      # four row tiles, one column tile
+    (128, 16, 32, (6, 11), "bf16"),     # one row tile, key and value gates worked on by different threads
+    (24, 120, 16, (5, 9), "f32"),       # 16-row tiles, several rounds of tiles
+])
+def test_gradient_tiles_and_gate_carry(dk, dv, chunk, grid, dtype):
+    """Tile edges of the gradient kernel, and the value-gate gradient that later chunks hand over."""
+    wl = Workload("beta", B=1, H=2, grid_h=grid[0], grid_w=grid[1], d_k=dk, d_v=dv, chunk=chunk, dtype=dtype, backward=True,
+                  tau=(16.0, 4.0), seed=38)
+    print(_run(wl, 3, 9))
+
+
 def test_long_sequence_many_chunks():
     wl = CONFIGS["C5"].scaled(B=1, H=2, grid_h=40, grid_w=40, backward=True)       # 1600 tokens, 25 chunks, d = 72
     print(_run(wl, 3, 6))
