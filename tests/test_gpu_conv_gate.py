@@ -82,6 +82,18 @@ def test_gate_transform(dtype):
     np.testing.assert_allclose(got, ref, rtol=3e-6, atol=1e-30)
 
 
+@pytest.mark.parametrize("H,dk,L,dtype", [(7, 72, 2407, "bf16"), (7, 72, 4813, "f32"), (256, 8, 1200, "bf16")])
+def test_gate_heads_over_several_passes(H, dk, L, dtype):
+    """More vectors than threads, in one, two and more passes with a ragged end: every head keeps its temperature."""
+    from paper_2405_18428_b200 import dig
+    rng = np.random.default_rng(2)
+    g = round_to_bf16(rng.standard_normal((1, L, H, dk)).astype(np.float32) * 4)
+    tau = np.linspace(0.5, 16, H).astype(np.float32)
+    t = torch.from_numpy(g).cuda()
+    got = dig.dig_gate_logsigmoid(t.to(torch.bfloat16) if dtype == "bf16" else t, tau).cpu().numpy()
+    np.testing.assert_allclose(got, oracle.gate(g, tau), rtol=3e-6, atol=1e-30)
+
+
 # ---- reverse mode of the SREM convolution ----------------------------------------------------------
 def _conv_bwd_case(B, gh, gw, D, dtype, direction, with_bias, seed=0):
     from paper_2405_18428_b200 import dig
