@@ -379,19 +379,23 @@ die:
 // segment's own contribution) becomes the gradient with respect to the state leaving segment s, seg_carry
 // the gate-gradient carried into the segment from later ones, seg_state16 an fp16 copy of the entry states
 // in the dense chunk-major order the backward sweep bulk-copies.
-// Bound by the latency of its loads, which do not depend on the recurrence: NB segments are in flight
-// together.  49 segments x 6 sequences, d = 64: 8.0 us with 8 lanes per row and fewer loads in flight, 6.1 us now;
-// backward flavour, 18 x 16, d = 72: 14.6 -> 10.1 us.  A whole warp per row: 12.9 us (five shuffles per row, half of
-// the lanes idle in the second piece).
+// Bound by the latency of its loads, which do not depend on the recurrence: NF (NB on the way back) segments are in
+// flight together.  Few segments get a kernel of their own with short loops, since fetching the instructions of the long
+// ones takes longer than they do (6 segments x 48 sequences, d = 64: 5.2 us in the long kernel, 3.6 in the short
+// one; backward flavour 9.1 and 5.6).  49 segments x 6 sequences, d = 64: 8.0 us with 8 lanes per row and fewer loads in
+// flight, 6.1 with 16 lanes, 5.5 us now; backward flavour, 18 x 16, d = 72: 14.6 -> 10.1 -> 7.9 us.  A whole warp
+// per row: 12.9 us (five shuffles per row, half of the lanes idle in the second piece).
 // =================================================================================================
 constexpr int kScanRows = 8;                          // state rows per block
-template <int D, bool BWD>
+constexpr int kScanFew = 8;                           // segments up to which the short kernel serves
+template <int D, bool BWD, bool MANY>
 __global__ void __launch_bounds__(16 * kScanRows)
 seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg_carry, __half *seg_state16,
          const float *s_in, float *s_out, const float *ds_out, float *ds_in, int nseg)
 {
     constexpr int NV = (D / 4 + 15) / 16;             // float4 pieces per lane
-    constexpr int NB = NV == 1 ? (BWD ? 8 : 16) : (BWD ? 6 : 12);         // segments whose loads are in flight together
+    // segments whose loads are in flight together, on the way forward and on the way back
+    constexpr int NF = MANY ? (NV == 1 ? 32 : 18) : (NV == 1 ? 8 : 6), NB = MANY ? (NV == 1 ? 16 : 9) : NF;
     const int bh = blockIdx.x, c = blockIdx.y * kScanRows + (threadIdx.x >> 4), lane = threadIdx.x & 15;
     static_assert(D % kScanRows == 0, "whole blocks of rows");
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -406,11 +410,11 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
     float4 s[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) s[i] = s_in ? ld(s_in + io, i) : zero;
-    for (int sg0 = 0; sg0 < nseg; sg0 += NB) {
-        float4 t[NB][NV];
-        float gam[NB];
+    for (int sg0 = 0; sg0 < nseg; sg0 += NF) {
+        float4 t[NF][NV];
+        float gam[NF];
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
+        for (int j = 0; j < NF; ++j) {
             const int sg = sg0 + j;
             if (sg < nseg) {
                 gam[j] = gam0[(size_t)sg * D];
@@ -419,7 +423,7 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
             }
         }
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
+        for (int j = 0; j < NF; ++j) {
             const int sg = sg0 + j;
             if (sg < nseg) {
                 const float gm = exp2f(gam[j]);
@@ -1109,7 +1113,7 @@ dig_status run(const GlaArgs &ga)
         if ((st = cuda_ok(cudaGetLastError())) != DIG_OK) return st;
     }
     if (scan) {
-        auto kern = seg_scan<D, BWD>;
+        auto kern = pl.nseg > kScanFew ? seg_scan<D, BWD, true> : seg_scan<D, BWD, false>;
         KernelTimer t(KID_SW_SCAN, ga.stream);
         launch_pdl(kern, dim3(g.B * g.H, D / kScanRows), dim3(16 * kScanRows), 0, ga.stream, w.seg_state, (const float *)w.seg_gamma, w.seg_dstate,
                    w.seg_carry, w.seg_state16, ga.sio.s_in, ga.sio.s_out, ga.sio.ds_out, ga.sio.ds_in, pl.nseg);

@@ -19,3 +19,11 @@ def test_segments_of_several_tiles(d, grid, B, H, chunk, tau, direction):
     wl = Workload("seg", B=B, H=H, grid_h=grid[0], grid_w=grid[1], d_k=d, d_v=d, chunk=chunk, dtype="bf16", backward=True,
                   tau=tau, seed=61)
     print(check_workload(wl, direction))
+
+
+@pytest.mark.parametrize("d,tiles,last", [(64, 8, 64), (64, 9, 1), (64, 33, 60), (72, 9, 64), (72, 19, 33), (72, 37, 64)])
+def test_scans_over_few_and_many_segments(d, tiles, last):
+    """One tile per segment: the scan over segment ends at the edges of its two kernels and of their passes."""
+    wl = Workload("scan", B=1, H=2, grid_h=1, grid_w=64 * (tiles - 1) + last, d_k=d, d_v=d, chunk=64, dtype="bf16", backward=True,
+                  tau=(16.0, 4.0), seed=62)
+    print(check_workload(wl, 1))
