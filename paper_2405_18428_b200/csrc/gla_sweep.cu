@@ -100,7 +100,7 @@ __device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, int *st
 // it lie the group sums of this tile and the operand rows of the one before, whose product is issued there;
 // operand tiles and sums have two buffers, and the rows of the next tile are loaded a whole tile ahead.
 // Bound by the latency of its phases (IPC 1.4); 48 sequences of 4096 tokens, d = 64: 40.3 us with the state in
-// registers, decayed once per tile in scan order, 30.2 us now; 16 of 16384, d = 72: 79 -> 48.5 us.
+// registers, decayed once per tile in scan order, 27 us now; 16 of 16384, d = 72: 79 -> 43 us.
 // =================================================================================================
 template <int D>
 struct LocalFwdSmem {
@@ -226,7 +226,7 @@ die:
 // tensor memory and are read once per segment.  A backward pass over uncut sequences needs only the states.
 // Pipelined over the (sub-)chunks: the products of one run while the next one's operand tiles are built (two
 // buffers of tiles and accumulators), and are folded into the state one step later.  48 sequences of 4096
-// tokens, d = 64: 66.6 us before (both sums in registers, no pipelining), 52.3 us now; 16 of 16384, d = 72: 122 -> 116 us.
+// tokens, d = 64: 66.6 us before (both sums in registers, no pipelining), 47 us now; 16 of 16384, d = 72: 122 -> 95 us.
 // =================================================================================================
 template <int D, bool GRAD>
 struct LocalBwdSmem {
@@ -500,8 +500,8 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
 // =================================================================================================
 // sweep_fwd: a segment from its entry state; writes out.
 // Bound by the latency of its phases (three barriers and two waits for products per tile; IPC 1.5, two CTAs per
-// SM).  16 sequences of 16384 tokens, d = 72: 114 us with the row-chunk work split, 84 us now; 768 of 256, d = 64
-// (uncut): 60 -> 52 us.  Three CTAs per SM on 80 registers: 72 us against 59 us on 48 sequences of 4096 tokens, d = 64.
+// SM).  16 sequences of 16384 tokens, d = 72: 114 us with the row-chunk work split, 76 us now; 768 of 256, d = 64
+// (uncut): 60 -> 48 us; 48 of 4096: 62 -> 51.  Three CTAs per SM on 80 registers: 72 us against 59 us on 48 sequences of 4096 tokens, d = 64.
 // =================================================================================================
 template <int D, typename TO>
 struct FwdSmem {
@@ -680,7 +680,7 @@ die:
 // operand tiles that are spent by then) to the column threads, which still hold the decay exponents of
 // their rows: they scale and store dq and dk, form q dq - k dk and sum it down their rows.
 // Bound by latency like the forward sweep.  48 sequences of 4096 tokens, d = 64: 140 us with the row-chunk work
-// split, 106 us now; 16 of 16384, d = 72: 252 -> 186 us (217 us before the L2 was asked for the next tile's rows early).
+// split, 94 us now; 16 of 16384, d = 72: 252 -> 181 us.
 // =================================================================================================
 template <int D, typename TO>
 struct BwdSmem {
