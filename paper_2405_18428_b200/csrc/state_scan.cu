@@ -10,6 +10,8 @@
 // Optional state arguments ([B*H][d_k][d_v] row-major fp32, null = zero / not wanted): the forward scan
 // starts from s_in and hands out the state after the last chunk; the backward scan starts from the
 // gradient with respect to that final state and hands out the gradient with respect to s_in.
+#include <type_traits>
+
 #include "dig_common.cuh"
 
 namespace dig {
@@ -17,6 +19,8 @@ namespace {
 
 constexpr int kScanThreads = 128;
 constexpr int kAhead = 16;
+constexpr int kAheadBeta = 4;      // with the value-channel gate, whose factors take as many registers as the states: at 16
+                                   // a third of the CTAs waits for a slot (16 chunks x 48 sequences, d = 64: 11.7 -> 7.9 us; 2: 9.2)
 
 __device__ __forceinline__ float round_tf32(float x)
 {
@@ -75,11 +79,12 @@ state_scan_fwd(float *__restrict__ states, const float *__restrict__ gamma, cons
     }
 }
 
-// The same scan with one element per thread and 16 chunks of loads in flight: four times the threads
+// The same scan with one element per thread and AHEAD chunks of loads in flight: four times the threads
 // of the kernel above, for calls with so few (batch, head) sequences that float4 threads would leave
-// most SMs idle and too few loads in flight (long sequences of a small batch).
-constexpr int kScan1Threads = 256, kAhead1 = 16;
-template <bool TF32>
+// most SMs idle and too few loads in flight (long sequences of a small batch).  Up to 16 chunks AHEAD is 8: fetching
+// the longer code takes longer than a second wait (16 chunks x 12 sequences, d = 64: 4.6 -> 3.6 us).
+constexpr int kScan1Threads = 256;
+template <bool TF32, int AHEAD>
 __global__ void __launch_bounds__(kScan1Threads)
 state_scan_fwd1(float *__restrict__ states, const float *__restrict__ gamma, const float *__restrict__ s_in,
                 float *__restrict__ s_final, int N, int dk, int dv)
@@ -94,12 +99,12 @@ state_scan_fwd1(float *__restrict__ states, const float *__restrict__ gamma, con
     const size_t sstride = (size_t)dk * dv;
     const size_t io = (size_t)blockIdx.y * dk * dv + (size_t)row * dv + col;
     float run = s_in != nullptr ? s_in[io] : 0.f;
-    for (int i = 0; i < N; i += kAhead1) {
-        float u[kAhead1], g[kAhead1];
+    for (int i = 0; i < N; i += AHEAD) {
+        float u[AHEAD], g[AHEAD];
         const float *pu = st;
         const float *pg = gm;
 #pragma unroll
-        for (int j = 0; j < kAhead1; ++j) {
+        for (int j = 0; j < AHEAD; ++j) {
             if (i + j < N) {
                 u[j] = *pu;
                 g[j] = *pg;
@@ -108,25 +113,24 @@ state_scan_fwd1(float *__restrict__ states, const float *__restrict__ gamma, con
             pg += dk;
         }
 #pragma unroll
-        for (int j = 0; j < kAhead1; ++j) {
+        for (int j = 0; j < AHEAD; ++j) {
             if (i + j < N) {
                 *st = TF32 ? round_tf32(run) : run;
                 run = fmaf(g[j], run, u[j]);
             }
             st += sstride;
         }
-        gm += (size_t)kAhead1 * dk;
+        gm += (size_t)AHEAD * dk;
     }
     if (s_final != nullptr) s_final[io] = run;
 }
 
-// One warp per key channel c; lanes stride over the value channels.
+// One warp per key channel c; lanes stride over the value channels, PL per lane (32 PL >= d_v).
 // TF32: dstates receives diag(gamma_i) D_[i] rounded to tf32, the form the warp-MMA gradient kernel
 // multiplies with, instead of D_[i].
 constexpr int kRowsPerBlock = 4;
-constexpr int kMaxPerLane = 4;     // d_v <= 128
 
-template <bool TF32>
+template <bool TF32, int PL>
 __global__ void __launch_bounds__(32 * kRowsPerBlock)
 state_scan_bwd(const float *__restrict__ states, float *__restrict__ dstates,
                const float *__restrict__ gamma, float *__restrict__ carry, const float *__restrict__ s_final,
@@ -143,10 +147,10 @@ state_scan_bwd(const float *__restrict__ states, float *__restrict__ dstates,
     float *D = dstates + base;
     const float *gm = gamma + (size_t)blockIdx.y * N * dk + c;
     float *cr = carry + (size_t)blockIdx.y * N * dk + c;
-    float run[kMaxPerLane];
+    float run[PL];
     const size_t io = ((size_t)blockIdx.y * dk + c) * dv;
 #pragma unroll
-    for (int r = 0; r < kMaxPerLane; ++r) {
+    for (int r = 0; r < PL; ++r) {
         const int e = lane + 32 * r;
         run[r] = (ds_out != nullptr && e < dv) ? ds_out[io + e] : 0.f;
     }
@@ -154,14 +158,14 @@ state_scan_bwd(const float *__restrict__ states, float *__restrict__ dstates,
     // once per kLook chunks and not once per chunk
     constexpr int kLook = 8;
     for (int i = N - 1; i >= 0; i -= kLook) {
-        float w[kLook][kMaxPerLane], sn[kLook][kMaxPerLane], g[kLook];
+        float w[kLook][PL], sn[kLook][PL], g[kLook];
 #pragma unroll
         for (int j = 0; j < kLook; ++j) {
             const int ch = i - j;
             g[j] = 0.f;
             if (ch >= 0) g[j] = gm[(size_t)ch * dk];
 #pragma unroll
-            for (int r = 0; r < kMaxPerLane; ++r) {
+            for (int r = 0; r < PL; ++r) {
                 const int e = lane + 32 * r;
                 w[j][r] = (ch >= 0 && e < dv) ? D[(size_t)ch * sstride + e] : 0.f;
                 sn[j][r] = 0.f;          // the state leaving chunk ch: the next chunk's entry, or the final state
@@ -177,7 +181,7 @@ state_scan_bwd(const float *__restrict__ states, float *__restrict__ dstates,
             if (ch < 0) break;          // uniform over the warp
             float dot = 0.f;
 #pragma unroll
-            for (int r = 0; r < kMaxPerLane; ++r) {
+            for (int r = 0; r < PL; ++r) {
                 const int e = lane + 32 * r;
                 if (e < dv) D[(size_t)ch * sstride + e] = TF32 ? round_tf32(g[j] * run[r]) : run[r];
                 dot = fmaf(sn[j][r], run[r], dot);
@@ -190,7 +194,7 @@ state_scan_bwd(const float *__restrict__ states, float *__restrict__ dstates,
     }
     if (ds_in != nullptr) {
 #pragma unroll
-        for (int r = 0; r < kMaxPerLane; ++r) {
+        for (int r = 0; r < PL; ++r) {
             const int e = lane + 32 * r;
             if (e < dv) ds_in[io + e] = run[r];
         }
@@ -215,10 +219,10 @@ state_scan_fwd_beta(float *__restrict__ states, const float *__restrict__ gamma,
     const float *gv = gamma_v + (size_t)blockIdx.y * N * dv + col;
     const size_t sstride = (size_t)dk * dv / 4;
     float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = 0; i < N; i += kAhead) {
-        float4 u[kAhead], g[kAhead];
+    for (int i = 0; i < N; i += kAheadBeta) {
+        float4 u[kAheadBeta], g[kAheadBeta];
 #pragma unroll
-        for (int j = 0; j < kAhead; ++j) {
+        for (int j = 0; j < kAheadBeta; ++j) {
             if (i + j < N) {
                 u[j] = st[(size_t)(i + j) * sstride];
                 const float gr = gm[(size_t)(i + j) * dk];
@@ -227,7 +231,7 @@ state_scan_fwd_beta(float *__restrict__ states, const float *__restrict__ gamma,
             }
         }
 #pragma unroll
-        for (int j = 0; j < kAhead; ++j) {
+        for (int j = 0; j < kAheadBeta; ++j) {
             if (i + j < N) {
                 st[(size_t)(i + j) * sstride] = tf32 ? round4_tf32(run) : run;
                 run.x = fmaf(g[j].x, run.x, u[j].x);
@@ -240,6 +244,7 @@ state_scan_fwd_beta(float *__restrict__ states, const float *__restrict__ gamma,
     if (s_final != nullptr) *reinterpret_cast<float4 *>(s_final + (size_t)blockIdx.y * dk * dv + (size_t)e4 * 4) = run;
 }
 
+template <int PL>
 __global__ void __launch_bounds__(32 * kRowsPerBlock)
 state_scan_bwd_beta(const float *__restrict__ states, float *__restrict__ dstates, const float *__restrict__ gamma,
                     const float *__restrict__ gamma_v, float *__restrict__ carry, int N, int dk, int dv, bool tf32)
@@ -256,18 +261,18 @@ state_scan_bwd_beta(const float *__restrict__ states, float *__restrict__ dstate
     const float *gm = gamma + (size_t)blockIdx.y * N * dk + c;
     const float *gv = gamma_v + (size_t)blockIdx.y * N * dv;
     float *cr = carry + (size_t)blockIdx.y * N * dk + c;
-    float run[kMaxPerLane];
+    float run[PL];
 #pragma unroll
-    for (int r = 0; r < kMaxPerLane; ++r) run[r] = 0.f;
+    for (int r = 0; r < PL; ++r) run[r] = 0.f;
     constexpr int kLook = 4;
     for (int i = N - 1; i >= 0; i -= kLook) {
-        float w[kLook][kMaxPerLane], sn[kLook][kMaxPerLane], g[kLook][kMaxPerLane];
+        float w[kLook][PL], sn[kLook][PL], g[kLook][PL];
 #pragma unroll
         for (int j = 0; j < kLook; ++j) {
             const int ch = i - j;
             const float gr = ch >= 0 ? gm[(size_t)ch * dk] : 0.f;
 #pragma unroll
-            for (int r = 0; r < kMaxPerLane; ++r) {
+            for (int r = 0; r < PL; ++r) {
                 const int e = lane + 32 * r;
                 const bool on = ch >= 0 && e < dv;
                 w[j][r] = on ? D[(size_t)ch * sstride + e] : 0.f;
@@ -281,7 +286,7 @@ state_scan_bwd_beta(const float *__restrict__ states, float *__restrict__ dstate
             if (ch < 0) break;          // uniform over the warp
             float dot = 0.f;
 #pragma unroll
-            for (int r = 0; r < kMaxPerLane; ++r) {
+            for (int r = 0; r < PL; ++r) {
                 const int e = lane + 32 * r;
                 if (e < dv) D[(size_t)ch * sstride + e] = tf32 ? round_tf32(g[j][r] * run[r]) : g[j][r] * run[r];
                 dot = fmaf(sn[j][r], run[r], dot);
@@ -292,6 +297,16 @@ state_scan_bwd_beta(const float *__restrict__ states, float *__restrict__ dstate
             if (lane == 0) cr[(size_t)ch * dk] = dot;
         }
     }
+}
+
+// Calls f(PL) with the value channels per lane that d_v needs (at most 128 of them): a bound of four for everything
+// doubled the code of the frequent 64 (16 chunks x 12 sequences 6.2 -> 5.4 us; with the value gate, x 48, 17 -> 13).
+template <typename F>
+void with_per_lane(int dv, F f)
+{
+    if (dv <= 64) f(std::integral_constant<int, 2>{});
+    else if (dv <= 96) f(std::integral_constant<int, 3>{});
+    else f(std::integral_constant<int, 4>{});
 }
 
 }  // namespace
@@ -305,10 +320,9 @@ dig_status launch_state_scan_fwd(const Workspace &w, const Geom &g, cudaStream_t
     KernelTimer t(KID_SCAN_FWD, s);
     if ((long long)grid.x * grid.y * kScanThreads < 16384) {       // few sequences: one element per thread
         const dim3 grid1((g.dk * g.dv + kScan1Threads - 1) / kScan1Threads, g.B * g.H);
-        if (tf32)
-            launch_pdl(state_scan_fwd1<true>, grid1, dim3(kScan1Threads), 0, s, w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
-        else
-            launch_pdl(state_scan_fwd1<false>, grid1, dim3(kScan1Threads), 0, s, w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
+        auto kern = g.N <= 16 ? (tf32 ? state_scan_fwd1<true, 8> : state_scan_fwd1<false, 8>)
+                              : (tf32 ? state_scan_fwd1<true, 16> : state_scan_fwd1<false, 16>);
+        launch_pdl(kern, grid1, dim3(kScan1Threads), 0, s, w.states, w.gamma, sio.s_in, fin, g.N, g.dk, g.dv);
         return cuda_ok(cudaGetLastError());
     }
     if (tf32)
@@ -323,12 +337,11 @@ dig_status launch_state_scan_bwd(const Workspace &w, const Geom &g, cudaStream_t
 {
     const dim3 grid((g.dk + kRowsPerBlock - 1) / kRowsPerBlock, g.B * g.H);
     KernelTimer t(KID_SCAN_BWD, s);
-    if (tf32)
-        launch_pdl(state_scan_bwd<true>, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, w.carry, w.sfinal, sio.ds_out,
-                                                                 sio.ds_in, g.N, g.dk, g.dv);
-    else
-        launch_pdl(state_scan_bwd<false>, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, w.carry, w.sfinal, sio.ds_out,
-                                                                  sio.ds_in, g.N, g.dk, g.dv);
+    with_per_lane(g.dv, [&](auto pl) {
+        constexpr int PL = decltype(pl)::value;
+        launch_pdl(tf32 ? state_scan_bwd<true, PL> : state_scan_bwd<false, PL>, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates,
+                   w.gamma, w.carry, w.sfinal, sio.ds_out, sio.ds_in, g.N, g.dk, g.dv);
+    });
     return cuda_ok(cudaGetLastError());
 }
 
@@ -344,7 +357,10 @@ dig_status launch_state_scan_bwd_beta(const Workspace &w, const float *gamma_v, 
 {
     const dim3 grid((g.dk + kRowsPerBlock - 1) / kRowsPerBlock, g.B * g.H);
     KernelTimer t(KID_SCAN_BWD, s);
-    launch_pdl(state_scan_bwd_beta, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, gamma_v, w.carry, g.N, g.dk, g.dv, tf32);
+    with_per_lane(g.dv, [&](auto pl) {
+        launch_pdl(state_scan_bwd_beta<decltype(pl)::value>, grid, dim3(32 * kRowsPerBlock), 0, s, w.states, w.dstates, w.gamma, gamma_v, w.carry,
+                   g.N, g.dk, g.dv, tf32);
+    });
     return cuda_ok(cudaGetLastError());
 }
 

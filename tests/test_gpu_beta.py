@@ -81,6 +81,16 @@ def test_gradient_tiles_and_gate_carry(dk, dv, chunk, grid, dtype):
     print(_run(wl, 3, 9))
 
 
+@pytest.mark.parametrize("dv,tokens", [(64, 16 * 16), (72, 16 * 17), (96, 16 * 5 - 3), (104, 16 * 4 + 1), (128, 16 * 16 + 1)])
+def test_state_scans_over_chunk_counts_and_value_widths(dv, tokens):
+    """The scans over chunk states at the edges of their passes and of the value channels a lane holds, with the value gate
+    and without it (fp32 storage, few sequences)."""
+    from parity import check_workload
+    wl = Workload("scan", B=1, H=2, grid_h=1, grid_w=tokens, d_k=16, d_v=dv, chunk=16, dtype="f32", backward=True, tau=(16.0, 4.0), seed=39)
+    print(_run(wl, 0, 11))
+    check_workload(wl, 1)
+
+
 def test_long_sequence_many_chunks():
     wl = CONFIGS["C5"].scaled(B=1, H=2, grid_h=40, grid_w=40, backward=True)       # 1600 tokens, 25 chunks, d = 72
     print(_run(wl, 3, 6))
