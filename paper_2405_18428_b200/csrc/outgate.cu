@@ -147,7 +147,9 @@ __device__ __forceinline__ float normalise(const Raw8<T> (&o)[CPL], const Lane<L
             if (!FULL && !ln.has_col(i)) x = make_float2(0.f, 0.f);
             v = fma2(x, x, v);
         }
-    const float rstd = rsqrtf(group_sum(v.x + v.y, ln.m) * inv_d + eps);
+    // slots past the last row hold zeros: with eps = 0 their 1/0 must not become 0 * inf in the affine gradients
+    const float var = group_sum(v.x + v.y, ln.m) * inv_d;
+    const float rstd = ln.row_ok ? rsqrtf(var + eps) : 0.f;
     const float2 sc = make_float2(rstd, rstd);
 #pragma unroll
     for (int i = 0; i < 4 * CPL; ++i) n[i] = mul2(n[i], sc);

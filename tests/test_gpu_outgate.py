@@ -68,6 +68,12 @@ def test_outgate_single_row_and_extremes():
     assert torch.isfinite(z).all() and float(z[:3].abs().max()) < 1e-6      # Swish(-100), Swish(-20), Swish(0)
 
 
+@pytest.mark.parametrize("dtype,d,rows", [("bf16", 64, 33), ("bf16", 72, 41), ("bf16", 128, 33), ("f32", 72, 13), ("f32", 24, 17)])
+def test_outgate_without_eps_on_a_partly_filled_tile(dtype, d, rows):
+    """eps = 0: row slots past the end of the last tile, whose variance is 0, must not reach the affine gradients."""
+    _case((rows, d), dtype, True, 5, eps=0.0)
+
+
 @pytest.mark.parametrize("cfg", ["C2", "C5"])
 def test_outgate_benchmark_shapes(cfg):
     wl = CONFIGS[cfg]
