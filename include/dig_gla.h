@@ -89,7 +89,9 @@ dig_status dig_gate_logsigmoid(const void *g, const float *tau_per_head, float *
  * to more than 15.9 in magnitude (any channel) the tile is worked in sub-chunks of 32, 16 or 8 tokens, so
  * results stay exact for any decay up to 15.9 per 8 consecutive scan positions (log alpha about -2 per
  * token).  Beyond that the call still completes with finite values, which are not the result, and
- * dig_last_device_status reports DIG_ERR_RANGE.  The other families form exp(+-sum) in fp32 / tf32: there
+ * dig_last_device_status reports DIG_ERR_RANGE.  Operands keep their 11 bits while |q| and |k| times
+ * exp(+-half of the (sub-)chunk's sum) stay in fp16's normal range, 6e-5 to 65504; smaller ones lose
+ * bits, larger ones saturate.  The other families form exp(+-sum) in fp32 / tf32: there
  * the magnitude of the gate summed over one chunk must stay below 80; beyond it results may overflow.
  * Sigmoid gates with temperature >= 1 are inside both ranges with a wide margin. */
 dig_status dig_gla_fwd(const void *q, const void *k, const void *v, const float *gate, void *out,

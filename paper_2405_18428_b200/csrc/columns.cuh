@@ -234,45 +234,8 @@ template <int D> __device__ __forceinline__ int item_offset(const Who<D> &w, int
     return j < 8 ? pair_offset<D>(8 * w.grp, w.c2) + 16 * j : pair_offset<D>(8 * w.grp + w.xrow, w.xc2);
 }
 
-// Operand tiles from the thread's rows; x = r.g[j] + off is the exponent (log2) of item j:
+// Operand tiles from the thread's rows, r.g[j] = x the exponent (log2) of item j:
 //   tK <- k 2^-x, tV <- v;  tQ <- q 2^x, tG <- dO.  `on` = false (uniform over the warp) writes zeros.
-template <int D, bool HQ, bool HD>
-__device__ __forceinline__ void build_kv_rows(const Cols<D, HQ, HD> &r, const Who<D> &w, float2 off, float2 xoff, char *tK, char *tV, bool on)
-{
-    if (on) {
-#pragma unroll
-        for (int j = 0; j < r.N; ++j) {
-            const int o = item_offset(w, j);
-            st_pair(tK, o, mul2(bf2(r.k[j]), ex2_neg2(add2(r.g[j], j < 8 ? off : xoff))));
-            st_pair(tV, o, bf2(r.v[j]));
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < r.N; ++j) {
-            st_zero(tK, item_offset(w, j));
-            st_zero(tV, item_offset(w, j));
-        }
-    }
-}
-template <int D, bool HQ, bool HD>
-__device__ __forceinline__ void build_qd_rows(const Cols<D, HQ, HD> &r, const Who<D> &w, float2 off, float2 xoff, char *tQ, char *tG, bool on)
-{
-    if (on) {
-#pragma unroll
-        for (int j = 0; j < r.N; ++j) {
-            const int o = item_offset(w, j);
-            st_pair(tQ, o, mul2(bf2(r.q[j]), ex2_2(add2(r.g[j], j < 8 ? off : xoff))));
-            if (HD) st_pair(tG, o, bf2(r.d[j]));
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < r.N; ++j) {
-            st_zero(tQ, item_offset(w, j));
-            if (HD) st_zero(tG, item_offset(w, j));
-        }
-    }
-}
-// All operand tiles; r.g[j] is the exponent itself.
 template <int D, bool HQ, bool HD>
 __device__ __forceinline__ void build_rows(const Cols<D, HQ, HD> &r, const Who<D> &w, char *tQ, char *tK, char *tV, char *tG, bool on)
 {
@@ -294,17 +257,6 @@ __device__ __forceinline__ void build_rows(const Cols<D, HQ, HD> &r, const Who<D
             if (HQ) st_zero(tQ, o);
             if (HD) st_zero(tG, o);
         }
-    }
-}
-// tK <- k 2^(off - r.g[j]): decay from the row to the point whose gate sum is off
-template <int D, bool HQ, bool HD>
-__device__ __forceinline__ void build_suffix_rows(const Cols<D, HQ, HD> &r, const Who<D> &w, float2 off, float2 xoff, char *tK, char *tV)
-{
-#pragma unroll
-    for (int j = 0; j < r.N; ++j) {
-        const int o = item_offset(w, j);
-        st_pair(tK, o, mul2(bf2(r.k[j]), ex2_2(sub2(j < 8 ? off : xoff, r.g[j]))));
-        st_pair(tV, o, bf2(r.v[j]));
     }
 }
 // Row sums of the gates -> exponents (log2) of the items' decay factors.
@@ -426,28 +378,50 @@ struct StateOf {
     __device__ __forceinline__ int chunk(int i) const { return (hf ? L::NV0 : 0) + idx(i); }
     __device__ __forceinline__ uint32_t tcol(int i) const { return corner(i) ? (uint32_t)L::HW : 8u * (uint32_t)idx(i); }
 };
-// Decay of one (sub-)chunk for the thread's state row: ec = 2^(t/2), e2c = 2^t with t the sum of the row
-// groups [w0, w1) of the key channel; x* the same for key channel 64 + lane % 8 of the corner.
+// Values per channel (the thread's own pairs, which every warp holds for all channels) -> the value of the thread's
+// state row, and of key channel 64 + lane % 8 of the corner.
+template <int D>
+__device__ __forceinline__ float of_row(const StateOf<D> &st, float2 x)
+{
+    const float a = __shfl_sync(0xffffffffu, x.x, st.row >> 1), b = __shfl_sync(0xffffffffu, x.y, st.row >> 1);
+    return (st.row & 1) ? b : a;
+}
+__device__ __forceinline__ float of_corner(float2 xx)
+{
+    const float a = __shfl_sync(0xffffffffu, xx.x, (threadIdx.x & 7) >> 1), b = __shfl_sync(0xffffffffu, xx.y, (threadIdx.x & 7) >> 1);
+    return (threadIdx.x & 1) ? b : a;
+}
+// Decay of one (sub-)chunk whose gates sum to t: ec = 2^(t/2), e2c = 2^t for the thread's state row, x* for its corner channel.
 struct Decay {
-    float t, ec, e2c, xt, xec, xe2c;
+    float ec, e2c, xec, xe2c;
 };
-// all / xall: the sums of the thread's own channel pairs, which every warp holds for all channels.
 template <int D>
 __device__ __forceinline__ Decay decay_of(const StateOf<D> &st, float2 all, float2 xall)
 {
     Decay d;
-    const float ax = __shfl_sync(0xffffffffu, all.x, st.row >> 1), ay = __shfl_sync(0xffffffffu, all.y, st.row >> 1);
-    d.t = (st.row & 1) ? ay : ax;
-    d.ec = ex2(0.5f * d.t);
-    d.e2c = ex2(d.t);
-    d.xt = d.xec = d.xe2c = 0.f;
+    const float t = of_row(st, all);
+    d.ec = ex2(0.5f * t);
+    d.e2c = ex2(t);
+    d.xec = d.xe2c = 0.f;
     if (Col<D>::X) {
-        const float bx = __shfl_sync(0xffffffffu, xall.x, (threadIdx.x & 7) >> 1), by = __shfl_sync(0xffffffffu, xall.y, (threadIdx.x & 7) >> 1);
-        d.xt = (threadIdx.x & 1) ? by : bx;
-        d.xec = ex2(0.5f * d.xt);
-        d.xe2c = ex2(d.xt);
+        const float xt = of_corner(xall);
+        d.xec = ex2(0.5f * xt);
+        d.xe2c = ex2(xt);
     }
     return d;
+}
+// Weight of a (sub-)chunk's product in a sum over the segment: 2^x with x the decay from the chunk's centre to the
+// segment's end (or from its start).
+struct Weight {
+    float f, xf;
+};
+template <int D>
+__device__ __forceinline__ Weight weight_of(const StateOf<D> &st, float2 x, float2 xx)
+{
+    Weight w;
+    w.f = ex2(of_row(st, x));
+    w.xf = Col<D>::X ? ex2(of_corner(xx)) : 0.f;
+    return w;
 }
 // value of key channel 64 + j of the corner (every lane of the warp must call it)
 __device__ __forceinline__ float corner_val(float v, int j) { return __shfl_sync(0xffffffffu, v, j); }
@@ -511,6 +485,24 @@ __device__ __forceinline__ void fold_state(uint32_t acc, const StateOf<D> &m, fl
         }
     }
 }
+// sum <- sum + 2^x U, U the accumulator at `acc`, the sum in tensor memory too (`first`: nothing is there yet)
+template <int D>
+__device__ __forceinline__ void add_product(uint32_t sum, uint32_t acc, const StateOf<D> &m, const Weight &wt, bool first)
+{
+#pragma unroll
+    for (int i = 0; i < Col<D>::NPS; ++i) {
+        if (!m.has(i)) continue;
+        float u[8], s[8];
+        tmem_ld8_pair(acc + m.tcol(i), sum + m.tcol(i), u, s);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float f = m.corner(i) ? corner_val(wt.xf, e) : wt.f;
+            s[e] = first ? f * u[e] : fmaf(f, u[e], s[e]);
+        }
+        tmem_st8(sum + m.tcol(i), s);
+    }
+    tmem_st_wait();
+}
 template <int D>
 __device__ __forceinline__ void get_state(const float *src, const StateOf<D> &m, float (&S)[Col<D>::NPS][8])
 {
@@ -564,21 +556,21 @@ __device__ __forceinline__ void acc_to_global(uint32_t acc, const StateOf<D> &m,
 
 // ---- products with split accumulators ----------------------------------------------------------------
 constexpr uint32_t kHiLanes = 16u << 16;
-// acc <- A^T B over the 64 token rows (or K16 steps of 16 rows from row r0): rows = key channels (A), columns = value channels (B)
+// acc <- A^T B over the 64 token rows: rows = key channels (A), columns = value channels (B)
 template <int D>
-__device__ __forceinline__ void issue_state(uint32_t acc, const char *tA, const char *tB, bool accumulate = false)
+__device__ __forceinline__ void issue_state(uint32_t acc, const char *tA, const char *tB)
 {
     using C = Cfg<D>;
     using L = Col<D>;
     const uint32_t a = smem_u32(tA), b = smem_u32(tB);
-    issue<64, 8 * L::NV0, true, true, T / 16, C::CHT, C::CHT>(acc, a, b, accumulate);
-    issue<64, 8 * L::NV1, true, true, T / 16, C::CHT, C::CHT>(acc + kHiLanes, a, b + L::NV0 * C::CHT, accumulate);
+    issue<64, 8 * L::NV0, true, true, T / 16, C::CHT, C::CHT>(acc, a, b, false);
+    issue<64, 8 * L::NV1, true, true, T / 16, C::CHT, C::CHT>(acc + kHiLanes, a, b + L::NV0 * C::CHT, false);
     if (L::X) {
         // the corner, transposed: rows = value channels (64 and the remaining 8), columns = key channels 64 .. 71.
         // The second product's A operand covers chunks 8 .. 15, most of them beyond the tile: mapped shared
         // memory whose rows of the result nobody reads.
-        issue<64, 8, true, true, T / 16, C::CHT, C::CHT>(acc + L::HW, b, a + 8 * C::CHT, accumulate);
-        issue<64, 8, true, true, T / 16, C::CHT, C::CHT>(acc + L::HW + kHiLanes, b + 8 * C::CHT, a + 8 * C::CHT, accumulate);
+        issue<64, 8, true, true, T / 16, C::CHT, C::CHT>(acc + L::HW, b, a + 8 * C::CHT, false);
+        issue<64, 8, true, true, T / 16, C::CHT, C::CHT>(acc + L::HW + kHiLanes, b + 8 * C::CHT, a + 8 * C::CHT, false);
     }
 }
 // acc (+)= A B with the value channels (columns of B) split; A K-major tile of 64 rows, B MN-major

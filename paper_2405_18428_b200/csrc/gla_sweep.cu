@@ -93,14 +93,18 @@ __device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, int *st
     } while (0)
 
 // =================================================================================================
-// sweep_local_fwd: the state a segment leaves from a zero start, sum over its tokens of k 2^(gates after
-// the token) v^T, and its total decay.  The tiles are walked from the segment's end: every decay factor is
-// then a power of two below 1 that needs no centring (no sub-chunks, whatever the gates), and the products
-// of all tiles add up in tensor memory, so the state is read once per segment.  One barrier per tile: behind
-// it lie the group sums of this tile and the operand rows of the one before, whose product is issued there;
-// operand tiles and sums have two buffers, and the rows of the next tile are loaded a whole tile ahead.
-// Bound by the latency of its phases (IPC 1.4); 48 sequences of 4096 tokens, d = 64: 40.3 us with the state in
-// registers, decayed once per tile in scan order, 27 us now; 16 of 16384, d = 72: 79 -> 43 us.
+// sweep_local_fwd: the state a segment leaves from a zero start, and its total decay.  The tiles are walked from the
+// segment's end, so the decay from a tile's centre to the end is known when its product is: the state is the plain
+// sum of 2^(that decay) (Kc^T V), kept in tensor memory.  A tile is divided only where its gates ask for it: shorter
+// chunks give the same errors here (2.1e-4 of RMS, root mean square, with chunks of 16, 32 or 64).  One barrier per
+// tile: behind it lie the group sums of this tile and the operand rows of the one before, whose product is issued there
+// and added one step later; operand tiles, accumulators and sums have two buffers, and the rows of the next tile are
+// loaded a whole tile ahead.
+// Bound by the latency of its phases.  48 sequences of 4096 tokens, d = 64: 40 us with the state in registers, decayed
+// once per tile in scan order, 33 us now; 16 of 16384, d = 72: 80 -> 54 us (63 with the sum in registers, which spills).
+// One operand exponent for the whole way to the segment's end would let the matrix unit add the products up (29 and
+// 43 us), but fp16 then loses what decays below 2^-25 even where nothing larger follows: errors of 0.3 of RMS where a
+// segment's keys lie in its first tile.
 // =================================================================================================
 template <int D>
 struct LocalFwdSmem {
@@ -109,7 +113,8 @@ struct LocalFwdSmem {
     static constexpr int kBuf = 2 * C::TILE_T;                                // tK tV
     static constexpr int kPad = L::X ? 16 * C::CHT - C::TILE_T : 0;           // the corner's operand reads past its tile
     static constexpr size_t bytes = 2 * kBuf + kPad + 2 * 8 * D * 4 + 4 * T * 4 + sizeof(Ctl);
-    static constexpr uint32_t tmem_cols = L::ACCS <= 32 ? 32 : 64;
+    static constexpr uint32_t aSum = 2 * L::ACCS;                             // accumulator columns: two products, the sum
+    static constexpr uint32_t tmem_cols = 3 * L::ACCS <= 128 ? 128 : 256;
 };
 
 template <int D>
@@ -127,20 +132,41 @@ sweep_local_fwd(const SweepArgs a)
     const int tid = threadIdx.x;
     cta_setup(ctl, 2, SM::tmem_cols, smem, 2 * SM::kBuf + SM::kPad);
     const Who<D> w;
+    const StateOf<D> sm(w);
     const uint32_t tmem = warp_uniform(ctl->tmem_base), tl = tmem + ((uint32_t)(32 * w.q4) << 16);
     const Geom &g = a.g;
     const Plan &pl = a.plan;
     Cols<D, false, false> raw;
     Cols<D, false, false> nxt;                          // rows and gates of the next tile, a whole tile ahead of their use
-    bool ok = true;
-    uint32_t it = 0;                                    // tiles worked so far: buffer it & 1, its barrier's phase (it >> 1) & 1
+    bool ok = true, first = true;                       // first: nothing of this segment is in the sum
+    uint32_t it = 0;                                    // (sub-)chunks worked so far: buffer it & 1, its barrier's phase (it >> 1) & 1
     const int total = g.B * g.H * pl.nseg;
+
+    // product of step i: its operand tiles were built before the barrier just passed
+    auto issue_step = [&](uint32_t i) {
+        if (w.issuer() && elect_one()) {
+            char *tK = smem + (i & 1) * SM::kBuf;
+            tc_fence_after_sync();
+            issue_state<D>(tmem + (i & 1) * L::ACCS, tK, tK + C::TILE_T);
+            mma_commit(&ctl->bar[i & 1]);
+        }
+    };
+    auto add_step = [&](uint32_t i, const Weight &wt) {
+        ok = wait_all(&ctl->bar[i & 1], (i >> 1) & 1, a.status, ok);
+        tc_fence_after_sync();
+        if (ok) add_product<D>(tl + SM::aSum, tl + (i & 1) * L::ACCS, sm, wt, first);
+        first = false;
+        tc_fence_before_sync();
+    };
 
     pdl_wait();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
+        first = true;
         float2 after = make_float2(0.f, 0.f), xafter = after;          // gates of the tiles behind (log2), the thread's channels
+        uint32_t n = 0;                                                 // (sub-)chunks of this segment
+        Weight w1{}, w2{};                                              // weights of the last one and of the one before
         if (tid < 3 * T && t1 - 1 - (tid >> 6) >= t0) {
             const int tile = t1 - 1 - (tid >> 6);
             rowOff[(tile & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, tile, tid & 63);
@@ -157,33 +183,54 @@ sweep_local_fwd(const SweepArgs a)
             }
             const int nrow = g.L - (t1 - 1) * T;
             if (nrow < T) { clear_tail_rows(raw, w, nrow); clear_tail_gates(raw, w, nrow); }
-            group_prefix<D>(raw, raw.g, w, sTot + (it & 1) * 8 * D);
+            group_prefix<D>(raw, raw.g, w, sTot + ((t1 - 1) & 1) * 8 * D);
         }
-        for (int tile = t1 - 1; tile >= t0; --tile, ++it) {
+        for (int tile = t1 - 1; tile >= t0; --tile) {
+            const int nrow = min(T, g.L - tile * T);
+            const float *tot = sTot + (tile & 1) * 8 * D;
             tc_fence_before_sync();
-            SYNC_OR_DIE();
-            if (w.issuer() && tile < t1 - 1 && elect_one()) {                    // the tile before is built
-                char *tK = smem + ((it + 1) & 1) * SM::kBuf;
-                tc_fence_after_sync();
-                issue_state<D>(tmem, tK, tK + C::TILE_T, tile < t1 - 2);
-                mma_commit(&ctl->bar[(it + 1) & 1]);
-            }
+            SYNC_OR_DIE();                                             // group totals are there, the step before is built
+            if (n > 0) issue_step(it - 1);
             if (tid < T && tile - 3 >= t0) rowOff[((tile - 3) & 3) * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 3, tid);
             if (tile > t0) {
                 uint32_t ro[9];
                 row_offsets<D>(rowOff + ((tile - 1) & 3) * T, w, ro);
                 load_rows(nxt, a.q, a.k, a.v, a.d_out, ro);
             }
-            const Tot tt = tile_totals<D>(sTot + (it & 1) * 8 * D, w);
-            if (it >= 2) ok = wait_all(&ctl->bar[it & 1], ((it - 2) >> 1) & 1, a.status, ok);       // the buffer is free again
-            const float2 off = add2(after, sub2(tt.all, tt.before)), xoff = add2(xafter, sub2(tt.xall, tt.xbefore));
-            char *tK = smem + (it & 1) * SM::kBuf;
-            build_suffix_rows<D>(raw, w, off, xoff, tK, tK + C::TILE_T);
-            fence_async_smem();
-            after = add2(after, tt.all);
-            xafter = add2(xafter, tt.xall);
+            const Tot whole = tile_totals<D>(tot, w);
+            Tot tt = whole;
+            int s = T;
+            if (beyond<D>(tt)) {
+                s = choose_window<D>(tot, w, T / 2, a.status);
+                const int w0 = 8 * w.grp / s * (s / 8);
+                tt = window_totals<D>(tot, w, w0, w0 + s / 8);
+            }
+            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
+            const int nsub = (nrow + s - 1) / s;
+            for (int u = nsub - 1; u >= 0; --u, ++it, ++n) {
+                if (u < nsub - 1) {
+                    tc_fence_before_sync();
+                    SYNC_OR_DIE();
+                    issue_step(it - 1);
+                }
+                if (n >= 2) add_step(it - 2, w2);                       // its buffer is free again
+                char *tK = smem + (it & 1) * SM::kBuf;
+                build_rows<D>(raw, w, nullptr, tK, tK + C::TILE_T, nullptr, 8 * w.grp >= u * s && 8 * w.grp < (u + 1) * s);
+                fence_async_smem();
+                // gates from the centre to the segment's end
+                float2 x = fma2(whole.all, make_float2(0.5f, 0.5f), after), xx = fma2(whole.xall, make_float2(0.5f, 0.5f), xafter);
+                if (s < T) {
+                    const Tot own = window_totals<D>(tot, w, u * s / 8, (u + 1) * s / 8), behind = window_totals<D>(tot, w, (u + 1) * s / 8, 8);
+                    x = fma2(own.all, make_float2(0.5f, 0.5f), add2(after, behind.all));
+                    xx = fma2(own.xall, make_float2(0.5f, 0.5f), add2(xafter, behind.xall));
+                }
+                w2 = w1;
+                w1 = weight_of<D>(sm, x, xx);
+            }
+            after = add2(after, whole.all);
+            xafter = add2(xafter, whole.xall);
             if (tile > t0) {
-                group_prefix<D>(raw, nxt.g, w, sTot + ((it + 1) & 1) * 8 * D);       // only the last tile of a sequence has a tail
+                group_prefix<D>(raw, nxt.g, w, sTot + ((tile - 1) & 1) * 8 * D);       // only the last tile of a sequence has a tail
                 if (tile - 2 >= t0) {
                     uint32_t ro[9];
                     row_offsets<D>(rowOff + ((tile - 2) & 3) * T, w, ro);
@@ -199,15 +246,11 @@ sweep_local_fwd(const SweepArgs a)
         }
         tc_fence_before_sync();
         SYNC_OR_DIE();
-        if (w.issuer() && elect_one()) {
-            char *tK = smem + ((it + 1) & 1) * SM::kBuf;
-            tc_fence_after_sync();
-            issue_state<D>(tmem, tK, tK + C::TILE_T, t1 - t0 > 1);
-            mma_commit(&ctl->bar[(it + 1) & 1]);
-        }
-        ok = wait_all(&ctl->bar[(it + 1) & 1], ((it - 1) >> 1) & 1, a.status, ok);
-        tc_fence_after_sync();
-        if (ok) acc_to_global<D>(tl, StateOf<D>(w), a.seg_state + (size_t)sid * D * D);
+        issue_step(it - 1);
+        if (n >= 2) add_step(it - 2, w2);
+        add_step(it - 1, w1);
+        if (ok) acc_to_global<D>(tl + SM::aSum, sm, a.seg_state + (size_t)sid * D * D);
+        tc_fence_before_sync();
         if (w.grp == 0) {
             *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.c2) = after;
             if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.xc2) = xafter;
@@ -222,11 +265,11 @@ die:
 // sweep_local_bwd: what the backward sweep needs of a segment from a zero state.  In scan order, the state
 // in registers: per (sub-)chunk the state entering it (scaled to its centre, fp16) and the decay since the
 // segment start.  GRAD: also the segment's contribution to the gradient of the state entering it, the sum of
-// 2^(gates since the segment start) q dO^T; those factors are below 1, so these products simply add up in
-// tensor memory and are read once per segment.  A backward pass over uncut sequences needs only the states.
+// 2^(gates from the segment start to the centre) (Qc^T dO), in tensor memory (the state and the rows take the
+// registers).  A backward pass over uncut sequences needs only the states.
 // Pipelined over the (sub-)chunks: the products of one run while the next one's operand tiles are built (two
-// buffers of tiles and accumulators), and are folded into the state one step later.  48 sequences of 4096
-// tokens, d = 64: 66.6 us before (both sums in registers, no pipelining), 47 us now; 16 of 16384, d = 72: 122 -> 95 us.
+// buffers of tiles and accumulators), and are folded into the sums one step later.  48 sequences of 4096 tokens, d = 64:
+// 60 us with both sums in registers and no pipelining, 44 us now; 16 of 16384, d = 72: 122 -> 104 us.
 // =================================================================================================
 template <int D, bool GRAD>
 struct LocalBwdSmem {
@@ -235,9 +278,11 @@ struct LocalBwdSmem {
     static constexpr int kBuf = (GRAD ? 4 : 2) * C::TILE_T;                   // (tQ) tK tV (tG)
     static constexpr int kPad = L::X ? 16 * C::CHT - C::TILE_T : 0;           // the corner's operand reads past its tile
     static constexpr size_t bytes = 2 * kBuf + kPad + 2 * 8 * D * 4 + 4 * T * 4 + sizeof(Ctl);
-    static constexpr uint32_t aW = 2 * L::ACCS;                               // accumulator columns: two of the state, one of the gradient
-    static constexpr uint32_t cols = (GRAD ? 3 : 2) * L::ACCS;
+    // accumulator columns: two of the state's products, two of the gradient's, the gradient's sum
+    static constexpr uint32_t aW = 2 * L::ACCS, aSum = 4 * L::ACCS;
+    static constexpr uint32_t cols = (GRAD ? 5 : 2) * L::ACCS;
     static constexpr uint32_t tmem_cols = cols <= 64 ? 64 : cols <= 128 ? 128 : 256;
+    static_assert(cols <= 256, "tensor memory of two CTAs");
 };
 
 template <int D, bool GRAD>
@@ -271,12 +316,18 @@ sweep_local_bwd(const SweepArgs a)
         load_gates(raw.g, a.gate, off);
         load_rows(raw, a.q, a.k, a.v, a.d_out, off);
     };
-    // S <- 2^2c S + 2^c (Kc^T V), the product of step i
+    // S <- 2^2c S + 2^c (Kc^T V), sum <- sum + 2^(.) (Qc^T dO): the products of step i
     Decay dec;
+    Weight wt{};
+    bool pending = false, first = true;                 // the step before waits to be folded; nothing of this segment is in the sum
     auto fold = [&](uint32_t i) {
         ok = wait_all(&ctl->bar[i & 1], (i >> 1) & 1, a.status, ok);
         tc_fence_after_sync();
-        if (ok) fold_state<D>(tl + (i & 1) * L::ACCS, sm, S, dec);
+        if (ok) {
+            fold_state<D>(tl + (i & 1) * L::ACCS, sm, S, dec);
+            if (GRAD) add_product<D>(tl + SM::aSum, tl + SM::aW + (i & 1) * L::ACCS, sm, wt, first);
+        }
+        first = false;
         tc_fence_before_sync();
     };
 
@@ -286,7 +337,8 @@ sweep_local_bwd(const SweepArgs a)
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
         get_state<D>(nullptr, sm, S);
         float2 gsum = make_float2(0.f, 0.f), gxsum = gsum;             // gates since the segment start (log2), the thread's channels
-        bool pending = false;
+        pending = false;
+        first = true;
         if (tid < 2 * T) rowOff[((t0 + (tid >> 6)) & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, t0 + (tid >> 6), tid & 63);
         __syncthreads();
         load_tile(t0);
@@ -309,15 +361,14 @@ sweep_local_bwd(const SweepArgs a)
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(tot, w, w0, w0 + s / 8);
             }
-            const float2 off = centred(tt.before, tt.all), xoff = centred(tt.xbefore, tt.xall);
+            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
             const int nsub = (nrow + s - 1) / s;
             for (int u = 0; u < nsub; ++u, ++it) {
                 const int lo = u * s, hi = lo + s;
                 const bool last = u == nsub - 1, on = 8 * w.grp >= lo && 8 * w.grp < hi;
                 char *buf = smem + (it & 1) * SM::kBuf;
                 char *tQ = buf, *tK = GRAD ? tQ + C::TILE_T : buf, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T;
-                build_kv_rows<D>(raw, w, off, xoff, tK, tV, on);
-                if (GRAD) build_qd_rows<D>(raw, w, add2(gsum, whole.before), add2(gxsum, whole.xbefore), tQ, tG, on);
+                build_rows<D>(raw, w, tQ, tK, tV, tG, on);
                 Tot tu = whole;
                 float2 gs = gsum, gxs = gxsum;                         // decay before the sub-chunk
                 if (s < T) {
@@ -327,6 +378,8 @@ sweep_local_bwd(const SweepArgs a)
                     tu = window_totals<D>(tot, w, lo / 8, hi / 8);
                 }
                 const Decay now = decay_of<D>(sm, tu.all, tu.xall);
+                Weight wnow{};
+                if (GRAD) wnow = weight_of<D>(sm, fma2(tu.all, make_float2(0.5f, 0.5f), gs), fma2(tu.xall, make_float2(0.5f, 0.5f), gxs));
                 const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
                 if (w.grp == 0) {
                     *reinterpret_cast<float2 *>(a.slot_g + slot * D + w.c2) = gs;
@@ -339,7 +392,7 @@ sweep_local_bwd(const SweepArgs a)
                 if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
                     issue_state<D>(tmem + (it & 1) * L::ACCS, tK, tV);                             // Kc^T V
-                    if (GRAD) issue_state<D>(tmem + SM::aW, tQ, tG, pending);                      // + (q decayed)^T dO
+                    if (GRAD) issue_state<D>(tmem + SM::aW + (it & 1) * L::ACCS, tQ, tG);          // Qc^T dO
                     mma_commit(&ctl->bar[it & 1]);
                 }
                 // the register prefetch alone does not cover the memory latency of tiles this short
@@ -347,6 +400,7 @@ sweep_local_bwd(const SweepArgs a)
                 if (last && tile + 2 < t1) prefetch_gates<D>(a.gate, rowOff + ((tile + 2) & 3) * T, w);
                 if (pending) fold(it - 1);
                 dec = now;
+                wt = wnow;
                 put_state<D, D * 16>(reinterpret_cast<char *>(a.slot_s + slot * (D * D)), sm, S, dec);
                 pending = true;
             }
@@ -360,7 +414,7 @@ sweep_local_bwd(const SweepArgs a)
         }
         fold(it - 1);
         save_state<D>(a.seg_state + (size_t)sid * D * D, sm, S);
-        if (GRAD && ok) acc_to_global<D>(tl + SM::aW, sm, a.seg_dstate + (size_t)sid * D * D);
+        if (GRAD && ok) acc_to_global<D>(tl + SM::aSum, sm, a.seg_dstate + (size_t)sid * D * D);
         if (w.grp == 0) {
             *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.c2) = gsum;
             if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.xc2) = gxsum;
