@@ -259,12 +259,14 @@ __device__ __forceinline__ void build_rows(const Cols<D, HQ, HD> &r, const Who<D
         }
     }
 }
-// Row sums of the gates -> exponents (log2) of the items' decay factors.
+// Row sums of the gates -> exponents (log2) of the items' decay factors.  Rows past the end of the sequence get 0: their
+// operands are zero, and where the gates are beyond the range 2^x would overflow there and make them 0 * inf.
 template <int D, bool HQ, bool HD>
-__device__ __forceinline__ void centre_rows(Cols<D, HQ, HD> &r, float2 off, float2 xoff)
+__device__ __forceinline__ void centre_rows(Cols<D, HQ, HD> &r, const Who<D> &w, float2 off, float2 xoff, int nrow)
 {
 #pragma unroll
     for (int j = 0; j < r.N; ++j) r.g[j] = add2(r.g[j], j < 8 ? off : xoff);
+    if (nrow < T) clear_tail_gates(r, w, nrow);
 }
 // exponent offset of a (sub-)chunk's rows: minus half its total, plus the groups before
 __device__ __forceinline__ float2 centred(float2 before, float2 all) { return fma2(all, make_float2(-0.5f, -0.5f), before); }

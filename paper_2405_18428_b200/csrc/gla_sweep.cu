@@ -205,7 +205,7 @@ sweep_local_fwd(const SweepArgs a)
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(tot, w, w0, w0 + s / 8);
             }
-            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
+            centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
             const int nsub = (nrow + s - 1) / s;
             for (int u = nsub - 1; u >= 0; --u, ++it, ++n) {
                 if (u < nsub - 1) {
@@ -361,7 +361,7 @@ sweep_local_bwd(const SweepArgs a)
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(tot, w, w0, w0 + s / 8);
             }
-            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
+            centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
             const int nsub = (nrow + s - 1) / s;
             for (int u = 0; u < nsub; ++u, ++it) {
                 const int lo = u * s, hi = lo + s;
@@ -640,7 +640,7 @@ sweep_fwd(const SweepArgs a)
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
             }
-            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
+            centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
             const int nsub = (nrow + s - 1) / s;
             for (int u = 0; u < nsub; ++u) {
                 const int lo = u * s, hi = lo + s;
@@ -864,7 +864,7 @@ sweep_bwd(const SweepArgs a)
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
             }
-            centre_rows<D>(raw, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall));
+            centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
             const int nsub = (nrow + s - 1) / s;
             float2 tot = make_float2(0.f, 0.f), xtot = tot;      // sums of q dq - k dk over the group
             for (int u = nsub - 1; u >= 0; --u) {

@@ -150,11 +150,11 @@ def test_decay_beyond_the_range_is_reported_not_silent():
 @pytest.mark.parametrize("d", [64, 72])
 @pytest.mark.parametrize("B,H", [(1, 3), (20, 16)])      # cut into one-tile segments; uncut
 def test_decay_beyond_the_range_in_a_partly_filled_window_stays_finite(d, B, H):
-    """log alpha = -60 per token, 203 = 3 * 64 + 11 tokens: the last 8-row window holds three rows whose gates sum to 2 * 130
+    """log alpha = -60 per token, 459 = 7 * 64 + 11 tokens: the last 8-row window holds three rows whose gates sum to 2 * 130
     in log2 units.  The empty rows behind them must stay zero operands although 2^130 overflows fp32."""
     from paper_2405_18428_b200 import dig
     from parity import to_dev
-    wl = _wl(d, 64, B=B, H=H, grid_h=7, grid_w=29)
+    wl = _wl(d, 64, B=B, H=H, grid_h=9, grid_w=51)
     x = make_inputs(wl, conv=False)
     q, k, v = (to_dev(x[n], wl) for n in ("q", "k", "v"))
     gate = torch.full(q.shape, -60.0, device="cuda")
