@@ -167,7 +167,7 @@ __device__ __forceinline__ float2 sigmoid2(float2 r)
     return make_float2(__fdividef(1.f, e.x), __fdividef(1.f, e.y));
 }
 
-// The affine parameters of a row in shared memory: weight (1 where absent), then bias (0).
+// The affine parameters of a row in shared memory: weight (1 where absent), then bias (0).  Ends with a barrier.
 template <int MAXD, int THREADS>
 __device__ __forceinline__ void stage_affine(float *sh, const float *ln_w, const float *ln_b, int dv)
 {
@@ -274,7 +274,6 @@ outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const floa
     ring.status = status;
     ring.rows = rows;
     ring_setup(bar);
-    stage_affine<kMaxD, kThreads>(aff, ln_w, ln_b, dv);
     Lane<LPR, CPL, kThreads, FULL> ln;
     ln.dv = dv;
     const float inv_d = 1.f / (float)dv;
@@ -283,6 +282,7 @@ outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const floa
         ring.fetch(0);
         ring.fetch(1);
     }
+    stage_affine<kMaxD, kThreads>(aff, ln_w, ln_b, dv);         // behind the wait: the kernel in front may have written them
     bool ok = true;
     int it = 0;
     for (; ok && ring.first(it) < rows; ++it) {
@@ -343,7 +343,6 @@ outgate_bwd(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln
     ring.status = status;
     ring.rows = rows;
     ring_setup(bar);
-    stage_affine<kMaxD, kThreads>(aff, ln_w, ln_b, dv);
     Lane<LPR, CPL, kThreads, FULL> ln;
     ln.dv = dv;
     const float inv_d = 1.f / (float)dv;
@@ -355,6 +354,7 @@ outgate_bwd(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln
         ring.fetch(0);
         ring.fetch(1);
     }
+    stage_affine<kMaxD, kThreads>(aff, ln_w, ln_b, dv);         // behind the wait: the kernel in front may have written them
     bool ok = true;
     int it = 0;
     for (; ok && ring.first(it) < rows; ++it) {

@@ -74,6 +74,28 @@ def test_outgate_without_eps_on_a_partly_filled_tile(dtype, d, rows):
     _case((rows, d), dtype, True, 5, eps=0.0)
 
 
+def test_affine_parameters_written_by_the_kernel_in_front():
+    """ln_w and ln_b come straight from the kernel before on the stream; every call sees their latest values."""
+    from paper_2405_18428_b200 import dig
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    n = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    o, r, dz = (n(333, 72).to(torch.bfloat16) for _ in range(3))
+    steps, d_w, d_b = 20, n(72), n(72)
+    w, b, got = torch.zeros(72, device="cuda"), torch.zeros(72, device="cuda"), []
+    for _ in range(steps):
+        w.add_(d_w)
+        b.add_(d_b)
+        got.append((dig.dig_gla_outgate_fwd(o, r, w, b, f32_out=True), dig.dig_gla_outgate_bwd(o, r, dz, w, b, f32_out=True)[:2]))
+    w, b = torch.zeros_like(w), torch.zeros_like(b)
+    for z, grads in got:
+        w.add_(d_w)
+        b.add_(d_b)
+        torch.cuda.synchronize()
+        assert torch.equal(z, dig.dig_gla_outgate_fwd(o, r, w, b, f32_out=True))
+        for x, y in zip(grads, dig.dig_gla_outgate_bwd(o, r, dz, w, b, f32_out=True)):
+            assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("cfg", ["C2", "C5"])
 def test_outgate_benchmark_shapes(cfg):
     wl = CONFIGS[cfg]
