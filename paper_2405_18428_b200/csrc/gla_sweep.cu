@@ -1060,34 +1060,6 @@ die:
 // ---- host side ----------------------------------------------------------------------------------
 constexpr int kPerSm = 2;       // CTAs of 256 threads that share an SM, for every kernel of the family
 
-// Segment length.  A pass costs (tiles of a segment + one of fill and drain) per round of resident CTAs.
-// Uncut sequences (one segment each) run the forward sweep alone; cut ones also run the local sweep, about
-// half of a forward sweep per tile, and the scan, and these two launches take about as long as three tiles
-// of a forward sweep when the machine is not full.  The backward pass needs the local sweep in either case.
-Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
-{
-    Plan p;
-    p.ntile = (g.L + T - 1) / T;
-    p.sub_max = g.C < T ? g.C : T;
-    p.gh_inv = g.gh > 1 ? (uint32_t)((1ull << 32) / (unsigned)g.gh) : 0xffffffffu;
-    const long long slots = (long long)sms * per_sm, bh = (long long)g.B * g.H;
-    long long best = -1;
-    p.G = p.ntile;
-    // the shortest G of every number of segments that occurs (about 2 sqrt(ntile) of them)
-    for (int nseg = 1, G = p.ntile;; nseg = (p.ntile + G - 2) / (G - 1), G = (p.ntile + nseg - 1) / nseg) {
-        const long long rounds = (bh * nseg + slots - 1) / slots;
-        long long cost = rounds * (G + 1) * 10;             // a segment costs about one tile of fill and drain
-        if (nseg > 1) cost += backward ? 15 : cost / 2 + 30;
-        if (best < 0 || cost < best) {
-            best = cost;
-            p.G = G;
-        }
-        if (G == 1) break;
-    }
-    p.nseg = (p.ntile + p.G - 1) / p.G;
-    return p;
-}
-
 struct SweepWs {
     float *seg_state, *seg_gamma, *seg_dstate, *seg_carry, *slot_g;
     __half *seg_state16, *slot_s;
@@ -1111,6 +1083,39 @@ SweepWs carve(char *base, const Geom &g, const Plan &pl, bool backward)
     }
     w.bytes = o;
     return w;
+}
+
+// Segment length.  A pass costs (tiles of a segment + one of fill and drain) per round of resident CTAs.
+// Uncut sequences (one segment each) run the forward sweep alone; cut ones also run the local sweep, about
+// half of a forward sweep per tile, and the scan, and these two launches take about as long as three tiles
+// of a forward sweep when the machine is not full.  The backward pass needs the local sweep in either case.
+// Chunks above 64 tokens: forward plans stay within the scratch of dig_gla_fwd_static where uncut sequences do (the
+// same plan serves dig_gla_fwd, so that both give the same bits).  No other family's workspace is counted there that
+// would be larger anyway; with chunks of up to 64 the per-chunk states of the other families always are.
+Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
+{
+    Plan p;
+    p.ntile = (g.L + T - 1) / T;
+    p.sub_max = g.C < T ? g.C : T;
+    p.gh_inv = g.gh > 1 ? (uint32_t)((1ull << 32) / (unsigned)g.gh) : 0xffffffffu;
+    const long long slots = (long long)sms * per_sm, bh = (long long)g.B * g.H;
+    long long best = -1;
+    p.G = p.ntile;
+    // the shortest G of every number of segments that occurs (about 2 sqrt(ntile) of them)
+    for (int nseg = 1, G = p.ntile;; nseg = (p.ntile + G - 2) / (G - 1), G = (p.ntile + nseg - 1) / nseg) {
+        const long long rounds = (bh * nseg + slots - 1) / slots;
+        long long cost = rounds * (G + 1) * 10;             // a segment costs about one tile of fill and drain
+        if (nseg > 1) cost += backward ? 15 : cost / 2 + 30;
+        p.nseg = nseg;
+        const bool fits = backward || g.C <= T || nseg == 1 || carve(nullptr, g, p, false).bytes <= DIG_GLA_STATIC_SCRATCH_BYTES;
+        if (best < 0 || (cost < best && fits)) {
+            best = cost;
+            p.G = G;
+        }
+        if (G == 1) break;
+    }
+    p.nseg = (p.ntile + p.G - 1) / p.G;
+    return p;
 }
 
 template <typename K>

@@ -83,3 +83,18 @@ def test_static_scratch_rejects_problems_beyond_its_limit():
         dig.dig_gla_fwd_static(t, t, t, gate, out, gh, gw, 64, 0)
     assert e.value.status == dig.DIG_ERR_SCRATCH_LIMIT
     assert "built-in scratch" in str(e.value)
+
+
+def test_static_scratch_serves_many_long_sequences_in_long_chunks():
+    """80 sequences of 4096 tokens, d = 72, chunks of 128: cut so that the segment states fit the array; the same bits as
+    dig_gla_fwd."""
+    import torch
+    from paper_2405_18428_b200 import dig
+    wl = Workload("static-c", B=5, H=16, grid_h=64, grid_w=64, d_k=72, d_v=72, chunk=128, dtype="bf16", tau=(16.0, 4.0), seed=13)
+    q, k, v, gate = _inputs(wl)
+    want = dig.dig_gla_fwd(q, k, v, gate, wl.grid_h, wl.grid_w, wl.chunk, 1)
+    out = torch.full_like(want, float("nan"))
+    dig.dig_gla_fwd_static(q, k, v, gate, out, wl.grid_h, wl.grid_w, wl.chunk, 1)
+    torch.cuda.synchronize()
+    assert dig.dig_last_device_status() == dig.DIG_OK
+    assert torch.equal(out, want)
