@@ -85,14 +85,19 @@ void *dev(const Tensor &t, ScalarType st, const char *name)
                                     c10::toString(t.scalar_type()) + " on " + t.device().str());
     return t.data_ptr();
 }
-void *dev(const Tensor &t, ScalarType st, at::IntArrayRef shape, const char *name)
+// ... of the given shape, on the device of `like`.
+void *dev(const Tensor &t, ScalarType st, at::IntArrayRef shape, const char *name, const Tensor &like)
 {
     void *p = dev(t, st, name);
     if (t.sizes() != shape) raise(PyExc_ValueError, std::string(name) + ": shape " + text(t.sizes()) + " != " + text(shape));
+    if (t.device() != like.device()) raise(PyExc_ValueError, std::string(name) + ": on " + t.device().str() + ", the other tensors on " + like.device().str());
     return p;
 }
-void *dev(PyObject *o, ScalarType st, at::IntArrayRef shape, const char *name) { return dev(tensor(o, name), st, shape, name); }
-void *dev_opt(PyObject *o, ScalarType st, at::IntArrayRef shape, const char *name) { return none(o) ? nullptr : dev(o, st, shape, name); }
+void *dev(PyObject *o, ScalarType st, at::IntArrayRef shape, const char *name, const Tensor &like) { return dev(tensor(o, name), st, shape, name, like); }
+void *dev_opt(PyObject *o, ScalarType st, at::IntArrayRef shape, const char *name, const Tensor &like)
+{
+    return none(o) ? nullptr : dev(o, st, shape, name, like);
+}
 
 Tensor empty(at::IntArrayRef shape, ScalarType st, const Tensor &like)
 {
@@ -134,8 +139,13 @@ struct Ws {
 Ws workspace(PyObject *o, size_t need, const Tensor &like)
 {
     Ws w;
-    if (none(o)) w.t = empty({(int64_t)(need > 16 ? need : 16)}, kByte, like);
-    else w.t = tensor(o, "workspace");
+    if (none(o)) {
+        w.t = empty({(int64_t)(need > 16 ? need : 16)}, kByte, like);
+    } else {                             // any type and shape: it is scratch
+        w.t = tensor(o, "workspace");
+        if (!w.t.is_cuda() || !w.t.is_non_overlapping_and_dense() || w.t.device() != like.device())
+            raise(PyExc_ValueError, "workspace: need a dense tensor on " + like.device().str() + ", got one on " + w.t.device().str());
+    }
     w.p = w.t.data_ptr();
     w.n = (size_t)w.t.numel() * w.t.element_size();
     return w;
@@ -163,9 +173,9 @@ struct Gla {
         st = storage(dtype);
         ost = out_storage(dtype);
         q = dev(q_t, st, "q");
-        k = dev(a[1], st, ks, "k");
-        v = dev(v_t, st, vs, "v");
-        gate = (float *)dev(a[3], kF32, ks, "gate");
+        k = dev(a[1], st, ks, "k", q_t);
+        v = dev(v_t, st, vs, "v", q_t);
+        gate = (float *)dev(a[3], kF32, ks, "gate", q_t);
     }
     std::vector<int64_t> state() const { return {B, H, dk, dv}; }
 };
@@ -200,7 +210,7 @@ PyObject *gate_logsigmoid(PyObject *const *a)
     Py_DECREF(seq);
     if (bad) throw Raised{};
     void *gp = dev(g, storage(dtype), "g");
-    float *op = (float *)dev(gate, kF32, g.sizes(), "gate");
+    float *op = (float *)dev(gate, kF32, g.sizes(), "gate", g);
     void *s = stream();
     CALL(dig_gate_logsigmoid(gp, tau.data(), op, B, L, H, dk, dtype, s), "dig_gate_logsigmoid");
     return wrap(gate);
@@ -212,7 +222,7 @@ PyObject *gla_fwd(PyObject *const *a)
     const Gla g(a, a[4], a[5], a[6], truth(a[8]));
     const int dir = integer(a[7]);
     Tensor out = given(a[9], g.vs, g.ost, g.q_t, "out");
-    void *op = dev(out, g.ost, g.vs, "out");
+    void *op = dev(out, g.ost, g.vs, "out", g.q_t);
     const Ws w = workspace(a[10], none(a[10]) ? dig_gla_workspace_bytes(g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, g.dtype, 0) : 0, g.q_t);
     void *s = stream();
     CALL(dig_gla_fwd(g.q, g.k, g.v, g.gate, op, g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, dir, g.dtype, w.p, w.n, s), "dig_gla_fwd");
@@ -247,10 +257,10 @@ struct Grads {
             Py_DECREF(seq);
             if (!tensors) raise(PyExc_ValueError, "grads: need four tensors (dq, dk, dv, dgate)");
         }
-        pq = dev(dq, g.ost, g.ks, "dq");
-        pk = dev(dk, g.ost, g.ks, "dk");
-        pv = dev(dv, g.ost, g.vs, "dv");
-        pg = (float *)dev(dg, kF32, g.ks, "dgate");
+        pq = dev(dq, g.ost, g.ks, "dq", g.q_t);
+        pk = dev(dk, g.ost, g.ks, "dk", g.q_t);
+        pv = dev(dv, g.ost, g.vs, "dv", g.q_t);
+        pg = (float *)dev(dg, kF32, g.ks, "dgate", g.q_t);
     }
 };
 
@@ -259,7 +269,7 @@ PyObject *gla_bwd(PyObject *const *a)
 {
     const Gla g(a, a[5], a[6], a[7], truth(a[9]));
     const int dir = integer(a[8]);
-    void *dop = dev(a[4], g.st, g.vs, "d_out");
+    void *dop = dev(a[4], g.st, g.vs, "d_out", g.q_t);
     const Grads r(a[10], g);
     const Ws w = workspace(a[11], none(a[11]) ? dig_gla_workspace_bytes(g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, g.dtype, 1) : 0, g.q_t);
     void *s = stream();
@@ -273,7 +283,7 @@ PyObject *gla_fwd_state(PyObject *const *a)
 {
     const Gla g(a, a[5], a[6], a[7], truth(a[9]));
     const int dir = integer(a[8]);
-    const float *si = (const float *)dev_opt(a[4], kF32, g.state(), "s_in");
+    const float *si = (const float *)dev_opt(a[4], kF32, g.state(), "s_in", g.q_t);
     Tensor out = empty(g.vs, g.ost, g.q_t), so;
     if (truth(a[10])) so = empty(g.state(), kF32, g.q_t);
     const Ws w = workspace(a[11], none(a[11]) ? dig_gla_workspace_bytes(g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, g.dtype, 0) : 0, g.q_t);
@@ -290,8 +300,8 @@ PyObject *gla_bwd_state(PyObject *const *a)
 {
     const Gla g(a, a[7], a[8], a[9], truth(a[11]));
     const int dir = integer(a[10]);
-    void *dop = dev(a[4], g.st, g.vs, "d_out");
-    const float *si = (const float *)dev_opt(a[5], kF32, g.state(), "s_in"), *dso = (const float *)dev_opt(a[6], kF32, g.state(), "ds_out");
+    void *dop = dev(a[4], g.st, g.vs, "d_out", g.q_t);
+    const float *si = (const float *)dev_opt(a[5], kF32, g.state(), "s_in", g.q_t), *dso = (const float *)dev_opt(a[6], kF32, g.state(), "ds_out", g.q_t);
     const Grads r(Py_None, g);
     Tensor dsi = empty(g.state(), kF32, g.q_t);
     float *dsip = (float *)dsi.data_ptr();
@@ -308,7 +318,7 @@ PyObject *gla_fwd_multi(PyObject *const *a)
     const Gla g(a, a[4], a[5], a[7], truth(a[8]));
     const unsigned mask = (unsigned)integer(a[6]);
     Tensor out = given(a[9], g.vs, g.ost, g.q_t, "out");
-    void *op = dev(out, g.ost, g.vs, "out");
+    void *op = dev(out, g.ost, g.vs, "out", g.q_t);
     const Ws w = workspace(a[10], none(a[10]) ? dig_gla_multi_workspace_bytes(g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, g.dtype, 0) : 0, g.q_t);
     void *s = stream();
     CALL(dig_gla_fwd_multi(g.q, g.k, g.v, g.gate, op, g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, mask, g.dtype, w.p, w.n, s), "dig_gla_fwd_multi");
@@ -320,7 +330,7 @@ PyObject *gla_bwd_multi(PyObject *const *a)
 {
     const Gla g(a, a[5], a[6], a[8], truth(a[9]));
     const unsigned mask = (unsigned)integer(a[7]);
-    void *dop = dev(a[4], g.st, g.vs, "d_out");
+    void *dop = dev(a[4], g.st, g.vs, "d_out", g.q_t);
     const Grads r(a[10], g);
     const Ws w = workspace(a[11], none(a[11]) ? dig_gla_multi_workspace_bytes(g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, g.dtype, 1) : 0, g.q_t);
     void *s = stream();
@@ -340,7 +350,7 @@ PyObject *gla_fwd_beta(PyObject *const *a)
 {
     const Gla g(a, a[5], a[6], a[7], truth(a[9]));
     const int dir = integer(a[8]);
-    const float *bg = (const float *)dev(a[4], kF32, g.vs, "bgate");
+    const float *bg = (const float *)dev(a[4], kF32, g.vs, "bgate", g.q_t);
     const Ws w = workspace(a[10], beta_need(g, 0), g.q_t);
     Tensor out = empty(g.vs, g.ost, g.q_t);
     void *op = out.data_ptr(), *s = stream();
@@ -352,8 +362,8 @@ PyObject *gla_bwd_beta(PyObject *const *a)
 {
     const Gla g(a, a[6], a[7], a[8], truth(a[10]));
     const int dir = integer(a[9]);
-    const float *bg = (const float *)dev(a[4], kF32, g.vs, "bgate");
-    void *dop = dev(a[5], g.st, g.vs, "d_out");
+    const float *bg = (const float *)dev(a[4], kF32, g.vs, "bgate", g.q_t);
+    void *dop = dev(a[5], g.st, g.vs, "d_out", g.q_t);
     const Ws w = workspace(a[11], beta_need(g, 1), g.q_t);
     const Grads r(Py_None, g);
     Tensor db = empty(g.vs, kF32, g.q_t);
@@ -369,8 +379,8 @@ PyObject *gla_fwd_outgate(PyObject *const *a)
 {
     const Gla g(a, a[5], a[6], a[7], truth(a[12]));
     const int dir = integer(a[8]);
-    const void *rp = dev(a[4], g.st, g.vs, "r");
-    const float *lw = (const float *)dev_opt(a[9], kF32, {g.dv}, "ln_w"), *lb = (const float *)dev_opt(a[10], kF32, {g.dv}, "ln_b");
+    const void *rp = dev(a[4], g.st, g.vs, "r", g.q_t);
+    const float *lw = (const float *)dev_opt(a[9], kF32, {g.dv}, "ln_w", g.q_t), *lb = (const float *)dev_opt(a[10], kF32, {g.dv}, "ln_b", g.q_t);
     const float eps = real(a[11]);
     Tensor out, z = empty(g.vs, g.ost, g.q_t);
     if (truth(a[13])) out = empty(g.vs, g.ost, g.q_t);
@@ -397,8 +407,8 @@ PyObject *outgate_fwd(PyObject *const *a)
     rows_of(o, d, rows);
     const int dtype = dtype_of(o, truth(a[5]));
     const ScalarType st = storage(dtype);
-    const void *op = dev(o, st, "o"), *rp = dev(a[1], st, o.sizes(), "r");
-    const float *lw = (const float *)dev_opt(a[2], kF32, {d}, "ln_w"), *lb = (const float *)dev_opt(a[3], kF32, {d}, "ln_b");
+    const void *op = dev(o, st, "o"), *rp = dev(a[1], st, o.sizes(), "r", o);
+    const float *lw = (const float *)dev_opt(a[2], kF32, {d}, "ln_w", o), *lb = (const float *)dev_opt(a[3], kF32, {d}, "ln_b", o);
     const float eps = real(a[4]);
     Tensor z = empty(o.sizes(), out_storage(dtype), o);
     void *zp = z.data_ptr(), *s = stream();
@@ -414,8 +424,8 @@ PyObject *outgate_bwd(PyObject *const *a)
     rows_of(o, d, rows);
     const int dtype = dtype_of(o, truth(a[7]));
     const ScalarType st = storage(dtype);
-    const void *op = dev(o, st, "o"), *rp = dev(a[1], st, o.sizes(), "r"), *zp = dev(a[2], st, o.sizes(), "dz");
-    const float *lw = (const float *)dev_opt(a[3], kF32, {d}, "ln_w"), *lb = (const float *)dev_opt(a[4], kF32, {d}, "ln_b");
+    const void *op = dev(o, st, "o"), *rp = dev(a[1], st, o.sizes(), "r", o), *zp = dev(a[2], st, o.sizes(), "dz", o);
+    const float *lw = (const float *)dev_opt(a[3], kF32, {d}, "ln_w", o), *lb = (const float *)dev_opt(a[4], kF32, {d}, "ln_b", o);
     const float eps = real(a[5]);
     Tensor d_o = empty(o.sizes(), out_storage(dtype), o), d_r = empty(o.sizes(), out_storage(dtype), o), dw, db;
     Ws w;
@@ -442,8 +452,8 @@ PyObject *dwconv(PyObject *const *a)
     const int dtype = dtype_of(x, truth(a[6]));
     const ScalarType st = storage(dtype), ost = out_storage(dtype);
     Tensor y = given(a[7], x.sizes(), ost, x, "y");
-    const void *xp = dev(x, st, "x"), *wp = dev(a[1], st, {3, 3, D}, "w"), *bp = dev_opt(a[2], st, {D}, "bias");
-    void *yp = dev(y, ost, x.sizes(), "y"), *s = stream();
+    const void *xp = dev(x, st, "x"), *wp = dev(a[1], st, {3, 3, D}, "w", x), *bp = dev_opt(a[2], st, {D}, "bias", x);
+    void *yp = dev(y, ost, x.sizes(), "y", x), *s = stream();
     const int B = (int)x.size(0);
     CALL(dig_srem_dwconv(xp, wp, bp, yp, B, gh, gw, (int)D, dir, dtype, s), "dig_srem_dwconv");
     return wrap(y);
@@ -460,7 +470,7 @@ PyObject *dwconv_bwd(PyObject *const *a)
     const ScalarType st = storage(dtype);
     const size_t need = dig_srem_dwconv_bwd_workspace_bytes(B, gh, gw, (int)D);
     if (need == 0) raise(PyExc_ValueError, "dig_srem_dwconv_bwd: unsupported sizes");
-    const void *xp = dev(x, st, "x"), *wp = dev(a[1], st, {3, 3, D}, "w"), *gp = dev(a[2], st, x.sizes(), "dy");
+    const void *xp = dev(x, st, "x"), *wp = dev(a[1], st, {3, 3, D}, "w", x), *gp = dev(a[2], st, x.sizes(), "dy", x);
     if (!none(a[8])) dev(tensor(a[8], "workspace"), kByte, "workspace");
     const Ws w = workspace(a[8], need, x);
     Tensor dx = empty(x.sizes(), out_storage(dtype), x), dw = empty({3, 3, D}, kF32, x), db;
