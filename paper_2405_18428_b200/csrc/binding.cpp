@@ -195,7 +195,6 @@ PyObject *gate_logsigmoid(PyObject *const *a)
     const Tensor &g = tensor(a[0], "g");
     if (g.dim() != 4) raise(PyExc_ValueError, "g: need 4 dimensions [B, L, H, d_k], got shape " + text(g.sizes()));
     const int B = (int)g.size(0), L = (int)g.size(1), H = (int)g.size(2), dk = (int)g.size(3), dtype = dtype_of(g, false);
-    Tensor gate = given(a[2], g.sizes(), kF32, g, "gate");
     PyObject *seq = PySequence_Fast(a[1], "tau_per_head: need a sequence of numbers");
     if (!seq) throw Raised{};
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
@@ -210,6 +209,7 @@ PyObject *gate_logsigmoid(PyObject *const *a)
     Py_DECREF(seq);
     if (bad) throw Raised{};
     void *gp = dev(g, storage(dtype), "g");
+    Tensor gate = given(a[2], g.sizes(), kF32, g, "gate");
     float *op = (float *)dev(gate, kF32, g.sizes(), "gate", g);
     void *s = stream();
     CALL(dig_gate_logsigmoid(gp, tau.data(), op, B, L, H, dk, dtype, s), "dig_gate_logsigmoid");
@@ -451,8 +451,8 @@ PyObject *dwconv(PyObject *const *a)
     if (x.size(1) != (int64_t)gh * gw) raise(PyExc_ValueError, "x: L != grid_h*grid_w");
     const int dtype = dtype_of(x, truth(a[6]));
     const ScalarType st = storage(dtype), ost = out_storage(dtype);
-    Tensor y = given(a[7], x.sizes(), ost, x, "y");
     const void *xp = dev(x, st, "x"), *wp = dev(a[1], st, {3, 3, D}, "w", x), *bp = dev_opt(a[2], st, {D}, "bias", x);
+    Tensor y = given(a[7], x.sizes(), ost, x, "y");
     void *yp = dev(y, ost, x.sizes(), "y", x), *s = stream();
     const int B = (int)x.size(0);
     CALL(dig_srem_dwconv(xp, wp, bp, yp, B, gh, gw, (int)D, dir, dtype, s), "dig_srem_dwconv");

@@ -24,3 +24,11 @@ def test_cpu_tensors_and_wrong_types_are_rejected(dig):
         dig.dig_srem_dwconv(torch.zeros(1, 4, 8), t, None, 3, 3)
     with pytest.raises(IndexError):
         dig.dig_gate_logsigmoid(t, [16.0, 16.0], t)
+
+
+def test_cpu_tensors_are_value_errors_where_the_result_is_not_given(dig):
+    """The check comes before the result is allocated on the input's device."""
+    with pytest.raises(ValueError, match="g: need a contiguous CUDA tensor"):
+        dig.dig_gate_logsigmoid(torch.zeros(1, 4, 1, 64), [16.0])
+    with pytest.raises(ValueError, match="x: need a contiguous CUDA tensor"):
+        dig.dig_srem_dwconv(torch.zeros(1, 4, 8), torch.zeros(3, 3, 8), None, 2, 2)
