@@ -351,6 +351,9 @@ struct StripCut {
     }
 };
 
+// What both directions take: the grid of the one-tile kernel, which serves small problems and bounds them all.
+bool sizes_served(int B, int gh, int nchb) { return (gh + TY - 1) / TY <= 65535 && (size_t)B * nchb <= 65535; }
+
 template <bool BWD>
 dig_status launch_strip(const void *src, const void *w, const void *bias, void *dst, const void *x, float *partial, int B, int gh,
                         int gw, int D, int dir, int dtype, dim3 grid, StripCut cut, int nstrips, cudaStream_t stream)
@@ -379,7 +382,7 @@ dig_status launch_dwconv(const void *x, const void *w, const void *bias, void *y
     const int CH = dtype == DIG_F32 ? Cfg<float>::CH : Cfg<__nv_bfloat16>::CH;
     const int nchb = (D + CH - 1) / CH;
     const dim3 grid((gw + TX - 1) / TX, (gh + TY - 1) / TY, B * nchb);
-    if (grid.y > 65535 || (size_t)B * nchb > 65535) return DIG_ERR_UNSUPPORTED;
+    if (!sizes_served(B, gh, nchb)) return DIG_ERR_UNSUPPORTED;
     KernelTimer t(KID_DWCONV, stream);
     // grids with at least one tile per resident CTA: strips of TX columns walked row by row, cut into row
     // segments so that as many CTAs as stay resident have work
@@ -426,7 +429,9 @@ dig_status launch_dwconv_bwd(const void *x, const void *w, const void *dy, void 
     // One partial sum per CTA row.  No more CTA rows than stay resident together so that their strip loops end together, never more than the workspace holds;
     // strips are cut into row segments until every CTA row has one.
     const int CHb = dtype == DIG_F32 ? Cfg<float>::CH : Cfg<__nv_bfloat16>::CH;
-    const int nchb = (D + CHb - 1) / CHb, resident = device_sm_count() * kStripCtas;
+    const int nchb = (D + CHb - 1) / CHb;
+    if (!sizes_served(B, gh, nchb)) return DIG_ERR_UNSUPPORTED;
+    const int resident = device_sm_count() * kStripCtas;
     if (resident <= 0) return DIG_ERR_CUDA;
     const long long npix = (long long)B * gh * gw;
     long long nslab = (npix + kWgPixels - 1) / kWgPixels;

@@ -85,6 +85,14 @@ def test_bad_arguments_are_rejected_on_the_host(L):
     assert L.dig_gate_logsigmoid(ok, None, ok, 1, 4, 2, 8, 0, None) == dig.DIG_ERR_INVALID_ARG
 
 
+def test_conv_reverse_mode_refuses_what_the_forward_call_refuses(L):
+    from paper_2405_18428_b200 import dig
+    ok = 0x1000
+    for B, gh, gw, D in [(70000, 8, 8, 64), (1, 4 * 65536, 1, 64), (22000, 4, 4, 512)]:       # sequences x channel blocks, grid rows
+        assert L.dig_srem_dwconv(ok, ok, None, ok, B, gh, gw, D, 0, dig.DIG_BF16, None) == dig.DIG_ERR_UNSUPPORTED
+        assert L.dig_srem_dwconv_bwd(ok, ok, ok, ok, ok, None, B, gh, gw, D, 0, dig.DIG_BF16, ok, 1 << 40, None) == dig.DIG_ERR_UNSUPPORTED
+
+
 def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     from paper_2405_18428_b200 import dig
     monkeypatch.setattr(dig, "_lib", None)
