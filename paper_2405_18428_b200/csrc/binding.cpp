@@ -58,6 +58,13 @@ int integer(PyObject *o)
     if (v < INT_MIN || v > INT_MAX) raise(PyExc_OverflowError, "integer argument out of range");
     return (int)v;
 }
+// A set of scan orders, one bit each, of which the library takes the lowest four and refuses the others up to 32.
+unsigned order_mask(PyObject *o)
+{
+    const unsigned long v = PyLong_AsUnsignedLongMask(o);
+    if (v == (unsigned long)-1 && PyErr_Occurred()) throw Raised{};
+    return (unsigned)v;
+}
 bool truth(PyObject *o)
 {
     const int v = PyObject_IsTrue(o);
@@ -316,7 +323,7 @@ PyObject *gla_bwd_state(PyObject *const *a)
 PyObject *gla_fwd_multi(PyObject *const *a)
 {
     const Gla g(a, a[4], a[5], a[7], truth(a[8]));
-    const unsigned mask = (unsigned)integer(a[6]);
+    const unsigned mask = order_mask(a[6]);
     Tensor out = given(a[9], g.vs, g.ost, g.q_t, "out");
     void *op = dev(out, g.ost, g.vs, "out", g.q_t);
     const Ws w = workspace(a[10], none(a[10]) ? dig_gla_multi_workspace_bytes(g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, g.dtype, 0) : 0, g.q_t);
@@ -329,7 +336,7 @@ PyObject *gla_fwd_multi(PyObject *const *a)
 PyObject *gla_bwd_multi(PyObject *const *a)
 {
     const Gla g(a, a[5], a[6], a[8], truth(a[9]));
-    const unsigned mask = (unsigned)integer(a[7]);
+    const unsigned mask = order_mask(a[7]);
     void *dop = dev(a[4], g.st, g.vs, "d_out", g.q_t);
     const Grads r(a[10], g);
     const Ws w = workspace(a[11], none(a[11]) ? dig_gla_multi_workspace_bytes(g.B, g.H, g.gh, g.gw, g.dk, g.dv, g.chunk, g.dtype, 1) : 0, g.q_t);

@@ -1,4 +1,5 @@
-"""The compiled binding checks the scratch memory it is given before any kernel is launched on it."""
+"""What the compiled binding hands to the library: scratch memory is checked before any kernel is launched on it, sets of
+scan orders keep their bits."""
 import pytest
 import torch
 
@@ -41,3 +42,14 @@ def test_workspace_has_to_be_dense_device_memory(call):
     flat = lambda r: [x for x in (r if isinstance(r, tuple) else (r,)) if x is not None]
     for a, b in zip(flat(f()), flat(f(workspace=torch.empty(n, dtype=torch.uint8, device="cuda")))):
         assert torch.equal(a, b)
+
+
+def test_scan_orders_beyond_the_four_are_the_librarys_refusal():
+    from paper_2405_18428_b200 import dig
+    q = torch.randn(1, 64, 1, 64, device="cuda").to(torch.bfloat16)
+    gate = torch.full(q.shape, -0.05, device="cuda")
+    for orders in ([4], [0, 31], []):
+        for f in (lambda: dig.dig_gla_fwd_multi(q, q, q, gate, 8, 8, orders), lambda: dig.dig_gla_bwd_multi(q, q, q, gate, q, 8, 8, orders)):
+            with pytest.raises(dig.DigError) as e:
+                f()
+            assert e.value.status == dig.DIG_ERR_INVALID_ARG
