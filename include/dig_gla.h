@@ -132,8 +132,9 @@ dig_status dig_gla_fwd_static(const void *q, const void *k, const void *v, const
  * (reverse-mode derivative of Eq. attn_gla; the paper trains through the operator but does not
  * print it).  Nothing is saved by the forward call: chunk states are recomputed here.
  *   d_out: [B][L][H][d_v]; dq, dk: [B][L][H][d_k]; dv: [B][L][H][d_v]; dgate: fp32 [B][L][H][d_k].
- * The fp32-FMA and warp-level families cover chunk <= 64 here (shared memory); chunk = 128 is served by
- * the tcgen05 family only (bf16 storage, d_k = d_v = 64 or 72, 64-token tiles). */
+ * The fp32-FMA and warp-level families cover what fits their shared memory here: chunk = 128 with small
+ * heads only (dig_gla_query_impl tells); the tcgen05 family serves it for d_k = d_v = 64 or 72 (bf16
+ * storage, 64-token tiles). */
 dig_status dig_gla_bwd(const void *q, const void *k, const void *v, const float *gate,
                        const void *d_out, void *dq, void *dk, void *dv, float *dgate,
                        int B, int H, int grid_h, int grid_w, int d_k, int d_v, int chunk,
@@ -173,7 +174,10 @@ dig_status dig_srem_dwconv_bwd(const void *x, const void *w, const void *dy, voi
  * The paper does not fix LN further; here it normalises each (token, head) row over its d_v values
  * (biased variance, `eps` added under the root) and applies an optional affine part shared by all
  * heads: ln_w, ln_b are fp32 [d_v] device arrays or NULL (weight 1 / bias 0).
- * d_v: a multiple of 8, at most 128.  fp32 arithmetic. */
+ * d_v: a multiple of 8, at most 128.  fp32 arithmetic.
+ * This kernel and its reverse mode wait for bulk copies, for at most 0.25 s: where such a wait expires, the rows
+ * after it stay unwritten and dig_last_device_status returns DIG_ERR_TIMEOUT (the call itself has returned
+ * DIG_OK by then, as with the tcgen05 kernels). */
 dig_status dig_gla_outgate_fwd(const void *o, const void *r, const float *ln_w, const float *ln_b, void *z,
                                long long rows, int d_v, float eps, int dtype, void *cuda_stream);
 

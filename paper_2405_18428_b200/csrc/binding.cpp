@@ -1,8 +1,8 @@
 // CPython module over the C ABI (include/dig_gla.h) for torch CUDA tensors: checks, allocation of results and
-// workspace, the current stream and the call, without a line of Python in between.  The same work through
-// ctypes took 10 to 20 us of host time per call (3.4 us of it to ask for the current stream, 2.6 us per
-// allocation, 0.6 us per checked tensor), more than the small problems take on the GPU; here it is about 2 us
-// beside the launches.  dig.py holds the documented functions, which hand their arguments over by position.
+// workspace, the current stream and the call, without a line of Python in between.  Through ctypes a call of one
+// launch took 14 to 19 us of host time (3.4 us of it to ask for the current stream, 2.6 us per allocation, 0.6 us
+// per checked tensor), more than the small problems take on the GPU; here it takes 4 to 5 us, the launch
+// included.  dig.py holds the documented functions, which hand their arguments over by position.
 // The interpreter lock is released around every library call.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>

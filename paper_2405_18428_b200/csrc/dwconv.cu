@@ -339,7 +339,8 @@ srem_dwconv_wgrad_sum(const float *__restrict__ partial, float *__restrict__ dw,
     else if (dbias != nullptr) dbias[idx - 9 * D] = sum;
 }
 
-// Rows of a strip cut into nseg segments of seg_rows, at least 8 rows each (two halo rows come on top).
+// Rows of a strip cut evenly into at most one segment per 8 rows (two halo rows come on top): 9 rows become 5 + 4, and the
+// last segment may be short (65 rows: eight of 8 and one of 1).
 struct StripCut {
     int nseg, seg_rows;
     StripCut(int want, int gh)

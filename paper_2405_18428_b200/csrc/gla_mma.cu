@@ -1,7 +1,7 @@
 // Warp-MMA kernel family for chunkwise gated linear attention (Eq. attn_gla, evaluated chunk by chunk
-// as Section 3.5 describes): serves bf16 requests whose head size or chunk size the tcgen05 family
-// does not cover (any d_k, d_v that is a multiple of 8 up to 128, chunks of 16, 32, 64 or 128 tokens
-// as far as shared memory allows), e.g. the 72-wide heads of the largest model.  Same decomposition
+// as Section 3.5 describes): serves bf16 requests whose head sizes the tcgen05 family does not cover (any
+// d_k, d_v that is a multiple of 8 up to 128, chunks of 16, 32, 64 or 128 tokens as far as shared memory
+// allows) and the full gate.  Same decomposition
 // as the other families: per-chunk state contributions, a scan over the chunks, then one CTA per
 // (chunk, batch*head) for the outputs or the gradients.  Every contraction runs on the tensor cores
 // through mma.sync.m16n8k8 (tf32 operands, fp32 accumulation) with fragments read straight from
@@ -888,8 +888,8 @@ dig_status bwd_dims(const GlaArgs &a)
 }
 
 // Head sizes and chunks of the paper's models get kernels with compile-time sizes (6 heads of 64, 8 x 1024 tokens in
-// chunks of 32 with the full gate: 546 -> 225 us; 4 x 1024 tokens in fp32: 249 -> 141); 64-wide heads in 64-token chunks without the full gate are the tcgen05
-// family's.
+// chunks of 32 with the full gate: 546 -> 225 us; 4 x 1024 tokens in fp32: 249 -> 141).  Without the full gate these heads
+// are the tcgen05 family's: the two instances kept there serve calls that force this family.
 template <bool BETA, typename F>
 dig_status with_dims(const Geom &g, F f)
 {

@@ -555,7 +555,7 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
 // sweep_fwd: a segment from its entry state; writes out.
 // Bound by the latency of its phases (three barriers and two waits for products per tile; IPC 1.5, two CTAs per
 // SM).  16 sequences of 16384 tokens, d = 72: 114 us with the row-chunk work split, 76 us now; 768 of 256, d = 64
-// (uncut): 60 -> 48 us; 48 of 4096: 62 -> 51.  Three CTAs per SM on 80 registers: 72 us against 59 us on 48 sequences of 4096 tokens, d = 64.
+// (uncut): 60 -> 48 us; 48 of 4096: 62 -> 51.  Three CTAs per SM on 80 registers spill: 72 us there.
 // =================================================================================================
 template <int D, typename TO>
 struct FwdSmem {

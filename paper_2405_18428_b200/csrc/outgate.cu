@@ -15,6 +15,8 @@
 // 72-value row share sectors, which the L1 loses when more CTAs are resident).
 // The affine gradients are summed per CTA in registers and shared memory and then across CTAs by a second
 // kernel in a fixed order.
+// The waits for the copies are bounded like those of the sweep kernels: where one expires the rows after it stay unwritten
+// and the device status word says so.
 #include <type_traits>
 
 #include "dig_common.cuh"

@@ -127,7 +127,7 @@ __device__ __forceinline__ uint64_t mdesc(uint32_t saddr, uint32_t ch) { return 
 template <int M, int N, bool A_MN, bool B_MN, int KSTEPS, uint32_t ACH, uint32_t BCH, uint32_t BSBO = 128>
 __device__ __forceinline__ void issue(uint32_t d_tmem, uint32_t a, uint32_t b, bool accumulate)
 {
-    static_assert((M == 64 && N % 8 == 0) || (M == 128 && N % 16 == 0), "instruction shape");
+    static_assert(M == 64 && N % 8 == 0, "instruction shape");
     constexpr uint32_t idesc = idesc_f16(M, N, A_MN, B_MN);
     const uint64_t da = A_MN ? mdesc(a, ACH) : kdesc(a, ACH), db = B_MN ? mdesc(b, BCH) : make_desc(b, BCH, BSBO, 0);
     constexpr uint32_t sa = A_MN ? 16u : (2u * ACH) >> 4, sb = B_MN ? 16u : (2u * BCH) >> 4;

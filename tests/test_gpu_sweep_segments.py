@@ -1,5 +1,7 @@
 """GPU parity of the sweep kernels where sequences are cut into segments of several tiles: the local sweeps
-accumulate over a segment, the last tile of the last segment is ragged, sub-chunks divide its tiles."""
+accumulate over a segment, the last tile of the last segment is ragged, sub-chunks divide its tiles.  The tests that need
+both passes cut assert the cut; in test_segments_of_several_tiles (99 to 108 sequences of 9 or 10 tiles) only the
+backward pass is."""
 import numpy as np
 import pytest
 import torch
