@@ -95,11 +95,9 @@ __device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, int *st
 // =================================================================================================
 // sweep_local_fwd: the state a segment leaves from a zero start, and its total decay.  The tiles are walked from the
 // segment's end, so the decay from a tile's centre to the end is known when its product is: the state is the plain
-// sum of 2^(that decay) (Kc^T V), kept in tensor memory.  A tile is divided only where its gates ask for it: shorter
-// chunks give the same errors here (2.1e-4 of RMS, root mean square, with chunks of 16, 32 or 64).  One barrier per
-// tile: behind it lie the group sums of this tile and the operand rows of the one before, whose product is issued there
-// and added one step later; operand tiles, accumulators and sums have two buffers, and the rows of the next tile are
-// loaded a whole tile ahead.
+// sum of 2^(that decay) (Kc^T V), kept in tensor memory.  One barrier per tile or sub-chunk: behind it lie the group sums of
+// this tile and the operand rows of the step before, whose product is issued there and added one step later; operand
+// tiles, accumulators and sums have two buffers, and the rows of the next tile are loaded a whole tile ahead.
 // Bound by the latency of its phases.  48 sequences of 4096 tokens, d = 64: 40 us with the state in registers, decayed
 // once per tile in scan order, 33 us now; 16 of 16384, d = 72: 80 -> 54 us (63 with the sum in registers, which spills).
 // One operand exponent for the whole way to the segment's end would let the matrix unit add the products up (29 and
@@ -200,8 +198,8 @@ sweep_local_fwd(const SweepArgs a)
             const Tot whole = tile_totals<D>(tot, w);
             Tot tt = whole;
             int s = T;
-            if (beyond<D>(tt)) {
-                s = choose_window<D>(tot, w, T / 2, a.status);
+            if (pl.sub_max < T || beyond<D>(tt)) {
+                s = choose_window<D>(tot, w, min(pl.sub_max, T / 2), a.status);
                 const int w0 = 8 * w.grp / s * (s / 8);
                 tt = window_totals<D>(tot, w, w0, w0 + s / 8);
             }

@@ -85,3 +85,14 @@ def test_both_passes_cut_into_segments_of_several_tiles(d, grid, B, H, chunk, ta
     wl = Workload("cut", B=B, H=H, grid_h=grid[0], grid_w=grid[1], d_k=d, d_v=d, chunk=chunk, dtype="bf16", backward=True,
                   tau=tau, seed=64)
     print(check_workload(wl, direction))
+
+
+@pytest.mark.parametrize("d,chunk", [(64, 16), (72, 32)])
+def test_short_chunks_keep_large_operands_in_range_in_every_kernel(d, chunk):
+    """Keys of size 30 times half of a 64-token tile's decay (up to 2^11.5) would saturate in fp16; chunks of 16 or 32 tokens,
+    which the caller asked for, keep them in range in the local sweeps too."""
+    wl = Workload("large", B=2, H=2, grid_h=41, grid_w=32, d_k=d, d_v=d, chunk=chunk, dtype="bf16", backward=True, tau=(4.0,), seed=65)
+    assert sweep_plan(4, 21, False)[0] > 1
+    x = make_inputs(wl, conv=False)
+    x["k"] = torch.from_numpy(x["k"] * np.float32(30)).to(torch.bfloat16).float().numpy()
+    print(check_workload(wl, 3, x=x))
