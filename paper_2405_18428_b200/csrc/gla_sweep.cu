@@ -1083,10 +1083,23 @@ SweepWs carve(char *base, const Geom &g, const Plan &pl, bool backward)
     return w;
 }
 
-// Segment length.  A pass costs (tiles of a segment + one of fill and drain) per round of resident CTAs.
-// Uncut sequences (one segment each) run the forward sweep alone; cut ones also run the local sweep, about
-// half of a forward sweep per tile, and the scan, and these two launches take about as long as three tiles
-// of a forward sweep when the machine is not full.  The backward pass needs the local sweep in either case.
+// Segment length.  Cost of a pass in 0.1 us, fitted to 1086 measured cuts of 2 to 768 sequences of 2 to 32 tiles, chunks of 16,
+// 32 and 64, d = 64 and 72 (root mean square of the fit's error 3 to 5%): launches, a fill per round of CTAs, tiles, and the
+// scan.  An SM with one CTA works a tile in two thirds of the time that two sharing it take.  Uncut sequences run the forward
+// sweep alone; cut ones also the local sweep and the scan; the backward pass needs the local sweep in either case.  Sub-chunks
+// multiply the tiles' cost, so short sequences in short chunks are cut where whole tiles would not be (3 tiles of 6
+// sequences, d = 64, chunks of 16: 24.4 us uncut, 18.7 cut; chunks of 64: 9.1 uncut).  A cut has to win by 2 us (backward: 1),
+// which its launches cost the host where nothing else keeps the device busy (a 256-token image: 19.2 us per block uncut, 22.6
+// cut, although the device is 0.6 us faster).  The cut chosen is within 19% of the best one, 0.3% off on average; a model of
+// rounds and tiles alone was 6% off on average and up to 2.2 times (5 tiles of 2 sequences, d = 72, chunks of 16: 53.6 us
+// uncut, 24.1 cut).
+struct PassCost {
+    int fixed[2], round[2], pair[2], alone[2];      // [cut]; pair: a tile on an SM with two CTAs, alone: with one
+    int scan;                                       // per machine full of segments
+    int chunk32, chunk16, d72;                      // factors of a tile's cost, per cent
+};
+constexpr PassCost kForward = {{21, 75}, {5, 8}, {32, 51}, {22, 37}, 35, 190, 310, 140};
+constexpr PassCost kBackward = {{14, 54}, {32, 23}, {88, 95}, {62, 73}, 67, 170, 280, 150};
 // Chunks above 64 tokens: forward plans stay within the scratch of dig_gla_fwd_static where uncut sequences do (the
 // same plan serves dig_gla_fwd, so that both give the same bits).  No other family's workspace is counted there that
 // would be larger anyway; with chunks of up to 64 the per-chunk states of the other families always are.
@@ -1096,14 +1109,18 @@ Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
     p.ntile = (g.L + T - 1) / T;
     p.sub_max = g.C < T ? g.C : T;
     p.gh_inv = g.gh > 1 ? (uint32_t)((1ull << 32) / (unsigned)g.gh) : 0xffffffffu;
+    const PassCost &c = backward ? kBackward : kForward;
     const long long slots = (long long)sms * per_sm, bh = (long long)g.B * g.H;
+    const long long tile = (p.sub_max == 16 ? c.chunk16 : p.sub_max == 32 ? c.chunk32 : 100) * (g.dk == 72 ? c.d72 : 100) / 100;      // per cent
     long long best = -1;
     p.G = p.ntile;
     // the shortest G of every number of segments that occurs (about 2 sqrt(ntile) of them)
     for (int nseg = 1, G = p.ntile;; nseg = (p.ntile + G - 2) / (G - 1), G = (p.ntile + nseg - 1) / nseg) {
-        const long long rounds = (bh * nseg + slots - 1) / slots;
-        long long cost = rounds * (G + 1) * 10;             // a segment costs about one tile of fill and drain
-        if (nseg > 1) cost += backward ? 15 : cost / 2 + 30;
+        const long long segs = bh * nseg, rest = segs % slots;
+        const long long pairs = segs / slots + (rest > sms), alone = rest > 0 && rest <= sms;          // rounds of either kind
+        const int cut = nseg > 1;
+        const long long cost = 100 * (c.fixed[cut] + (pairs + alone) * c.round[cut]) + tile * G * (pairs * c.pair[cut] + alone * c.alone[cut]) +
+                               (cut ? 100 * c.scan * segs / slots : 0);
         p.nseg = nseg;
         const bool fits = backward || g.C <= T || nseg == 1 || carve(nullptr, g, p, false).bytes <= DIG_GLA_STATIC_SCRATCH_BYTES;
         if (best < 0 || (cost < best && fits)) {

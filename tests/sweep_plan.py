@@ -9,15 +9,25 @@ def segment_bytes(segments: int, d: int) -> int:
     return up(segments * d * d * 4) + up(segments * d * 4)
 
 
-def sweep_plan(sequences: int, ntile: int, backward: bool, limit: tuple[int, int] | None = None) -> tuple[int, int]:
-    """(segments per sequence, tiles per segment); limit = (bytes, head size) for forward passes in chunks above 64."""
-    slots, best, best_g = 148 * 2, None, ntile
+# per pass: launches, fill per round, a tile beside another CTA, a tile alone (each uncut, cut), scan; per cent for
+# chunks of 32 and 16 and for d = 72
+FORWARD = ((21, 75), (5, 8), (32, 51), (22, 37), 35, {32: 190, 16: 310}, 140)
+BACKWARD = ((14, 54), (32, 23), (88, 95), (62, 73), 67, {32: 170, 16: 280}, 150)
+
+
+def sweep_plan(sequences: int, ntile: int, backward: bool, chunk: int = 64, d: int = 64, limit: int | None = None) -> tuple[int, int]:
+    """(segments per sequence, tiles per segment); limit: bytes that forward passes in chunks above 64 keep to."""
+    fixed, fill, pair, alone, scan, sub, d72 = BACKWARD if backward else FORWARD
+    tile = sub.get(chunk, 100) * (d72 if d == 72 else 100) // 100
+    sms, best, best_g = 148, None, ntile
     nseg, g = 1, ntile
     while True:
-        cost = -(-sequences * nseg // slots) * (g + 1) * 10
-        if nseg > 1:
-            cost += 15 if backward else cost // 2 + 30
-        fits = limit is None or nseg == 1 or segment_bytes(sequences * nseg, limit[1]) <= limit[0]
+        segs, cut = sequences * nseg, int(nseg > 1)
+        rounds, rest = divmod(segs, 2 * sms)
+        pairs, single = rounds + (rest > sms), int(0 < rest <= sms)
+        cost = 100 * (fixed[cut] + (pairs + single) * fill[cut]) + tile * g * (pairs * pair[cut] + single * alone[cut])
+        cost += 100 * scan * segs // (2 * sms) if cut else 0
+        fits = backward or chunk <= 64 or nseg == 1 or limit is None or segment_bytes(segs, d) <= limit
         if best is None or (cost < best and fits):
             best, best_g = cost, g
         if g == 1:

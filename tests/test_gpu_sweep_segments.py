@@ -46,7 +46,7 @@ def test_states_of_segments_keep_their_relative_precision(d, case):
     import oracle
     from paper_2405_18428_b200 import dig
     wl = Workload("prec", B=4, H=12, grid_h=25, grid_w=91, d_k=d, d_v=d, chunk=64, dtype="bf16", backward=True, tau=(16.0,), seed=63)
-    assert sweep_plan(48, 36, False) == sweep_plan(48, 36, True) == (6, 6) and -(-wl.L // 64) == 36
+    assert sweep_plan(48, 36, False, 64, d) == sweep_plan(48, 36, True, 64, d) == (6, 6) and -(-wl.L // 64) == 36
     x = make_inputs(wl, conv=False)
     if case == "small":
         for n in ("q", "k"):
@@ -80,7 +80,7 @@ def test_both_passes_cut_into_segments_of_several_tiles(d, grid, B, H, chunk, ta
     """(The gate gradient is a sum over all later tokens of products of 11-bit operands, so its error grows with the length:
     2.1e-2 of RMS for tau = 1 over 1953 tokens; hence tau = 2 on the longest.)"""
     for backward in (False, True):
-        nseg, g = sweep_plan(B * H, -(-grid[0] * grid[1] // 64), backward)
+        nseg, g = sweep_plan(B * H, -(-grid[0] * grid[1] // 64), backward, chunk, d)
         assert nseg > 1 and g > 1
     wl = Workload("cut", B=B, H=H, grid_h=grid[0], grid_w=grid[1], d_k=d, d_v=d, chunk=chunk, dtype="bf16", backward=True,
                   tau=tau, seed=64)
@@ -92,7 +92,23 @@ def test_short_chunks_keep_large_operands_in_range_in_every_kernel(d, chunk):
     """Keys of size 30 times half of a 64-token tile's decay (up to 2^11.5) would saturate in fp16; chunks of 16 or 32 tokens,
     which the caller asked for, keep them in range in the local sweeps too."""
     wl = Workload("large", B=2, H=2, grid_h=41, grid_w=32, d_k=d, d_v=d, chunk=chunk, dtype="bf16", backward=True, tau=(4.0,), seed=65)
-    assert sweep_plan(4, 21, False)[0] > 1
+    assert sweep_plan(4, 21, False, chunk, d)[0] > 1
     x = make_inputs(wl, conv=False)
     x["k"] = torch.from_numpy(x["k"] * np.float32(30)).to(torch.bfloat16).float().numpy()
     print(check_workload(wl, 3, x=x))
+
+
+@pytest.mark.parametrize("d", [64, 72])
+@pytest.mark.parametrize("chunk,tiles,cut", [(16, 3, True), (16, 5, True), (64, 2, False), (32, 5, True)])
+def test_short_sequences_are_cut_where_their_chunks_make_them_long(d, chunk, tiles, cut):
+    """The forward launches of 6 sequences: a sub-chunk costs most of a tile, the launches of a cut pass stay the same."""
+    from paper_2405_18428_b200 import dig
+    assert (sweep_plan(6, tiles, False, chunk, d)[0] > 1) == cut
+    q = torch.randn(1, 64 * tiles, 6, d, device="cuda").to(torch.bfloat16)
+    gate = torch.full(q.shape, -0.05, device="cuda")
+    dig.dig_profile_enable(True)
+    try:
+        dig.dig_gla_fwd(q, q, q, gate, 64, tiles, chunk, 0)
+        assert ("sweep_local" in dig.dig_profile_read()) == cut
+    finally:
+        dig.dig_profile_enable(False)

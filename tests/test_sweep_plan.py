@@ -20,7 +20,7 @@ def test_restated_plan_gives_the_librarys_workspace(dig, backward):
     """d = 72 in chunks of 128, which no other family serves: the sweep workspace alone counts."""
     d, up = 72, lambda x: -(-x // 256) * 256
     for bh, t in SHAPES:
-        nseg, _ = sweep_plan(bh, t, backward, None if backward else (dig.DIG_GLA_STATIC_SCRATCH_BYTES, d))
+        nseg, _ = sweep_plan(bh, t, backward, 128, d, dig.DIG_GLA_STATIC_SCRATCH_BYTES)
         segs, want = bh * nseg, segment_bytes(bh * nseg, d)
         if backward:
             want += up(segs * d * d * 4) + up(segs * d * 4) + up(segs * d * d * 2) + up(8 * bh * t * d * d * 2) + up(8 * bh * t * d * 4)
