@@ -96,6 +96,22 @@ def test_affine_parameters_written_by_the_kernel_in_front():
             assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("d", [40, 72, 96])
+def test_rows_far_from_zero_lose_only_what_the_reciprocal_of_their_length_loses(d):
+    """Rows of mean 0.5 and deviation 0.03 (sums of bf16 values, exact in fp32): the mean enters as sum * (1 / d) without a rounding
+    of its own, so z is off by the relative error of 1 / d in fp32 times mean / deviation, and by 9e-8 (RMS) of everything else.
+    A rounded mean adds 2^-25 * 0.5 / 0.03 or so."""
+    from paper_2405_18428_b200 import dig
+    rng = np.random.default_rng(9)
+    o = round_to_bf16((0.5 + 0.03 * rng.standard_normal((4099, d))).astype(np.float32))
+    r = round_to_bf16(rng.standard_normal((4099, d)).astype(np.float32))
+    ref = oracle.outgate(o, r, None, None, 1e-5)
+    dev = lambda a: torch.from_numpy(a).cuda().to(torch.bfloat16)
+    z = dig.dig_gla_outgate_fwd(dev(o), dev(r), None, None, 1e-5, f32_out=True).double().cpu().numpy()
+    err = np.sqrt(np.mean((z - ref) ** 2) / np.mean(ref ** 2))
+    assert err <= 1.2 * (abs(float(np.float32(1) / np.float32(d)) * d - 1) * 0.5 / 0.03 + 9e-8), err
+
+
 @pytest.mark.parametrize("cfg", ["C2", "C5"])
 def test_outgate_benchmark_shapes(cfg):
     wl = CONFIGS[cfg]
