@@ -1,18 +1,16 @@
 // Output gate of the GLA layer (Eq. attn_gla, the line that forms Y_t before the projection W_O):
 //     z = Swish(r) (.) LN(o)      per (token, head) row of d_v values,
 // and its reverse mode.  Elementwise plus two row reductions, so bandwidth-bound once the instruction count
-// allows it.  The rows are contiguous in memory: a CTA walks over tiles of as many rows as it holds, each
-// tensor's tile fetched by one bulk copy (two tiles in flight) and the results written by one, so no thread
-// spends instructions on global addresses and every line moves once, whatever the row length.
-// A row is held by LPR lanes with CPL neighbouring chunks of 8 values each.  bf16 rows: 4 lanes x 2 chunks up
-// to 64 values, 3 x 3 for 72 (ten rows per warp), 4 x 4 above: few lanes per row keep the shuffles of the row
-// sums (two per sum) small against the arithmetic, which is done on packed fp32 pairs.  fp32 rows, whose
-// chunks take twice the registers: one chunk per lane (8, 9 or 16 lanes).
-// 262144 rows of 72 in bf16: forward 30.0 us with nine lanes of one chunk, unpacked arithmetic and loads by
-// every thread, 21.2 us
-// now (5.3 TB/s); reverse 54.0 -> 33.4 us (5.7 TB/s); 196608 rows of 64: 17.5 -> 15.6 and 29.8 -> 25.2 us.
-// With loads by every thread and the split above: 23.0 / 42.5 and 14.7 / 26.4 us (the 48-byte pieces of a
-// 72-value row share sectors, which the L1 loses when more CTAs are resident).
+// allows it.  Two ways, by row length and storage type (Split, below):
+//   - Through shared memory.  The rows are contiguous in memory: a CTA walks over tiles of as many rows as it holds, each
+//     tensor's tile fetched by one bulk copy (two tiles in flight) and the results written by one, so no thread
+//     spends instructions on global addresses and every line moves once, whatever the row length.  A row is held by LPR
+//     lanes with CPL neighbouring chunks of 8 values each, 4 lanes x 2 chunks up to 64 values, 3 x 3 for 72 (ten rows
+//     per warp): few lanes per row keep the shuffles of the row sums small against the arithmetic.  What it is for are rows of 72:
+//     the 48-byte pieces that three lanes would load share sectors, which the L1 loses when more CTAs are resident.
+//   - Directly.  Every lane loads one chunk (8, 9 or 16 lanes a row).
+// 262144 rows of 72 in bf16: forward 30.0 us with nine lanes of one chunk, unpacked arithmetic and loads by every
+// thread, 18 us now (6.3 TB/s); reverse 54.5 -> 33.5 us (5.6 TB/s).
 // The affine gradients are summed per CTA in registers and shared memory and then across CTAs by a second
 // kernel in a fixed order.
 // The waits for the copies are bounded like those of the sweep kernels: where one expires the rows after it stay unwritten
@@ -63,6 +61,20 @@ __device__ __forceinline__ void store8(__nv_bfloat16 *p, const float2 *f)
     t = __float22bfloat162_rn(f[3]); u.w = *reinterpret_cast<uint32_t *>(&t);
     *reinterpret_cast<uint4 *>(p) = u;
 }
+
+// Arithmetic on pairs: packed instructions for bf16 rows, whose bound they are; one by one for fp32 rows, which the packed
+// form slows down (196608 rows of 64 without shared memory: 19 -> 16.5 us, reverse 33 -> 32; of 8 values 14 -> 11.7 and 27 -> 22).
+struct Packed {
+    static __device__ __forceinline__ float2 add(float2 a, float2 b) { return add2(a, b); }
+    static __device__ __forceinline__ float2 mul(float2 a, float2 b) { return mul2(a, b); }
+    static __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
+};
+struct Single {
+    static __device__ __forceinline__ float2 add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+    static __device__ __forceinline__ float2 mul(float2 a, float2 b) { return make_float2(a.x * b.x, a.y * b.y); }
+    static __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)); }
+};
+template <typename T> using OpsFor = std::conditional_t<sizeof(T) == 2, Packed, Single>;
 
 // Thread -> (row slot of the CTA, lane of the row's group): 32 / LPR rows per warp.
 template <int LPR, int THREADS>
@@ -126,7 +138,7 @@ __device__ __forceinline__ void load_row(Raw8<T> (&x)[CPL], const T *p, const LN
     }
 }
 // Normalised row n = (o - mean) * rstd (zero where the lane holds none).
-template <typename T, int LPR, int CPL, int THREADS, bool FULL>
+template <typename V, typename T, int LPR, int CPL, int THREADS, bool FULL>
 __device__ __forceinline__ float normalise(const Raw8<T> (&o)[CPL], const Lane<LPR, CPL, THREADS, FULL> &ln, float inv_d, float eps, float2 (&n)[4 * CPL])
 {
     float2 s = make_float2(0.f, 0.f);
@@ -135,7 +147,7 @@ __device__ __forceinline__ float normalise(const Raw8<T> (&o)[CPL], const Lane<L
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             n[4 * i + j] = o[i].pair(j);
-            s = add2(s, n[4 * i + j]);
+            s = V::add(s, n[4 * i + j]);
         }
     // minus the mean as sum * (1 / d) inside a fused multiply-add: rounded on its own it costs rows far from zero (mean 16
     // deviations) three times the error
@@ -147,27 +159,28 @@ __device__ __forceinline__ float normalise(const Raw8<T> (&o)[CPL], const Lane<L
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             float2 &x = n[4 * i + j];
-            x = fma2(minus, scale, x);
+            x = V::fma(minus, scale, x);
             if (!FULL && !ln.has_col(i)) x = make_float2(0.f, 0.f);
-            v = fma2(x, x, v);
+            v = V::fma(x, x, v);
         }
     // slots past the last row hold zeros: with eps = 0 their 1/0 must not become 0 * inf in the affine gradients
     const float var = group_sum(v.x + v.y, ln.m) * inv_d;
     const float rstd = ln.row_ok ? rsqrtf(var + eps) : 0.f;
     const float2 sc = make_float2(rstd, rstd);
 #pragma unroll
-    for (int i = 0; i < 4 * CPL; ++i) n[i] = mul2(n[i], sc);
+    for (int i = 0; i < 4 * CPL; ++i) n[i] = V::mul(n[i], sc);
     return rstd;
 }
 
 // 1 / (1 + e^-r) with the fast exponential and the fast reciprocal (2 ulp each; e^-r = inf gives 0)
+template <typename V>
 __device__ __forceinline__ float2 sigmoid2(float2 r)
 {
-    const float2 t = mul2(r, make_float2(-1.4426950408889634f, -1.4426950408889634f));
+    const float2 t = V::mul(r, make_float2(-1.4426950408889634f, -1.4426950408889634f));
     float2 e;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(t.x));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(t.y));
-    e = add2(e, make_float2(1.f, 1.f));
+    e = V::add(e, make_float2(1.f, 1.f));
     return make_float2(__fdividef(1.f, e.x), __fdividef(1.f, e.y));
 }
 
@@ -297,7 +310,7 @@ outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const floa
         load_row(ov, reinterpret_cast<const TA *>(ring.in_buf(0, it)) + ln.m.slot * dv, ln);
         load_row(rv, reinterpret_cast<const TR *>(ring.in_buf(1, it)) + ln.m.slot * dv, ln);
         float2 n[4 * CPL];
-        normalise(ov, ln, inv_d, eps, n);
+        normalise<Packed>(ov, ln, inv_d, eps, n);
         TZ *zb = reinterpret_cast<TZ *>(ring.out_buf(0, it)) + ln.m.slot * dv;
 #pragma unroll
         for (int i = 0; i < CPL; ++i) {
@@ -307,7 +320,7 @@ outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const floa
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float2 x = rv[i].pair(j);
-                out[j] = mul2(mul2(x, sigmoid2(x)), fma2(n[4 * i + j], w[j], b[j]));
+                out[j] = mul2(mul2(x, sigmoid2<Packed>(x)), fma2(n[4 * i + j], w[j], b[j]));
             }
             if (ln.ok(i)) store8(zb + ln.col(i), out);
         }
@@ -316,6 +329,61 @@ outgate_fwd(const TA *o, const TR *r, const float *__restrict__ ln_w, const floa
     }
     pdl_launch_dependents();
     ring.drain(it, ok);
+}
+
+// What the reverse mode keeps of a row: with n the normalised row, dy = dz Swish(r), dn = dy w,
+//   dr = dz y Swish'(r),   do = rstd (dn - mean(dn) - n mean(dn n)),   dw += dy n,   db += dy.
+template <typename V, int CPL>
+struct RowGrad {
+    float2 n[4 * CPL], dn[4 * CPL], s1, s2;
+    float rstd, m1, m2;
+    __device__ __forceinline__ void start(float rstd_)
+    {
+        rstd = rstd_;
+        s1 = s2 = make_float2(0.f, 0.f);
+    }
+    template <typename T>
+    __device__ __forceinline__ void chunk(int i, const Raw8<T> &rv, const Raw8<T> &gv, const float2 (&w)[4], const float2 (&b)[4], float2 (&aw)[4 * CPL],
+                                          float2 (&ab)[4 * CPL], float2 (&dr)[4])
+    {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int e = 4 * i + j;
+            const float2 x = rv.pair(j), g = gv.pair(j), sg = sigmoid2<V>(x), sw = V::mul(x, sg);
+            const float2 y = V::fma(n[e], w[j], b[j]), dy = V::mul(g, sw);
+            dr[j] = V::mul(V::mul(g, y), V::fma(sw, V::fma(sg, make_float2(-1.f, -1.f), make_float2(1.f, 1.f)), sg));
+            aw[e] = V::fma(dy, n[e], aw[e]);
+            ab[e] = V::add(ab[e], dy);
+            dn[e] = V::mul(dy, w[j]);
+            s1 = V::add(s1, dn[e]);
+            s2 = V::fma(dn[e], n[e], s2);
+        }
+    }
+    template <typename M>
+    __device__ __forceinline__ void finish(const M &m, float inv_d)
+    {
+        m1 = group_sum(s1.x + s1.y, m) * inv_d;
+        m2 = group_sum(s2.x + s2.y, m) * inv_d;
+    }
+    __device__ __forceinline__ void d_o(int i, float2 (&x)[4]) const
+    {
+        const float2 k0 = make_float2(-rstd * m1, -rstd * m1), k1 = make_float2(-rstd * m2, -rstd * m2), k2 = make_float2(rstd, rstd);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = V::fma(k2, dn[4 * i + j], V::fma(k1, n[4 * i + j], k0));
+    }
+};
+// partial[cta][2][dv]: the row slots' sums of dw and db
+template <int ROWS, int MAXD, int THREADS>
+__device__ __forceinline__ void write_partial(const float (*red)[2][MAXD], float *partial, int dv)
+{
+    for (int idx = threadIdx.x; idx < 2 * MAXD; idx += THREADS) {
+        const int which = idx / MAXD, c = idx - which * MAXD;
+        if (c >= dv) continue;
+        float sum = 0.f;
+#pragma unroll 8
+        for (int s = 0; s < ROWS; ++s) sum += red[s][which][c];
+        partial[((size_t)blockIdx.x * 2 + which) * dv + c] = sum;
+    }
 }
 
 template <typename TI, typename TO, int LPR, int CPL, bool FULL>
@@ -369,34 +437,21 @@ outgate_bwd(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln
         load_row(rv, reinterpret_cast<const TI *>(ring.in_buf(1, it)) + ln.m.slot * dv, ln);
         load_row(gv, reinterpret_cast<const TI *>(ring.in_buf(2, it)) + ln.m.slot * dv, ln);       // zero where the lane holds no value: it adds nothing
         TO *dob = reinterpret_cast<TO *>(ring.out_buf(0, it)) + ln.m.slot * dv, *drb = reinterpret_cast<TO *>(ring.out_buf(1, it)) + ln.m.slot * dv;
-        float2 n[NP], dn[NP], s1 = make_float2(0.f, 0.f), s2 = s1;
-        const float rstd = normalise(ov, ln, inv_d, eps, n);
+        RowGrad<Packed, CPL> g;
+        g.start(normalise<Packed>(ov, ln, inv_d, eps, g.n));
 #pragma unroll
         for (int i = 0; i < CPL; ++i) {
             float2 w[4], b[4], dr[4];
             pairs8(aff + ln.col(i), w);
             pairs8(aff + kMaxD + ln.col(i), b);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int e = 4 * i + j;
-                const float2 x = rv[i].pair(j), g = gv[i].pair(j), sg = sigmoid2(x), sw = mul2(x, sg);
-                const float2 y = fma2(n[e], w[j], b[j]), dy = mul2(g, sw);
-                dr[j] = mul2(mul2(g, y), fma2(sw, sub2(make_float2(1.f, 1.f), sg), sg));
-                aw[e] = fma2(dy, n[e], aw[e]);
-                ab[e] = add2(ab[e], dy);
-                dn[e] = mul2(dy, w[j]);
-                s1 = add2(s1, dn[e]);
-                s2 = fma2(dn[e], n[e], s2);
-            }
+            g.chunk(i, rv[i], gv[i], w, b, aw, ab, dr);
             if (ln.ok(i)) store8(drb + ln.col(i), dr);
         }
-        const float m1 = group_sum(s1.x + s1.y, ln.m) * inv_d, m2 = group_sum(s2.x + s2.y, ln.m) * inv_d;
-        const float2 k0 = make_float2(-rstd * m1, -rstd * m1), k1 = make_float2(-rstd * m2, -rstd * m2), k2 = make_float2(rstd, rstd);
+        g.finish(ln.m, inv_d);
 #pragma unroll
         for (int i = 0; i < CPL; ++i) {
             float2 x[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) x[j] = fma2(k2, dn[4 * i + j], fma2(k1, n[4 * i + j], k0));
+            g.d_o(i, x);
             if (ln.ok(i)) store8(dob + ln.col(i), x);
         }
         ok = ring.hand_over(it, ok);
@@ -417,15 +472,98 @@ outgate_bwd(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln
             }
     }
     __syncthreads();
-    // partial[cta][2][dv]
-    for (int idx = threadIdx.x; idx < 2 * kMaxD; idx += kThreads) {
-        const int which = idx / kMaxD, c = idx - which * kMaxD;
-        if (c >= dv) continue;
-        float sum = 0.f;
-#pragma unroll 8
-        for (int s = 0; s < kRows; ++s) sum += red[s][which][c];
-        partial[((size_t)blockIdx.x * 2 + which) * dv + c] = sum;
+    write_partial<kRows, kMaxD, kThreads>(red, partial, dv);
+}
+
+// The same without shared memory: every lane loads its chunk of a row from global memory, one chunk per lane (8, 9 or 16
+// lanes a row).
+template <int LPR>
+struct Direct {
+    static constexpr int kThreads = 256, kRows = RowMap<LPR, kThreads>::kRows, kMaxD = 8 * LPR;
+    using LN = Lane<LPR, 1, kThreads, false>;
+};
+__device__ __forceinline__ void load_affine(const float *p, int col, float absent, bool has, float2 (&x)[4])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = p != nullptr && has ? make_float2(p[col + 2 * j], p[col + 2 * j + 1]) : make_float2(absent, absent);
+}
+template <typename TA, typename TR, typename TZ, int LPR>
+__global__ void __launch_bounds__(Direct<LPR>::kThreads, LPR == 9 ? 4 : sizeof(TR) == 2 ? 5 : 1)
+outgate_fwd_direct(const TA *o, const TR *r, const float *__restrict__ ln_w, const float *__restrict__ ln_b, TZ *z, long long rows, int dv, float eps)
+{
+    using DR = Direct<LPR>;
+    using V = OpsFor<TR>;
+    typename DR::LN ln;
+    ln.dv = dv;
+    const int col = ln.col(0);
+    const float inv_d = 1.f / (float)dv;
+    pdl_wait();
+    float2 w[4], b[4];
+    load_affine(ln_w, col, 1.f, ln.has_col(0), w);
+    load_affine(ln_b, col, 0.f, ln.has_col(0), b);
+    for (long long base = (long long)blockIdx.x * DR::kRows; base < rows; base += (long long)gridDim.x * DR::kRows) {
+        const long long row = base + ln.m.slot;
+        ln.row_ok = row < rows;
+        Raw8<TA> ov[1];
+        Raw8<TR> rv[1];
+        load_row(ov, o + row * dv, ln);
+        load_row(rv, r + row * dv, ln);
+        float2 n[4], out[4];
+        normalise<V>(ov, ln, inv_d, eps, n);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 x = rv[0].pair(j);
+            out[j] = V::mul(V::mul(x, sigmoid2<V>(x)), V::fma(n[j], w[j], b[j]));
+        }
+        if (ln.ok(0)) store8(z + row * dv + col, out);
     }
+    pdl_launch_dependents();
+}
+template <typename TI, typename TO, int LPR>
+__global__ void __launch_bounds__(Direct<LPR>::kThreads, kBwdPerSM)
+outgate_bwd_direct(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln_w, const float *__restrict__ ln_b, TO *d_o, TO *d_r,
+                   float *__restrict__ partial, long long rows, int dv, float eps)
+{
+    using DR = Direct<LPR>;
+    using V = OpsFor<TI>;
+    __shared__ float red[DR::kRows][2][DR::kMaxD];
+    typename DR::LN ln;
+    ln.dv = dv;
+    const int col = ln.col(0);
+    const float inv_d = 1.f / (float)dv;
+    pdl_wait();
+    float2 w[4], b[4], aw[4], ab[4];
+    load_affine(ln_w, col, 1.f, ln.has_col(0), w);
+    load_affine(ln_b, col, 0.f, ln.has_col(0), b);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) aw[j] = ab[j] = make_float2(0.f, 0.f);
+    for (long long base = (long long)blockIdx.x * DR::kRows; base < rows; base += (long long)gridDim.x * DR::kRows) {
+        const long long row = base + ln.m.slot;
+        ln.row_ok = row < rows;
+        Raw8<TI> ov[1], rv[1], gv[1];
+        load_row(ov, o + row * dv, ln);
+        load_row(rv, r + row * dv, ln);
+        load_row(gv, dz + row * dv, ln);
+        RowGrad<V, 1> g;
+        g.start(normalise<V>(ov, ln, inv_d, eps, g.n));
+        float2 dr[4], dx[4];
+        g.chunk(0, rv[0], gv[0], w, b, aw, ab, dr);
+        if (ln.ok(0)) store8(d_r + row * dv + col, dr);
+        g.finish(ln.m, inv_d);
+        g.d_o(0, dx);
+        if (ln.ok(0)) store8(d_o + row * dv + col, dx);
+    }
+    pdl_launch_dependents();
+    if (partial == nullptr) return;
+    if (ln.m.valid) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            *reinterpret_cast<float2 *>(&red[ln.m.slot][0][col + 2 * j]) = aw[j];
+            *reinterpret_cast<float2 *>(&red[ln.m.slot][1][col + 2 * j]) = ab[j];
+        }
+    }
+    __syncthreads();
+    write_partial<DR::kRows, DR::kMaxD, DR::kThreads>(red, partial, dv);
 }
 
 // Sums of the CTAs' partial sums: lanes hold neighbouring parameters (whole lines per load), warp s of the
@@ -458,30 +596,44 @@ outgate_affine_sum(const float *__restrict__ partial, float *__restrict__ dln_w,
     }
 }
 
-// Calls f(LPR, CPL, FULL) with the row split of a storage type and row length.
-template <typename T, typename F>
-void with_split(int dv, F f)
+// Rows through shared memory or directly, and their split over lanes.  Measured on 196608 rows (us, forward / reverse, through
+// shared memory | directly): bf16 rows of 72 13.6 / 26.3 | 19.1 / 39.0, of 64 12.5 / 28.0 | 13.5 / 23.6 (fp32 results 15.1 / 28.3 |
+// 15.9 / 30.8), of 32 12.2 / 23.7 | 13.1 / 23.1 (786432 rows 43.8 / 76.4 | 52.4 / 81.1), of 40 13.7 / 24.6 | 13.4 / 23.5 (fp32
+// results 17.6 / 31.1 | 13.7 / 24.1: odd multiples of 16 bytes meet in banks), of 128 45.6 / 92.5 | 30.9 / 47.6; fp32 rows of 64
+// 21.9 / 46.0 | 16.5 / 31.9, of 72 31.3 / 63.0 | 23.8 / 42.9, of 128 52.9 / 101.8 | 35.6 / 58.8.  Hence shared memory for bf16 rows of
+// 72 values and of multiples of 16 up to 64, the reverse mode of 64 excepted.  One rule for both result types of bf16
+// rows, whose results have to agree to the bit.
+struct Split {
+    bool ring;
+    int lpr;
+    Split(int dv, bool narrow, bool reverse)
+        : ring(narrow && (dv == 72 || (dv <= 64 && dv % 16 == 0 && !(reverse && dv == 64)))),
+          lpr(ring ? (dv == 72 ? 3 : 4) : (dv <= 64 ? 8 : dv == 72 ? 9 : 16)) {}
+    int threads() const { return ring ? kThreads : Direct<8>::kThreads; }
+};
+// Calls f(LPR, CPL, FULL) with the split of rows that go through shared memory, or f(LPR) with that of the others.
+template <bool REVERSE, typename F>
+void with_ring(int dv, F f)
 {
     using std::integral_constant;
-    if constexpr (sizeof(T) == 2) {
-        if (dv == 64) f(integral_constant<int, 4>{}, integral_constant<int, 2>{}, std::true_type{});
-        else if (dv < 64) f(integral_constant<int, 4>{}, integral_constant<int, 2>{}, std::false_type{});
-        else if (dv == 72) f(integral_constant<int, 3>{}, integral_constant<int, 3>{}, std::true_type{});
-        else f(integral_constant<int, 4>{}, integral_constant<int, 4>{}, std::false_type{});
-    } else {
-        if (dv <= 64) f(integral_constant<int, 8>{}, integral_constant<int, 1>{}, std::false_type{});
-        else if (dv == 72) f(integral_constant<int, 9>{}, integral_constant<int, 1>{}, std::false_type{});
-        else f(integral_constant<int, 16>{}, integral_constant<int, 1>{}, std::false_type{});
-    }
+    if (!REVERSE && dv == 64) f(integral_constant<int, 4>{}, integral_constant<int, 2>{}, std::bool_constant<!REVERSE>{});
+    else if (dv < 64) f(integral_constant<int, 4>{}, integral_constant<int, 2>{}, std::false_type{});
+    else f(integral_constant<int, 3>{}, integral_constant<int, 3>{}, std::true_type{});
 }
-// lanes per row of that split
-int lanes_for(int dv, bool narrow) { return narrow ? (dv == 72 ? 3 : 4) : (dv <= 64 ? 8 : dv == 72 ? 9 : 16); }
-int grid_for(long long rows, int lpr, int per_sm)
+template <typename F>
+void with_direct(int dv, F f)
+{
+    using std::integral_constant;
+    if (dv <= 64) f(integral_constant<int, 8>{});
+    else if (dv == 72) f(integral_constant<int, 9>{});
+    else f(integral_constant<int, 16>{});
+}
+int grid_for(long long rows, const Split &sp, int per_sm)
 {
     int sms = device_sm_count();
     if (sms <= 0) sms = 148;            // sizing call without a device: the count the launch will most likely see
     const int kMaxCtas = sms * per_sm;
-    const long long per = (kThreads / 32) * (32 / lpr), need = (rows + per - 1) / per;
+    const long long per = (sp.threads() / 32) * (32 / sp.lpr), need = (rows + per - 1) / per;
     return (int)(need < kMaxCtas ? need : kMaxCtas);
 }
 
@@ -489,41 +641,61 @@ template <typename TA, typename TR, typename TZ>
 dig_status fwd_dispatch(const void *o, const void *r, const float *w, const float *b, void *z, long long rows, int dv,
                         float eps, cudaStream_t stream)
 {
-    int *status = device_status_ptr();
-    if (!status) return DIG_ERR_CUDA;
-    dig_status st = DIG_OK;
-    with_split<TR>(dv, [&](auto lpr, auto cpl, auto full) {
-        constexpr int LPR = decltype(lpr)::value, CPL = decltype(cpl)::value, ROWS = RowMap<LPR, kThreads>::kRows;
-        auto kern = outgate_fwd<TA, TR, TZ, LPR, CPL, decltype(full)::value>;
-        const size_t smem = (size_t)kStages * ROWS * dv * (sizeof(TA) + sizeof(TR) + sizeof(TZ));
-        if ((st = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem)) != DIG_OK) return;
-        const int fit = (int)(kSmemPerSM / (smem + 3072));           // + 1 KB of the system's and the static arrays
-        const int per_sm = fit < 1 ? 1 : fit < kFwdPerSM ? fit : kFwdPerSM;
-        launch_pdl(kern, dim3(grid_for(rows, LPR, per_sm)), dim3(kThreads), smem, stream, (const TA *)o, (const TR *)r, w, b,
-                   (TZ *)z, rows, dv, eps, status);
-        st = cuda_ok(cudaGetLastError());
+    const Split sp(dv, sizeof(TR) == 2, false);
+    if constexpr (sizeof(TR) == 2) {
+        if (sp.ring) {
+            int *status = device_status_ptr();
+            if (!status) return DIG_ERR_CUDA;
+            dig_status st = DIG_OK;
+            with_ring<false>(dv, [&](auto lpr, auto cpl, auto full) {
+                constexpr int LPR = decltype(lpr)::value, CPL = decltype(cpl)::value, ROWS = RowMap<LPR, kThreads>::kRows;
+                auto kern = outgate_fwd<TA, TR, TZ, LPR, CPL, decltype(full)::value>;
+                const size_t smem = (size_t)kStages * ROWS * dv * (sizeof(TA) + sizeof(TR) + sizeof(TZ));
+                if ((st = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem)) != DIG_OK) return;
+                const int fit = (int)(kSmemPerSM / (smem + 3072));           // + 1 KB of the system's and the static arrays
+                const int per_sm = fit < 1 ? 1 : fit < kFwdPerSM ? fit : kFwdPerSM;
+                launch_pdl(kern, dim3(grid_for(rows, sp, per_sm)), dim3(kThreads), smem, stream, (const TA *)o, (const TR *)r, w, b,
+                           (TZ *)z, rows, dv, eps, status);
+                st = cuda_ok(cudaGetLastError());
+            });
+            return st;
+        }
+    }
+    with_direct(dv, [&](auto lpr) {
+        launch_pdl(outgate_fwd_direct<TA, TR, TZ, decltype(lpr)::value>, dim3(grid_for(rows, sp, kFwdPerSM)), dim3(sp.threads()), 0, stream,
+                   (const TA *)o, (const TR *)r, w, b, (TZ *)z, rows, dv, eps);
     });
-    return st;
+    return cuda_ok(cudaGetLastError());
 }
 
 template <typename TI, typename TO>
 dig_status bwd_dispatch(const void *o, const void *r, const void *dz, const float *w, const float *b, void *d_o, void *d_r,
                         float *partial, long long rows, int dv, float eps, cudaStream_t stream)
 {
-    int *status = device_status_ptr();
-    if (!status) return DIG_ERR_CUDA;
-    dig_status st = DIG_OK;
-    with_split<TI>(dv, [&](auto lpr, auto cpl, auto full) {
-        constexpr int LPR = decltype(lpr)::value, CPL = decltype(cpl)::value, ROWS = RowMap<LPR, kThreads>::kRows;
-        auto kern = outgate_bwd<TI, TO, LPR, CPL, decltype(full)::value>;
-        const size_t ring = (size_t)kStages * ROWS * dv * (3 * sizeof(TI) + 2 * sizeof(TO)), red = (size_t)ROWS * 2 * 8 * LPR * CPL * sizeof(float);
-        const size_t smem = ring > red ? ring : red;
-        if ((st = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem)) != DIG_OK) return;
-        launch_pdl(kern, dim3(grid_for(rows, LPR, kBwdPerSM)), dim3(kThreads), smem, stream, (const TI *)o, (const TI *)r,
-                   (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps, status);
-        st = cuda_ok(cudaGetLastError());
+    const Split sp(dv, sizeof(TI) == 2, true);
+    if constexpr (sizeof(TI) == 2) {
+        if (sp.ring) {
+            int *status = device_status_ptr();
+            if (!status) return DIG_ERR_CUDA;
+            dig_status st = DIG_OK;
+            with_ring<true>(dv, [&](auto lpr, auto cpl, auto full) {
+                constexpr int LPR = decltype(lpr)::value, CPL = decltype(cpl)::value, ROWS = RowMap<LPR, kThreads>::kRows;
+                auto kern = outgate_bwd<TI, TO, LPR, CPL, decltype(full)::value>;
+                const size_t ring = (size_t)kStages * ROWS * dv * (3 * sizeof(TI) + 2 * sizeof(TO)), red = (size_t)ROWS * 2 * 8 * LPR * CPL * sizeof(float);
+                const size_t smem = ring > red ? ring : red;
+                if ((st = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem)) != DIG_OK) return;
+                launch_pdl(kern, dim3(grid_for(rows, sp, kBwdPerSM)), dim3(kThreads), smem, stream, (const TI *)o, (const TI *)r,
+                           (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps, status);
+                st = cuda_ok(cudaGetLastError());
+            });
+            return st;
+        }
+    }
+    with_direct(dv, [&](auto lpr) {
+        launch_pdl(outgate_bwd_direct<TI, TO, decltype(lpr)::value>, dim3(grid_for(rows, sp, kBwdPerSM)), dim3(sp.threads()), 0, stream, (const TI *)o,
+                   (const TI *)r, (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps);
     });
-    return st;
+    return cuda_ok(cudaGetLastError());
 }
 
 }  // namespace
@@ -531,7 +703,7 @@ dig_status bwd_dispatch(const void *o, const void *r, const void *dz, const floa
 // the wider of the two storage types' grids
 size_t outgate_bwd_workspace_bytes(long long rows, int dv)
 {
-    const int a = grid_for(rows, lanes_for(dv, true), kBwdPerSM), b = grid_for(rows, lanes_for(dv, false), kBwdPerSM);
+    const int a = grid_for(rows, Split(dv, true, true), kBwdPerSM), b = grid_for(rows, Split(dv, false, true), kBwdPerSM);
     return (size_t)(a > b ? a : b) * 2 * (size_t)dv * sizeof(float);
 }
 
@@ -571,7 +743,7 @@ dig_status launch_outgate_bwd(const void *o, const void *r, const void *dz, cons
     if (st != DIG_OK || !affine) return st;
     KernelTimer t(KID_OUTGATE, stream);
     launch_pdl(outgate_affine_sum, dim3((2 * dv + 31) / 32), dim3(32 * kSumWarps), 0, stream, (const float *)partial, dln_w,
-               dln_b, grid_for(rows, lanes_for(dv, dtype != DIG_F32), kBwdPerSM), dv);
+               dln_b, grid_for(rows, Split(dv, dtype != DIG_F32, true), kBwdPerSM), dv);
     return cuda_ok(cudaGetLastError());
 }
 

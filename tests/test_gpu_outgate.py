@@ -56,6 +56,13 @@ def test_outgate_small_ragged(dtype, d):
     _case((3, 37, 5, d), dtype, affine=(d != 24), seed=d)
 
 
+@pytest.mark.parametrize("dtype,d,rows", [("bf16", 48, 40 * 148 * 8 + 7), ("bf16", 80, 20011), ("bf16", 56, 33), ("f32", 120, 20011), ("f32", 16, 31)])
+def test_outgate_lengths_at_the_edges_of_the_row_split(dtype, d, rows):
+    """Row lengths on either side of the rule that picks shared memory or direct loads; more rows than one pass of the grid, and
+    fewer than a CTA."""
+    _case((rows, d), dtype, True, d)
+
+
 def test_outgate_single_row_and_extremes():
     from paper_2405_18428_b200 import dig
     _case((1, 1, 1, 64), "f32", True, 1)
