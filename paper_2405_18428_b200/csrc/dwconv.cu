@@ -144,7 +144,7 @@ srem_dwconv3x3(const T *__restrict__ x, const T *__restrict__ w, const T *__rest
 // one pass 34 us, where dx and the filter sums in a pass each took 21 + 25.5.
 constexpr int kRing = 6;
 constexpr int kStripCtas = 4;        // per SM: what 128 registers allow (five at 100 registers were no faster)
-constexpr int kWgPixels = 128;       // pixels per partial sum (sizes the workspace)
+constexpr int kWgPixels = 32;        // pixels per partial sum at least
 
 __device__ __forceinline__ float2 load_pair(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 __device__ __forceinline__ float2 load_pair(const __nv_bfloat16 *p) { return bf2(*reinterpret_cast<const uint32_t *>(p)); }
@@ -418,26 +418,32 @@ dig_status launch_dwconv(const void *x, const void *w, const void *bias, void *y
     return cuda_ok(cudaGetLastError());
 }
 
+// CTA rows of the reverse mode, one partial sum each: no more than stay resident together, so that their strip loops end
+// together, and no more than one per kWgPixels pixels (with one per 128, which the filter sums alone wanted, small grids
+// had too few CTAs for dx: 11 x 5 x 8 pixels of 712 channels 11.0 us, 8 x 11 x 32 of 592 23.9, 6.6 and 11.8 now; 8 x 32 x 32 of 384 18.8 -> 13.9).
+static long long slabs_for(int B, int gh, int gw, int nchb)
+{
+    int sms = device_sm_count();
+    if (sms <= 0) sms = 148;            // sizing call without a device: the count the launch will most likely see
+    const long long cap = sms * kStripCtas / nchb, n = ((long long)B * gh * gw + kWgPixels - 1) / kWgPixels;
+    return n < cap ? n : cap > 0 ? cap : 1;
+}
+
 size_t dwconv_bwd_workspace_bytes(int B, int gh, int gw, int D)
 {
-    const size_t nslab = ((size_t)B * gh * gw + kWgPixels - 1) / kWgPixels;
-    return nslab * 10 * (size_t)D * sizeof(float);
+    const int CH = Cfg<__nv_bfloat16>::CH;         // the wider block of the two storage types: the most CTA rows
+    return (size_t)slabs_for(B, gh, gw, (D + CH - 1) / CH) * 10 * (size_t)D * sizeof(float);
 }
 
 dig_status launch_dwconv_bwd(const void *x, const void *w, const void *dy, void *dx, float *dw, float *dbias,
                              int B, int gh, int gw, int D, int dir, int dtype, float *partial, cudaStream_t stream)
 {
-    // One partial sum per CTA row.  No more CTA rows than stay resident together so that their strip loops end together, never more than the workspace holds;
-    // strips are cut into row segments until every CTA row has one.
+    // Strips are cut into row segments until every CTA row has one.
     const int CHb = dtype == DIG_F32 ? Cfg<float>::CH : Cfg<__nv_bfloat16>::CH;
     const int nchb = (D + CHb - 1) / CHb;
     if (!sizes_served(B, gh, nchb)) return DIG_ERR_UNSUPPORTED;
-    const int resident = device_sm_count() * kStripCtas;
-    if (resident <= 0) return DIG_ERR_CUDA;
-    const long long npix = (long long)B * gh * gw;
-    long long nslab = (npix + kWgPixels - 1) / kWgPixels;
-    const int cap = resident / nchb > 0 ? resident / nchb : 1;
-    if (nslab > cap) nslab = cap;
+    if (device_sm_count() <= 0) return DIG_ERR_CUDA;
+    long long nslab = slabs_for(B, gh, gw, nchb);
     const int strips_x = (gw + TX - 1) / TX;
     const long long base = (long long)B * strips_x;
     const StripCut cut((int)(nslab / base), gh);                    // rounded down: no CTA row gets a second strip while others have one

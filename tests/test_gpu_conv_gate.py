@@ -141,6 +141,22 @@ def test_conv_bwd_strip_edges(B, gh, gw, D, dtype, direction):
     _conv_bwd_case(B, gh, gw, D, dtype, direction, with_bias=True, seed=20 + direction)
 
 
+@pytest.mark.parametrize("B,gh,gw,D,dtype", [(11, 5, 8, 712, "bf16"), (8, 11, 32, 592, "f32"), (1, 4, 9, 8, "bf16"), (2, 200, 3, 40, "bf16")])
+def test_conv_bwd_partial_sums_of_small_grids(B, gh, gw, D, dtype):
+    """One partial sum per 32 pixels at most: one to two strips per CTA row, strips of one column, a single partial sum; the call
+    stays within the workspace it asks for."""
+    from paper_2405_18428_b200 import dig
+    _conv_bwd_case(B, gh, gw, D, dtype, 1, with_bias=True, seed=30)
+    st = torch.bfloat16 if dtype == "bf16" else torch.float32
+    x, w = torch.randn(B, gh * gw, D, device="cuda").to(st), torch.randn(3, 3, D, device="cuda").to(st)
+    need = dig.lib().dig_srem_dwconv_bwd_workspace_bytes(B, gh, gw, D)
+    ws = torch.full((need + 4096,), 77, dtype=torch.uint8, device="cuda")
+    a = dig.dig_srem_dwconv_bwd(x, w, x, gh, gw, 1, workspace=ws[:need])
+    assert bool((ws[need:] == 77).all())
+    for s, t in zip(a, dig.dig_srem_dwconv_bwd(x, w, x, gh, gw, 1)):
+        assert torch.equal(s, t)
+
+
 @pytest.mark.parametrize("cfg", ["C2", "C5"])
 def test_conv_bwd_benchmark_shapes(cfg):
     from paper_2405_18428_b200 import dig
