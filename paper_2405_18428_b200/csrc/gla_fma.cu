@@ -47,10 +47,11 @@ __device__ __forceinline__ void mm_nt(float (&acc)[4][4], const float *A, int ld
     }
 }
 // acc[i][j] += sum_{k<K} A[(r0+i)*lda + k] * Bm[k*ldb + c0 + j]
+template <int UNROLL>
 __device__ __forceinline__ void mm_nn(float (&acc)[4][4], const float *A, int lda, int r0,
                                       const float *Bm, int ldb, int c0, int K)
 {
-#pragma unroll 4
+#pragma unroll UNROLL
     for (int k = 0; k < K; k += 4) {
         float4 a[4], b[4];
 #pragma unroll
@@ -336,8 +337,11 @@ __device__ __forceinline__ void score_block(float *sP, int ldp, const float *sA,
 
 // ---- kernel 3: outputs ---------------------------------------------------------------------------
 // out = tril(Qt Kt^T) V + Qt S
-template <typename T, typename TO>
-__global__ void __launch_bounds__(kThreads)
+// PERSM: CTAs per SM that the registers allow, three, or four on shorter loops where a launch has more CTAs than three per SM and
+// shared memory holds four (chunks below 64): 180 sequences of 250 tokens in chunks of 16 (d = 64) take 82 us with three, 70
+// with four.  Fewer CTAs are faster with three (12 sequences of 1024 tokens in chunks of 32: 31.0 us a pass, 34.7 with four).
+template <typename T, typename TO, int PERSM>
+__global__ void __launch_bounds__(kThreads, PERSM)
 fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v,
               const float *__restrict__ gate, const float *__restrict__ states,
               TO *__restrict__ out, Geom g)
@@ -375,13 +379,14 @@ fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     for (int blk = threadIdx.x; blk < nb * nb; blk += kThreads) score_block(sP, ldp, sQ, ldk, sK, ldk, g.C, g.dk, blk);
     loads_done();
     __syncthreads();
+    constexpr int UN = PERSM > 3 ? 1 : 4;
     const int nrb = g.C >> 2, ncb = g.dv >> 2;
     for (int blk = threadIdx.x; blk < nrb * ncb; blk += kThreads) {
         const int r0 = (blk / ncb) << 2, c0 = (blk % ncb) << 2;
         float acc[4][4];
         zero(acc);
-        mm_nn(acc, sP, ldp, r0, sV, ldv, c0, r0 + 4);       // columns beyond the diagonal are zero
-        mm_nn(acc, sQ, ldk, r0, sS, ldv, c0, g.dk);
+        mm_nn<UN>(acc, sP, ldp, r0, sV, ldv, c0, r0 + 4);       // columns beyond the diagonal are zero
+        mm_nn<UN>(acc, sQ, ldk, r0, sS, ldv, c0, g.dk);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int row = sRow[r0 + i];
@@ -587,7 +592,7 @@ dig_status fwd_typed(const GlaArgs &a)
     launch_pdl(k1, grid, dim3(kThreads), smem_state(g, false), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
                (const T *)nullptr, w.states, w.gamma, (float *)nullptr, g); }
     if ((st = launch_state_scan_fwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
-    auto k3 = fma_chunk_out<T, TO>;
+    auto k3 = g.C < 64 && (long long)grid.x * grid.y > 3ll * device_sm_count() ? fma_chunk_out<T, TO, 4> : fma_chunk_out<T, TO, 3>;
     if ((st = set_smem(k3, smem_out(g))) != DIG_OK) return st;
     KernelTimer t(KID_FMA_OUT, a.stream);
     launch_pdl(k3, grid, dim3(kThreads), smem_out(g), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
