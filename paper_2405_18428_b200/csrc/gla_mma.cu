@@ -397,8 +397,12 @@ __device__ __forceinline__ void masked_scores(float *sP, int ldp, const float *A
 // U = Kh^T V (and, for the backward pass, W = Qt^T dO); gamma = exp(Lam_{C-1}).
 // BETA: with the value-channel gate the value side mirrors the key side: M = prefix sums of log(beta),
 // gamma_v = exp(M_{C-1}), U = Kh^T Vh with Vh = v*exp(M_{C-1}-M), W = Qt^T G with G = dO*exp(M).
+// CTAs per SM that the registers have to allow: with sizes not known at compile time two, which chunks that are short have the
+// shared memory for (24 sequences of 6561 tokens, d = 48 x 88, chunks of 16 with the full gate: 493 us with 72 registers and one
+// CTA, 312 with 64 and two); the others what their tiles allow.
+template <typename DM> constexpr int kStateCtas = DM::kC == 0 ? 2 : DM::kC == 32 && DM::kDK == 64 ? 4 : 3;
 template <bool BWD, typename DM, bool BETA, typename TI>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, kStateCtas<DM>)
 mma_chunk_state(const TI *__restrict__ q, const TI *__restrict__ k, const TI *__restrict__ v, const float *__restrict__ gate,
                 const TI *__restrict__ d_out, float *__restrict__ states, float *__restrict__ gamma,
                 float *__restrict__ dstates, BetaDev bd, Geom g)
