@@ -205,6 +205,23 @@ template <int D> __device__ __forceinline__ bool beyond(const Tot &t)        // 
     const bool b = fmaxf(fabsf(t.all.x), fabsf(t.all.y)) > kSubLimit || (Col<D>::X && fmaxf(fabsf(t.xall.x), fabsf(t.xall.y)) > kSubLimit);
     return __any_sync(0xffffffffu, b) != 0;
 }
+// Sums over one half of the tile's groups (HALF = 0, 1).
+template <int D, int HALF>
+__device__ __forceinline__ Tot half_totals(const float *sTot, const Who<D> &w)
+{
+    Tot t;
+    t.before = t.all = t.xbefore = t.xall = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int s = 4 * HALF; s < 4 * HALF + 4; ++s) {
+        if (s == w.grp) {
+            t.before = t.all;
+            t.xbefore = t.xall;
+        }
+        t.all = add2(t.all, *reinterpret_cast<const float2 *>(sTot + s * D + w.c2));
+        if (Col<D>::X) t.xall = add2(t.xall, *reinterpret_cast<const float2 *>(sTot + s * D + w.xc2));
+    }
+    return t;
+}
 // Longest sub-chunk length (a power of two between kMinSub and `start`) for which every aligned window of
 // the tile keeps |sum of gates| <= kSubLimit in every channel; kMinSub if none does (then the range bit of
 // *status is set).  Uniform over the CTA.
@@ -223,6 +240,24 @@ __device__ __noinline__ int choose_window(const float *sTot, Who<D> w, int start
             return s;
         }
     }
+}
+// Sub-chunk length of a tile whose totals are tt; tt becomes the totals of the (sub-)chunk the thread's rows are in.  Halves,
+// which chunks of 32 ask for and which suffice for most tiles beyond the limit, are tried with sums over fixed groups (the
+// search takes a few hundred cycles).
+template <int D>
+__device__ __forceinline__ int divide_tile(const float *sTot, const Who<D> &w, int sub_max, int *status, Tot &tt)
+{
+    if (sub_max >= T && !beyond<D>(tt)) return T;
+    if (sub_max >= T / 2) {
+        const Tot lo = half_totals<D, 0>(sTot, w), hi = half_totals<D, 1>(sTot, w);
+        if (!beyond<D>(lo) && !beyond<D>(hi)) {
+            tt = w.grp < 4 ? lo : hi;
+            return T / 2;
+        }
+    }
+    const int s = choose_window<D>(sTot, w, min(sub_max, T / 4), status), w0 = 8 * w.grp / s * (s / 8);
+    tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
+    return s;
 }
 
 __device__ __forceinline__ void st_pair(char *tile, int o, float2 a) { *reinterpret_cast<uint32_t *>(tile + o) = pack_h2(a.x, a.y); }
@@ -393,37 +428,46 @@ __device__ __forceinline__ float of_corner(float2 xx)
     const float a = __shfl_sync(0xffffffffu, xx.x, (threadIdx.x & 7) >> 1), b = __shfl_sync(0xffffffffu, xx.y, (threadIdx.x & 7) >> 1);
     return (threadIdx.x & 1) ? b : a;
 }
+// Gates (log2) summed over one (sub-)chunk or more, for the thread's state row and its corner channel.
+struct RowSum {
+    float t, xt;
+};
+template <int D>
+__device__ __forceinline__ RowSum row_sum(const StateOf<D> &st, const Tot &tt)
+{
+    return RowSum{of_row(st, tt.all), Col<D>::X ? of_corner(tt.xall) : 0.f};
+}
+__device__ __forceinline__ RowSum operator+(RowSum a, RowSum b) { return RowSum{a.t + b.t, a.xt + b.xt}; }
 // Decay of one (sub-)chunk whose gates sum to t: ec = 2^(t/2), e2c = 2^t for the thread's state row, x* for its corner channel.
 struct Decay {
     float ec, e2c, xec, xe2c;
 };
 template <int D>
-__device__ __forceinline__ Decay decay_of(const StateOf<D> &st, float2 all, float2 xall)
+__device__ __forceinline__ Decay decay_of(RowSum r)
 {
     Decay d;
-    const float t = of_row(st, all);
-    d.ec = ex2(0.5f * t);
-    d.e2c = ex2(t);
-    d.xec = d.xe2c = 0.f;
-    if (Col<D>::X) {
-        const float xt = of_corner(xall);
-        d.xec = ex2(0.5f * xt);
-        d.xe2c = ex2(xt);
-    }
+    d.ec = ex2(0.5f * r.t);
+    d.e2c = ex2(r.t);
+    d.xec = Col<D>::X ? ex2(0.5f * r.xt) : 0.f;
+    d.xe2c = Col<D>::X ? ex2(r.xt) : 0.f;
     return d;
 }
 // Weight of a (sub-)chunk's product in a sum over the segment: 2^x with x the decay from the chunk's centre to the
-// segment's end (or from its start).
+// segment's end (or from its start): half of the chunk's own gates `r` and those between, `far`.
 struct Weight {
     float f, xf;
 };
 template <int D>
-__device__ __forceinline__ Weight weight_of(const StateOf<D> &st, float2 x, float2 xx)
+__device__ __forceinline__ Weight weight_of(RowSum r, RowSum far)
 {
-    Weight w;
-    w.f = ex2(of_row(st, x));
-    w.xf = Col<D>::X ? ex2(of_corner(xx)) : 0.f;
-    return w;
+    return Weight{ex2(fmaf(0.5f, r.t, far.t)), Col<D>::X ? ex2(fmaf(0.5f, r.xt, far.xt)) : 0.f};
+}
+// the threads' row sums as an array over the channels (once per CTA)
+template <int D>
+__device__ __forceinline__ void put_row_sums(float *dst, const Who<D> &w, const StateOf<D> &st, RowSum r)
+{
+    if (w.cg == 0 && w.hf == 0) dst[st.row] = r.t;
+    if (Col<D>::X && threadIdx.x < 8) dst[64 + threadIdx.x] = r.xt;
 }
 // value of key channel 64 + j of the corner (every lane of the warp must call it)
 __device__ __forceinline__ float corner_val(float v, int j) { return __shfl_sync(0xffffffffu, v, j); }
@@ -558,32 +602,37 @@ __device__ __forceinline__ void acc_to_global(uint32_t acc, const StateOf<D> &m,
 
 // ---- products with split accumulators ----------------------------------------------------------------
 constexpr uint32_t kHiLanes = 16u << 16;
-// acc <- A^T B over the 64 token rows: rows = key channels (A), columns = value channels (B)
-template <int D>
+// Rows a product takes: all of the tile, or one half where each half is a sub-chunk (the value is the quarters of the
+// accumulator's lanes that hold the other rows).
+enum Rows : uint32_t { kAllRows = 0, kLowRows = 0xc, kHighRows = 0x3 };
+// acc <- A^T B over the token rows: rows = key channels (A), columns = value channels (B)
+template <int D, Rows ROWS = kAllRows>
 __device__ __forceinline__ void issue_state(uint32_t acc, const char *tA, const char *tB)
 {
     using C = Cfg<D>;
     using L = Col<D>;
-    const uint32_t a = smem_u32(tA), b = smem_u32(tB);
-    issue<64, 8 * L::NV0, true, true, T / 16, C::CHT, C::CHT>(acc, a, b, false);
-    issue<64, 8 * L::NV1, true, true, T / 16, C::CHT, C::CHT>(acc + kHiLanes, a, b + L::NV0 * C::CHT, false);
+    constexpr int KS = ROWS == kAllRows ? T / 16 : T / 32;
+    constexpr uint32_t first = ROWS == kHighRows ? T / 2 * 16 : 0;
+    const uint32_t a = smem_u32(tA) + first, b = smem_u32(tB) + first;
+    issue<64, 8 * L::NV0, true, true, KS, C::CHT, C::CHT>(acc, a, b, false);
+    issue<64, 8 * L::NV1, true, true, KS, C::CHT, C::CHT>(acc + kHiLanes, a, b + L::NV0 * C::CHT, false);
     if (L::X) {
         // the corner, transposed: rows = value channels (64 and the remaining 8), columns = key channels 64 .. 71.
         // The second product's A operand covers chunks 8 .. 15, most of them beyond the tile: mapped shared
         // memory whose rows of the result nobody reads.
-        issue<64, 8, true, true, T / 16, C::CHT, C::CHT>(acc + L::HW, b, a + 8 * C::CHT, false);
-        issue<64, 8, true, true, T / 16, C::CHT, C::CHT>(acc + L::HW + kHiLanes, b + 8 * C::CHT, a + 8 * C::CHT, false);
+        issue<64, 8, true, true, KS, C::CHT, C::CHT>(acc + L::HW, b, a + 8 * C::CHT, false);
+        issue<64, 8, true, true, KS, C::CHT, C::CHT>(acc + L::HW + kHiLanes, b + 8 * C::CHT, a + 8 * C::CHT, false);
     }
 }
 // acc (+)= A B with the value channels (columns of B) split; A K-major tile of 64 rows, B MN-major
-template <int D, int KSTEPS, uint32_t BCH>
+template <int D, int KSTEPS, uint32_t BCH, Rows ROWS = kAllRows>
 __device__ __forceinline__ void issue_split(uint32_t acc, const char *tA, const char *tB, bool accumulate)
 {
     using C = Cfg<D>;
     using L = Col<D>;
     const uint32_t a = smem_u32(tA), b = smem_u32(tB);
-    issue<64, 8 * L::NV0, false, true, KSTEPS, C::CHT, BCH>(acc, a, b, accumulate);
-    issue<64, 8 * L::NV1, false, true, KSTEPS, C::CHT, BCH>(acc + kHiLanes, a, b + L::NV0 * BCH, accumulate);
+    issue<64, 8 * L::NV0, false, true, KSTEPS, C::CHT, BCH, 128, ROWS>(acc, a, b, accumulate);
+    issue<64, 8 * L::NV1, false, true, KSTEPS, C::CHT, BCH, 128, ROWS>(acc + kHiLanes, a, b + L::NV0 * BCH, accumulate);
 }
 // acc <- A B^T (scores), columns split into even (lanes 0-15) and odd (lanes 16-31) 8-token chunks
 template <int D>

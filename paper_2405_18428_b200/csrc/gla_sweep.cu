@@ -24,6 +24,13 @@
 // In the backward sweep S_in = S_local + diag(G) S_segment, G the decay since the segment start, so
 // dO Sc^T = dO Sc_local^T + (dO S_segment^T) diag(exp(c) G): two products and one fused multiply-add.
 //
+// A tile whose gates sum to too much for one centring, or that was asked for in shorter chunks, is worked in sub-chunks.  Two
+// of 32 rows share one pass through a kernel's phases: operands are built once, each row centred on its own half, scores are
+// block-diagonal, and only what acts through the state or its gradient is done per half, the later half with the second
+// group of products.  The results are those of two passes bit for bit.  48 sequences of 1961 tokens in chunks of 32, d = 72:
+// the four kernels 42 + 56 + 76 + 108 us with a pass per half, 28 + 38 + 56 + 84 now; 48 of 4096, d = 64, half of the heads at
+// tau = 4, where one tile in six is divided and the CTA with most of them is the last: 35 + 49 + 48 + 94, now 30 + 43 + 46 + 86.
+//
 // Every product is a tcgen05.mma (kind::f16, fp16 operands, fp32 accumulators in tensor memory) issued by
 // one thread of the last warp, which otherwise works like the others: all threads build operand tiles, mask the
 // scores and post-process accumulators, phase by phase (columns.cuh holds the work split).  Rows of the
@@ -95,9 +102,10 @@ __device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, int *st
 // =================================================================================================
 // sweep_local_fwd: the state a segment leaves from a zero start, and its total decay.  The tiles are walked from the
 // segment's end, so the decay from a tile's centre to the end is known when its product is: the state is the plain
-// sum of 2^(that decay) (Kc^T V), kept in tensor memory.  One barrier per tile or sub-chunk: behind it lie the group sums of
-// this tile and the operand rows of the step before, whose product is issued there and added one step later; operand
-// tiles, accumulators and sums have two buffers, and the rows of the next tile are loaded a whole tile ahead.
+// sum of 2^(that decay) (Kc^T V), kept in tensor memory.  One barrier per tile or sub-chunk (two sub-chunks of 32 rows are
+// one step with two products): behind it lie the group sums of this tile and the operand rows of the step before, whose
+// product is issued there and added once this step's operands are built; operand tiles and sums have two buffers, and the
+// rows of the next tile are loaded a whole tile ahead.
 // Bound by the latency of its phases.  48 sequences of 4096 tokens, d = 64: 40 us with the state in registers, decayed
 // once per tile in scan order, 33 us now; 16 of 16384, d = 72: 80 -> 54 us (63 with the sum in registers, which spills).
 // One operand exponent for the whole way to the segment's end would let the matrix unit add the products up (29 and
@@ -111,7 +119,7 @@ struct LocalFwdSmem {
     static constexpr int kBuf = 2 * C::TILE_T;                                // tK tV
     static constexpr int kPad = L::X ? 16 * C::CHT - C::TILE_T : 0;           // the corner's operand reads past its tile
     static constexpr size_t bytes = 2 * kBuf + kPad + 2 * 8 * D * 4 + 4 * T * 4 + sizeof(Ctl);
-    static constexpr uint32_t aSum = 2 * L::ACCS;                             // accumulator columns: two products, the sum
+    static constexpr uint32_t aSum = 2 * L::ACCS;                             // accumulator columns: products of one pass (of two halves), the sum
     static constexpr uint32_t tmem_cols = 3 * L::ACCS <= 128 ? 128 : 256;
 };
 
@@ -128,7 +136,7 @@ sweep_local_fwd(const SweepArgs a)
     Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 4 * T);
 
     const int tid = threadIdx.x;
-    cta_setup(ctl, 2, SM::tmem_cols, smem, 2 * SM::kBuf + SM::kPad);
+    cta_setup(ctl, 1, SM::tmem_cols, smem, 2 * SM::kBuf + SM::kPad);
     const Who<D> w;
     const StateOf<D> sm(w);
     const uint32_t tmem = warp_uniform(ctl->tmem_base), tl = tmem + ((uint32_t)(32 * w.q4) << 16);
@@ -137,22 +145,32 @@ sweep_local_fwd(const SweepArgs a)
     Cols<D, false, false> raw;
     Cols<D, false, false> nxt;                          // rows and gates of the next tile, a whole tile ahead of their use
     bool ok = true, first = true;                       // first: nothing of this segment is in the sum
-    uint32_t it = 0;                                    // (sub-)chunks worked so far: buffer it & 1, its barrier's phase (it >> 1) & 1
+    uint32_t it = 0;                                    // operand tiles built so far: buffer it & 1, phase of their products' barrier it & 1
     const int total = g.B * g.H * pl.nseg;
 
-    // product of step i: its operand tiles were built before the barrier just passed
-    auto issue_step = [&](uint32_t i) {
+    // products of the tiles built last (before the barrier just passed), one or one per half
+    Weight w1{}, w2{};                                  // their weights
+    bool pending = false, pair = false;
+    auto issue_step = [&]() {
         if (w.issuer() && elect_one()) {
-            char *tK = smem + (i & 1) * SM::kBuf;
+            char *tK = smem + ((it - 1) & 1) * SM::kBuf;
             tc_fence_after_sync();
-            issue_state<D>(tmem + (i & 1) * L::ACCS, tK, tK + C::TILE_T);
-            mma_commit(&ctl->bar[i & 1]);
+            if (!pair) {
+                issue_state<D>(tmem, tK, tK + C::TILE_T);
+            } else {
+                issue_state<D, kHighRows>(tmem, tK, tK + C::TILE_T);
+                issue_state<D, kLowRows>(tmem + L::ACCS, tK, tK + C::TILE_T);
+            }
+            mma_commit(&ctl->bar[0]);
         }
     };
-    auto add_step = [&](uint32_t i, const Weight &wt) {
-        ok = wait_all(&ctl->bar[i & 1], (i >> 1) & 1, a.status, ok);
+    auto add_step = [&](uint32_t parity) {
+        ok = wait_all(&ctl->bar[0], parity, a.status, ok);
         tc_fence_after_sync();
-        if (ok) add_product<D>(tl + SM::aSum, tl + (i & 1) * L::ACCS, sm, wt, first);
+        if (ok) {
+            add_product<D>(tl + SM::aSum, tl, sm, w1, first);
+            if (pair) add_product<D>(tl + SM::aSum, tl + L::ACCS, sm, w2, false);
+        }
         first = false;
         tc_fence_before_sync();
     };
@@ -162,9 +180,8 @@ sweep_local_fwd(const SweepArgs a)
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
         first = true;
-        float2 after = make_float2(0.f, 0.f), xafter = after;          // gates of the tiles behind (log2), the thread's channels
-        uint32_t n = 0;                                                 // (sub-)chunks of this segment
-        Weight w1{}, w2{};                                              // weights of the last one and of the one before
+        RowSum after{0.f, 0.f};                                         // gates of the tiles behind
+        pending = false;
         if (tid < 3 * T && t1 - 1 - (tid >> 6) >= t0) {
             const int tile = t1 - 1 - (tid >> 6);
             rowOff[(tile & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, tile, tid & 63);
@@ -188,45 +205,45 @@ sweep_local_fwd(const SweepArgs a)
             const float *tot = sTot + (tile & 1) * 8 * D;
             tc_fence_before_sync();
             SYNC_OR_DIE();                                             // group totals are there, the step before is built
-            if (n > 0) issue_step(it - 1);
+            if (pending) issue_step();
             if (tid < T && tile - 3 >= t0) rowOff[((tile - 3) & 3) * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 3, tid);
             if (tile > t0) {
                 uint32_t ro[9];
                 row_offsets<D>(rowOff + ((tile - 1) & 3) * T, w, ro);
                 load_rows(nxt, a.q, a.k, a.v, a.d_out, ro);
             }
-            const Tot whole = tile_totals<D>(tot, w);
-            Tot tt = whole;
-            int s = T;
-            if (pl.sub_max < T || beyond<D>(tt)) {
-                s = choose_window<D>(tot, w, min(pl.sub_max, T / 2), a.status);
-                const int w0 = 8 * w.grp / s * (s / 8);
-                tt = window_totals<D>(tot, w, w0, w0 + s / 8);
-            }
+            Tot tt = tile_totals<D>(tot, w);
+            const RowSum mine = row_sum<D>(sm, tt);
+            const int s = divide_tile<D>(tot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
-            const int nsub = (nrow + s - 1) / s;
-            for (int u = nsub - 1; u >= 0; --u, ++it, ++n) {
+            const bool halves = s == T / 2 && nrow > T / 2;            // two sub-chunks at once, a product each
+            const int step = halves ? T : s, nsub = (nrow + step - 1) / step;
+            for (int u = nsub - 1; u >= 0; --u) {
                 if (u < nsub - 1) {
                     tc_fence_before_sync();
                     SYNC_OR_DIE();
-                    issue_step(it - 1);
+                    issue_step();
                 }
-                if (n >= 2) add_step(it - 2, w2);                       // its buffer is free again
-                char *tK = smem + (it & 1) * SM::kBuf;
-                build_rows<D>(raw, w, nullptr, tK, tK + C::TILE_T, nullptr, 8 * w.grp >= u * s && 8 * w.grp < (u + 1) * s);
+                char *tK = smem + (it & 1) * SM::kBuf;                  // what read it last has been added
+                build_rows<D>(raw, w, nullptr, tK, tK + C::TILE_T, nullptr, 8 * w.grp >= u * step && 8 * w.grp < (u + 1) * step);
                 fence_async_smem();
+                if (pending) add_step((it - 1) & 1);
+                pending = true;
+                pair = halves;
+                ++it;
                 // gates from the centre to the segment's end
-                float2 x = fma2(whole.all, make_float2(0.5f, 0.5f), after), xx = fma2(whole.xall, make_float2(0.5f, 0.5f), xafter);
-                if (s < T) {
-                    const Tot own = window_totals<D>(tot, w, u * s / 8, (u + 1) * s / 8), behind = window_totals<D>(tot, w, (u + 1) * s / 8, 8);
-                    x = fma2(own.all, make_float2(0.5f, 0.5f), add2(after, behind.all));
-                    xx = fma2(own.xall, make_float2(0.5f, 0.5f), add2(xafter, behind.xall));
+                if (halves) {
+                    const RowSum low = row_sum<D>(sm, half_totals<D, 0>(tot, w)), high = row_sum<D>(sm, half_totals<D, 1>(tot, w));
+                    w1 = weight_of<D>(high, after);
+                    w2 = weight_of<D>(low, after + high);
+                } else if (s < T) {
+                    w1 = weight_of<D>(row_sum<D>(sm, window_totals<D>(tot, w, u * s / 8, (u + 1) * s / 8)),
+                                      after + row_sum<D>(sm, window_totals<D>(tot, w, (u + 1) * s / 8, 8)));
+                } else {
+                    w1 = weight_of<D>(mine, after);
                 }
-                w2 = w1;
-                w1 = weight_of<D>(sm, x, xx);
             }
-            after = add2(after, whole.all);
-            xafter = add2(xafter, whole.xall);
+            after = after + mine;
             if (tile > t0) {
                 group_prefix<D>(raw, nxt.g, w, sTot + ((tile - 1) & 1) * 8 * D);       // only the last tile of a sequence has a tail
                 if (tile - 2 >= t0) {
@@ -244,15 +261,11 @@ sweep_local_fwd(const SweepArgs a)
         }
         tc_fence_before_sync();
         SYNC_OR_DIE();
-        issue_step(it - 1);
-        if (n >= 2) add_step(it - 2, w2);
-        add_step(it - 1, w1);
+        issue_step();
+        add_step((it - 1) & 1);
         if (ok) acc_to_global<D>(tl + SM::aSum, sm, a.seg_state + (size_t)sid * D * D);
         tc_fence_before_sync();
-        if (w.grp == 0) {
-            *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.c2) = after;
-            if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.xc2) = xafter;
-        }
+        put_row_sums<D>(a.seg_gamma + (size_t)sid * D, w, sm, after);
     }
 die:
     cta_teardown(ctl, SM::tmem_cols);
@@ -305,7 +318,8 @@ sweep_local_bwd(const SweepArgs a)
     float S[L::NPS][8];
     Cols<D, GRAD, GRAD> raw;
     bool ok = true;
-    uint32_t it = 0;                                    // (sub-)chunks worked so far: buffer it & 1, its barrier's phase (it >> 1) & 1
+    uint32_t it = 0;                                    // (sub-)chunks worked so far: accumulators it & 1, their barrier's phase (it >> 1) & 1
+    uint32_t nbuf = 0;                                  // operand tiles built so far: buffer nbuf & 1
     const int total = g.B * g.H * pl.nseg;
 
     auto load_tile = [&](int tile) {
@@ -334,7 +348,7 @@ sweep_local_bwd(const SweepArgs a)
         const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
         get_state<D>(nullptr, sm, S);
-        float2 gsum = make_float2(0.f, 0.f), gxsum = gsum;             // gates since the segment start (log2), the thread's channels
+        RowSum since{0.f, 0.f};                                         // gates since the segment start
         pending = false;
         first = true;
         if (tid < 2 * T) rowOff[((t0 + (tid >> 6)) & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, t0 + (tid >> 6), tid & 63);
@@ -351,47 +365,58 @@ sweep_local_bwd(const SweepArgs a)
             float *tot = sTot + (tile & 1) * 8 * D;
             SYNC_OR_DIE();                                             // group totals are there
             if (tid < T && tile + 2 < t1) rowOff[((tile + 2) & 3) * T + tid] = tile_row_offset(g, pl, b, h, D, tile + 2, tid);
-            const Tot whole = tile_totals<D>(tot, w);
-            Tot tt = whole;
-            int s = T;
-            if (pl.sub_max < T || beyond<D>(tt)) {
-                s = choose_window<D>(tot, w, min(pl.sub_max, T / 2), a.status);
-                const int w0 = 8 * w.grp / s * (s / 8);
-                tt = window_totals<D>(tot, w, w0, w0 + s / 8);
-            }
+            Tot tt = tile_totals<D>(tot, w);
+            const RowSum mine = row_sum<D>(sm, tt);
+            const int s = divide_tile<D>(tot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
-            const int nsub = (nrow + s - 1) / s;
-            for (int u = 0; u < nsub; ++u, ++it) {
-                const int lo = u * s, hi = lo + s;
-                const bool last = u == nsub - 1, on = 8 * w.grp >= lo && 8 * w.grp < hi;
-                char *buf = smem + (it & 1) * SM::kBuf;
+            // Two sub-chunks of 32 rows: one pass, a product each in either accumulator, the state between them as soon as the
+            // first is done (nothing of them stays for the next pass).
+            const bool halves = s == T / 2 && nrow > T / 2;
+            const int step = halves ? T : s, nsub = (nrow + step - 1) / step, nslot = halves ? 2 : nsub;
+            for (int u = 0; u < nsub; ++u, ++it, ++nbuf) {
+                const int lo = u * step;
+                const bool last = u == nsub - 1, on = 8 * w.grp >= lo && 8 * w.grp < lo + step;
+                char *buf = smem + (nbuf & 1) * SM::kBuf;
                 char *tQ = buf, *tK = GRAD ? tQ + C::TILE_T : buf, *tV = tK + C::TILE_T, *tG = tV + C::TILE_T;
                 build_rows<D>(raw, w, tQ, tK, tV, tG, on);
-                Tot tu = whole;
-                float2 gs = gsum, gxs = gxsum;                         // decay before the sub-chunk
-                if (s < T) {
-                    tu = window_totals<D>(tot, w, 0, lo / 8);
-                    gs = add2(gs, tu.all);
-                    gxs = add2(gxs, tu.xall);
-                    tu = window_totals<D>(tot, w, lo / 8, hi / 8);
+                RowSum own, before = since;                            // gates of the sub-chunk and before it
+                if (halves) {
+                    own = row_sum<D>(sm, half_totals<D, 0>(tot, w));
+                } else if (s < T) {
+                    before = since + row_sum<D>(sm, window_totals<D>(tot, w, 0, lo / 8));
+                    own = row_sum<D>(sm, window_totals<D>(tot, w, lo / 8, (lo + s) / 8));
+                } else {
+                    own = mine;
                 }
-                const Decay now = decay_of<D>(sm, tu.all, tu.xall);
+                const Decay now = decay_of<D>(own);
                 Weight wnow{};
-                if (GRAD) wnow = weight_of<D>(sm, fma2(tu.all, make_float2(0.5f, 0.5f), gs), fma2(tu.xall, make_float2(0.5f, 0.5f), gxs));
-                const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
-                if (w.grp == 0) {
-                    *reinterpret_cast<float2 *>(a.slot_g + slot * D + w.c2) = gs;
-                    if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.slot_g + slot * D + w.xc2) = gxs;
+                if (GRAD) wnow = weight_of<D>(own, before);
+                size_t slot = ((size_t)(nslot - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
+                put_row_sums<D>(a.slot_g + slot * D, w, sm, before);
+                const bool late = L::X && halves;                      // registers: rows after the second half's state
+                if (last && more && !late) load_tile(tile + 1);
+                if (halves && pending) {                               // both accumulators have to be free
+                    fold(it - 1);
+                    pending = false;
                 }
-                if (last && more) load_tile(tile + 1);
                 fence_async_smem();
                 tc_fence_before_sync();
                 __syncthreads();
                 if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
-                    issue_state<D>(tmem + (it & 1) * L::ACCS, tK, tV);                             // Kc^T V
-                    if (GRAD) issue_state<D>(tmem + SM::aW + (it & 1) * L::ACCS, tQ, tG);          // Qc^T dO
-                    mma_commit(&ctl->bar[it & 1]);
+                    const uint32_t x = (it & 1) * L::ACCS, y = L::ACCS - x;
+                    if (!halves) {
+                        issue_state<D>(tmem + x, tK, tV);                                          // Kc^T V
+                        if (GRAD) issue_state<D>(tmem + SM::aW + x, tQ, tG);                       // Qc^T dO
+                        mma_commit(&ctl->bar[it & 1]);
+                    } else {
+                        issue_state<D, kLowRows>(tmem + x, tK, tV);
+                        if (GRAD) issue_state<D, kLowRows>(tmem + SM::aW + x, tQ, tG);
+                        mma_commit(&ctl->bar[it & 1]);
+                        issue_state<D, kHighRows>(tmem + y, tK, tV);
+                        if (GRAD) issue_state<D, kHighRows>(tmem + SM::aW + y, tQ, tG);
+                        mma_commit(&ctl->bar[(it + 1) & 1]);
+                    }
                 }
                 // the register prefetch alone does not cover the memory latency of tiles this short
                 if (last && tile + 2 < t1) prefetch_rows<D, GRAD, GRAD>(a.q, a.k, a.v, a.d_out, rowOff + ((tile + 2) & 3) * T, w);
@@ -401,9 +426,19 @@ sweep_local_bwd(const SweepArgs a)
                 wt = wnow;
                 put_state<D, D * 16>(reinterpret_cast<char *>(a.slot_s + slot * (D * D)), sm, S, dec);
                 pending = true;
+                if (halves) {
+                    fold(it++);
+                    before = since + own;
+                    own = row_sum<D>(sm, half_totals<D, 1>(tot, w));
+                    slot -= (size_t)g.B * g.H * pl.ntile;
+                    put_row_sums<D>(a.slot_g + slot * D, w, sm, before);
+                    dec = decay_of<D>(own);
+                    if (GRAD) wt = weight_of<D>(own, before);
+                    put_state<D, D * 16>(reinterpret_cast<char *>(a.slot_s + slot * (D * D)), sm, S, dec);
+                    if (late && more) load_tile(tile + 1);
+                }
             }
-            gsum = add2(gsum, whole.all);
-            gxsum = add2(gxsum, whole.xall);
+            since = since + mine;
             if (more) {                                                // the next tile's gate sums while the products run
                 const int nr = g.L - (tile + 1) * T;
                 if (nr < T) { clear_tail_rows(raw, w, nr); clear_tail_gates(raw, w, nr); }
@@ -413,10 +448,7 @@ sweep_local_bwd(const SweepArgs a)
         fold(it - 1);
         save_state<D>(a.seg_state + (size_t)sid * D * D, sm, S);
         if (GRAD && ok) acc_to_global<D>(tl + SM::aSum, sm, a.seg_dstate + (size_t)sid * D * D);
-        if (w.grp == 0) {
-            *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.c2) = gsum;
-            if (L::X && w.xrow == 0) *reinterpret_cast<float2 *>(a.seg_gamma + (size_t)sid * D + w.xc2) = gxsum;
-        }
+        put_row_sums<D>(a.seg_gamma + (size_t)sid * D, w, sm, since);
         tc_fence_before_sync();
     }
 die:
@@ -629,24 +661,23 @@ sweep_fwd(const SweepArgs a)
             SYNC_OR_DIE();                                       // group totals are there, the previous tile's products are done
             if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile + 1, tid);
             // Where some channel's gates sum to too much for one centring (or shorter chunks were asked for) the tile
-            // is worked in sub-chunks: the other rows of the operand tiles are zero, each has its own centring.
+            // is worked in sub-chunks with their own centring.  Two of 32 rows share one pass through the phases below
+            // (`halves`): both are built and scored at once, the state between them is formed after the scores and read by the
+            // upper half's rows alone.  Shorter ones take a pass each, the other rows of the operand tiles zero.
             const Tot whole = tile_totals<D>(sTot, w);
             Tot tt = whole;
-            int s = T;
-            if (pl.sub_max < T || beyond<D>(tt)) {
-                s = choose_window<D>(sTot, w, min(pl.sub_max, T / 2), a.status);
-                const int w0 = 8 * w.grp / s * (s / 8);
-                tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
-            }
+            const int s = divide_tile<D>(sTot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
-            const int nsub = (nrow + s - 1) / s;
+            const bool halves = s == T / 2 && nrow > T / 2;
+            const int step = halves ? T : s, nsub = (nrow + step - 1) / step;
             for (int u = 0; u < nsub; ++u) {
-                const int lo = u * s, hi = lo + s;
+                const int lo = u * step, hi = lo + step;
                 const bool last = u == nsub - 1;
                 build_rows<D>(raw, w, tQ, tK, tV, nullptr, 8 * w.grp >= lo && 8 * w.grp < hi);
                 Tot tu = whole;
-                if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
-                const Decay dec = decay_of<D>(sm, tu.all, tu.xall);
+                if (halves) tu = half_totals<D, 0>(sTot, w);
+                else if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
+                Decay dec = decay_of<D>(row_sum<D>(sm, tu));
                 put_state<D, C::CHS>(tS, sm, S, dec);            // Sc = diag(2^c) S
                 fence_async_smem();
                 tc_fence_before_sync();
@@ -654,15 +685,26 @@ sweep_fwd(const SweepArgs a)
                 if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
                     issue_scores<D>(tmem + SM::aP, tQ, tK);                                       // Qc Kc^T
-                    mma_commit(&ctl->bar[0]);
+                    if (!halves) mma_commit(&ctl->bar[0]);
                     issue_split<D, C::KS, C::CHS>(tmem + SM::aO, tQ, tS, false);                  // Qc Sc
-                    issue_state<D>(tmem + SM::aU, tK, tV);                                        // Kc^T V
+                    if (!halves) {
+                        issue_state<D>(tmem + SM::aU, tK, tV);                                    // Kc^T V
+                    } else {
+                        issue_state<D, kLowRows>(tmem + SM::aU, tK, tV);
+                        mma_commit(&ctl->bar[0]);
+                    }
                 }
                 if (staged) flush_rows<D>(out, stage, rowOff + prv * T, w, staged, a.accumulate != 0);
                 staged = 0;
                 if (last && more) load_tile(nxt);
                 ok = wait_all(&ctl->bar[0], 0, a.status, ok);          // completes twice per iteration: parities 0, 1
                 tc_fence_after_sync();
+                if (halves && ok) {                                    // the state between the halves
+                    fold_state<D>(tl + SM::aU, sm, S, dec);
+                    tu = half_totals<D, 1>(sTot, w);
+                    dec = decay_of<D>(row_sum<D>(sm, tu));
+                    put_state<D, C::CHS>(tS, sm, S, dec);
+                }
                 // Scores of row r16: lanes 0-15 hold the even 8-token chunks, lanes 16-31 the odd ones.  Keep s <= t, the
                 // diagonal has weight 1.  Chunks above the diagonal of all 16 rows of the warp are never written (the tile
                 // starts out zero), pairs below it need no selects.
@@ -676,6 +718,9 @@ sweep_fwd(const SweepArgs a)
                         if (pr == w.q4) {
 #pragma unroll
                             for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= w.r16) ? p[e] : 0.f;
+                        } else if (halves && pr < 2 && w.q4 >= 2) {        // the lower half acts on the upper one through the state
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) p[e] = 0.f;
                         }
                         *reinterpret_cast<uint4 *>(tP + sc * C::CHT + w.r16 * 16) = pack_h8(p);
                     }
@@ -685,6 +730,10 @@ sweep_fwd(const SweepArgs a)
                 __syncthreads();
                 if (w.issuer() && elect_one()) {
                     tc_fence_after_sync();
+                    if (halves) {
+                        issue_split<D, C::KS, C::CHS, kHighRows>(tmem + SM::aO, tQ, tS, false);
+                        issue_state<D, kHighRows>(tmem + SM::aU, tK, tV);
+                    }
                     issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);                  // + P V
                     mma_commit(&ctl->bar[0]);
                 }
@@ -749,7 +798,7 @@ struct BwdSmem {
     static constexpr bool kStage = D == 64 || sizeof(TO) == 2, kOwnStage = D == 64;
     static constexpr int kStageBytes = kOwnStage ? Staging<D, TO>::kBytes : 0;
     static_assert(!kStage || kOwnStage || Staging<D, TO>::kBytes <= C::NCH * C::CHS, "the state tile's zero chunk stays clean");
-    static constexpr size_t bytes = kTiles + kStageBytes + (2 * 8 * D + D) * 4 + 2 * T * 4 + sizeof(Ctl);
+    static constexpr size_t bytes = kTiles + kStageBytes + (2 * 8 * D + 2 * D) * 4 + 2 * T * 4 + sizeof(Ctl);
     static constexpr uint32_t aP = 0, aQK = 64, aV = aQK + D, aW = aV + D;     // accumulator columns
     static constexpr uint32_t tmem_cols = 256;
     static_assert(aW + L::ACCS <= tmem_cols, "tensor memory");
@@ -775,7 +824,7 @@ sweep_bwd(const SweepArgs a)
     float *bufQ = reinterpret_cast<float *>(tV), *bufK = bufQ + T * SM::LDP;
     char *stage = SM::kOwnStage ? smem + SM::kTiles : tS;
     float *sTot = reinterpret_cast<float *>(smem + SM::kTiles + SM::kStageBytes), *sX = sTot + 8 * D, *sAux = sX + 8 * D;
-    int *rowOff = reinterpret_cast<int *>(sAux + D);
+    int *rowOff = reinterpret_cast<int *>(sAux + 2 * D);
     Ctl *ctl = reinterpret_cast<Ctl *>(rowOff + 2 * T);
 
     const int tid = threadIdx.x;
@@ -856,23 +905,23 @@ sweep_bwd(const SweepArgs a)
             if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 1, tid);
             const Tot whole = tile_totals<D>(sTot, w);
             Tot tt = whole;
-            int s = T;
-            if (pl.sub_max < T || beyond<D>(tt)) {
-                s = choose_window<D>(sTot, w, min(pl.sub_max, T / 2), a.status);
-                const int w0 = 8 * w.grp / s * (s / 8);
-                tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
-            }
+            const int s = divide_tile<D>(sTot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
-            const int nsub = (nrow + s - 1) / s;
+            // Two sub-chunks of 32 rows share one pass: both are built, scored and finished at once; the upper half's products
+            // with the gradient and the states come with the scores, the lower half's with the second group of products, once
+            // the gradient between the halves is known.
+            const bool halves = s == T / 2 && nrow > T / 2;
+            const int step = halves ? T : s, nsub = (nrow + step - 1) / step;
             float2 tot = make_float2(0.f, 0.f), xtot = tot;      // sums of q dq - k dk over the group
             for (int u = nsub - 1; u >= 0; --u) {
-                const int lo = u * s, hi = lo + s;
+                const int lo = u * step, hi = lo + step;
                 const bool mine = 8 * w.grp >= lo && 8 * w.grp < hi;
                 const size_t slot = ((size_t)(nsub - 1 - u) * g.B * g.H + bh) * pl.ntile + tile;
                 build_rows<D>(raw, w, tQ, tK, tV, tG, mine);
                 Tot tu = whole;
-                if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
-                const Decay dec = decay_of<D>(sm, tu.all, tu.xall);
+                if (halves) tu = half_totals<D, 1>(sTot, w);
+                else if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
+                Decay dec = decay_of<D>(row_sum<D>(sm, tu));
                 put_state<D, C::CHS>(tD, sm, Dst, dec);          // Dc = diag(2^c) D
                 if (L::X) clear_pads<D>(tV, tG, tD);
                 fence_async_smem();
@@ -885,20 +934,30 @@ sweep_bwd(const SweepArgs a)
                     const uint32_t sS = smem_u32(tS), sI = smem_u32(tI), sD = smem_u32(tD);
                     issue<64, 64, false, false, C::KS, C::CHT, C::CHT>(tmem + SM::aP, sQ, sK, false);                   // Qc Kc^T
                     issue<64, 64, false, false, C::KS, C::CHT, C::CHT>(tmem + SM::aP + kHiLanes, sG, sV, false);        // dO V^T
-                    mma_commit(barG1);
+                    if (!halves) mma_commit(barG1);
                     issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + SM::aQK, sG, sS, false);                   // dO Sc_local^T
                     if (entry) issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + SM::aV, sG, sI, false);         // dO S_segment^T
                     issue<64, D, false, false, C::KS, C::CHT, C::CHS>(tmem + SM::aQK + kHiLanes, sV, sD, false);        // V Dc^T
                     issue<64, D, false, true, C::KS, C::CHT, C::CHS>(tmem + SM::aV + kHiLanes, sK, sD, false);          // Kc Dc
-                    issue_state<D>(tmem + SM::aW, tQ, tG);                                                              // Qc^T dO
-                }
-                if (entry && w.grp == 0) {                       // decay from the segment start to the sub-chunk's centre
-                    const float2 G = *reinterpret_cast<const float2 *>(a.slot_g + slot * D + w.c2);
-                    *reinterpret_cast<float2 *>(sAux + w.c2) = make_float2(ex2(0.5f * tu.all.x + G.x), ex2(0.5f * tu.all.y + G.y));
-                    if (L::X && w.xrow == 0) {
-                        const float2 X = *reinterpret_cast<const float2 *>(a.slot_g + slot * D + w.xc2);
-                        *reinterpret_cast<float2 *>(sAux + w.xc2) = make_float2(ex2(0.5f * tu.xall.x + X.x), ex2(0.5f * tu.xall.y + X.y));
+                    if (!halves) {
+                        issue_state<D>(tmem + SM::aW, tQ, tG);                                                          // Qc^T dO
+                    } else {
+                        issue_state<D, kHighRows>(tmem + SM::aW, tQ, tG);
+                        mma_commit(barG1);
                     }
+                }
+                // decay from the segment start to a sub-chunk's centre; the lower half's in the second row of sAux
+                auto put_aux = [&](float *aux, size_t sl, const Tot &t) {
+                    const float2 G = *reinterpret_cast<const float2 *>(a.slot_g + sl * D + w.c2);
+                    *reinterpret_cast<float2 *>(aux + w.c2) = make_float2(ex2(0.5f * t.all.x + G.x), ex2(0.5f * t.all.y + G.y));
+                    if (L::X && w.xrow == 0) {
+                        const float2 X = *reinterpret_cast<const float2 *>(a.slot_g + sl * D + w.xc2);
+                        *reinterpret_cast<float2 *>(aux + w.xc2) = make_float2(ex2(0.5f * t.xall.x + X.x), ex2(0.5f * t.xall.y + X.y));
+                    }
+                };
+                if (entry && w.grp == 0) {
+                    put_aux(sAux, slot, tu);
+                    if (halves) put_aux(sAux + D, slot + (size_t)g.B * g.H * pl.ntile, half_totals<D, 0>(sTot, w));
                 }
                 if (u == 0 && more) {
                     prefetch_gates<D>(a.gate, rowOff + nxt * T, w);
@@ -911,6 +970,14 @@ sweep_bwd(const SweepArgs a)
                 }
                 ok = wait_all(barG1, 0, a.status, ok);         // completes twice per iteration: parities 0, 1
                 tc_fence_after_sync();
+                if (halves && ok) {
+                    fetch_next(bh, slot, 1, tile, more);         // the lower half's state
+                    fold_state<D>(tl + SM::aW, sm, Dst, dec);
+                    tu = half_totals<D, 0>(sTot, w);
+                    dec = decay_of<D>(row_sum<D>(sm, tu));
+                    put_state<D, C::CHS>(tD, sm, Dst, dec);
+                    par ^= 1;
+                }
                 // lanes 0-15: scores, lanes 16-31: dO V^T; keep s <= t, the diagonal has weight 1.  Column chunks
                 // entirely above the diagonal for all rows of the warp are never written (the tiles start out zero),
                 // chunks entirely below it need no selects.
@@ -924,6 +991,9 @@ sweep_bwd(const SweepArgs a)
                             if (i == w.q4) {
 #pragma unroll
                                 for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= w.r16) ? p[e] : 0.f;
+                            } else if (halves && i < 2 && w.q4 >= 2) {       // the halves meet through the states only
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) p[e] = 0.f;
                             }
                             *reinterpret_cast<uint4 *>((w.hf ? tdP : tP) + sc * C::CHT + w.r16 * 16) = pack_h8(p);
                         }
@@ -936,9 +1006,19 @@ sweep_bwd(const SweepArgs a)
                     tc_fence_after_sync();
                     const uint32_t sQ = smem_u32(tQ), sK = smem_u32(tK), sG = smem_u32(tG);
                     const uint32_t sP = smem_u32(tP), sdP = smem_u32(tdP);
-                    issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK, sdP, sK, true);                   // + dP Kc
+                    if (halves) {
+                        const uint32_t sV = smem_u32(tV), sD = smem_u32(tD);
+                        issue<64, D, false, false, C::KS, C::CHT, C::CHS, 128, kLowRows>(tmem + SM::aQK + kHiLanes, sV, sD, false);
+                        issue<64, D, false, true, C::KS, C::CHT, C::CHS, 128, kLowRows>(tmem + SM::aV + kHiLanes, sK, sD, false);
+                        issue_state<D, kLowRows>(tmem + SM::aW, tQ, tG);
+                    }
                     issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK + kHiLanes, sdP, sQ, true);         // + dP^T Qc
                     issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aV + kHiLanes, sP, sG, true);           // + P^T dO
+                    if (halves) {
+                        ok = mbar_wait(barS, par, a.status) && ok;
+                        issue<64, D, false, false, C::KS, C::CHT, C::CHS, 128, kLowRows>(tmem + SM::aQK, sG, smem_u32(tS), false);
+                    }
+                    issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK, sdP, sK, true);                   // + dP Kc
                     mma_commit(barG1);
                 }
                 ok = wait_all(barG1, 1, a.status, ok);
@@ -961,7 +1041,7 @@ sweep_bwd(const SweepArgs a)
                                 }
                             } else if (entry) {
                                 float hh[8];
-                                ld8(sAux + 8 * jc, hh);
+                                ld8((halves && w.q4 < 2 ? sAux + D : sAux) + 8 * jc, hh);
 #pragma unroll
                                 for (int e = 0; e < 8; ++e) x0[e] = fmaf(hh[e], x1[e], x0[e]);
                             }

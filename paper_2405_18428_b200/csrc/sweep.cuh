@@ -123,8 +123,9 @@ __device__ __forceinline__ uint64_t mdesc(uint32_t saddr, uint32_t ch) { return 
 // of the first element the product uses (a row or chunk offset selects a slice), ach / bch: chunk
 // strides of the tiles (compile-time, so every descriptor is the first one plus a constant in its
 // low word: shared-memory addresses stay below 2^18, the address field cannot carry into the next).
-// BSBO: distance of the 8-row groups of a K-major B (256 takes every other group).
-template <int M, int N, bool A_MN, bool B_MN, int KSTEPS, uint32_t ACH, uint32_t BCH, uint32_t BSBO = 128>
+// BSBO: distance of the 8-row groups of a K-major B (256 takes every other group).  SKIP: quarters of the
+// accumulator's lanes that stay as they are (rows 16 q .. 16 q + 15 of an M = 64 product are in quarter q).
+template <int M, int N, bool A_MN, bool B_MN, int KSTEPS, uint32_t ACH, uint32_t BCH, uint32_t BSBO = 128, uint32_t SKIP = 0>
 __device__ __forceinline__ void issue(uint32_t d_tmem, uint32_t a, uint32_t b, bool accumulate)
 {
     static_assert(M == 64 && N % 8 == 0, "instruction shape");
@@ -135,7 +136,8 @@ __device__ __forceinline__ void issue(uint32_t d_tmem, uint32_t a, uint32_t b, b
 #pragma unroll
     for (int kk = 0; kk < KSTEPS; ++kk) {
         const uint64_t xa = ((uint64_t)ahi << 32) | (alo + kk * sa), xb = ((uint64_t)bhi << 32) | (blo + kk * sb);
-        mma_f16(d_tmem, xa, xb, idesc, accumulate || kk > 0);
+        if constexpr (SKIP == 0) mma_f16(d_tmem, xa, xb, idesc, accumulate || kk > 0);
+        else mma_f16_part<SKIP>(d_tmem, xa, xb, idesc, accumulate || kk > 0);
     }
 }
 

@@ -53,6 +53,17 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
 }
+// The same for the accumulator lanes outside the quarters of 32 lanes named by SKIP (bit q: lanes 32 q .. 32 q + 31 keep
+// what they hold).
+template <uint32_t SKIP>
+__device__ __forceinline__ void mma_f16_part(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate)
+{
+    constexpr uint32_t m0 = SKIP & 1 ? ~0u : 0u, m1 = SKIP & 2 ? ~0u : 0u, m2 = SKIP & 4 ? ~0u : 0u, m3 = SKIP & 8 ? ~0u : 0u;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+        :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(m0), "r"(m1), "r"(m2), "r"(m3) : "memory");
+}
 
 // Arrive on an mbarrier once every tcgen05.mma issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
