@@ -29,7 +29,8 @@
 // block-diagonal, and only what acts through the state or its gradient is done per half, the later half with the second
 // group of products.  The results are those of two passes bit for bit.  48 sequences of 1961 tokens in chunks of 32, d = 72:
 // the four kernels 42 + 56 + 76 + 108 us with a pass per half, 28 + 38 + 56 + 84 now; 48 of 4096, d = 64, half of the heads at
-// tau = 4, where one tile in six is divided and the CTA with most of them is the last: 35 + 49 + 48 + 94, now 30 + 43 + 46 + 86.
+// tau = 4, where one tile in six is divided and the CTA with most of them is the last: 35 + 49 + 48 + 94, now 30 + 42 + 46 + 94 (the
+// backward sweep shares a pass in chunks of 32 only).
 //
 // Every product is a tcgen05.mma (kind::f16, fp16 operands, fp32 accumulators in tensor memory) issued by
 // one thread of the last warp, which otherwise works like the others: all threads build operand tiles, mask the
@@ -59,6 +60,11 @@ struct SweepArgs {
     int scanned;            // backward pass: a segment scan ran (else every segment's entry state, gradient and carry are zero)
     Geom g;
     Plan plan;
+};
+
+// A condition known to the compiler, for code that also takes a bool.
+template <bool B> struct Const {
+    __device__ constexpr operator bool() const { return B; }
 };
 
 // ---- shared phases ------------------------------------------------------------------------------
@@ -668,99 +674,112 @@ sweep_fwd(const SweepArgs a)
             Tot tt = whole;
             const int s = divide_tile<D>(sTot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
-            const bool halves = s == T / 2 && nrow > T / 2;
-            const int step = halves ? T : s, nsub = (nrow + step - 1) / step;
-            for (int u = 0; u < nsub; ++u) {
-                const int lo = u * step, hi = lo + step;
-                const bool last = u == nsub - 1;
-                build_rows<D>(raw, w, tQ, tK, tV, nullptr, 8 * w.grp >= lo && 8 * w.grp < hi);
-                Tot tu = whole;
-                if (halves) tu = half_totals<D, 0>(sTot, w);
-                else if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
-                Decay dec = decay_of<D>(row_sum<D>(sm, tu));
-                put_state<D, C::CHS>(tS, sm, S, dec);            // Sc = diag(2^c) S
-                fence_async_smem();
-                tc_fence_before_sync();
-                __syncthreads();
-                if (w.issuer() && elect_one()) {
+            // At d = 64 the two kinds of pass are compiled apart (768 sequences of 256 tokens 49.2 us without halves, 50.9
+            // with the branches, 50.0 so); at d = 72 registers would spill.
+            auto passes = [&](auto kind) {
+                const bool halves = kind;
+                const int step = halves ? T : s, nsub = halves ? 1 : (nrow + step - 1) / step;
+                for (int u = 0; u < nsub; ++u) {
+                    const int lo = u * step, hi = lo + step;
+                    const bool last = u == nsub - 1;
+                    build_rows<D>(raw, w, tQ, tK, tV, nullptr, 8 * w.grp >= lo && 8 * w.grp < hi);
+                    Tot tu = whole;
+                    if (halves) tu = half_totals<D, 0>(sTot, w);
+                    else if (s < T) tu = window_totals<D>(sTot, w, lo / 8, hi / 8);
+                    Decay dec = decay_of<D>(row_sum<D>(sm, tu));
+                    put_state<D, C::CHS>(tS, sm, S, dec);            // Sc = diag(2^c) S
+                    fence_async_smem();
+                    tc_fence_before_sync();
+                    __syncthreads();
+                    if (w.issuer() && elect_one()) {
+                        tc_fence_after_sync();
+                        issue_scores<D>(tmem + SM::aP, tQ, tK);                                       // Qc Kc^T
+                        if (!halves) mma_commit(&ctl->bar[0]);
+                        issue_split<D, C::KS, C::CHS>(tmem + SM::aO, tQ, tS, false);                  // Qc Sc
+                        if (!halves) {
+                            issue_state<D>(tmem + SM::aU, tK, tV);                                    // Kc^T V
+                        } else {
+                            issue_state<D, kLowRows>(tmem + SM::aU, tK, tV);
+                            mma_commit(&ctl->bar[0]);
+                        }
+                    }
+                    if (staged) flush_rows<D>(out, stage, rowOff + prv * T, w, staged, a.accumulate != 0);
+                    staged = 0;
+                    if (last && more) load_tile(nxt);
+                    ok = wait_all(&ctl->bar[0], 0, a.status, ok);          // completes twice per iteration: parities 0, 1
                     tc_fence_after_sync();
-                    issue_scores<D>(tmem + SM::aP, tQ, tK);                                       // Qc Kc^T
-                    if (!halves) mma_commit(&ctl->bar[0]);
-                    issue_split<D, C::KS, C::CHS>(tmem + SM::aO, tQ, tS, false);                  // Qc Sc
-                    if (!halves) {
-                        issue_state<D>(tmem + SM::aU, tK, tV);                                    // Kc^T V
-                    } else {
-                        issue_state<D, kLowRows>(tmem + SM::aU, tK, tV);
+                    if (halves && ok) {                                    // the state between the halves
+                        fold_state<D>(tl + SM::aU, sm, S, dec);
+                        tu = half_totals<D, 1>(sTot, w);
+                        dec = decay_of<D>(row_sum<D>(sm, tu));
+                        put_state<D, C::CHS>(tS, sm, S, dec);
+                    }
+                    // Scores of row r16: lanes 0-15 hold the even 8-token chunks, lanes 16-31 the odd ones.  Keep s <= t, the
+                    // diagonal has weight 1.  Chunks above the diagonal of all 16 rows of the warp are never written (the tile
+                    // starts out zero), pairs below it need no selects.
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int pr = w.cg + 2 * i;
+                        if (ok && pr <= w.q4) {                // uniform over the warp
+                            float p[8];
+                            tmem_ld8(tl + SM::aP + 8 * pr, p);
+                            const int sc = 2 * pr + w.hf;
+                            if (pr == w.q4) {
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= w.r16) ? p[e] : 0.f;
+                            } else if (halves && pr < 2 && w.q4 >= 2) {        // the lower half acts on the upper one through the state
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) p[e] = 0.f;
+                            }
+                            *reinterpret_cast<uint4 *>(tP + sc * C::CHT + w.r16 * 16) = pack_h8(p);
+                        }
+                    }
+                    fence_async_smem();
+                    tc_fence_before_sync();
+                    __syncthreads();
+                    if (w.issuer() && elect_one()) {
+                        tc_fence_after_sync();
+                        if (halves) {
+                            issue_split<D, C::KS, C::CHS, kHighRows>(tmem + SM::aO, tQ, tS, false);
+                            issue_state<D, kHighRows>(tmem + SM::aU, tK, tV);
+                        }
+                        issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);                  // + P V
                         mma_commit(&ctl->bar[0]);
                     }
-                }
-                if (staged) flush_rows<D>(out, stage, rowOff + prv * T, w, staged, a.accumulate != 0);
-                staged = 0;
-                if (last && more) load_tile(nxt);
-                ok = wait_all(&ctl->bar[0], 0, a.status, ok);          // completes twice per iteration: parities 0, 1
-                tc_fence_after_sync();
-                if (halves && ok) {                                    // the state between the halves
-                    fold_state<D>(tl + SM::aU, sm, S, dec);
-                    tu = half_totals<D, 1>(sTot, w);
-                    dec = decay_of<D>(row_sum<D>(sm, tu));
-                    put_state<D, C::CHS>(tS, sm, S, dec);
-                }
-                // Scores of row r16: lanes 0-15 hold the even 8-token chunks, lanes 16-31 the odd ones.  Keep s <= t, the
-                // diagonal has weight 1.  Chunks above the diagonal of all 16 rows of the warp are never written (the tile
-                // starts out zero), pairs below it need no selects.
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int pr = w.cg + 2 * i;
-                    if (ok && pr <= w.q4) {                // uniform over the warp
-                        float p[8];
-                        tmem_ld8(tl + SM::aP + 8 * pr, p);
-                        const int sc = 2 * pr + w.hf;
-                        if (pr == w.q4) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) p[e] = (8 * sc + e <= w.r16) ? p[e] : 0.f;
-                        } else if (halves && pr < 2 && w.q4 >= 2) {        // the lower half acts on the upper one through the state
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) p[e] = 0.f;
-                        }
-                        *reinterpret_cast<uint4 *>(tP + sc * C::CHT + w.r16 * 16) = pack_h8(p);
+                    if (last && more) {                                // the next tile's gate sums while the products run
+                        const int nr = g.L - (tile + 1) * T;
+                        if (nr < T) { clear_tail_rows(raw, w, nr); clear_tail_gates(raw, w, nr); }
+                        group_prefix<D>(raw, raw.g, w, sTot);
                     }
-                }
-                fence_async_smem();
-                tc_fence_before_sync();
-                __syncthreads();
-                if (w.issuer() && elect_one()) {
+                    ok = wait_all(&ctl->bar[0], 1, a.status, ok);
                     tc_fence_after_sync();
-                    if (halves) {
-                        issue_split<D, C::KS, C::CHS, kHighRows>(tmem + SM::aO, tQ, tS, false);
-                        issue_state<D, kHighRows>(tmem + SM::aU, tK, tV);
-                    }
-                    issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);                  // + P V
-                    mma_commit(&ctl->bar[0]);
-                }
-                if (last && more) {                                // the next tile's gate sums while the products run
-                    const int nr = g.L - (tile + 1) * T;
-                    if (nr < T) { clear_tail_rows(raw, w, nr); clear_tail_gates(raw, w, nr); }
-                    group_prefix<D>(raw, raw.g, w, sTot);
-                }
-                ok = wait_all(&ctl->bar[0], 1, a.status, ok);
-                tc_fence_after_sync();
-                if (ok) {
-                    const bool inrow = w.r16 >= lo && w.r16 < min(hi, nrow);
+                    if (ok) {
+                        const bool inrow = w.r16 >= lo && w.r16 < min(hi, nrow);
 #pragma unroll
-                    for (int i = 0; i < L::NPO; ++i) {
-                        const int jc = w.cg + 2 * i;
-                        if (jc < L::NV0) {                        // uniform over the warp
-                            float o[8];
-                            tmem_ld8(tl + SM::aO + 8 * jc, o);
-                            if (inrow && jc < (w.hf ? L::NV1 : L::NV0)) stage_row<D, TO>(stage, w.r16, (w.hf ? L::NV0 : 0) + jc, o);
+                        for (int i = 0; i < L::NPO; ++i) {
+                            const int jc = w.cg + 2 * i;
+                            if (jc < L::NV0) {                        // uniform over the warp
+                                float o[8];
+                                tmem_ld8(tl + SM::aO + 8 * jc, o);
+                                if (inrow && jc < (w.hf ? L::NV1 : L::NV0)) stage_row<D, TO>(stage, w.r16, (w.hf ? L::NV0 : 0) + jc, o);
+                            }
                         }
+                        fold_state<D>(tl + SM::aU, sm, S, dec);
                     }
-                    fold_state<D>(tl + SM::aU, sm, S, dec);
+                    if (!last) {                              // the operand tiles and the accumulators are free again
+                        tc_fence_before_sync();
+                        if (!__syncthreads_and(ok)) return false;
+                    }
                 }
-                if (!last) {                              // the operand tiles and the accumulators are free again
-                    tc_fence_before_sync();
-                    SYNC_OR_DIE();
-                }
+                return true;
+            };
+            const bool two = s == T / 2 && nrow > T / 2;
+            bool done;
+            if constexpr (L::X) done = passes(two);
+            else done = two ? passes(Const<true>{}) : passes(Const<false>{});
+            if (!done) {
+                ok = false;
+                goto die;
             }
             staged = nrow;
             cur = nxt;
@@ -780,6 +799,10 @@ die:
 // After the second group of products the dq and dk accumulators go through shared memory (over the
 // operand tiles that are spent by then) to the column threads, which still hold the decay exponents of
 // their rows: they scale and store dq and dk, form q dq - k dk and sum it down their rows.
+// PAIRS: two sub-chunks of 32 rows share a pass.  Only for chunks of 32: the code for it slows whole tiles down by 4% at
+// d = 64 (92.4 -> 96 us on 768 sequences of 256 tokens) and 2.5% at d = 72, also compiled apart per tile (101 us, spills) or per
+// CTA (98.7; short launches then wait for instructions: 25.4 -> 34 us on 48 sequences of 1024).  Tiles that are divided
+// without it take a pass per half, with the same bits and the same slots.
 // Bound by latency like the forward sweep.  48 sequences of 4096 tokens, d = 64: 140 us with the row-chunk work
 // split, 94 us now; 16 of 16384, d = 72: 252 -> 181 us.
 // =================================================================================================
@@ -811,7 +834,7 @@ __device__ __forceinline__ void store_pair(float *p, float x, float y, bool add)
 }
 __device__ __forceinline__ void store_pair(bf16 *p, float x, float y, bool) { *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(x, y); }
 
-template <int D, typename TO>
+template <int D, typename TO, bool PAIRS>
 __global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_bwd(const SweepArgs a)
 {
@@ -910,7 +933,7 @@ sweep_bwd(const SweepArgs a)
             // Two sub-chunks of 32 rows share one pass: both are built, scored and finished at once; the upper half's products
             // with the gradient and the states come with the scores, the lower half's with the second group of products, once
             // the gradient between the halves is known.
-            const bool halves = s == T / 2 && nrow > T / 2;
+            const bool halves = PAIRS && s == T / 2 && nrow > T / 2;
             const int step = halves ? T : s, nsub = (nrow + step - 1) / step;
             float2 tot = make_float2(0.f, 0.f), xtot = tot;      // sums of q dq - k dk over the group
             for (int u = nsub - 1; u >= 0; --u) {
@@ -1012,13 +1035,13 @@ sweep_bwd(const SweepArgs a)
                         issue<64, D, false, true, C::KS, C::CHT, C::CHS, 128, kLowRows>(tmem + SM::aV + kHiLanes, sK, sD, false);
                         issue_state<D, kLowRows>(tmem + SM::aW, tQ, tG);
                     }
-                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK + kHiLanes, sdP, sQ, true);         // + dP^T Qc
-                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aV + kHiLanes, sP, sG, true);           // + P^T dO
                     if (halves) {
                         ok = mbar_wait(barS, par, a.status) && ok;
                         issue<64, D, false, false, C::KS, C::CHT, C::CHS, 128, kLowRows>(tmem + SM::aQK, sG, smem_u32(tS), false);
                     }
                     issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK, sdP, sK, true);                   // + dP Kc
+                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK + kHiLanes, sdP, sQ, true);         // + dP^T Qc
+                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aV + kHiLanes, sP, sG, true);           // + P^T dO
                     mma_commit(barG1);
                 }
                 ok = wait_all(barG1, 1, a.status, ok);
@@ -1283,8 +1306,9 @@ dig_status run(const GlaArgs &ga)
         launch_pdl(f32 ? k32 : k16, grid, block, f32 ? smem32 : smem16, ga.stream, a);
     } else {
         constexpr size_t smem16 = BwdSmem<D, bf16>::bytes, smem32 = BwdSmem<D, float>::bytes;
-        auto k16 = sweep_bwd<D, bf16>;
-        auto k32 = sweep_bwd<D, float>;
+        const bool pairs = pl.sub_max == T / 2;
+        auto k16 = pairs ? sweep_bwd<D, bf16, true> : sweep_bwd<D, bf16, false>;
+        auto k32 = pairs ? sweep_bwd<D, float, true> : sweep_bwd<D, float, false>;
         if ((st = set_smem(k16, smem16)) != DIG_OK || (st = set_smem(k32, smem32)) != DIG_OK) return st;
         KernelTimer t(KID_SW_BWD, ga.stream);
         launch_pdl(f32 ? k32 : k16, grid, block, f32 ? smem32 : smem16, ga.stream, a);
