@@ -369,10 +369,10 @@ __device__ __forceinline__ void put_pair(float *dst, float2 v, bool add)
     else *reinterpret_cast<float2 *>(dst) = v;
 }
 __device__ __forceinline__ void put_pair(bf16 *dst, uint32_t v, bool) { *reinterpret_cast<uint32_t *>(dst) = v; }
-// The thread's items of the staged tile to global memory (rows below nrow).  All shared-memory loads first: a
+// The thread's items of the staged tile to global memory (rows below nrow), `oo` elements behind dst.  All shared-memory loads first: a
 // load and a store per row in turn took 850 cycles per tile.
 template <int D, typename TO>
-__device__ __forceinline__ void flush_rows(TO *dst, const char *stage, const int *row_off, const Who<D> &w, int nrow, bool add)
+__device__ __forceinline__ void flush_rows(TO *dst, uint32_t oo, const char *stage, const int *row_off, const Who<D> &w, int nrow, bool add)
 {
     constexpr int N = Col<D>::X ? 9 : 8;
     uint32_t off[9];
@@ -383,11 +383,11 @@ __device__ __forceinline__ void flush_rows(TO *dst, const char *stage, const int
         v[j] = *reinterpret_cast<const typename Pair<TO>::type *>(stage + item_row(w, j) * Staging<D, TO>::kStride + (j < 8 ? w.c2 : w.xc2) * (int)sizeof(TO));
     if (nrow == T) {
 #pragma unroll
-        for (int j = 0; j < N; ++j) put_pair(dst + off[j], v[j], add);
+        for (int j = 0; j < N; ++j) put_pair(dst + (off[j] + oo), v[j], add);
     } else {
 #pragma unroll
         for (int j = 0; j < N; ++j)
-            if (item_row(w, j) < nrow) put_pair(dst + off[j], v[j], add);
+            if (item_row(w, j) < nrow) put_pair(dst + (off[j] + oo), v[j], add);
     }
 }
 

@@ -60,7 +60,30 @@ struct SweepArgs {
     int scanned;            // backward pass: a segment scan ran (else every segment's entry state, gradient and carry are zero)
     Geom g;
     Plan plan;
+    // Several scan orders in one forward launch: g.B = batch * orders sequences per head; order i (two bits each in dirs) reads
+    // the same inputs and writes out_stride elements behind the one before.
+    int batch;
+    uint32_t dirs, out_stride;
 };
+
+// Batch entry, head, scan order and place of the results of sequence bh.  ORDERS: of several scan orders in one launch.
+struct Seq {
+    int b, h, dir;
+    uint32_t oo;
+};
+template <bool ORDERS>
+__device__ __forceinline__ Seq seq_of(const SweepArgs &a, int bh)
+{
+    Seq s{bh / a.g.H, 0, a.g.dir, 0u};
+    s.h = bh - s.b * a.g.H;
+    if (ORDERS) {
+        const int i = s.b / a.batch;
+        s.b -= i * a.batch;
+        s.dir = (int)(a.dirs >> (2 * i)) & 3;
+        s.oo = (uint32_t)i * a.out_stride;
+    }
+    return s;
+}
 
 // A condition known to the compiler, for code that also takes a bool.
 template <bool B> struct Const {
@@ -129,7 +152,7 @@ struct LocalFwdSmem {
     static constexpr uint32_t tmem_cols = 3 * L::ACCS <= 128 ? 128 : 256;
 };
 
-template <int D>
+template <int D, bool ORDERS>
 __global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_local_fwd(const SweepArgs a)
 {
@@ -183,14 +206,15 @@ sweep_local_fwd(const SweepArgs a)
 
     pdl_wait();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
-        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
+        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg;
+        const Seq sq = seq_of<ORDERS>(a, bh);
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
         first = true;
         RowSum after{0.f, 0.f};                                         // gates of the tiles behind
         pending = false;
         if (tid < 3 * T && t1 - 1 - (tid >> 6) >= t0) {
             const int tile = t1 - 1 - (tid >> 6);
-            rowOff[(tile & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, tile, tid & 63);
+            rowOff[(tile & 3) * T + (tid & 63)] = tile_row_offset(g, pl, sq.dir, sq.b, sq.h, D, tile, tid & 63);
         }
         __syncthreads();
         {
@@ -212,7 +236,7 @@ sweep_local_fwd(const SweepArgs a)
             tc_fence_before_sync();
             SYNC_OR_DIE();                                             // group totals are there, the step before is built
             if (pending) issue_step();
-            if (tid < T && tile - 3 >= t0) rowOff[((tile - 3) & 3) * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 3, tid);
+            if (tid < T && tile - 3 >= t0) rowOff[((tile - 3) & 3) * T + tid] = tile_row_offset(g, pl, sq.dir, sq.b, sq.h, D, tile - 3, tid);
             if (tile > t0) {
                 uint32_t ro[9];
                 row_offsets<D>(rowOff + ((tile - 1) & 3) * T, w, ro);
@@ -357,7 +381,7 @@ sweep_local_bwd(const SweepArgs a)
         RowSum since{0.f, 0.f};                                         // gates since the segment start
         pending = false;
         first = true;
-        if (tid < 2 * T) rowOff[((t0 + (tid >> 6)) & 3) * T + (tid & 63)] = tile_row_offset(g, pl, b, h, D, t0 + (tid >> 6), tid & 63);
+        if (tid < 2 * T) rowOff[((t0 + (tid >> 6)) & 3) * T + (tid & 63)] = tile_row_offset(g, pl, g.dir, b, h, D, t0 + (tid >> 6), tid & 63);
         __syncthreads();
         load_tile(t0);
         {
@@ -370,7 +394,7 @@ sweep_local_bwd(const SweepArgs a)
             const bool more = tile + 1 < t1;
             float *tot = sTot + (tile & 1) * 8 * D;
             SYNC_OR_DIE();                                             // group totals are there
-            if (tid < T && tile + 2 < t1) rowOff[((tile + 2) & 3) * T + tid] = tile_row_offset(g, pl, b, h, D, tile + 2, tid);
+            if (tid < T && tile + 2 < t1) rowOff[((tile + 2) & 3) * T + tid] = tile_row_offset(g, pl, g.dir, b, h, D, tile + 2, tid);
             Tot tt = tile_totals<D>(tot, w);
             const RowSum mine = row_sum<D>(sm, tt);
             const int s = divide_tile<D>(tot, w, pl.sub_max, a.status, tt);
@@ -611,6 +635,7 @@ sweep_fwd(const SweepArgs a)
     using C = Cfg<D>;
     using L = Col<D>;
     using SM = FwdSmem<D, TO>;
+    constexpr bool ORDERS = sizeof(TO) == 4;            // sums over scan orders have fp32 results
     extern __shared__ __align__(128) char smem[];
     char *tQ = smem, *tK = tQ + C::TILE_T, *tV = tK + C::TILE_T, *tS = tV + C::TILE_T, *tP = tS + C::TILE_S;
     char *stage = smem + SM::kTiles;
@@ -641,8 +666,9 @@ sweep_fwd(const SweepArgs a)
     // The first tile's rows are inputs of the call: their loads need not wait for the scan kernel (whose own
     // wait covered whatever produced them).  Uncut sequences have no kernel in front that has waited: wait first.
     auto prime = [&](int sid) {
-        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
-        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, pl, b, h, D, sg * pl.G, tid);
+        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg;
+        const Seq sq = seq_of<ORDERS>(a, bh);
+        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, pl, sq.dir, sq.b, sq.h, D, sg * pl.G, tid);
         __syncthreads();
         load_tile(cur);
     };
@@ -650,7 +676,8 @@ sweep_fwd(const SweepArgs a)
     if ((int)blockIdx.x < total) prime(blockIdx.x);
     pdl_wait();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
-        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
+        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg;
+        const Seq sq = seq_of<ORDERS>(a, bh);
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
         if (pl.nseg == 1) get_state<D>(a.s_in ? a.s_in + (size_t)sid * D * D : nullptr, sm, S);      // uncut: no scan ran
         else get_state<D>(a.seg_state + (size_t)sid * D * D, sm, S);
@@ -665,7 +692,7 @@ sweep_fwd(const SweepArgs a)
             const bool more = tile + 1 < t1;
             tc_fence_before_sync();
             SYNC_OR_DIE();                                       // group totals are there, the previous tile's products are done
-            if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile + 1, tid);
+            if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, sq.dir, sq.b, sq.h, D, tile + 1, tid);
             // Where some channel's gates sum to too much for one centring (or shorter chunks were asked for) the tile
             // is worked in sub-chunks with their own centring.  Two of 32 rows share one pass through the phases below
             // (`halves`): both are built and scored at once, the state between them is formed after the scores and read by the
@@ -703,7 +730,7 @@ sweep_fwd(const SweepArgs a)
                             mma_commit(&ctl->bar[0]);
                         }
                     }
-                    if (staged) flush_rows<D>(out, stage, rowOff + prv * T, w, staged, a.accumulate != 0);
+                    if (staged) flush_rows<D>(out, sq.oo, stage, rowOff + prv * T, w, staged, a.accumulate != 0);
                     staged = 0;
                     if (last && more) load_tile(nxt);
                     ok = wait_all(&ctl->bar[0], 0, a.status, ok);          // completes twice per iteration: parities 0, 1
@@ -785,7 +812,7 @@ sweep_fwd(const SweepArgs a)
             cur = nxt;
         }
         SYNC_OR_DIE();
-        flush_rows<D>(out, stage, rowOff + ((cur + 3) & 3) * T, w, staged, a.accumulate != 0);
+        flush_rows<D>(out, sq.oo, stage, rowOff + ((cur + 3) & 3) * T, w, staged, a.accumulate != 0);
         staged = 0;
         if (pl.nseg == 1 && a.s_out) save_state<D>(a.s_out + (size_t)sid * D * D, sm, S);
     }
@@ -885,16 +912,18 @@ sweep_bwd(const SweepArgs a)
     };
     // the first tile's rows are inputs of the call: their loads need not wait for the scan kernel
     auto prime = [&](int sid) {
-        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
+        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg;
+        const Seq sq = seq_of<false>(a, bh);
         const int t1 = min(sg * pl.G + pl.G, pl.ntile);
-        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, pl, b, h, D, t1 - 1, tid);
+        if (tid < T) rowOff[cur * T + tid] = tile_row_offset(g, pl, sq.dir, sq.b, sq.h, D, t1 - 1, tid);
         __syncthreads();
         load_all(cur);
     };
     if ((int)blockIdx.x < total) prime(blockIdx.x);
     pdl_wait();
     for (int sid = blockIdx.x; sid < total; sid += gridDim.x) {
-        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg, b = bh / g.H, h = bh - b * g.H;
+        const int bh = sid / pl.nseg, sg = sid - bh * pl.nseg;
+        const Seq sq = seq_of<false>(a, bh);
         const int t0 = sg * pl.G, t1 = min(t0 + pl.G, pl.ntile);
         // without a scan (uncut sequences, no state arguments) the entry state, the incoming state gradient and the carry are zero
         get_state<D>(entry ? a.seg_dstate + (size_t)sid * D * D : nullptr, sm, Dst);
@@ -925,7 +954,7 @@ sweep_bwd(const SweepArgs a)
             const int nrow = min(T, g.L - tile * T), nxt = cur ^ 1;
             const bool more = tile > t0;
             SYNC_OR_DIE();                                       // group totals are there, the accumulator buffers are free
-            if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, b, h, D, tile - 1, tid);
+            if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, sq.dir, sq.b, sq.h, D, tile - 1, tid);
             const Tot whole = tile_totals<D>(sTot, w);
             Tot tt = whole;
             const int s = divide_tile<D>(sTot, w, pl.sub_max, a.status, tt);
@@ -1114,7 +1143,7 @@ sweep_bwd(const SweepArgs a)
                     }
                 }
                 // the state tile as staging holds this sub-chunk's rows only
-                if (SM::kStage && (!SM::kOwnStage || u == 0)) flush_rows<D>(dv, stage, rowOff + cur * T, w, SM::kOwnStage || mine ? nrow : 0, acc_out);
+                if (SM::kStage && (!SM::kOwnStage || u == 0)) flush_rows<D>(dv, 0u, stage, rowOff + cur * T, w, SM::kOwnStage || mine ? nrow : 0, acc_out);
                 if (u > 0) {
                     fence_async_smem();
                     __syncthreads();                             // the accumulator buffers become operand tiles again
@@ -1206,7 +1235,7 @@ constexpr PassCost kBackward = {{14, 54}, {32, 23}, {88, 95}, {62, 73}, 67, 170,
 // Chunks above 64 tokens: forward plans stay within the scratch of dig_gla_fwd_static where uncut sequences do (the
 // same plan serves dig_gla_fwd, so that both give the same bits).  No other family's workspace is counted there that
 // would be larger anyway; with chunks of up to 64 the per-chunk states of the other families always are.
-Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
+Plan make_plan(const Geom &g, int sms, int per_sm, bool backward, long long *least = nullptr)
 {
     Plan p;
     p.ntile = (g.L + T - 1) / T;
@@ -1233,6 +1262,7 @@ Plan make_plan(const Geom &g, int sms, int per_sm, bool backward)
         if (G == 1) break;
     }
     p.nseg = (p.ntile + p.G - 1) / p.G;
+    if (least) *least = best;
     return p;
 }
 
@@ -1242,10 +1272,12 @@ dig_status set_smem(K kern, size_t bytes)
     return ensure_dynamic_smem(reinterpret_cast<const void *>(kern), bytes);
 }
 
+// n scan orders (two bits each in dirs) of the same inputs; results of order i stand i * stride elements behind the first's.
 template <int D, bool BWD>
-dig_status run(const GlaArgs &ga)
+dig_status run(const GlaArgs &ga, int n, uint32_t dirs, size_t stride)
 {
-    const Geom &g = ga.g;
+    Geom g = ga.g;
+    g.B *= n;
     const int sms = device_sm_count();
     int *status = device_status_ptr();
     if (!status || sms <= 0) return DIG_ERR_CUDA;
@@ -1261,6 +1293,9 @@ dig_status run(const GlaArgs &ga)
     a.seg_state16 = w.seg_state16; a.slot_s = w.slot_s; a.slot_g = w.slot_g;
     a.status = status;
     a.accumulate = ga.accumulate;
+    a.batch = ga.g.B;
+    a.dirs = dirs;
+    a.out_stride = (uint32_t)stride;
     a.g = g;
     a.plan = pl;
     const dim3 grid((unsigned)(total < (long long)sms * kPerSm ? total : (long long)sms * kPerSm)), block(Col<D>::NT);
@@ -1281,7 +1316,7 @@ dig_status run(const GlaArgs &ga)
             kern = states_only ? sweep_local_bwd<D, false> : sweep_local_bwd<D, true>;
             smem = states_only ? LocalBwdSmem<D, false>::bytes : LocalBwdSmem<D, true>::bytes;
         } else {
-            kern = sweep_local_fwd<D>;
+            kern = n > 1 ? sweep_local_fwd<D, true> : sweep_local_fwd<D, false>;
             smem = LocalFwdSmem<D>::bytes;
         }
         if ((st = set_smem(kern, smem)) != DIG_OK) return st;
@@ -1335,93 +1370,158 @@ size_t sweep_workspace_bytes(const Geom &g, bool backward)
 
 namespace {
 
-// fp32 sums -> bf16 results (round to nearest even), 8 elements per thread; blockIdx.y selects the tensor.
-struct RoundArgs {
-    const float *src[3];
-    bf16 *dst[3];
+dig_status sweep_orders(const GlaArgs &a, bool backward, int n, uint32_t dirs, size_t stride)
+{
+    if (backward) return a.g.dk == 64 ? run<64, true>(a, n, dirs, stride) : run<72, true>(a, n, dirs, stride);
+    return a.g.dk == 64 ? run<64, false>(a, n, dirs, stride) : run<72, false>(a, n, dirs, stride);
+}
+
+// Sums over n buffers of fp32 results, in order, to the caller's tensors (fp32, or rounded to the nearest even bf16), 8
+// elements per thread; blockIdx.y selects the tensor.
+struct SumArgs {
+    const float *src[4];
+    void *dst[4];
+    bool f32[4];
 };
-__global__ void __launch_bounds__(256) round_to_bf16(const RoundArgs a, size_t n8)
+__global__ void __launch_bounds__(256) sum_orders(const SumArgs a, int n, size_t stride, size_t n8)
 {
     pdl_wait();
     pdl_launch_dependents();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n8) return;
-    float f[8];
-    ld8(a.src[blockIdx.y] + 8 * i, f);
-    store_out8(a.dst[blockIdx.y] + 8 * i, f);
+    const float *src = a.src[blockIdx.y] + 8 * i;
+    float f[4][8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (k < n) ld8(src + k * stride, f[k]);
+#pragma unroll
+    for (int k = 1; k < 4; ++k)
+        if (k < n)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) f[0][e] += f[k][e];
+    if (a.f32[blockIdx.y]) store_out8(static_cast<float *>(a.dst[blockIdx.y]) + 8 * i, f[0]);
+    else store_out8(static_cast<bf16 *>(a.dst[blockIdx.y]) + 8 * i, f[0]);
 }
-dig_status launch_round(const RoundArgs &a, int tensors, size_t n, cudaStream_t s)
+
+// Scan orders of a forward pass that share a launch.  Where a sequence has too few tiles to fill the machine, orders side by
+// side need fewer cuts or none, so no local sweep and no scan; the results of a launch's orders then stand in buffers of their
+// own, later launches add to them, and one pass sums the buffers.  Costs as in make_plan, plus the buffers beyond the first,
+// written and read at 0.6 MB per 0.1 us.  768 tiles in 48 sequences, d = 64, four orders: 127 us one after the other, 82 side by
+// side.  Backward passes keep one order per launch: pairs took 180 instead of 198 us there, but their four tensors' buffers
+// cost as much more in the sum.  Offsets of the results have 31 bits.
+int orders_together(const Geom &g, int sms, bool backward, int n)
 {
-    const size_t n8 = n / 8;
-    launch_pdl(round_to_bf16, dim3((unsigned)((n8 + 255) / 256), tensors), dim3(256), 0, s, a, n8);
+    const size_t elems = (size_t)g.B * g.L * g.H * g.dk;
+    long long best = -1;
+    int k = 1;
+    for (int j = 1; j <= (backward ? 1 : n); j *= 2) {
+        if (j > 1 && elems * j >= (1ull << 31)) break;
+        Geom h = g;
+        h.B *= j;
+        long long cost = 0;
+        make_plan(h, sms, kPerSm, backward, &cost);
+        cost = cost * ((n + j - 1) / j) + (long long)(100 * (j - 1) * 8 * elems / 600000);
+        if (best < 0 || cost < best) {
+            best = cost;
+            k = j;
+        }
+    }
+    return k;
+}
+// Bytes of one tensor's buffers: bf16 results and results of several orders are summed in the workspace.
+size_t multi_buffer_bytes(const Geom &g, int k) { return align256((size_t)g.B * g.L * g.H * g.dk * 4 * k); }
+
+size_t multi_bytes(const Geom &g, int sms, bool backward, int dtype, int n)
+{
+    const int k = orders_together(g, sms, backward, n);
+    Geom h = g;
+    h.B *= k;
+    size_t bytes = align256(sweep_workspace_bytes(h, backward));
+    if (k > 1) bytes += multi_buffer_bytes(g, k) * (backward ? 4 : 1);
+    else if (dtype == DIG_BF16) bytes += multi_buffer_bytes(g, 1) * (backward ? 3 : 1);
+    return bytes;
+}
+
+}  // namespace
+
+// Several scan orders summed (Algorithm 2 / Algorithm 3): groups of orders one after the other, each launch adding
+// its fp32 results to the same buffers, which are summed and rounded to the storage type once at the end.  An element of a
+// buffer gets one addition per launch and the launches follow one another on the stream, so the sum does not depend on
+// scheduling.
+size_t sweep_multi_workspace_bytes(const Geom &g, bool backward, int dtype)
+{
+    int sms = device_sm_count();
+    if (sms <= 0) sms = 148;
+    size_t most = 0;
+    for (int n = 1; n <= 4; ++n) {
+        const size_t b = multi_bytes(g, sms, backward, dtype, n);
+        most = b > most ? b : most;
+    }
+    return most;
+}
+
+namespace {
+
+dig_status sweep_multi(const GlaArgs &a0, bool backward, unsigned mask)
+{
+    const int sms = device_sm_count();
+    if (sms <= 0) return DIG_ERR_CUDA;
+    GlaArgs a = a0;
+    const size_t elems = (size_t)a.g.B * a.g.L * a.g.H * a.g.dk;          // d_k = d_v
+    const int n = __builtin_popcount(mask), k = orders_together(a.g, sms, backward, n);
+    Geom h = a.g;
+    h.B *= k;
+    char *extra = reinterpret_cast<char *>(a0.ws) + align256(sweep_workspace_bytes(h, backward));
+    const bool narrow = a0.dtype == DIG_BF16;
+    void *const result[4] = {backward ? a0.dq : a0.out, a0.dk, a0.dv, a0.dgate};
+    SumArgs sum{};
+    int sums = 0;
+    auto buffer = [&](int t) -> void * {
+        const bool f32 = !narrow || t == 3;
+        if (k == 1 && f32) return result[t];
+        float *p = reinterpret_cast<float *>(extra);
+        extra += multi_buffer_bytes(a.g, k);
+        sum.src[sums] = p;
+        sum.dst[sums] = result[t];
+        sum.f32[sums++] = f32;
+        return p;
+    };
+    a.dtype = DIG_BF16_F32OUT;
+    if (backward) {
+        a.dq = buffer(0);
+        a.dk = buffer(1);
+        a.dv = buffer(2);
+        a.dgate = static_cast<float *>(buffer(3));
+    } else {
+        a.out = buffer(0);
+    }
+    a.accumulate = 0;
+    uint32_t dirs = 0;
+    int held = 0, left = n;
+    for (uint32_t d = 0; d < 4; ++d) {
+        if (!(mask >> d & 1)) continue;
+        dirs |= d << (2 * held++);
+        --left;
+        if (held < k && left > 0) continue;
+        a.g.dir = (int)d;                             // of a single order
+        const dig_status st = sweep_orders(a, backward, held, dirs, elems);
+        if (st != DIG_OK) return st;
+        a.accumulate = 1;
+        dirs = 0;
+        held = 0;
+    }
+    if (sums == 0) return DIG_OK;
+    const size_t n8 = elems / 8;
+    launch_pdl(sum_orders, dim3((unsigned)((n8 + 255) / 256), sums), dim3(256), 0, a.stream, sum, k, elems, n8);
     return cuda_ok(cudaGetLastError());
 }
 
 }  // namespace
 
-// Several scan orders summed (Algorithm 2 / Algorithm 3): the orders run one after the other, each
-// adding its fp32 results to the same buffers, which are rounded to the storage type once at the end.
-size_t sweep_multi_workspace_bytes(const Geom &g, bool backward, int dtype)
-{
-    size_t n = align256(sweep_workspace_bytes(g, backward));
-    if (dtype == DIG_BF16) {
-        const size_t tok = (size_t)g.B * g.L * g.H;
-        n += backward ? align256(tok * g.dk * 4) * 2 + align256(tok * g.dv * 4) : align256(tok * g.dv * 4);
-    }
-    return n;
-}
+dig_status sweep_gla_fwd_multi(const GlaArgs &a, unsigned mask) { return sweep_multi(a, false, mask); }
+dig_status sweep_gla_bwd_multi(const GlaArgs &a, unsigned mask) { return sweep_multi(a, true, mask); }
 
-dig_status sweep_gla_fwd_multi(const GlaArgs &a0, unsigned mask)
-{
-    GlaArgs a = a0;
-    const size_t tok = (size_t)a.g.B * a.g.L * a.g.H;
-    char *extra = reinterpret_cast<char *>(a0.ws) + align256(sweep_workspace_bytes(a.g, false));
-    const bool narrow = a0.dtype == DIG_BF16;
-    a.dtype = DIG_BF16_F32OUT;
-    if (narrow) a.out = extra;
-    bool first = true;
-    for (int d = 0; d < 4; ++d) {
-        if (!(mask >> d & 1)) continue;
-        a.g.dir = d;
-        a.accumulate = first ? 0 : 1;
-        first = false;
-        const dig_status st = sweep_gla_fwd(a);
-        if (st != DIG_OK) return st;
-    }
-    if (!narrow) return DIG_OK;
-    return launch_round(RoundArgs{{reinterpret_cast<const float *>(extra)}, {(bf16 *)a0.out}}, 1, tok * a.g.dv, a.stream);
-}
-
-dig_status sweep_gla_bwd_multi(const GlaArgs &a0, unsigned mask)
-{
-    GlaArgs a = a0;
-    const size_t tok = (size_t)a.g.B * a.g.L * a.g.H;
-    char *extra = reinterpret_cast<char *>(a0.ws) + align256(sweep_workspace_bytes(a.g, true));
-    const bool narrow = a0.dtype == DIG_BF16;
-    a.dtype = DIG_BF16_F32OUT;
-    float *sq = reinterpret_cast<float *>(extra), *sk = reinterpret_cast<float *>(extra + align256(tok * a.g.dk * 4));
-    float *sv = reinterpret_cast<float *>(extra + 2 * align256(tok * a.g.dk * 4));
-    if (narrow) { a.dq = sq; a.dk = sk; a.dv = sv; }
-    bool first = true;
-    for (int d = 0; d < 4; ++d) {
-        if (!(mask >> d & 1)) continue;
-        a.g.dir = d;
-        a.accumulate = first ? 0 : 1;
-        first = false;
-        const dig_status st = sweep_gla_bwd(a);
-        if (st != DIG_OK) return st;
-    }
-    if (!narrow) return DIG_OK;
-    return launch_round(RoundArgs{{sq, sk, sv}, {(bf16 *)a0.dq, (bf16 *)a0.dk, (bf16 *)a0.dv}}, 3, tok * a.g.dk, a.stream);      // d_k = d_v
-}
-
-dig_status sweep_gla_fwd(const GlaArgs &a)
-{
-    return a.g.dk == 64 ? run<64, false>(a) : run<72, false>(a);
-}
-dig_status sweep_gla_bwd(const GlaArgs &a)
-{
-    return a.g.dk == 64 ? run<64, true>(a) : run<72, true>(a);
-}
+dig_status sweep_gla_fwd(const GlaArgs &a) { return sweep_orders(a, false, 1, (uint32_t)a.g.dir, 0); }
+dig_status sweep_gla_bwd(const GlaArgs &a) { return sweep_orders(a, true, 1, (uint32_t)a.g.dir, 0); }
 
 }  // namespace dig

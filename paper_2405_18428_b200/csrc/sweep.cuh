@@ -150,12 +150,12 @@ struct Ctl {
 // Element offset of the (batch b, head h) row of the token at scan position 64*tile + row in a
 // [B][L][H][D] tensor; positions past the end of the sequence give its first row (what is read there is
 // cleared).  The host checks that offsets fit 31 bits.
-__device__ __forceinline__ int tile_row_offset(const Geom &g, const Plan &pl, int b, int h, int d, int tile, int row)
+__device__ __forceinline__ int tile_row_offset(const Geom &g, const Plan &pl, int dir, int b, int h, int d, int tile, int row)
 {
     int p = tile * T + row;
     if (p >= g.L) p = 0;
-    if (g.dir & 1) p = g.L - 1 - p;
-    if (g.dir & 2) {
+    if (dir & 1) p = g.L - 1 - p;
+    if (dir & 2) {
         // p / gh with a reciprocal rounded down: the estimate is at most one too small for p < 2^24
         int x = (int)__umulhi((uint32_t)p, pl.gh_inv), y = p - x * g.gh;
         if (y >= g.gh) { y -= g.gh; ++x; }
