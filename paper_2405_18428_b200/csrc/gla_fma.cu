@@ -183,22 +183,25 @@ __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool on
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(on ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void loads_done() { asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void load_tile(float *dst, int ld, const float *src, const Rows &sRow, int C, int d)
+// Rows j0 .. j1 - 1 (kept at their places), `w` of the d columns from src on.
+__device__ __forceinline__ void load_tile(float *dst, int ld, const float *src, const Rows &sRow, int j0, int j1, int d, int w)
 {
-    const int per_row = d >> 2, n = C * per_row;
+    const int per_row = w >> 2, n = (j1 - j0) * per_row;
     for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        const int j = idx / per_row, c = (idx - j * per_row) << 2, row = sRow[j];
+        const int r = idx / per_row, j = j0 + r, c = (idx - r * per_row) << 2, row = sRow[j];
         cp_async16(dst + j * ld + c, src + (size_t)max(row, 0) * d + c, row >= 0);
     }
 }
-__device__ __forceinline__ void load_tile(float *dst, int ld, const __nv_bfloat16 *src, const Rows &sRow, int C, int d)
+__device__ __forceinline__ void load_tile(float *dst, int ld, const __nv_bfloat16 *src, const Rows &sRow, int j0, int j1, int d, int w)
 {
-    const int per_row = d >> 2, n = C * per_row;
+    const int per_row = w >> 2, n = (j1 - j0) * per_row;
     for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        const int j = idx / per_row, c = (idx - j * per_row) << 2, row = sRow[j];
+        const int r = idx / per_row, j = j0 + r, c = (idx - r * per_row) << 2, row = sRow[j];
         *reinterpret_cast<float4 *>(dst + j * ld + c) = row >= 0 ? load4(src + (size_t)row * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
+template <typename T>
+__device__ __forceinline__ void load_tile(float *dst, int ld, const T *src, const Rows &sRow, int C, int d) { load_tile(dst, ld, src, sRow, 0, C, d, d); }
 // A [dk][dv] state of the workspace -> [dk][ld] tile.
 __device__ __forceinline__ void load_state(float *dst, int ld, const float *src, int dk, int dv)
 {
@@ -237,8 +240,9 @@ __device__ __forceinline__ float4 exp4(float4 x) { return make_float4(expf(x.x),
 __device__ __forceinline__ float4 mul4(float4 a, float4 b) { return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w); }
 
 // ---- kernel 1: chunk-local state contributions ------------------------------------------------
-// U = Kh^T V  (and, for the backward pass, W = Qt^T dO); gamma = exp(Lam_{C-1}).
-template <typename T, bool BWD>
+// U = Kh^T V  (and, for the backward pass, W = Qt^T dO); gamma = exp(Lam_{C-1}).  CTA z of a chunk takes a slice of the key
+// channels (SHARED: where the chunks leave SMs idle).
+template <typename T, bool BWD, bool SHARED>
 __global__ void __launch_bounds__(kThreads)
 fma_chunk_state(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v,
                 const float *__restrict__ gate, const T *__restrict__ d_out,
@@ -247,12 +251,13 @@ fma_chunk_state(const T *__restrict__ q, const T *__restrict__ k, const T *__res
 {
     extern __shared__ __align__(16) float smem[];
     const int chunk = blockIdx.x, bh = blockIdx.y, b = bh / g.H, h = bh - b * g.H;
-    const int ldk = g.dk + 4, ldv = g.dv + 4;
+    const int w = SHARED ? g.dk / gridDim.z : g.dk, k0 = SHARED ? blockIdx.z * w : 0;      // the CTA's key channels
+    const int ldk = w + 4, ldv = g.dv + 4;
     float *sLam = smem;                     // gates -> Lam
     float *sX = sLam + g.C * ldk;           // k -> Kh
     float *sV = sX + g.C * ldk;
-    float *sSeg = sV + g.C * ldv;           // [8][dk]
-    float *sQ = sSeg + 8 * g.dk;            // BWD: Qt
+    float *sSeg = sV + g.C * ldv;           // [8][w]
+    float *sQ = sSeg + 8 * w;               // BWD: Qt
     float *sG = sQ + (BWD ? g.C * ldk : 0); // BWD: dO
 
     const Rows sRow(sV, ldv, g.dv);
@@ -260,21 +265,21 @@ fma_chunk_state(const T *__restrict__ q, const T *__restrict__ k, const T *__res
     pdl_wait();
     pdl_launch_dependents();
     __syncthreads();
-    load_tile(sLam, ldk, gate, sRow, g.C, g.dk);
-    load_tile(sX, ldk, k, sRow, g.C, g.dk);
+    load_tile(sLam, ldk, gate + k0, sRow, 0, g.C, g.dk, w);
+    load_tile(sX, ldk, k + k0, sRow, 0, g.C, g.dk, w);
     load_tile(sV, ldv, v, sRow, g.C, g.dv);
     if (BWD) {
-        load_tile(sQ, ldk, q, sRow, g.C, g.dk);
+        load_tile(sQ, ldk, q + k0, sRow, 0, g.C, g.dk, w);
         load_tile(sG, ldv, d_out, sRow, g.C, g.dv);
     }
     loads_done();
     __syncthreads();
-    prefix_gates(sLam, ldk, g.C, g.dk, sSeg);
+    prefix_gates(sLam, ldk, g.C, w, sSeg);
     const size_t chunk_id = (size_t)bh * g.N + chunk;
     const float *sLast = sLam + (g.C - 1) * ldk;
-    for (int c = threadIdx.x; c < g.dk; c += kThreads) gamma[chunk_id * g.dk + c] = expf(sLast[c]);
+    for (int c = threadIdx.x; c < w; c += kThreads) gamma[chunk_id * g.dk + k0 + c] = expf(sLast[c]);
     {
-        const int per_row = g.dk >> 2;
+        const int per_row = w >> 2;
         for (int idx = threadIdx.x; idx < g.C * per_row; idx += kThreads) {
             const int j = idx / per_row, o = j * ldk + ((idx - j * per_row) << 2);
             const float4 lam = *reinterpret_cast<const float4 *>(sLam + o), last = *reinterpret_cast<const float4 *>(sLast + o - j * ldk);
@@ -284,9 +289,9 @@ fma_chunk_state(const T *__restrict__ q, const T *__restrict__ k, const T *__res
         }
     }
     __syncthreads();
-    const int nrb = g.dk >> 2, ncb = g.dv >> 2;
-    float *U = states + chunk_id * g.dk * g.dv;
-    float *W = BWD ? dstates + chunk_id * g.dk * g.dv : nullptr;
+    const int nrb = w >> 2, ncb = g.dv >> 2;
+    float *U = states + (chunk_id * g.dk + k0) * g.dv;
+    float *W = BWD ? dstates + (chunk_id * g.dk + k0) * g.dv : nullptr;
     for (int blk = threadIdx.x; blk < nrb * ncb; blk += kThreads) {
         const int r0 = (blk / ncb) << 2, c0 = (blk % ncb) << 2;
         float acc[4][4];
@@ -305,15 +310,15 @@ fma_chunk_state(const T *__restrict__ q, const T *__restrict__ k, const T *__res
     }
 }
 
-// In place: q -> Qt = q exp(Lam), k -> Kt = k exp(-Lam), Lam -> exp(Lam).
-__device__ __forceinline__ void make_qt_kt(float *sQ, float *sK, float *sLam, int ldk, int C, int dk)
+// In place: q -> Qt = q exp(Lam), k -> Kt = k exp(-Lam), Lam -> exp(Lam); q from row q0 on.
+__device__ __forceinline__ void make_qt_kt(float *sQ, float *sK, float *sLam, int ldk, int C, int dk, int q0 = 0)
 {
     const int per_row = dk >> 2;
     for (int idx = threadIdx.x; idx < C * per_row; idx += blockDim.x) {
         const int j = idx / per_row, o = j * ldk + ((idx - j * per_row) << 2);
         const float4 lam = *reinterpret_cast<const float4 *>(sLam + o), e = exp4(lam);
         *reinterpret_cast<float4 *>(sLam + o) = e;
-        *reinterpret_cast<float4 *>(sQ + o) = mul4(*reinterpret_cast<const float4 *>(sQ + o), e);
+        if (j >= q0) *reinterpret_cast<float4 *>(sQ + o) = mul4(*reinterpret_cast<const float4 *>(sQ + o), e);
         *reinterpret_cast<float4 *>(sK + o) = mul4(*reinterpret_cast<const float4 *>(sK + o), exp4(make_float4(-lam.x, -lam.y, -lam.z, -lam.w)));
     }
 }
@@ -337,10 +342,12 @@ __device__ __forceinline__ void score_block(float *sP, int ldp, const float *sA,
 
 // ---- kernel 3: outputs ---------------------------------------------------------------------------
 // out = tril(Qt Kt^T) V + Qt S
+// CTA z of a chunk takes a part of its rows, for which it needs the keys up to them (SHARED: where the chunks leave SMs
+// idle; parts are whole quarters, so that the interleaved columns of a score block stay below the part's last row).
 // PERSM: CTAs per SM that the registers allow, three, or four on shorter loops where a launch has more CTAs than three per SM and
 // shared memory holds four (chunks below 64): 180 sequences of 250 tokens in chunks of 16 (d = 64) take 82 us with three, 70
 // with four.  Fewer CTAs are faster with three (12 sequences of 1024 tokens in chunks of 32: 31.0 us a pass, 34.7 with four).
-template <typename T, typename TO, int PERSM>
+template <typename T, typename TO, int PERSM, bool SHARED>
 __global__ void __launch_bounds__(kThreads, PERSM)
 fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v,
               const float *__restrict__ gate, const float *__restrict__ states,
@@ -349,6 +356,7 @@ fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     extern __shared__ __align__(16) float smem[];
     const int chunk = blockIdx.x, bh = blockIdx.y, b = bh / g.H, h = bh - b * g.H;
     const int ldk = g.dk + 4, ldv = g.dv + 4, ldp = g.C + 4;
+    const int rows = SHARED ? g.C / gridDim.z : g.C, lo = SHARED ? blockIdx.z * rows : 0, hi = lo + rows;     // the CTA's rows; keys below hi
     float *sLam = smem;
     float *sQ = sLam + g.C * ldk;
     float *sK = sQ + g.C * ldk;
@@ -363,26 +371,26 @@ fma_chunk_out(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     fill_rows(sRow, g, b, h, chunk);
     __syncthreads();
     // the inputs of the call: whatever produced them has completed before the kernels in front of this one started
-    load_tile(sLam, ldk, gate, sRow, g.C, g.dk);
-    load_tile(sV, ldv, v, sRow, g.C, g.dv);
-    load_tile(sQ, ldk, q, sRow, g.C, g.dk);
-    load_tile(sK, ldk, k, sRow, g.C, g.dk);
+    load_tile(sLam, ldk, gate, sRow, hi, g.dk);
+    load_tile(sV, ldv, v, sRow, hi, g.dv);
+    load_tile(sQ, ldk, q, sRow, lo, hi, g.dk, g.dk);
+    load_tile(sK, ldk, k, sRow, hi, g.dk);
     loads_done();
     __syncthreads();
-    prefix_gates(sLam, ldk, g.C, g.dk, sSeg);
-    make_qt_kt(sQ, sK, sLam, ldk, g.C, g.dk);
+    prefix_gates(sLam, ldk, hi, g.dk, sSeg);
+    make_qt_kt(sQ, sK, sLam, ldk, hi, g.dk, lo);
     __syncthreads();
     pdl_wait();                             // the states come from the scan in front
     pdl_launch_dependents();
     load_state(sS, ldv, states + ((size_t)bh * g.N + chunk) * g.dk * g.dv, g.dk, g.dv);
     const int nb = g.C >> 2;
-    for (int blk = threadIdx.x; blk < nb * nb; blk += kThreads) score_block(sP, ldp, sQ, ldk, sK, ldk, g.C, g.dk, blk);
+    for (int blk = (lo >> 2) * nb + threadIdx.x; blk < (hi >> 2) * nb; blk += kThreads) score_block(sP, ldp, sQ, ldk, sK, ldk, g.C, g.dk, blk);
     loads_done();
     __syncthreads();
     constexpr int UN = PERSM > 3 ? 1 : 4;
-    const int nrb = g.C >> 2, ncb = g.dv >> 2;
+    const int nrb = rows >> 2, ncb = g.dv >> 2;
     for (int blk = threadIdx.x; blk < nrb * ncb; blk += kThreads) {
-        const int r0 = (blk / ncb) << 2, c0 = (blk % ncb) << 2;
+        const int r0 = lo + ((blk / ncb) << 2), c0 = (blk % ncb) << 2;
         float acc[4][4];
         zero(acc);
         mm_nn<UN>(acc, sP, ldp, r0, sV, ldv, c0, r0 + 4);       // columns beyond the diagonal are zero
@@ -571,7 +579,15 @@ size_t smem_bwd(const Geom &g)
     return sizeof(float) * n;
 }
 constexpr size_t kMaxSmem = 227 * 1024;
-
+// CTAs that share a chunk where the chunks leave SMs idle.  24 chunks of 64 tokens, d = 64: state kernel 7.7 us alone, 6.1 in two
+// slices, 5.8 in four; outputs 14.2, 12.4 in two parts, 12.6 in four.  192 chunks: state 10.4, 9.8, 14.1, outputs 20.8, 25.7, 36.8.
+int share(const Geom &g, int n, bool whole) { return whole && (long long)n * g.N * g.B * g.H <= device_sm_count() ? n : 1; }
+int state_slices(const Geom &g)                 // whole vectors of channels
+{
+    const int n = share(g, 4, g.dk % 16 == 0);
+    return n > 1 ? n : share(g, 2, g.dk % 8 == 0);
+}
+int row_parts(const Geom &g) { return share(g, 2, true); }
 template <typename K>
 dig_status set_smem(K kernel, size_t bytes)
 {
@@ -584,18 +600,20 @@ dig_status fwd_typed(const GlaArgs &a)
 {
     const Geom &g = a.g;
     const Workspace w = carve_workspace(a.ws, g, false);
-    const dim3 grid(g.N, g.B * g.H);
+    const dim3 grid(g.N, g.B * g.H), grid1(g.N, g.B * g.H, state_slices(g));
     dig_status st;
-    auto k1 = fma_chunk_state<T, false>;
+    auto k1 = grid1.z > 1 ? fma_chunk_state<T, false, true> : fma_chunk_state<T, false, false>;
     if ((st = set_smem(k1, smem_state(g, false))) != DIG_OK) return st;
     { KernelTimer t(KID_FMA_STATE, a.stream);
-    launch_pdl(k1, grid, dim3(kThreads), smem_state(g, false), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+    launch_pdl(k1, grid1, dim3(kThreads), smem_state(g, false), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
                (const T *)nullptr, w.states, w.gamma, (float *)nullptr, g); }
     if ((st = launch_state_scan_fwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
-    auto k3 = g.C < 64 && (long long)grid.x * grid.y > 3ll * device_sm_count() ? fma_chunk_out<T, TO, 4> : fma_chunk_out<T, TO, 3>;
+    const int parts = row_parts(g);
+    auto k3 = parts > 1 ? fma_chunk_out<T, TO, 3, true>
+              : g.C < 64 && (long long)grid.x * grid.y > 3ll * device_sm_count() ? fma_chunk_out<T, TO, 4, false> : fma_chunk_out<T, TO, 3, false>;
     if ((st = set_smem(k3, smem_out(g))) != DIG_OK) return st;
     KernelTimer t(KID_FMA_OUT, a.stream);
-    launch_pdl(k3, grid, dim3(kThreads), smem_out(g), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+    launch_pdl(k3, dim3(grid.x, grid.y, parts), dim3(kThreads), smem_out(g), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
                (const float *)w.states, (TO *)a.out, g);
     return cuda_ok(cudaGetLastError());
 }
@@ -605,14 +623,14 @@ dig_status bwd_typed(const GlaArgs &a)
 {
     const Geom &g = a.g;
     const Workspace w = carve_workspace(a.ws, g, true);
-    const dim3 grid(g.N, g.B * g.H);
+    const dim3 grid(g.N, g.B * g.H), grid1(g.N, g.B * g.H, state_slices(g));
     dig_status st;
-    auto k1 = fma_chunk_state<T, true>;
+    auto k1 = grid1.z > 1 ? fma_chunk_state<T, true, true> : fma_chunk_state<T, true, false>;
     if ((st = set_smem(k1, smem_state(g, true))) != DIG_OK) return st;
     auto k4 = fma_chunk_bwd<T, TO>;
     if ((st = set_smem(k4, smem_bwd(g))) != DIG_OK) return st;
     { KernelTimer t(KID_FMA_STATE, a.stream);
-    launch_pdl(k1, grid, dim3(kThreads), smem_state(g, true), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
+    launch_pdl(k1, grid1, dim3(kThreads), smem_state(g, true), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
                (const T *)a.d_out, w.states, w.gamma, w.dstates, g); }
     if ((st = launch_state_scan_fwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
     if ((st = launch_state_scan_bwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
