@@ -26,7 +26,7 @@ namespace {
 // Threads per CTA and CTAs per SM (what the grid is capped at, so that the grid-stride loops end together): the
 // forward kernel as many as shared memory holds, up to 8 (4, 5, 6 and 8 were measured: 17.7, 17.2, 16.7, 15.6 us on
 // 196608 rows of 64), the reverse one 3 (2, 3, 4: 37, 33, 45 us on 262144 rows of 72).
-constexpr int kThreads = 128, kFwdPerSM = 8, kBwdPerSM = 3;
+constexpr int kThreads = 128, kFwdPerSM = 8, kBwdPerSM = 3, kAheadPerSM = 2;
 constexpr size_t kSmemPerSM = 228 * 1024;
 
 // Eight values as they are stored.
@@ -520,7 +520,7 @@ outgate_fwd_direct(const TA *o, const TR *r, const float *__restrict__ ln_w, con
     pdl_launch_dependents();
 }
 template <typename TI, typename TO, int LPR>
-__global__ void __launch_bounds__(Direct<LPR>::kThreads, kBwdPerSM)
+__global__ void __launch_bounds__(Direct<LPR>::kThreads, sizeof(TI) == 2 ? kAheadPerSM : kBwdPerSM)
 outgate_bwd_direct(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln_w, const float *__restrict__ ln_b, TO *d_o, TO *d_r,
                    float *__restrict__ partial, long long rows, int dv, float eps)
 {
@@ -537,13 +537,28 @@ outgate_bwd_direct(const TI *o, const TI *r, const TI *dz, const float *__restri
     load_affine(ln_b, col, 0.f, ln.has_col(0), b);
 #pragma unroll
     for (int j = 0; j < 4; ++j) aw[j] = ab[j] = make_float2(0.f, 0.f);
-    for (long long base = (long long)blockIdx.x * DR::kRows; base < rows; base += (long long)gridDim.x * DR::kRows) {
-        const long long row = base + ln.m.slot;
+    // bf16: the next row is asked for before this one is worked, which takes the registers of two CTAs per SM
+    constexpr bool AHEAD = sizeof(TI) == 2;
+    const long long step = (long long)gridDim.x * DR::kRows;
+    Raw8<TI> ov[1], rv[1], gv[1], no[1], nr[1], ng[1];
+    auto load = [&](long long row, Raw8<TI> (&x)[1], Raw8<TI> (&y)[1], Raw8<TI> (&z)[1]) {
         ln.row_ok = row < rows;
-        Raw8<TI> ov[1], rv[1], gv[1];
-        load_row(ov, o + row * dv, ln);
-        load_row(rv, r + row * dv, ln);
-        load_row(gv, dz + row * dv, ln);
+        load_row(x, o + row * dv, ln);
+        load_row(y, r + row * dv, ln);
+        load_row(z, dz + row * dv, ln);
+    };
+    if (AHEAD) load((long long)blockIdx.x * DR::kRows + ln.m.slot, no, nr, ng);
+    for (long long base = (long long)blockIdx.x * DR::kRows; base < rows; base += step) {
+        const long long row = base + ln.m.slot;
+        if (AHEAD) {
+            ov[0] = no[0];
+            rv[0] = nr[0];
+            gv[0] = ng[0];
+            load(row + step, no, nr, ng);
+            ln.row_ok = row < rows;
+        } else {
+            load(row, ov, rv, gv);
+        }
         RowGrad<V, 1> g;
         g.start(normalise<V>(ov, ln, inv_d, eps, g.n));
         float2 dr[4], dx[4];
@@ -628,6 +643,8 @@ void with_direct(int dv, F f)
     else if (dv == 72) f(integral_constant<int, 9>{});
     else f(integral_constant<int, 16>{});
 }
+// CTAs per SM of the reverse mode
+int bwd_per_sm(const Split &sp, bool narrow) { return narrow && !sp.ring ? kAheadPerSM : kBwdPerSM; }
 int grid_for(long long rows, const Split &sp, int per_sm)
 {
     int sms = device_sm_count();
@@ -692,7 +709,7 @@ dig_status bwd_dispatch(const void *o, const void *r, const void *dz, const floa
         }
     }
     with_direct(dv, [&](auto lpr) {
-        launch_pdl(outgate_bwd_direct<TI, TO, decltype(lpr)::value>, dim3(grid_for(rows, sp, kBwdPerSM)), dim3(sp.threads()), 0, stream, (const TI *)o,
+        launch_pdl(outgate_bwd_direct<TI, TO, decltype(lpr)::value>, dim3(grid_for(rows, sp, bwd_per_sm(sp, sizeof(TI) == 2))), dim3(sp.threads()), 0, stream, (const TI *)o,
                    (const TI *)r, (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps);
     });
     return cuda_ok(cudaGetLastError());
@@ -743,7 +760,7 @@ dig_status launch_outgate_bwd(const void *o, const void *r, const void *dz, cons
     if (st != DIG_OK || !affine) return st;
     KernelTimer t(KID_OUTGATE, stream);
     launch_pdl(outgate_affine_sum, dim3((2 * dv + 31) / 32), dim3(32 * kSumWarps), 0, stream, (const float *)partial, dln_w,
-               dln_b, grid_for(rows, Split(dv, dtype != DIG_F32, true), kBwdPerSM), dv);
+               dln_b, grid_for(rows, Split(dv, dtype != DIG_F32, true), bwd_per_sm(Split(dv, dtype != DIG_F32, true), dtype != DIG_F32)), dv);
     return cuda_ok(cudaGetLastError());
 }
 
