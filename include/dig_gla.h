@@ -247,10 +247,10 @@ dig_status dig_gla_bwd_beta(const void *q, const void *k, const void *v, const f
  *     out = sum over the directions d in direction_mask of dig_gla_fwd(..., direction = d),
  * bit d of direction_mask (1 .. 15) selecting dig_dir d, all orders reading the same q, k, v and gate and
  * writing canonical positions.  dig_gla_bwd_multi returns the gradients of <d_out, out> (the sums of the
- * single-order gradients).  The orders run one after the other on the stream; each adds its fp32 results
- * to the same buffers (caller's for DIG_BF16_F32OUT, workspace for DIG_BF16), so the sum is formed in fp32
- * and rounded to bf16 once.  Served by the tcgen05 kernels only (bf16 storage, d_k = d_v = 64 or 72; else
- * DIG_ERR_UNSUPPORTED); workspace from dig_gla_multi_workspace_bytes (0 for invalid or unsupported sizes).
+ * single-order gradients).  The orders run one after the other on the stream, or, in forward passes over short
+ * sequences, several in a launch with buffers of their own that are added in a fixed order; each adds its fp32 results
+ * to its buffer (caller's or workspace), so the sum is formed in fp32 and rounded to bf16 once.  Served by the
+ * tcgen05 kernels only (bf16 storage, d_k = d_v = 64 or 72; else DIG_ERR_UNSUPPORTED); workspace from dig_gla_multi_workspace_bytes (0 for invalid or unsupported sizes).
  * Tensors, sizes and the gate range are those of dig_gla_fwd / dig_gla_bwd. */
 size_t dig_gla_multi_workspace_bytes(int B, int H, int grid_h, int grid_w, int d_k, int d_v, int chunk, int dtype,
                                      int backward);

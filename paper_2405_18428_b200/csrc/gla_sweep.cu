@@ -136,7 +136,7 @@ __device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity, int *st
 // product is issued there and added once this step's operands are built; operand tiles and sums have two buffers, and the
 // rows of the next tile are loaded a whole tile ahead.
 // Bound by the latency of its phases.  48 sequences of 4096 tokens, d = 64: 40 us with the state in registers, decayed
-// once per tile in scan order, 33 us now; 16 of 16384, d = 72: 80 -> 54 us (63 with the sum in registers, which spills).
+// once per tile in scan order, 30 us now; 16 of 16384, d = 72: 80 -> 52 us (63 with the sum in registers, which spills).
 // One operand exponent for the whole way to the segment's end would let the matrix unit add the products up (29 and
 // 43 us), but fp16 then loses what decays below 2^-25 even where nothing larger follows: errors of 0.3 of RMS where a
 // segment's keys lie in its first tile.
@@ -310,7 +310,7 @@ die:
 // registers).  A backward pass over uncut sequences needs only the states.
 // Pipelined over the (sub-)chunks: the products of one run while the next one's operand tiles are built (two
 // buffers of tiles and accumulators), and are folded into the sums one step later.  48 sequences of 4096 tokens, d = 64:
-// 60 us with both sums in registers and no pipelining, 44 us now; 16 of 16384, d = 72: 122 -> 104 us.
+// 60 us with both sums in registers and no pipelining, 45 us now; 16 of 16384, d = 72: 122 -> 101 us.
 // =================================================================================================
 template <int D, bool GRAD>
 struct LocalBwdSmem {
