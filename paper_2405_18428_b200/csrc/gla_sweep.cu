@@ -617,6 +617,10 @@ seg_scan(float *seg_state, const float *seg_gamma, float *seg_dstate, float *seg
 // SM).  16 sequences of 16384 tokens, d = 72: 114 us with the row-chunk work split, 76 us now; 768 of 256, d = 64
 // (uncut): 60 -> 48 us; 48 of 4096: 62 -> 51.  Three CTAs per SM on 80 registers spill: 72 us there.
 // =================================================================================================
+// PAIRS: two sub-chunks of 32 rows share a pass.  Not in short sweeps of whole tiles, which wait for the instructions (one tile
+// per CTA, 294 CTAs: 8.6 us without, 9.0 with; four tiles, 768 CTAs: 49.2 and 50.0); tiles that are divided there take a pass
+// per half, with the same bits.
+constexpr int kPlainTiles = 4;
 template <int D, typename TO>
 struct FwdSmem {
     using C = Cfg<D>;
@@ -628,7 +632,7 @@ struct FwdSmem {
     static_assert(aU + L::ACCS <= tmem_cols, "tensor memory");
 };
 
-template <int D, typename TO>
+template <int D, typename TO, bool PAIRS>
 __global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_fwd(const SweepArgs a)
 {
@@ -800,9 +804,10 @@ sweep_fwd(const SweepArgs a)
                 }
                 return true;
             };
-            const bool two = s == T / 2 && nrow > T / 2;
+            [[maybe_unused]] const bool two = s == T / 2 && nrow > T / 2;
             bool done;
-            if constexpr (L::X) done = passes(two);
+            if constexpr (!PAIRS) done = passes(Const<false>{});
+            else if constexpr (L::X) done = passes(two);
             else done = two ? passes(Const<true>{}) : passes(Const<false>{});
             if (!done) {
                 ok = false;
@@ -1334,8 +1339,9 @@ dig_status run(const GlaArgs &ga, int n, uint32_t dirs, size_t stride)
     const bool f32 = ga.dtype == DIG_BF16_F32OUT;
     if constexpr (!BWD) {
         constexpr size_t smem16 = FwdSmem<D, bf16>::bytes, smem32 = FwdSmem<D, float>::bytes;
-        auto k16 = sweep_fwd<D, bf16>;
-        auto k32 = sweep_fwd<D, float>;
+        const bool pairs = pl.sub_max == T / 2 || (pl.sub_max == T && pl.G > kPlainTiles);
+        auto k16 = pairs ? sweep_fwd<D, bf16, true> : sweep_fwd<D, bf16, false>;
+        auto k32 = pairs ? sweep_fwd<D, float, true> : sweep_fwd<D, float, false>;
         if ((st = set_smem(k16, smem16)) != DIG_OK || (st = set_smem(k32, smem32)) != DIG_OK) return st;
         KernelTimer t(KID_SW_FWD, ga.stream);
         launch_pdl(f32 ? k32 : k16, grid, block, f32 ? smem32 : smem16, ga.stream, a);
