@@ -39,6 +39,7 @@
 // other's products are in the tensor pipe.
 #include "columns.cuh"
 #include "sweep.cuh"
+#include "sweep_plan.cuh"
 
 namespace dig {
 namespace {
@@ -1193,84 +1194,6 @@ die:
 #undef SYNC_OR_DIE
 
 // ---- host side ----------------------------------------------------------------------------------
-constexpr int kPerSm = 2;       // CTAs of 256 threads that share an SM, for every kernel of the family
-
-struct SweepWs {
-    float *seg_state, *seg_gamma, *seg_dstate, *seg_carry, *slot_g;
-    __half *seg_state16, *slot_s;
-    size_t bytes;
-};
-SweepWs carve(char *base, const Geom &g, const Plan &pl, bool backward)
-{
-    SweepWs w{};
-    const size_t segs = (size_t)g.B * g.H * pl.nseg, dd = (size_t)g.dk * g.dv;
-    size_t o = 0;
-    auto take = [&](size_t bytes) { char *p = base + o; o += align256(bytes); return p; };
-    w.seg_state = reinterpret_cast<float *>(take(segs * dd * 4));
-    w.seg_gamma = reinterpret_cast<float *>(take(segs * g.dk * 4));
-    if (backward) {
-        const size_t slots = (size_t)kSlots * g.B * g.H * pl.ntile;
-        w.seg_dstate = reinterpret_cast<float *>(take(segs * dd * 4));
-        w.seg_carry = reinterpret_cast<float *>(take(segs * g.dk * 4));
-        w.seg_state16 = reinterpret_cast<__half *>(take(segs * dd * 2));
-        w.slot_s = reinterpret_cast<__half *>(take(slots * dd * 2));
-        w.slot_g = reinterpret_cast<float *>(take(slots * g.dk * 4));
-    }
-    w.bytes = o;
-    return w;
-}
-
-// Segment length.  Cost of a pass in 0.1 us, fitted to 1086 measured cuts of 2 to 768 sequences of 2 to 32 tiles, chunks of 16,
-// 32 and 64, d = 64 and 72 (root mean square of the fit's error 3 to 5%): launches, a fill per round of CTAs, tiles, and the
-// scan.  An SM with one CTA works a tile in two thirds of the time that two sharing it take.  Uncut sequences run the forward
-// sweep alone; cut ones also the local sweep and the scan; the backward pass needs the local sweep in either case.  Sub-chunks
-// multiply the tiles' cost, so short sequences in short chunks are cut where whole tiles would not be (3 tiles of 6
-// sequences, d = 64, chunks of 16: 24.4 us uncut, 18.7 cut; chunks of 64: 9.1 uncut).  A cut has to win by 2 us (backward: 1),
-// which its launches cost the host where nothing else keeps the device busy (a 256-token image: 19.2 us per block uncut, 22.6
-// cut, although the device is 0.6 us faster).  The cut chosen is within 19% of the best one, 0.3% off on average; a model of
-// rounds and tiles alone was 6% off on average and up to 2.2 times (5 tiles of 2 sequences, d = 72, chunks of 16: 53.6 us
-// uncut, 24.1 cut).
-struct PassCost {
-    int fixed[2], round[2], pair[2], alone[2];      // [cut]; pair: a tile on an SM with two CTAs, alone: with one
-    int scan;                                       // per machine full of segments
-    int chunk32, chunk16, d72;                      // factors of a tile's cost, per cent
-};
-constexpr PassCost kForward = {{21, 75}, {5, 8}, {32, 51}, {22, 37}, 35, 190, 310, 140};
-constexpr PassCost kBackward = {{14, 54}, {32, 23}, {88, 95}, {62, 73}, 67, 170, 280, 150};
-// Chunks above 64 tokens: forward plans stay within the scratch of dig_gla_fwd_static where uncut sequences do (the
-// same plan serves dig_gla_fwd, so that both give the same bits).  No other family's workspace is counted there that
-// would be larger anyway; with chunks of up to 64 the per-chunk states of the other families always are.
-Plan make_plan(const Geom &g, int sms, int per_sm, bool backward, long long *least = nullptr)
-{
-    Plan p;
-    p.ntile = (g.L + T - 1) / T;
-    p.sub_max = g.C < T ? g.C : T;
-    p.gh_inv = g.gh > 1 ? (uint32_t)((1ull << 32) / (unsigned)g.gh) : 0xffffffffu;
-    const PassCost &c = backward ? kBackward : kForward;
-    const long long slots = (long long)sms * per_sm, bh = (long long)g.B * g.H;
-    const long long tile = (p.sub_max == 16 ? c.chunk16 : p.sub_max == 32 ? c.chunk32 : 100) * (g.dk == 72 ? c.d72 : 100) / 100;      // per cent
-    long long best = -1;
-    p.G = p.ntile;
-    // the shortest G of every number of segments that occurs (about 2 sqrt(ntile) of them)
-    for (int nseg = 1, G = p.ntile;; nseg = (p.ntile + G - 2) / (G - 1), G = (p.ntile + nseg - 1) / nseg) {
-        const long long segs = bh * nseg, rest = segs % slots;
-        const long long pairs = segs / slots + (rest > sms), alone = rest > 0 && rest <= sms;          // rounds of either kind
-        const int cut = nseg > 1;
-        const long long cost = 100 * (c.fixed[cut] + (pairs + alone) * c.round[cut]) + tile * G * (pairs * c.pair[cut] + alone * c.alone[cut]) +
-                               (cut ? 100 * c.scan * segs / slots : 0);
-        p.nseg = nseg;
-        const bool fits = backward || g.C <= T || nseg == 1 || carve(nullptr, g, p, false).bytes <= DIG_GLA_STATIC_SCRATCH_BYTES;
-        if (best < 0 || (cost < best && fits)) {
-            best = cost;
-            p.G = G;
-        }
-        if (G == 1) break;
-    }
-    p.nseg = (p.ntile + p.G - 1) / p.G;
-    if (least) *least = best;
-    return p;
-}
-
 template <typename K>
 dig_status set_smem(K kern, size_t bytes)
 {
@@ -1409,31 +1332,6 @@ __global__ void __launch_bounds__(256) sum_orders(const SumArgs a, int n, size_t
     else store_out8(static_cast<bf16 *>(a.dst[blockIdx.y]) + 8 * i, f[0]);
 }
 
-// Scan orders of a forward pass that share a launch.  Where a sequence has too few tiles to fill the machine, orders side by
-// side need fewer cuts or none, so no local sweep and no scan; the results of a launch's orders then stand in buffers of their
-// own, later launches add to them, and one pass sums the buffers.  Costs as in make_plan, plus the buffers beyond the first,
-// written and read at 0.6 MB per 0.1 us.  768 tiles in 48 sequences, d = 64, four orders: 127 us one after the other, 82 side by
-// side.  Backward passes keep one order per launch: pairs took 180 instead of 198 us there, but their four tensors' buffers
-// cost as much more in the sum.  Offsets of the results have 31 bits.
-int orders_together(const Geom &g, int sms, bool backward, int n)
-{
-    const size_t elems = (size_t)g.B * g.L * g.H * g.dk;
-    long long best = -1;
-    int k = 1;
-    for (int j = 1; j <= (backward ? 1 : n); j *= 2) {
-        if (j > 1 && elems * j >= (1ull << 31)) break;
-        Geom h = g;
-        h.B *= j;
-        long long cost = 0;
-        make_plan(h, sms, kPerSm, backward, &cost);
-        cost = cost * ((n + j - 1) / j) + (long long)(100 * (j - 1) * 8 * elems / 600000);
-        if (best < 0 || cost < best) {
-            best = cost;
-            k = j;
-        }
-    }
-    return k;
-}
 // Bytes of one tensor's buffers: bf16 results and results of several orders are summed in the workspace.
 size_t multi_buffer_bytes(const Geom &g, int k) { return align256((size_t)g.B * g.L * g.H * g.dk * 4 * k); }
 
