@@ -231,6 +231,7 @@ dig_status dig_gla_fwd_state(const void *q, const void *k, const void *v, const 
     a.sio.s_in = s_in; a.sio.s_out = s_out;
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.out = out;
     a.ws = reinterpret_cast<float *>(workspace);
+    a.ws_bytes = workspace_bytes;
     a.g = make_geom(B, H, grid_h, grid_w, d_k, d_v, tile_chunk(impl, chunk), direction);
     a.dtype = dtype;
     a.stream = (cudaStream_t)cuda_stream;
@@ -258,6 +259,7 @@ dig_status dig_gla_bwd_state(const void *q, const void *k, const void *v, const 
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.d_out = d_out;
     a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate;
     a.ws = reinterpret_cast<float *>(workspace);
+    a.ws_bytes = workspace_bytes;
     a.g = make_geom(B, H, grid_h, grid_w, d_k, d_v, tile_chunk(impl, chunk), direction);
     a.dtype = dtype;
     a.stream = (cudaStream_t)cuda_stream;
@@ -364,6 +366,7 @@ dig_status dig_gla_fwd_outgate(const void *q, const void *k, const void *v, cons
     GlaArgs a{};
     a.q = q; a.k = k; a.v = v; a.gate = gate;
     a.ws = reinterpret_cast<float *>(workspace);
+    a.ws_bytes = workspace_bytes;
     a.g = make_geom(B, H, grid_h, grid_w, d_k, d_v, tile_chunk(impl, chunk), direction);
     a.dtype = dtype;
     a.stream = (cudaStream_t)cuda_stream;
@@ -398,6 +401,7 @@ dig_status dig_gla_fwd_beta(const void *q, const void *k, const void *v, const f
     a.bio.bgate = bgate;
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.out = out;
     a.ws = reinterpret_cast<float *>(workspace);
+    a.ws_bytes = workspace_bytes;
     a.g = make_geom(B, H, grid_h, grid_w, d_k, d_v, chunk, direction);
     a.dtype = dtype;
     a.stream = (cudaStream_t)cuda_stream;
@@ -422,6 +426,7 @@ dig_status dig_gla_bwd_beta(const void *q, const void *k, const void *v, const f
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.d_out = d_out;
     a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate;
     a.ws = reinterpret_cast<float *>(workspace);
+    a.ws_bytes = workspace_bytes;
     a.g = make_geom(B, H, grid_h, grid_w, d_k, d_v, chunk, direction);
     a.dtype = dtype;
     a.stream = (cudaStream_t)cuda_stream;
@@ -450,6 +455,7 @@ dig_status dig_gla_fwd_multi(const void *q, const void *k, const void *v, const 
     GlaArgs a{};
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.out = out;
     a.ws = reinterpret_cast<float *>(workspace);
+    a.ws_bytes = workspace_bytes;
     a.g = make_geom(B, H, grid_h, grid_w, d_k, d_v, chunk, 0);
     a.dtype = dtype;
     a.stream = (cudaStream_t)cuda_stream;
@@ -474,6 +480,7 @@ dig_status dig_gla_bwd_multi(const void *q, const void *k, const void *v, const 
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.d_out = d_out;
     a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate;
     a.ws = reinterpret_cast<float *>(workspace);
+    a.ws_bytes = workspace_bytes;
     a.g = make_geom(B, H, grid_h, grid_w, d_k, d_v, chunk, 0);
     a.dtype = dtype;
     a.stream = (cudaStream_t)cuda_stream;

@@ -114,6 +114,7 @@ struct GlaArgs {
     void *dq, *dk, *dv;
     float *dgate;
     float *ws;                   // workspace base (fp32 view)
+    size_t ws_bytes;
     Geom g;
     int dtype;
     int accumulate;              // outputs are added to what the (fp32) output buffers hold

@@ -1211,6 +1211,7 @@ dig_status run(const GlaArgs &ga, int n, uint32_t dirs, size_t stride)
     if (!status || sms <= 0) return DIG_ERR_CUDA;
     const Plan pl = make_plan(g, sms, kPerSm, BWD);
     const SweepWs w = carve(reinterpret_cast<char *>(ga.ws), g, pl, BWD);
+    if (w.bytes > ga.ws_bytes) return DIG_ERR_WORKSPACE;
     const long long total = (long long)g.B * g.H * pl.nseg;
     if (total > (1ll << 30) || (long long)g.B * g.L * g.H * D >= (1ll << 31)) return DIG_ERR_UNSUPPORTED;     // 31-bit row offsets
     SweepArgs a{};
@@ -1293,8 +1294,7 @@ size_t sweep_workspace_bytes(const Geom &g, bool backward)
 {
     int sms = device_sm_count();
     if (sms <= 0) sms = 148;
-    const Plan pl = make_plan(g, sms, kPerSm, backward);
-    return carve(nullptr, g, pl, backward).bytes;
+    return launch_bytes(g, sms, backward, 1);
 }
 
 namespace {
@@ -1332,20 +1332,6 @@ __global__ void __launch_bounds__(256) sum_orders(const SumArgs a, int n, size_t
     else store_out8(static_cast<bf16 *>(a.dst[blockIdx.y]) + 8 * i, f[0]);
 }
 
-// Bytes of one tensor's buffers: bf16 results and results of several orders are summed in the workspace.
-size_t multi_buffer_bytes(const Geom &g, int k) { return align256((size_t)g.B * g.L * g.H * g.dk * 4 * k); }
-
-size_t multi_bytes(const Geom &g, int sms, bool backward, int dtype, int n)
-{
-    const int k = orders_together(g, sms, backward, n);
-    Geom h = g;
-    h.B *= k;
-    size_t bytes = align256(sweep_workspace_bytes(h, backward));
-    if (k > 1) bytes += multi_buffer_bytes(g, k) * (backward ? 4 : 1);
-    else if (dtype == DIG_BF16) bytes += multi_buffer_bytes(g, 1) * (backward ? 3 : 1);
-    return bytes;
-}
-
 }  // namespace
 
 // Several scan orders summed (Algorithm 2 / Algorithm 3): groups of orders one after the other, each launch adding
@@ -1358,7 +1344,7 @@ size_t sweep_multi_workspace_bytes(const Geom &g, bool backward, int dtype)
     if (sms <= 0) sms = 148;
     size_t most = 0;
     for (int n = 1; n <= 4; ++n) {
-        const size_t b = multi_bytes(g, sms, backward, dtype, n);
+        const size_t b = multi_ws(g, sms, backward, dtype, n, orders_together(g, sms, backward, n)).bytes();
         most = b > most ? b : most;
     }
     return most;
@@ -1373,18 +1359,20 @@ dig_status sweep_multi(const GlaArgs &a0, bool backward, unsigned mask)
     GlaArgs a = a0;
     const size_t elems = (size_t)a.g.B * a.g.L * a.g.H * a.g.dk;          // d_k = d_v
     const int n = __builtin_popcount(mask), k = orders_together(a.g, sms, backward, n);
-    Geom h = a.g;
-    h.B *= k;
-    char *extra = reinterpret_cast<char *>(a0.ws) + align256(sweep_workspace_bytes(h, backward));
     const bool narrow = a0.dtype == DIG_BF16;
+    const MultiWs ws = multi_ws(a.g, sms, backward, a0.dtype, n, k);
+    if (a0.ws_bytes < ws.bytes()) return DIG_ERR_WORKSPACE;
+    char *buffers = reinterpret_cast<char *>(a0.ws);
+    a.ws = reinterpret_cast<float *>(buffers + ws.buffer * ws.buffers);
+    a.ws_bytes = ws.launch;
     void *const result[4] = {backward ? a0.dq : a0.out, a0.dk, a0.dv, a0.dgate};
     SumArgs sum{};
     int sums = 0;
     auto buffer = [&](int t) -> void * {
         const bool f32 = !narrow || t == 3;
         if (k == 1 && f32) return result[t];
-        float *p = reinterpret_cast<float *>(extra);
-        extra += multi_buffer_bytes(a.g, k);
+        float *p = reinterpret_cast<float *>(buffers);
+        buffers += ws.buffer;
         sum.src[sums] = p;
         sum.dst[sums] = result[t];
         sum.f32[sums++] = f32;

@@ -111,5 +111,33 @@ inline int orders_together(const Geom &g, int sms, bool backward, int n)
     return k;
 }
 
+// Workspace of one launch of `orders` scan orders, without buffers of results.
+inline size_t launch_bytes(const Geom &g, int sms, bool backward, int orders)
+{
+    Geom h = g;
+    h.B *= orders;
+    return carve(nullptr, h, make_plan(h, sms, kPerSm, backward), backward).bytes;
+}
+// Workspace of a sum over n orders, k to a launch: the buffers of bf16 results and of results of several orders in front, and
+// behind them what the largest of its launches needs.  A last launch of fewer orders is planned by itself and may be cut where
+// the others are not: three orders of 8 x 32 x 32 tokens, 6 heads of 64, are a pair in 1.6 MB and one order in 4.8 MB.
+struct MultiWs {
+    size_t buffer;              // bytes of one tensor's buffers
+    int buffers;                // tensors that have them
+    size_t launch;
+    size_t bytes() const { return buffer * buffers + launch; }
+};
+inline MultiWs multi_ws(const Geom &g, int sms, bool backward, int dtype, int n, int k)
+{
+    MultiWs w{align256((size_t)g.B * g.L * g.H * g.dk * 4 * k), 0, launch_bytes(g, sms, backward, k)};
+    if (k > 1) w.buffers = backward ? 4 : 1;
+    else if (dtype == DIG_BF16) w.buffers = backward ? 3 : 1;
+    if (n % k) {
+        const size_t rest = launch_bytes(g, sms, backward, n % k);
+        w.launch = rest > w.launch ? rest : w.launch;
+    }
+    return w;
+}
+
 }  // namespace sw
 }  // namespace dig

@@ -15,8 +15,8 @@ FORWARD = ((21, 75), (5, 8), (32, 51), (22, 37), 35, {32: 190, 16: 310}, 140)
 BACKWARD = ((14, 54), (32, 23), (88, 95), (62, 73), 67, {32: 170, 16: 280}, 150)
 
 
-def sweep_plan(sequences: int, ntile: int, backward: bool, chunk: int = 64, d: int = 64, limit: int | None = None) -> tuple[int, int]:
-    """(segments per sequence, tiles per segment); limit: bytes that forward passes in chunks above 64 keep to."""
+def costed_plan(sequences: int, ntile: int, backward: bool, chunk: int = 64, d: int = 64, limit: int | None = None) -> tuple[int, int, int]:
+    """(segments per sequence, tiles per segment, cost); limit: bytes that forward passes in chunks above 64 keep to."""
     fixed, fill, pair, alone, scan, sub, d72 = BACKWARD if backward else FORWARD
     tile = sub.get(chunk, 100) * (d72 if d == 72 else 100) // 100
     sms, best, best_g = 148, None, ntile
@@ -34,4 +34,33 @@ def sweep_plan(sequences: int, ntile: int, backward: bool, chunk: int = 64, d: i
             break
         nseg = -(-ntile // (g - 1))
         g = -(-ntile // nseg)
-    return -(-ntile // best_g), best_g
+    return -(-ntile // best_g), best_g, best
+
+
+def sweep_plan(*args, **kw) -> tuple[int, int]:
+    """(segments per sequence, tiles per segment)."""
+    return costed_plan(*args, **kw)[:2]
+
+
+def orders_together(B: int, H: int, L: int, d: int, chunk: int, orders: int) -> int:
+    """Scan orders that share a launch of a forward sum (chunks of up to 64)."""
+    elems, best, k, j = B * L * H * d, None, 1, 1
+    while j <= orders and (j == 1 or elems * j < 1 << 31):
+        cost = costed_plan(B * H * j, -(-L // 64), False, chunk, d)[2] * -(-orders // j) + 100 * (j - 1) * 8 * elems // 600000
+        if best is None or cost < best:
+            best, k = cost, j
+        j *= 2
+    return k
+
+
+def launch_bytes(B: int, H: int, L: int, d: int, chunk: int, orders: int) -> int:
+    """Workspace of one launch of so many orders of a forward sum, without the buffers of the results."""
+    nseg, _ = sweep_plan(B * H * orders, -(-L // 64), False, chunk, d)
+    return segment_bytes(B * H * orders * nseg, d)
+
+
+def multi_bytes(B: int, H: int, L: int, d: int, chunk: int, orders: int, bf16_out: bool) -> int:
+    """Workspace of a forward sum over so many orders: the buffers and the largest of its launches."""
+    k = orders_together(B, H, L, d, chunk, orders)
+    buffers = -(-B * L * H * d * 4 * k // 256) * 256 if k > 1 or bf16_out else 0
+    return buffers + max(launch_bytes(B, H, L, d, chunk, n) for n in (k, orders % k) if n)

@@ -1,8 +1,11 @@
 """The cut of the tcgen05 kernels as the workspace sizes show it: against its restatement, and against the scratch of
 dig_gla_fwd_static, whose limit is what dig_gla_workspace_bytes asks for."""
+import os
+import subprocess
+
 import pytest
 
-from sweep_plan import segment_bytes, sweep_plan
+from sweep_plan import multi_bytes, segment_bytes, sweep_plan
 
 
 @pytest.fixture(scope="module")
@@ -35,3 +38,55 @@ def test_cutting_sequences_does_not_exceed_the_static_scratch(dig):
     for bh, t in SHAPES:
         if segment_bytes(bh, 72) <= limit:
             assert need(1, bh, 8, 8 * t, 72) <= limit, (bh, t)
+
+
+def test_restated_orders_give_the_librarys_workspace(dig):
+    for B, H in [(1, 6), (2, 6), (4, 6), (8, 6), (2, 16), (16, 12)]:
+        for t in (1, 2, 3, 5, 7, 9, 16, 20, 36):
+            for d in (64, 72):
+                for chunk in (16, 32, 64):
+                    for dtype in (dig.DIG_BF16, dig.DIG_BF16_F32OUT):
+                        want = max(multi_bytes(B, H, 64 * t, d, chunk, n, dtype == dig.DIG_BF16) for n in (1, 2, 3, 4))
+                        assert dig.dig_gla_multi_workspace_bytes(B, H, 8, 8 * t, d, d, chunk, dtype, 0) == want, (B, H, t, d, chunk)
+
+
+def test_launches_of_a_sum_stay_clear_of_its_buffers(tmp_path):
+    """The layout itself, compiled from the plan's header: behind the buffers there is room for every launch of a sum, a last
+    one of fewer orders among them, which may be cut into more segments than the launches in front of it."""
+    from paper_2405_18428_b200 import build
+    src = tmp_path / "layout.cu"
+    src.write_text(r"""
+#include <cstdio>
+#include "sweep_plan.cuh"
+using namespace dig;
+using namespace dig::sw;
+int main()
+{
+    long short_last = 0, over = 0;
+    for (int B : {1, 2, 4, 8, 16, 40}) for (int H : {1, 6, 12, 16}) for (int t = 1; t <= 64; ++t)
+    for (int d : {64, 72}) for (int C : {16, 32, 64, 128}) for (int bwd = 0; bwd < 2; ++bwd) for (int n = 1; n <= 4; ++n) {
+        Geom g{};
+        g.B = B; g.H = H; g.gh = 8; g.gw = 8 * t; g.L = 64 * t; g.dk = g.dv = d; g.C = C; g.N = (g.L + C - 1) / C;
+        const int k = orders_together(g, 148, bwd, n);
+        const MultiWs w = multi_ws(g, 148, bwd, DIG_BF16, n, k);
+        for (int left = n; left > 0; left -= k) {
+            Geom h = g;
+            h.B *= left < k ? left : k;
+            const size_t need = carve(nullptr, h, make_plan(h, 148, kPerSm, bwd), bwd).bytes;
+            over += w.buffer * w.buffers + need > w.bytes();
+            if (left < k) {
+                Geom f = g;
+                f.B *= k;
+                short_last += need > carve(nullptr, f, make_plan(f, 148, kPerSm, bwd), bwd).bytes;
+            }
+        }
+    }
+    printf("%ld %ld\n", short_last, over);
+    return 0;
+}
+""")
+    exe = tmp_path / "layout"
+    subprocess.run([os.environ.get("NVCC", "nvcc"), *build.NVCC_FLAGS, str(src), "-o", str(exe)], check=True, capture_output=True)
+    short_last, over = map(int, subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split())
+    assert over == 0
+    assert short_last > 100        # the sizes at which the last launch needs the most are among them
