@@ -634,6 +634,16 @@ __device__ __forceinline__ void issue_split(uint32_t acc, const char *tA, const 
     issue<64, 8 * L::NV0, false, true, KSTEPS, C::CHT, BCH, 128, ROWS>(acc, a, b, accumulate);
     issue<64, 8 * L::NV1, false, true, KSTEPS, C::CHT, BCH, 128, ROWS>(acc + kHiLanes, a, b + L::NV0 * BCH, accumulate);
 }
+// acc += P V, P the masked scores, the value channels split
+template <int D>
+__device__ __forceinline__ void issue_weighted(uint32_t acc, const char *tP, const char *tV)
+{
+    using C = Cfg<D>;
+    using L = Col<D>;
+    const uint32_t a = smem_u32(tP), b = smem_u32(tV);
+    issue_triangle<8 * L::NV0, false, C::CHT, C::CHT>(acc, a, b);
+    issue_triangle<8 * L::NV1, false, C::CHT, C::CHT>(acc + kHiLanes, a, b + L::NV0 * C::CHT);
+}
 // acc <- A B^T (scores), columns split into even (lanes 0-15) and odd (lanes 16-31) 8-token chunks
 template <int D>
 __device__ __forceinline__ void issue_scores(uint32_t acc, const char *tA, const char *tB)

@@ -775,7 +775,8 @@ sweep_fwd(const SweepArgs a)
                             issue_split<D, C::KS, C::CHS, kHighRows>(tmem + SM::aO, tQ, tS, false);
                             issue_state<D, kHighRows>(tmem + SM::aU, tK, tV);
                         }
-                        issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);                  // + P V
+                        if (PAIRS) issue_weighted<D>(tmem + SM::aO, tP, tV);                          // + P V
+                        else issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);
                         mma_commit(&ctl->bar[0]);
                     }
                     if (last && more) {                                // the next tile's gate sums while the products run
@@ -1074,9 +1075,15 @@ sweep_bwd(const SweepArgs a)
                         ok = mbar_wait(barS, par, a.status) && ok;
                         issue<64, D, false, false, C::KS, C::CHT, C::CHS, 128, kLowRows>(tmem + SM::aQK, sG, smem_u32(tS), false);
                     }
-                    issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK, sdP, sK, true);                   // + dP Kc
-                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK + kHiLanes, sdP, sQ, true);         // + dP^T Qc
-                    issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aV + kHiLanes, sP, sG, true);           // + P^T dO
+                    if (PAIRS) {
+                        issue_triangle<D, false, C::CHT, C::CHT>(tmem + SM::aQK, sdP, sK);                              // + dP Kc
+                        issue_triangle<D, true, C::CHT, C::CHT>(tmem + SM::aQK + kHiLanes, sdP, sQ);                    // + dP^T Qc
+                        issue_triangle<D, true, C::CHT, C::CHT>(tmem + SM::aV + kHiLanes, sP, sG);                      // + P^T dO
+                    } else {
+                        issue<64, D, false, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK, sdP, sK, true);
+                        issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aQK + kHiLanes, sdP, sQ, true);
+                        issue<64, D, true, true, T / 16, C::CHT, C::CHT>(tmem + SM::aV + kHiLanes, sP, sG, true);
+                    }
                     mma_commit(barG1);
                 }
                 ok = wait_all(barG1, 1, a.status, ok);

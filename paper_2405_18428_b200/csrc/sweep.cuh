@@ -125,8 +125,8 @@ __device__ __forceinline__ uint64_t mdesc(uint32_t saddr, uint32_t ch) { return 
 // low word: shared-memory addresses stay below 2^18, the address field cannot carry into the next).
 // BSBO: distance of the 8-row groups of a K-major B (256 takes every other group).  SKIP: quarters of the
 // accumulator's lanes that stay as they are (rows 16 q .. 16 q + 15 of an M = 64 product are in quarter q).
-template <int M, int N, bool A_MN, bool B_MN, int KSTEPS, uint32_t ACH, uint32_t BCH, uint32_t BSBO = 128, uint32_t SKIP = 0>
-__device__ __forceinline__ void issue(uint32_t d_tmem, uint32_t a, uint32_t b, bool accumulate)
+template <int M, int N, bool A_MN, bool B_MN, int KSTEPS, uint32_t ACH, uint32_t BCH, uint32_t BSBO, class F>
+__device__ __forceinline__ void each_step(uint32_t a, uint32_t b, F mma)
 {
     static_assert(M == 64 && N % 8 == 0, "instruction shape");
     constexpr uint32_t idesc = idesc_f16(M, N, A_MN, B_MN);
@@ -134,11 +134,26 @@ __device__ __forceinline__ void issue(uint32_t d_tmem, uint32_t a, uint32_t b, b
     constexpr uint32_t sa = A_MN ? 16u : (2u * ACH) >> 4, sb = B_MN ? 16u : (2u * BCH) >> 4;
     const uint32_t alo = (uint32_t)da, ahi = (uint32_t)(da >> 32), blo = (uint32_t)db, bhi = (uint32_t)(db >> 32);
 #pragma unroll
-    for (int kk = 0; kk < KSTEPS; ++kk) {
-        const uint64_t xa = ((uint64_t)ahi << 32) | (alo + kk * sa), xb = ((uint64_t)bhi << 32) | (blo + kk * sb);
+    for (int kk = 0; kk < KSTEPS; ++kk) mma(kk, ((uint64_t)ahi << 32) | (alo + kk * sa), ((uint64_t)bhi << 32) | (blo + kk * sb), idesc);
+}
+template <int M, int N, bool A_MN, bool B_MN, int KSTEPS, uint32_t ACH, uint32_t BCH, uint32_t BSBO = 128, uint32_t SKIP = 0>
+__device__ __forceinline__ void issue(uint32_t d_tmem, uint32_t a, uint32_t b, bool accumulate)
+{
+    each_step<M, N, A_MN, B_MN, KSTEPS, ACH, BCH, BSBO>(a, b, [&](int kk, uint64_t xa, uint64_t xb, uint32_t idesc) {
         if constexpr (SKIP == 0) mma_f16(d_tmem, xa, xb, idesc, accumulate || kk > 0);
         else mma_f16_part<SKIP>(d_tmem, xa, xb, idesc, accumulate || kk > 0);
-    }
+    });
+}
+// D += A * B with the 64 x 64 lower triangle A (TRANSPOSED: upper), in as many instructions: where half of A's rows are zero along
+// half of the contraction, they keep what they hold.  Zeros would do but for NaN, which they spread: where the halves are
+// sub-chunks, to rows that do not depend on it (in the other direction the state carries a NaN over in any case).
+template <int N, bool TRANSPOSED, uint32_t ACH, uint32_t BCH>
+__device__ __forceinline__ void issue_triangle(uint32_t d_tmem, uint32_t a, uint32_t b)
+{
+    each_step<64, N, TRANSPOSED, true, T / 16, ACH, BCH, 128>(a, b, [&](int kk, uint64_t xa, uint64_t xb, uint32_t idesc) {
+        if (TRANSPOSED != (kk < T / 32)) mma_f16(d_tmem, xa, xb, idesc, true);
+        else mma_f16_part<TRANSPOSED ? 0xcu : 0x3u>(d_tmem, xa, xb, idesc, true);
+    });
 }
 
 struct Ctl {

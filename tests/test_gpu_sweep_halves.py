@@ -1,7 +1,9 @@
 """GPU parity of the sweep kernels on tiles worked as two 32-row sub-chunks in one pass: last tiles that end around
 the middle, tiles of either kind side by side, short and uncut sequences, with a start state and its gradient."""
 import pytest
+import torch
 
+from paper_2405_18428_b200 import dig
 from paper_2405_18428_b200.inputs import Workload
 from test_gpu_state_io import _run
 
@@ -20,3 +22,30 @@ pytestmark = pytest.mark.gpu
 def test_tiles_in_two_halves(d, direction, L, B, H, chunk, tau):
     wl = Workload("halves", B=B, H=H, grid_h=1, grid_w=L, d_k=d, d_v=d, chunk=chunk, dtype="bf16", backward=True, tau=tau, seed=71)
     print(_run(wl, direction, 9))
+
+
+@pytest.mark.parametrize("d,direction", [(64, 0), (72, 0), (64, 1)])
+def test_a_nan_stays_in_its_half(d, direction):
+    """Two sub-chunks of a tile meet through the state alone: a NaN in the upper one leaves the rows before it as they were, a
+    NaN in the lower one the gradients of the rows behind it."""
+    L, H, at = 64 * 5 + 50, 2, 64 * 2
+    gen = torch.Generator(device="cuda").manual_seed(91)
+    x = {n: torch.randn((1, L, H, d), generator=gen, device="cuda").to(torch.bfloat16) for n in ("q", "k", "v", "dO")}
+    gate = dig.dig_gate_logsigmoid(torch.randn((1, L, H, d), generator=gen, device="cuda"), [16.0] * H)
+    rows = lambda lo, hi: slice(lo, hi) if direction == 0 else slice(L - hi, L - lo)        # scan positions -> tokens
+
+    def run(**bad):
+        y = dict(x)
+        for n, p in bad.items():
+            y[n] = x[n].clone()
+            y[n][:, rows(p, p + 1)] = float("nan")
+        out = dig.dig_gla_fwd(y["q"], y["k"], y["v"], gate, 1, L, 32, direction)
+        return out, *dig.dig_gla_bwd(y["q"], y["k"], y["v"], gate, y["dO"], 1, L, 32, direction)
+
+    clean, before, behind = run(), rows(0, at + 32), rows(at + 32, L)
+    for n in ("k", "v"):
+        for got, want, name in zip(run(**{n: at + 40})[:4], clean, ("out", "dq", "dk", "dv")):
+            assert torch.equal(got[:, before], want[:, before]), (n, name)
+    for n in ("q", "dO"):
+        for got, want, name in zip(run(**{n: at + 10}), clean, ("out", "dq", "dk", "dv", "dgate")):
+            assert torch.equal(got[:, behind], want[:, behind]), (n, name)
