@@ -250,7 +250,12 @@ dig_status dig_gla_bwd_beta(const void *q, const void *k, const void *v, const f
  * single-order gradients).  The orders run one after the other on the stream, or, in forward passes over short
  * sequences, several in a launch with buffers of their own that are added in a fixed order; each adds its fp32 results
  * to its buffer (caller's or workspace), so the sum is formed in fp32 and rounded to bf16 once.  Served by the
- * tcgen05 kernels only (bf16 storage, d_k = d_v = 64 or 72; else DIG_ERR_UNSUPPORTED); workspace from dig_gla_multi_workspace_bytes (0 for invalid or unsupported sizes).
+ * tcgen05 kernels only (bf16 storage, d_k = d_v = 64 or 72; else DIG_ERR_UNSUPPORTED).
+ * Workspace: dig_gla_multi_workspace_bytes (0 for invalid or unsupported sizes) is enough for every mask, in forward passes
+ * with up to four fp32 copies of out for orders that share a launch (8 x 32 x 32 tokens, 6 heads of 64: 53.5 MB).  A
+ * forward call takes less too and then runs fewer orders together, which is slower and may differ in the last bits: what
+ * dig_gla_workspace_bytes gives for the same sizes and, for DIG_BF16, one fp32 copy of out (its bytes rounded up to a
+ * multiple of 256) is enough for every mask.  Anything smaller may be refused (DIG_ERR_WORKSPACE).
  * Tensors, sizes and the gate range are those of dig_gla_fwd / dig_gla_bwd. */
 size_t dig_gla_multi_workspace_bytes(int B, int H, int grid_h, int grid_w, int d_k, int d_v, int chunk, int dtype,
                                      int backward);

@@ -450,8 +450,7 @@ dig_status dig_gla_fwd_multi(const void *q, const void *k, const void *v, const 
     if (direction_mask == 0 || direction_mask > 15u) return DIG_ERR_INVALID_ARG;
     if (!valid_geometry(B, H, grid_h, grid_w, d_k, d_v, chunk, 0, dtype)) return DIG_ERR_INVALID_ARG;
     if (!sweep_supports(d_k, d_v, chunk, dtype)) return DIG_ERR_UNSUPPORTED;
-    const size_t need = dig_gla_multi_workspace_bytes(B, H, grid_h, grid_w, d_k, d_v, chunk, dtype, 0);
-    if (!workspace || !aligned16(workspace) || workspace_bytes < need) return DIG_ERR_WORKSPACE;
+    if (!workspace || !aligned16(workspace)) return DIG_ERR_WORKSPACE;        // its size: sweep_gla_fwd_multi
     GlaArgs a{};
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.out = out;
     a.ws = reinterpret_cast<float *>(workspace);
@@ -474,8 +473,7 @@ dig_status dig_gla_bwd_multi(const void *q, const void *k, const void *v, const 
     if (direction_mask == 0 || direction_mask > 15u) return DIG_ERR_INVALID_ARG;
     if (!valid_geometry(B, H, grid_h, grid_w, d_k, d_v, chunk, 0, dtype)) return DIG_ERR_INVALID_ARG;
     if (!sweep_supports(d_k, d_v, chunk, dtype)) return DIG_ERR_UNSUPPORTED;
-    const size_t need = dig_gla_multi_workspace_bytes(B, H, grid_h, grid_w, d_k, d_v, chunk, dtype, 1);
-    if (!workspace || !aligned16(workspace) || workspace_bytes < need) return DIG_ERR_WORKSPACE;
+    if (!workspace || !aligned16(workspace)) return DIG_ERR_WORKSPACE;        // its size: sweep_gla_bwd_multi
     GlaArgs a{};
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.d_out = d_out;
     a.dq = dq; a.dk = dk; a.dv = dv; a.dgate = dgate;

@@ -1297,11 +1297,16 @@ bool sweep_supports(int dk, int dv, int chunk, int dtype)
     return dk == dv && (dk == 64 || dk == 72);
 }
 
+// SMs for sizes, which can be asked for without a device.
+static int device_sms()
+{
+    const int sms = device_sm_count();
+    return sms > 0 ? sms : 148;
+}
+
 size_t sweep_workspace_bytes(const Geom &g, bool backward)
 {
-    int sms = device_sm_count();
-    if (sms <= 0) sms = 148;
-    return launch_bytes(g, sms, backward, 1);
+    return launch_bytes(g, device_sms(), backward, 1);
 }
 
 namespace {
@@ -1347,11 +1352,10 @@ __global__ void __launch_bounds__(256) sum_orders(const SumArgs a, int n, size_t
 // scheduling.
 size_t sweep_multi_workspace_bytes(const Geom &g, bool backward, int dtype)
 {
-    int sms = device_sm_count();
-    if (sms <= 0) sms = 148;
+    const SumPlans plans(g, device_sms(), backward, dtype);
     size_t most = 0;
     for (int n = 1; n <= 4; ++n) {
-        const size_t b = multi_ws(g, sms, backward, dtype, n, orders_together(g, sms, backward, n)).bytes();
+        const size_t b = plans.of(n, SIZE_MAX).bytes();
         most = b > most ? b : most;
     }
     return most;
@@ -1361,25 +1365,23 @@ namespace {
 
 dig_status sweep_multi(const GlaArgs &a0, bool backward, unsigned mask)
 {
-    const int sms = device_sm_count();
-    if (sms <= 0) return DIG_ERR_CUDA;
     GlaArgs a = a0;
     const size_t elems = (size_t)a.g.B * a.g.L * a.g.H * a.g.dk;          // d_k = d_v
-    const int n = __builtin_popcount(mask), k = orders_together(a.g, sms, backward, n);
-    const bool narrow = a0.dtype == DIG_BF16;
-    const MultiWs ws = multi_ws(a.g, sms, backward, a0.dtype, n, k);
-    if (a0.ws_bytes < ws.bytes()) return DIG_ERR_WORKSPACE;
+    const int n = __builtin_popcount(mask);
+    const SumPlan plan = SumPlans(a.g, device_sms(), backward, a0.dtype).of(n, a0.ws_bytes);
+    if (plan.bytes() > a0.ws_bytes) return DIG_ERR_WORKSPACE;
+    const int k = plan.k;
     char *buffers = reinterpret_cast<char *>(a0.ws);
-    a.ws = reinterpret_cast<float *>(buffers + ws.buffer * ws.buffers);
-    a.ws_bytes = ws.launch;
+    a.ws = reinterpret_cast<float *>(buffers + plan.buffer * plan.buffers);
+    a.ws_bytes = plan.launch;
     void *const result[4] = {backward ? a0.dq : a0.out, a0.dk, a0.dv, a0.dgate};
     SumArgs sum{};
     int sums = 0;
     auto buffer = [&](int t) -> void * {
-        const bool f32 = !narrow || t == 3;
+        const bool f32 = a0.dtype != DIG_BF16 || t == 3;
         if (k == 1 && f32) return result[t];
         float *p = reinterpret_cast<float *>(buffers);
-        buffers += ws.buffer;
+        buffers += plan.buffer;
         sum.src[sums] = p;
         sum.dst[sums] = result[t];
         sum.f32[sums++] = f32;

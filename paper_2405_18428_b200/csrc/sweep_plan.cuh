@@ -85,59 +85,61 @@ inline Plan make_plan(const Geom &g, int sms, int per_sm, bool backward, long lo
     return p;
 }
 
-// Scan orders of a forward pass that share a launch.  Where a sequence has too few tiles to fill the machine, orders side by
-// side need fewer cuts or none, so no local sweep and no scan; the results of a launch's orders then stand in buffers of their
-// own, later launches add to them, and one pass sums the buffers.  Costs as in make_plan, plus the buffers beyond the first,
-// written and read at 0.6 MB per 0.1 us.  768 tiles in 48 sequences, d = 64, four orders: 127 us one after the other, 82 side by
-// side.  Backward passes keep one order per launch: pairs took 180 instead of 198 us there, but their four tensors' buffers
-// cost as much more in the sum.  Offsets of the results have 31 bits.
-inline int orders_together(const Geom &g, int sms, bool backward, int n)
-{
-    const size_t elems = (size_t)g.B * g.L * g.H * g.dk;
-    long long best = -1;
-    int k = 1;
-    for (int j = 1; j <= (backward ? 1 : n); j *= 2) {
-        if (j > 1 && elems * j >= (1ull << 31)) break;
-        Geom h = g;
-        h.B *= j;
-        long long cost = 0;
-        make_plan(h, sms, kPerSm, backward, &cost);
-        cost = cost * ((n + j - 1) / j) + (long long)(100 * (j - 1) * 8 * elems / 600000);
-        if (best < 0 || cost < best) {
-            best = cost;
-            k = j;
-        }
-    }
-    return k;
-}
-
 // Workspace of one launch of `orders` scan orders, without buffers of results.
-inline size_t launch_bytes(const Geom &g, int sms, bool backward, int orders)
+inline size_t launch_bytes(const Geom &g, int sms, bool backward, int orders, long long *cost = nullptr)
 {
     Geom h = g;
     h.B *= orders;
-    return carve(nullptr, h, make_plan(h, sms, kPerSm, backward), backward).bytes;
+    return carve(nullptr, h, make_plan(h, sms, kPerSm, backward, cost), backward).bytes;
 }
-// Workspace of a sum over n orders, k to a launch: the buffers of bf16 results and of results of several orders in front, and
-// behind them what the largest of its launches needs.  A last launch of fewer orders is planned by itself and may be cut where
-// the others are not: three orders of 8 x 32 x 32 tokens, 6 heads of 64, are a pair in 1.6 MB and one order in 4.8 MB.
-struct MultiWs {
+
+// A sum over scan orders: k of them to a launch.  Its workspace has the buffers of bf16 results and of results of several
+// orders in front, and behind them what the largest of its launches needs.  A last launch of fewer orders is planned by itself
+// and may be cut where the others are not: three orders of 8 x 32 x 32 tokens, 6 heads of 64, are a pair in 1.6 MB and one order
+// in 4.8 MB.
+struct SumPlan {
+    int k;
     size_t buffer;              // bytes of one tensor's buffers
     int buffers;                // tensors that have them
     size_t launch;
     size_t bytes() const { return buffer * buffers + launch; }
 };
-inline MultiWs multi_ws(const Geom &g, int sms, bool backward, int dtype, int n, int k)
-{
-    MultiWs w{align256((size_t)g.B * g.L * g.H * g.dk * 4 * k), 0, launch_bytes(g, sms, backward, k)};
-    if (k > 1) w.buffers = backward ? 4 : 1;
-    else if (dtype == DIG_BF16) w.buffers = backward ? 3 : 1;
-    if (n % k) {
-        const size_t rest = launch_bytes(g, sms, backward, n % k);
-        w.launch = rest > w.launch ? rest : w.launch;
+// Where a sequence has too few tiles to fill the machine, orders of a forward pass side by side need fewer cuts or none, so no
+// local sweep and no scan; the results of a launch's orders then stand in buffers of their own, later launches add to them, and
+// one pass sums the buffers.  Costs as in make_plan, plus the buffers beyond the first, written and read at 0.6 MB per 0.1 us.
+// 768 tiles in 48 sequences, d = 64, four orders: 127 us one after the other, 82 side by side.  Backward passes keep one order
+// per launch: pairs took 180 instead of 198 us there, but their four tensors' buffers cost as much more in the sum.  Offsets of
+// the results have 31 bits.
+class SumPlans {
+    const Geom &g;
+    const bool backward, narrow;
+    size_t elems, launch[3];    // of launches of 1, 2 and 4 orders
+    long long cost[3];
+    int sizes;
+
+public:
+    SumPlans(const Geom &geom, int sms, bool bwd, int dtype) : g(geom), backward(bwd), narrow(dtype == DIG_BF16), elems((size_t)g.B * g.L * g.H * g.dk)
+    {
+        for (sizes = 0; sizes < (backward ? 1 : 3) && (sizes == 0 || elems << sizes < 1ull << 31); ++sizes) launch[sizes] = launch_bytes(g, sms, backward, 1 << sizes, cost + sizes);
     }
-    return w;
-}
+    // n orders, the cheapest way whose workspace is at most `limit`; one order per launch where none is
+    SumPlan of(int n, size_t limit) const
+    {
+        SumPlan best{};
+        long long least = -1;
+        for (int i = 0; i < sizes && 1 << i <= n; ++i) {
+            SumPlan p{1 << i, align256(elems * 4 << i), 0, launch[i]};
+            p.buffers = backward ? (narrow ? 3 : 0) : (narrow || i > 0);
+            if (n == 3 && i == 1 && launch[0] > launch[1]) p.launch = launch[0];          // the third order's launch
+            const long long c = cost[i] * ((n + p.k - 1) / p.k) + (long long)(100 * (p.k - 1) * 8 * elems / 600000);
+            if (least < 0 || (c < least && p.bytes() <= limit)) {
+                least = c;
+                best = p;
+            }
+        }
+        return best;
+    }
+};
 
 }  // namespace sw
 }  // namespace dig

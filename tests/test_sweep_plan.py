@@ -52,7 +52,8 @@ def test_restated_orders_give_the_librarys_workspace(dig):
 
 def test_launches_of_a_sum_stay_clear_of_its_buffers(tmp_path):
     """The layout itself, compiled from the plan's header: behind the buffers there is room for every launch of a sum, a last
-    one of fewer orders among them, which may be cut into more segments than the launches in front of it."""
+    one of fewer orders among them, which may be cut into more segments than the launches in front of it.  A workspace for one
+    order per launch is enough for every sum."""
     from paper_2405_18428_b200 import build
     src = tmp_path / "layout.cu"
     src.write_text(r"""
@@ -62,31 +63,35 @@ using namespace dig;
 using namespace dig::sw;
 int main()
 {
-    long short_last = 0, over = 0;
+    long short_last = 0, over = 0, fewer = 0;
     for (int B : {1, 2, 4, 8, 16, 40}) for (int H : {1, 6, 12, 16}) for (int t = 1; t <= 64; ++t)
-    for (int d : {64, 72}) for (int C : {16, 32, 64, 128}) for (int bwd = 0; bwd < 2; ++bwd) for (int n = 1; n <= 4; ++n) {
+    for (int d : {64, 72}) for (int C : {16, 32, 64, 128}) for (int bwd = 0; bwd < 2; ++bwd) for (int dt : {DIG_BF16, DIG_BF16_F32OUT}) {
         Geom g{};
         g.B = B; g.H = H; g.gh = 8; g.gw = 8 * t; g.L = 64 * t; g.dk = g.dv = d; g.C = C; g.N = (g.L + C - 1) / C;
-        const int k = orders_together(g, 148, bwd, n);
-        const MultiWs w = multi_ws(g, 148, bwd, DIG_BF16, n, k);
-        for (int left = n; left > 0; left -= k) {
+        const SumPlans plans(g, 148, bwd, dt);
+        auto bytes = [&](int orders) {
             Geom h = g;
-            h.B *= left < k ? left : k;
-            const size_t need = carve(nullptr, h, make_plan(h, 148, kPerSm, bwd), bwd).bytes;
-            over += w.buffer * w.buffers + need > w.bytes();
-            if (left < k) {
-                Geom f = g;
-                f.B *= k;
-                short_last += need > carve(nullptr, f, make_plan(f, 148, kPerSm, bwd), bwd).bytes;
+            h.B *= orders;
+            return carve(nullptr, h, make_plan(h, 148, kPerSm, bwd), bwd).bytes;
+        };
+        const size_t one = bytes(1) + (dt == DIG_BF16 ? (bwd ? 3 : 1) * align256((size_t)B * g.L * H * d * 4) : 0);      // one order per launch
+        for (int n = 1; n <= 4; ++n) for (size_t limit : {SIZE_MAX, one}) {
+            const SumPlan p = plans.of(n, limit);
+            over += p.bytes() > limit;
+            fewer += limit == one && p.k < plans.of(n, SIZE_MAX).k;
+            for (int left = n; left > 0; left -= p.k) {
+                const size_t need = bytes(left < p.k ? left : p.k);
+                over += p.buffer * p.buffers + need > p.bytes();
+                short_last += left < p.k && need > bytes(p.k);
             }
         }
     }
-    printf("%ld %ld\n", short_last, over);
+    printf("%ld %ld %ld\n", short_last, over, fewer);
     return 0;
 }
 """)
     exe = tmp_path / "layout"
     subprocess.run([os.environ.get("NVCC", "nvcc"), *build.NVCC_FLAGS, str(src), "-o", str(exe)], check=True, capture_output=True)
-    short_last, over = map(int, subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split())
+    short_last, over, fewer = map(int, subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split())
     assert over == 0
-    assert short_last > 100        # the sizes at which the last launch needs the most are among them
+    assert short_last > 100 and fewer > 1000       # sizes at which the last launch needs the most, or orders part, are among them
