@@ -241,21 +241,21 @@ __device__ __noinline__ int choose_window(const float *sTot, Who<D> w, int start
         }
     }
 }
-// Sub-chunk length of a tile whose totals are tt; tt becomes the totals of the (sub-)chunk the thread's rows are in.  Halves,
+// Sub-chunk length of a tile whose totals are tt; tt becomes the totals of the (sub-)chunk the thread's rows are in.  HALVES: halves,
 // which chunks of 32 ask for and which suffice for most tiles beyond the limit, are tried with sums over fixed groups (the
 // search takes a few hundred cycles).
-template <int D>
+template <int D, bool HALVES>
 __device__ __forceinline__ int divide_tile(const float *sTot, const Who<D> &w, int sub_max, int *status, Tot &tt)
 {
     if (sub_max >= T && !beyond<D>(tt)) return T;
-    if (sub_max >= T / 2) {
+    if (HALVES && sub_max >= T / 2) {
         const Tot lo = half_totals<D, 0>(sTot, w), hi = half_totals<D, 1>(sTot, w);
         if (!beyond<D>(lo) && !beyond<D>(hi)) {
             tt = w.grp < 4 ? lo : hi;
             return T / 2;
         }
     }
-    const int s = choose_window<D>(sTot, w, min(sub_max, T / 4), status), w0 = 8 * w.grp / s * (s / 8);
+    const int s = choose_window<D>(sTot, w, min(sub_max, HALVES ? T / 4 : T / 2), status), w0 = 8 * w.grp / s * (s / 8);
     tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
     return s;
 }
