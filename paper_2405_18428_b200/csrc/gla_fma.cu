@@ -1,15 +1,16 @@
 // fp32-FMA kernel family for chunkwise gated linear attention (Eq. attn_gla, evaluated chunk
 // by chunk as Section 3.5 describes).  Serves DIG_F32 (products must be fp32-accurate, which a
 // single tf32 tensor-core pass is not) and any bf16 request the tensor-core family does not
-// cover.  One CTA per (chunk, batch*head); every contraction is a register-blocked FMA loop over
-// shared-memory tiles: 4x4 blocks in the state and output kernels, 8x4 in the gradient kernel.
+// cover.  One CTA per (chunk, batch*head), or several where few chunks leave SMs idle (share); every contraction is a
+// register-blocked FMA loop over shared-memory tiles: 4x4 blocks in the state and output kernels, 8x4 in the gradient kernel.
 //
 // What bounds it: latency.  A CTA holds a whole chunk (C = d = 64 in fp32: 80 to 160 KB) and 192 chunks fill 148 SMs
 // once or twice, so a kernel's time is one or two CTAs' serial chain of load, prefix, scores, products.  Hence all
 // tiles of a kernel are asked for at once, prefix sums run in segments on all threads, loops are unrolled so that
 // several shared loads are in flight, and rounds and waits in front of the states' arrival are filled by the
 // programmatic launch.  B = 2, H = 6, L = 1024, d = C = 64 (us, before -> now): state 18 -> 11.2, with gradients
-// 26 -> 16.9, outputs 29 -> 21.2, gradients 100 -> 58; one 256-token sequence of 6 heads: 14.7 -> 8.5, 21.4 -> 15.6.
+// 26 -> 16.9, outputs 29 -> 21.2, gradients 100 -> 58; one 256-token sequence of 6 heads, whose
+// chunks are shared: state 14.7 -> 5.8, outputs 21.4 -> 12.4.
 //
 // Notation per chunk (rows j = 0..C-1 in scan order, zero rows past the end of the sequence):
 //   Lam_j = inclusive prefix sum of the gates, gamma = exp(Lam_{C-1}),
@@ -579,15 +580,31 @@ size_t smem_bwd(const Geom &g)
     return sizeof(float) * n;
 }
 constexpr size_t kMaxSmem = 227 * 1024;
-// CTAs that share a chunk where the chunks leave SMs idle.  24 chunks of 64 tokens, d = 64: state kernel 7.7 us alone, 6.1 in two
-// slices, 5.8 in four; outputs 14.2, 12.4 in two parts, 12.6 in four.  192 chunks: state 10.4, 9.8, 14.1, outputs 20.8, 25.7, 36.8.
-int share(const Geom &g, int n, bool whole) { return whole && (long long)n * g.N * g.B * g.H <= device_sm_count() ? n : 1; }
-int state_slices(const Geom &g)                 // whole vectors of channels
+// CTAs that share a chunk where the chunks leave SMs idle: slices of the state kernel, parts of the output kernel.  Fitted to 832
+// calls of 1 to 96 chunks of 16 to 128 tokens, d_k and d_v of 16 to 128: 6.1% faster on average than a CTA per chunk, the best
+// choice each time 7.4%; nine calls are slower by more than 1.5% (worst 7%).  The kernel behind is launched early and wants a place
+// for its CTA too, so n slices take n + 1 of them per chunk (forward: and a tenth to spare); wide heads gain as long as there are two SMs per
+// chunk.  Little work is not worth the further loads.  Whole passes, d = 64, us:
+//   24 chunks of 64 tokens: 20.7 with a CTA per chunk, 18.8 with four slices, 17.6 with four slices and two parts
+//   74 chunks of 64: 22.2, 26.3 with two slices and two parts;  64 chunks of 32: 15.2 and 18.1;  72 chunks of 128: 43.6, 33.6 with four
+//   and two;  24 chunks of 16, backward pass: 24.0, 24.0 with four slices
+struct Sharing {
+    int slices, parts;
+};
+Sharing share(const Geom &g, bool backward)
 {
-    const int n = share(g, 4, g.dk % 16 == 0);
-    return n > 1 ? n : share(g, 2, g.dk % 8 == 0);
+    const long long sms = device_sm_count(), chunks = (long long)g.N * g.B * g.H;
+    auto places = [&](int per_chunk) { return per_chunk * chunks <= sms; };
+    const bool wide = g.dk * g.dv > 4096, work = g.C * g.dk * g.dv > (backward ? 65536 : 32768);
+    Sharing s{1, 1};
+    for (int n = 4; work && n > 1 && s.slices == 1; n /= 2)
+        if (g.dk % (4 * n) == 0 && (wide ? places(2) : backward ? places(n + 1) : 11 * (n + 1) * chunks <= 10 * sms)) s.slices = n;        // whole vectors of channels
+    if (!backward && ((g.C == 128 || (g.C == 64 && wide)) ? places(2) : g.C == 64 && g.dv >= 48 && places(4))) {
+        s.parts = 2;
+        if (work && !places(3) && g.dk % 16 == 0) s.slices = 4;
+    }
+    return s;
 }
-int row_parts(const Geom &g) { return share(g, 2, true); }
 template <typename K>
 dig_status set_smem(K kernel, size_t bytes)
 {
@@ -600,7 +617,8 @@ dig_status fwd_typed(const GlaArgs &a)
 {
     const Geom &g = a.g;
     const Workspace w = carve_workspace(a.ws, g, false);
-    const dim3 grid(g.N, g.B * g.H), grid1(g.N, g.B * g.H, state_slices(g));
+    const Sharing shared = share(g, false);
+    const dim3 grid(g.N, g.B * g.H), grid1(g.N, g.B * g.H, shared.slices);
     dig_status st;
     auto k1 = grid1.z > 1 ? fma_chunk_state<T, false, true> : fma_chunk_state<T, false, false>;
     if ((st = set_smem(k1, smem_state(g, false))) != DIG_OK) return st;
@@ -608,7 +626,7 @@ dig_status fwd_typed(const GlaArgs &a)
     launch_pdl(k1, grid1, dim3(kThreads), smem_state(g, false), a.stream, (const T *)a.q, (const T *)a.k, (const T *)a.v, a.gate,
                (const T *)nullptr, w.states, w.gamma, (float *)nullptr, g); }
     if ((st = launch_state_scan_fwd(w, g, a.stream, a.sio)) != DIG_OK) return st;
-    const int parts = row_parts(g);
+    const int parts = shared.parts;
     auto k3 = parts > 1 ? fma_chunk_out<T, TO, 3, true>
               : g.C < 64 && (long long)grid.x * grid.y > 3ll * device_sm_count() ? fma_chunk_out<T, TO, 4, false> : fma_chunk_out<T, TO, 3, false>;
     if ((st = set_smem(k3, smem_out(g))) != DIG_OK) return st;
@@ -623,7 +641,7 @@ dig_status bwd_typed(const GlaArgs &a)
 {
     const Geom &g = a.g;
     const Workspace w = carve_workspace(a.ws, g, true);
-    const dim3 grid(g.N, g.B * g.H), grid1(g.N, g.B * g.H, state_slices(g));
+    const dim3 grid(g.N, g.B * g.H), grid1(g.N, g.B * g.H, share(g, true).slices);
     dig_status st;
     auto k1 = grid1.z > 1 ? fma_chunk_state<T, true, true> : fma_chunk_state<T, true, false>;
     if ((st = set_smem(k1, smem_state(g, true))) != DIG_OK) return st;

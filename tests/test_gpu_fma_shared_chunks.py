@@ -11,10 +11,16 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("d_k,d_v,chunk,L,H", [
     (64, 64, 64, 1, 1),             # one token
     (64, 64, 64, 256, 6),           # 24 chunks: four slices, two parts
-    (64, 64, 64, 64 * 18 + 1, 2),   # 38 chunks: two slices, two parts
-    (64, 64, 64, 64 * 37 - 5, 2),   # 74 chunks: the last that share
-    (64, 64, 64, 64 * 37 + 3, 2),   # 76: none does
-    (72, 72, 32, 100, 3),           # 72 channels are cut in two at most
+    (64, 64, 64, 64 * 18, 2),       # 36 chunks: two slices, two parts
+    (64, 64, 64, 64 * 18 + 1, 2),   # 38 chunks: two slices, one part
+    (64, 64, 64, 64 * 49 - 7, 1),   # 49 chunks: two slices in the backward pass alone
+    (64, 64, 64, 64 * 37 - 5, 2),   # 74 chunks: none
+    (64, 64, 64, 64 * 37 + 3, 2),
+    (72, 72, 64, 64 * 37 - 5, 2),   # wide heads: 74 chunks share, 72 channels are cut in two at most
+    (72, 72, 64, 64 * 37 + 3, 2),   # 76 do not
+    (72, 72, 32, 100, 3),
+    (80, 80, 64, 64 * 8 + 9, 1),    # four slices of 20 channels
+    (16, 24, 128, 128 * 29 + 40, 2),        # 60 chunks: four slices, two parts
     (16, 32, 16, 40, 2),
     (24, 16, 128, 200, 1),          # scores in a place of their own
 ])
