@@ -25,7 +25,7 @@ namespace {
 
 // Threads per CTA and CTAs per SM (what the grid is capped at, so that the grid-stride loops end together): the
 // forward kernel as many as shared memory holds, up to 8 (4, 5, 6 and 8 were measured: 17.7, 17.2, 16.7, 15.6 us on
-// 196608 rows of 64), the reverse one 3 (2, 3, 4: 37, 33, 45 us on 262144 rows of 72).
+// 196608 rows of 64), the reverse one 3 (2, 3, 4: 37, 33, 45 us on 262144 rows of 72), or 2 with the next row ahead.
 constexpr int kThreads = 128, kFwdPerSM = 8, kBwdPerSM = 3, kAheadPerSM = 2;
 constexpr size_t kSmemPerSM = 228 * 1024;
 
@@ -519,8 +519,8 @@ outgate_fwd_direct(const TA *o, const TR *r, const float *__restrict__ ln_w, con
     }
     pdl_launch_dependents();
 }
-template <typename TI, typename TO, int LPR>
-__global__ void __launch_bounds__(Direct<LPR>::kThreads, sizeof(TI) == 2 ? kAheadPerSM : kBwdPerSM)
+template <typename TI, typename TO, int LPR, bool AHEAD>
+__global__ void __launch_bounds__(Direct<LPR>::kThreads, AHEAD ? kAheadPerSM : kBwdPerSM)
 outgate_bwd_direct(const TI *o, const TI *r, const TI *dz, const float *__restrict__ ln_w, const float *__restrict__ ln_b, TO *d_o, TO *d_r,
                    float *__restrict__ partial, long long rows, int dv, float eps)
 {
@@ -537,9 +537,6 @@ outgate_bwd_direct(const TI *o, const TI *r, const TI *dz, const float *__restri
     load_affine(ln_b, col, 0.f, ln.has_col(0), b);
 #pragma unroll
     for (int j = 0; j < 4; ++j) aw[j] = ab[j] = make_float2(0.f, 0.f);
-    // bf16: the next row is asked for before this one is worked, which takes the registers of two CTAs per SM (196608 rows of 64
-    // in a training step: 28.5 -> 28.0 us, and 5.3 instead of 6.1 us to add the partial sums)
-    constexpr bool AHEAD = sizeof(TI) == 2;
     const long long step = (long long)gridDim.x * DR::kRows;
     Raw8<TI> ov[1], rv[1], gv[1], no[1], nr[1], ng[1];
     auto load = [&](long long row, Raw8<TI> (&x)[1], Raw8<TI> (&y)[1], Raw8<TI> (&z)[1]) {
@@ -612,13 +609,14 @@ outgate_affine_sum(const float *__restrict__ partial, float *__restrict__ dln_w,
     }
 }
 
-// Rows through shared memory or directly, and their split over lanes.  Measured on 196608 rows (us, forward / reverse, through
-// shared memory | directly): bf16 rows of 72 13.6 / 26.3 | 19.1 / 39.0, of 64 12.5 / 28.0 | 13.5 / 23.6 (fp32 results 15.1 / 28.3 |
-// 15.9 / 30.8), of 32 12.2 / 23.7 | 13.1 / 23.1 (786432 rows 43.8 / 76.4 | 52.4 / 81.1), of 40 13.7 / 24.6 | 13.4 / 23.5 (fp32
-// results 17.6 / 31.1 | 13.7 / 24.1: odd multiples of 16 bytes meet in banks), of 128 45.6 / 92.5 | 30.9 / 47.6; fp32 rows of 64
-// 21.9 / 46.0 | 16.5 / 31.9, of 72 31.3 / 63.0 | 23.8 / 42.9, of 128 52.9 / 101.8 | 35.6 / 58.8.  Hence shared memory for bf16 rows of
-// 72 values and of multiples of 16 up to 64, the reverse mode of 64 excepted.  One rule for both result types of bf16
-// rows, whose results have to agree to the bit.
+// Rows through shared memory or directly, and their split over lanes.  Measured on 196608 rows (us, through shared memory |
+// directly).  Forward: bf16 rows of 72 13.6 | 19.1, of 64 12.5 | 13.5 (fp32 results 15.1 | 15.9), of 32 12.2 | 13.1 (786432 rows
+// 43.8 | 52.4), of 40 13.7 | 13.4 (fp32 results 17.6 | 13.7: odd multiples of 16 bytes meet in banks), of 128 45.6 | 30.9; fp32 rows of
+// 64 21.9 | 16.5, of 72 31.3 | 23.8, of 128 52.9 | 35.6.  Reverse, kernel alone, the direct one with the next row ahead: bf16 rows of
+// 72 24.1 | 36.5 (fp32 results 39.6 | 42.0), of 32 19.9 | 19.4 (20.9 | 20.1), of 48 20.9 | 20.6 (25.6 | 27.7), directly of 40 19.9 (24.4), of 64
+// 25.6 (32.2), of 128 50.0 (62.5); without the row ahead of 64 28.0 | 25.6 (28.3 | 31.7), of 128 92.5 | 57.2; fp32 rows of 64 46.0 | 31.9, of 72
+// 63.0 | 42.9, of 128 101.8 | 58.8.  Hence shared memory for bf16 rows of 72 values and of multiples of 16 up to 64, the reverse
+// mode of 64 excepted.  One rule for both result types of bf16 rows, whose results have to agree to the bit.
 struct Split {
     bool ring;
     int lpr;
@@ -644,8 +642,6 @@ void with_direct(int dv, F f)
     else if (dv == 72) f(integral_constant<int, 9>{});
     else f(integral_constant<int, 16>{});
 }
-// CTAs per SM of the reverse mode
-int bwd_per_sm(const Split &sp, bool narrow) { return narrow && !sp.ring ? kAheadPerSM : kBwdPerSM; }
 int grid_for(long long rows, const Split &sp, int per_sm)
 {
     int sms = device_sm_count();
@@ -654,6 +650,16 @@ int grid_for(long long rows, const Split &sp, int per_sm)
     const long long per = (sp.threads() / 32) * (32 / sp.lpr), need = (rows + per - 1) / per;
     return (int)(need < kMaxCtas ? need : kMaxCtas);
 }
+// Reverse mode of bf16 rows without shared memory: where a thread works more than one row, the next one is asked for before
+// this one is worked.  That takes the registers of two CTAs per SM instead of three and leaves a third fewer partial sums to
+// add.  Rows of 64: 196608 in a training step 28.5 -> 28.0 us and 6.1 -> 5.3 for the sums; alone, kernel and sums, 16384 rows 7.36 ->
+// 6.51 (of 128: 9.30 -> 8.15), 262144 36.3 -> 35.9 (78.9 -> 68.5), but 12288 rows 6.02 -> 6.14 and 4096 3.68 -> 3.85.
+bool rows_ahead(long long rows, const Split &sp, bool narrow)
+{
+    const long long per = (sp.threads() / 32) * (32 / sp.lpr);
+    return narrow && !sp.ring && rows > grid_for(rows, sp, kBwdPerSM) * per;
+}
+int bwd_grid(long long rows, const Split &sp, bool narrow) { return grid_for(rows, sp, rows_ahead(rows, sp, narrow) ? kAheadPerSM : kBwdPerSM); }
 
 template <typename TA, typename TR, typename TZ>
 dig_status fwd_dispatch(const void *o, const void *r, const float *w, const float *b, void *z, long long rows, int dv,
@@ -710,8 +716,12 @@ dig_status bwd_dispatch(const void *o, const void *r, const void *dz, const floa
         }
     }
     with_direct(dv, [&](auto lpr) {
-        launch_pdl(outgate_bwd_direct<TI, TO, decltype(lpr)::value>, dim3(grid_for(rows, sp, bwd_per_sm(sp, sizeof(TI) == 2))), dim3(sp.threads()), 0, stream, (const TI *)o,
-                   (const TI *)r, (const TI *)dz, w, b, (TO *)d_o, (TO *)d_r, partial, rows, dv, eps);
+        auto kern = outgate_bwd_direct<TI, TO, decltype(lpr)::value, false>;
+        if constexpr (sizeof(TI) == 2) {
+            if (rows_ahead(rows, sp, true)) kern = outgate_bwd_direct<TI, TO, decltype(lpr)::value, true>;
+        }
+        launch_pdl(kern, dim3(bwd_grid(rows, sp, sizeof(TI) == 2)), dim3(sp.threads()), 0, stream, (const TI *)o, (const TI *)r, (const TI *)dz, w, b,
+                   (TO *)d_o, (TO *)d_r, partial, rows, dv, eps);
     });
     return cuda_ok(cudaGetLastError());
 }
@@ -761,7 +771,7 @@ dig_status launch_outgate_bwd(const void *o, const void *r, const void *dz, cons
     if (st != DIG_OK || !affine) return st;
     KernelTimer t(KID_OUTGATE, stream);
     launch_pdl(outgate_affine_sum, dim3((2 * dv + 31) / 32), dim3(32 * kSumWarps), 0, stream, (const float *)partial, dln_w,
-               dln_b, grid_for(rows, Split(dv, dtype != DIG_F32, true), bwd_per_sm(Split(dv, dtype != DIG_F32, true), dtype != DIG_F32)), dv);
+               dln_b, bwd_grid(rows, Split(dv, dtype != DIG_F32, true), dtype != DIG_F32), dv);
     return cuda_ok(cudaGetLastError());
 }
 

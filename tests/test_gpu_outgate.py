@@ -63,6 +63,13 @@ def test_outgate_lengths_at_the_edges_of_the_row_split(dtype, d, rows):
     _case((rows, d), dtype, True, d)
 
 
+@pytest.mark.parametrize("d,per", [(64, 32), (128, 16)])
+@pytest.mark.parametrize("more", [0, 1, 40])
+def test_outgate_reverse_mode_on_either_side_of_rows_ahead(d, per, more):
+    """As many rows as three CTAs per SM take at once, and more, where the next row is asked for ahead."""
+    _case((3 * torch.cuda.get_device_properties(0).multi_processor_count * per + more, d), "bf16", True, d + more)
+
+
 def test_outgate_single_row_and_extremes():
     from paper_2405_18428_b200 import dig
     _case((1, 1, 1, 64), "f32", True, 1)
