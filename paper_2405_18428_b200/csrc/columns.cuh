@@ -241,13 +241,15 @@ __device__ __noinline__ int choose_window(const float *sTot, Who<D> w, int start
         }
     }
 }
-// Sub-chunk length of a tile whose totals are tt; tt becomes the totals of the (sub-)chunk the thread's rows are in.  HALVES: halves,
+// How a kernel works a tile of two sub-chunks of 32 rows, with the same bits: not looked for (a pass each where the search finds
+// them), looked for first and a pass each, or both in one pass.
+enum Halves { kNoHalves, kHalvesApart, kHalvesTogether };
+// Sub-chunk length of a tile whose totals are tt; tt becomes the totals of the (sub-)chunk the thread's rows are in.  Halves,
 // which chunks of 32 ask for and which suffice for most tiles beyond the limit, are tried with sums over fixed groups (the
 // search takes a few hundred cycles).
 template <int D, bool HALVES>
-__device__ __forceinline__ int divide_tile(const float *sTot, const Who<D> &w, int sub_max, int *status, Tot &tt)
+__device__ __forceinline__ int divide_below(const float *sTot, const Who<D> &w, int sub_max, int *status, Tot &tt)
 {
-    if (sub_max >= T && !beyond<D>(tt)) return T;
     if (HALVES && sub_max >= T / 2) {
         const Tot lo = half_totals<D, 0>(sTot, w), hi = half_totals<D, 1>(sTot, w);
         if (!beyond<D>(lo) && !beyond<D>(hi)) {
@@ -258,6 +260,27 @@ __device__ __forceinline__ int divide_tile(const float *sTot, const Who<D> &w, i
     const int s = choose_window<D>(sTot, w, min(sub_max, HALVES ? T / 4 : T / 2), status), w0 = 8 * w.grp / s * (s / 8);
     tt = window_totals<D>(sTot, w, w0, w0 + s / 8);
     return s;
+}
+struct Divided {
+    Tot tt;
+    int s;
+};
+template <int D>
+__device__ __noinline__ Divided divide_away(const float *sTot, Who<D> w, int sub_max, int *status)
+{
+    Divided d;
+    d.s = divide_below<D, true>(sTot, w, sub_max, status, d.tt);
+    return d;
+}
+// AWAY: in a function of its own, out of the way of launches that wait for their instructions.
+template <int D, Halves HALVES, bool AWAY = false>
+__device__ __forceinline__ int divide_tile(const float *sTot, const Who<D> &w, int sub_max, int *status, Tot &tt)
+{
+    if (sub_max >= T && !beyond<D>(tt)) return T;
+    if (!AWAY) return divide_below<D, HALVES != kNoHalves>(sTot, w, sub_max, status, tt);
+    const Divided d = divide_away<D>(sTot, w, sub_max, status);
+    tt = d.tt;
+    return d.s;
 }
 
 __device__ __forceinline__ void st_pair(char *tile, int o, float2 a) { *reinterpret_cast<uint32_t *>(tile + o) = pack_h2(a.x, a.y); }

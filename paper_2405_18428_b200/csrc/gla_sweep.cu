@@ -91,14 +91,14 @@ template <bool B> struct Const {
     __device__ constexpr operator bool() const { return B; }
 };
 
-// How the kernels work a tile of two sub-chunks of 32 rows: in one pass, or in a pass each, with the same bits.  The code for one
-// pass costs tiles that are not divided so; short launches also wait for its instructions.  The forward and the local sweeps
-// (PAIRS) leave it out of sweeps of up to four tiles (one tile per CTA, 294 CTAs: forward sweep 8.6 us without, 9.0 with; 144 CTAs:
-// backward local sweep 6.4 and 6.8; four tiles, 768 CTAs: 49.2 and 50.0) and for chunks of 16 (48 sequences of 12544 tokens: local
-// sweeps 227 -> 238 and 274 -> 303 us with it, 233 and 280 without).  The backward sweep has it for chunks of 32 only and also the
-// search for halves (kHalvesApart) for longer ones only.
+// Tiles of two 32-row sub-chunks (Halves).  The code that works both in one pass costs tiles that are not divided so.
+//   Local sweeps and, in sweeps of more than kPlainTiles tiles, the forward sweep have it for chunks of 32 and more.  The forward
+//   sweep of fewer tiles takes a pass each: its launches wait for instructions (one tile per CTA, 144 CTAs, d = 64: a forward
+//   pass of 12.6 us against 13.0; four tiles, 768 CTAs: 46.2 and 46.9).
+//   The backward sweep has it for chunks of 32 only (see there).
+//   Chunks of 16, whose tiles are never divided so, have instances without any of it: 48 sequences of 12544 tokens, d = 64, local
+//   sweeps 238 us forward and 303 backward with it, 233 and 280 without; 16 of 16384, d = 72, backward sweep 427 and 419.
 constexpr int kPlainTiles = 4;
-enum Halves { kNoHalves, kHalvesApart, kHalvesTogether };
 
 // ---- shared phases ------------------------------------------------------------------------------
 __device__ __forceinline__ void cta_setup(Ctl *ctl, int nbar, uint32_t tmem_cols, char *tiles, int tile_bytes)
@@ -162,7 +162,7 @@ struct LocalFwdSmem {
     static constexpr uint32_t tmem_cols = 3 * L::ACCS <= 128 ? 128 : 256;
 };
 
-template <int D, bool ORDERS, bool PAIRS>
+template <int D, bool ORDERS, Halves HALVES>
 __global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_local_fwd(const SweepArgs a)
 {
@@ -194,7 +194,7 @@ sweep_local_fwd(const SweepArgs a)
         if (w.issuer() && elect_one()) {
             char *tK = smem + ((it - 1) & 1) * SM::kBuf;
             tc_fence_after_sync();
-            if (!PAIRS || !pair) {
+            if (HALVES != kHalvesTogether || !pair) {
                 issue_state<D>(tmem, tK, tK + C::TILE_T);
             } else {
                 issue_state<D, kHighRows>(tmem, tK, tK + C::TILE_T);
@@ -208,7 +208,7 @@ sweep_local_fwd(const SweepArgs a)
         tc_fence_after_sync();
         if (ok) {
             add_product<D>(tl + SM::aSum, tl, sm, w1, first);
-            if (PAIRS && pair) add_product<D>(tl + SM::aSum, tl + L::ACCS, sm, w2, false);
+            if (HALVES == kHalvesTogether && pair) add_product<D>(tl + SM::aSum, tl + L::ACCS, sm, w2, false);
         }
         first = false;
         tc_fence_before_sync();
@@ -254,9 +254,9 @@ sweep_local_fwd(const SweepArgs a)
             }
             Tot tt = tile_totals<D>(tot, w);
             const RowSum mine = row_sum<D>(sm, tt);
-            const int s = divide_tile<D, PAIRS>(tot, w, pl.sub_max, a.status, tt);
+            const int s = divide_tile<D, HALVES>(tot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
-            const bool halves = PAIRS && s == T / 2 && nrow > T / 2;            // two sub-chunks at once, a product each
+            const bool halves = HALVES == kHalvesTogether && s == T / 2 && nrow > T / 2;            // two sub-chunks at once, a product each
             const int step = halves ? T : s, nsub = (nrow + step - 1) / step;
             for (int u = nsub - 1; u >= 0; --u) {
                 if (u < nsub - 1) {
@@ -336,7 +336,7 @@ struct LocalBwdSmem {
     static_assert(cols <= 256, "tensor memory of two CTAs");
 };
 
-template <int D, bool GRAD, bool PAIRS>
+template <int D, bool GRAD, Halves HALVES>
 __global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_local_bwd(const SweepArgs a)
 {
@@ -407,11 +407,11 @@ sweep_local_bwd(const SweepArgs a)
             if (tid < T && tile + 2 < t1) rowOff[((tile + 2) & 3) * T + tid] = tile_row_offset(g, pl, g.dir, b, h, D, tile + 2, tid);
             Tot tt = tile_totals<D>(tot, w);
             const RowSum mine = row_sum<D>(sm, tt);
-            const int s = divide_tile<D, PAIRS>(tot, w, pl.sub_max, a.status, tt);
+            const int s = divide_tile<D, HALVES>(tot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
             // Two sub-chunks of 32 rows: one pass, a product each in either accumulator, the state between them as soon as the
             // first is done (nothing of them stays for the next pass).
-            const bool halves = PAIRS && s == T / 2 && nrow > T / 2;
+            const bool halves = HALVES == kHalvesTogether && s == T / 2 && nrow > T / 2;
             const int step = halves ? T : s, nsub = (nrow + step - 1) / step, nslot = halves ? 2 : nsub;
             for (int u = 0; u < nsub; ++u, ++it, ++nbuf) {
                 const int lo = u * step;
@@ -638,7 +638,7 @@ struct FwdSmem {
     static_assert(aU + L::ACCS <= tmem_cols, "tensor memory");
 };
 
-template <int D, typename TO, bool PAIRS>
+template <int D, typename TO, Halves HALVES>
 __global__ void __launch_bounds__(Col<D>::NT, 2)
 sweep_fwd(const SweepArgs a)
 {
@@ -709,7 +709,7 @@ sweep_fwd(const SweepArgs a)
             // upper half's rows alone.  Shorter ones take a pass each, the other rows of the operand tiles zero.
             const Tot whole = tile_totals<D>(sTot, w);
             Tot tt = whole;
-            const int s = divide_tile<D, PAIRS>(sTot, w, pl.sub_max, a.status, tt);
+            const int s = divide_tile<D, HALVES, HALVES == kHalvesApart>(sTot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
             // At d = 64 the two kinds of pass are compiled apart (768 sequences of 256 tokens 49.2 us without halves, 50.9
             // with the branches, 50.0 so); at d = 72 registers would spill.
@@ -780,7 +780,7 @@ sweep_fwd(const SweepArgs a)
                             issue_split<D, C::KS, C::CHS, kHighRows>(tmem + SM::aO, tQ, tS, false);
                             issue_state<D, kHighRows>(tmem + SM::aU, tK, tV);
                         }
-                        if (PAIRS) issue_weighted<D>(tmem + SM::aO, tP, tV);                          // + P V
+                        if (HALVES == kHalvesTogether) issue_weighted<D>(tmem + SM::aO, tP, tV);                          // + P V
                         else issue_split<D, T / 16, C::CHT>(tmem + SM::aO, tP, tV, true);
                         mma_commit(&ctl->bar[0]);
                     }
@@ -813,7 +813,7 @@ sweep_fwd(const SweepArgs a)
             };
             [[maybe_unused]] const bool two = s == T / 2 && nrow > T / 2;
             bool done;
-            if constexpr (!PAIRS) done = passes(Const<false>{});
+            if constexpr (HALVES != kHalvesTogether) done = passes(Const<false>{});
             else if constexpr (L::X) done = passes(two);
             else done = two ? passes(Const<true>{}) : passes(Const<false>{});
             if (!done) {
@@ -838,11 +838,10 @@ die:
 // After the second group of products the dq and dk accumulators go through shared memory (over the
 // operand tiles that are spent by then) to the column threads, which still hold the decay exponents of
 // their rows: they scale and store dq and dk, form q dq - k dk and sum it down their rows.
-// HALVES: one pass for two sub-chunks of 32 rows only in chunks of 32: the code for it slows whole tiles down by 4% at d = 64
-// (92.4 -> 96 us on 768 sequences of 256 tokens) and 2.5% at d = 72, also compiled apart per tile (101 us, spills) or per CTA
-// (98.7; short launches then wait for instructions: 25.4 -> 34 us on 48 sequences of 1024).  In chunks of 64 halves are still
-// looked for first (48 sequences of 4096, half of the heads at tau = 4: 97 us, 100 with the search alone), in chunks of 16 the
-// code for that costs more (16 of 16384, d = 72: 427 us, 418 without).
+// Two sub-chunks of 32 rows in one pass only for chunks of 32: the code for it slows whole tiles down by 4% at d = 64 (92.4 -> 96 us
+// on 768 sequences of 256 tokens) and 2.5% at d = 72, also compiled apart per tile (101 us, spills) or per CTA (98.7; short launches
+// then wait for instructions: 25.4 -> 34 us on 48 sequences of 1024).  Heads of low gate temperature in chunks of 32 pay for it: tiles
+// in sub-chunks of 16 or 8 rows (tau = 2) take 5% longer than without that code.
 // Bound by latency like the forward sweep.  48 sequences of 4096 tokens, d = 64: 140 us with the row-chunk work
 // split, 94 us now; 16 of 16384, d = 72: 252 -> 181 us.
 // =================================================================================================
@@ -970,7 +969,7 @@ sweep_bwd(const SweepArgs a)
             if (tid < T && more) rowOff[nxt * T + tid] = tile_row_offset(g, pl, sq.dir, sq.b, sq.h, D, tile - 1, tid);
             const Tot whole = tile_totals<D>(sTot, w);
             Tot tt = whole;
-            const int s = divide_tile<D, HALVES != kNoHalves>(sTot, w, pl.sub_max, a.status, tt);
+            const int s = divide_tile<D, HALVES>(sTot, w, pl.sub_max, a.status, tt);
             centre_rows<D>(raw, w, centred(tt.before, tt.all), centred(tt.xbefore, tt.xall), nrow);
             // Two sub-chunks of 32 rows share one pass: both are built, scored and finished at once; the upper half's products
             // with the gradient and the states come with the scores, the lower half's with the second group of products, once
@@ -1244,7 +1243,7 @@ dig_status run(const GlaArgs &ga, int n, uint32_t dirs, size_t stride)
     a.s_in = ga.sio.s_in;
     a.s_out = ga.sio.s_out;
     const bool sweep_only = !BWD && pl.nseg == 1;      // uncut sequences: the forward sweep starts from the start state itself
-    const bool pairs = pl.sub_max == T / 2 || (pl.sub_max == T && pl.G > kPlainTiles);
+    const bool none = pl.sub_max < T / 2;                // chunks of 16: no tile is divided in two
     dig_status st;
     // backward pass over uncut sequences whose start-state gradient is not asked for: the segment's own
     // contribution to the state gradient is never used, the local sweep only has to store the states
@@ -1256,12 +1255,12 @@ dig_status run(const GlaArgs &ga, int n, uint32_t dirs, size_t stride)
         void (*kern)(SweepArgs) = nullptr;
         size_t smem = 0;
         if constexpr (BWD) {
-            kern = states_only ? (pairs ? sweep_local_bwd<D, false, true> : sweep_local_bwd<D, false, false>)
-                               : (pairs ? sweep_local_bwd<D, true, true> : sweep_local_bwd<D, true, false>);
+            kern = states_only ? (none ? sweep_local_bwd<D, false, kNoHalves> : sweep_local_bwd<D, false, kHalvesTogether>)
+                               : (none ? sweep_local_bwd<D, true, kNoHalves> : sweep_local_bwd<D, true, kHalvesTogether>);
             smem = states_only ? LocalBwdSmem<D, false>::bytes : LocalBwdSmem<D, true>::bytes;
         } else {
-            kern = n > 1 ? (pairs ? sweep_local_fwd<D, true, true> : sweep_local_fwd<D, true, false>)
-                         : (pairs ? sweep_local_fwd<D, false, true> : sweep_local_fwd<D, false, false>);
+            kern = n > 1 ? (none ? sweep_local_fwd<D, true, kNoHalves> : sweep_local_fwd<D, true, kHalvesTogether>)
+                         : (none ? sweep_local_fwd<D, false, kNoHalves> : sweep_local_fwd<D, false, kHalvesTogether>);
             smem = LocalFwdSmem<D>::bytes;
         }
         if ((st = set_smem(kern, smem)) != DIG_OK) return st;
@@ -1279,16 +1278,17 @@ dig_status run(const GlaArgs &ga, int n, uint32_t dirs, size_t stride)
     const bool f32 = ga.dtype == DIG_BF16_F32OUT;
     if constexpr (!BWD) {
         constexpr size_t smem16 = FwdSmem<D, bf16>::bytes, smem32 = FwdSmem<D, float>::bytes;
-        auto k16 = pairs ? sweep_fwd<D, bf16, true> : sweep_fwd<D, bf16, false>;
-        auto k32 = pairs ? sweep_fwd<D, float, true> : sweep_fwd<D, float, false>;
+        const bool two = pl.sub_max == T / 2 || pl.G > kPlainTiles;
+        auto k16 = none ? sweep_fwd<D, bf16, kNoHalves> : two ? sweep_fwd<D, bf16, kHalvesTogether> : sweep_fwd<D, bf16, kHalvesApart>;
+        auto k32 = none ? sweep_fwd<D, float, kNoHalves> : two ? sweep_fwd<D, float, kHalvesTogether> : sweep_fwd<D, float, kHalvesApart>;
         if ((st = set_smem(k16, smem16)) != DIG_OK || (st = set_smem(k32, smem32)) != DIG_OK) return st;
         KernelTimer t(KID_SW_FWD, ga.stream);
         launch_pdl(f32 ? k32 : k16, grid, block, f32 ? smem32 : smem16, ga.stream, a);
     } else {
         constexpr size_t smem16 = BwdSmem<D, bf16>::bytes, smem32 = BwdSmem<D, float>::bytes;
-        const bool two = pl.sub_max == T / 2, none = pl.sub_max < T / 2;
-        auto k16 = two ? sweep_bwd<D, bf16, kHalvesTogether> : none ? sweep_bwd<D, bf16, kNoHalves> : sweep_bwd<D, bf16, kHalvesApart>;
-        auto k32 = two ? sweep_bwd<D, float, kHalvesTogether> : none ? sweep_bwd<D, float, kNoHalves> : sweep_bwd<D, float, kHalvesApart>;
+        const bool two = pl.sub_max == T / 2;
+        auto k16 = none ? sweep_bwd<D, bf16, kNoHalves> : two ? sweep_bwd<D, bf16, kHalvesTogether> : sweep_bwd<D, bf16, kHalvesApart>;
+        auto k32 = none ? sweep_bwd<D, float, kNoHalves> : two ? sweep_bwd<D, float, kHalvesTogether> : sweep_bwd<D, float, kHalvesApart>;
         if ((st = set_smem(k16, smem16)) != DIG_OK || (st = set_smem(k32, smem32)) != DIG_OK) return st;
         KernelTimer t(KID_SW_BWD, ga.stream);
         launch_pdl(f32 ? k32 : k16, grid, block, f32 ? smem32 : smem16, ga.stream, a);
