@@ -34,23 +34,25 @@ inline SweepWs carve(char *base, const Geom &g, const Plan &pl, bool backward)
     return w;
 }
 
-// Segment length.  Cost of a pass in 0.1 us, fitted to 1086 measured cuts of 2 to 768 sequences of 2 to 32 tiles, chunks of 16,
-// 32 and 64, d = 64 and 72 (root mean square of the fit's error 3 to 5%): launches, a fill per round of CTAs, tiles, and the
-// scan.  An SM with one CTA works a tile in two thirds of the time that two sharing it take.  Uncut sequences run the forward
-// sweep alone; cut ones also the local sweep and the scan; the backward pass needs the local sweep in either case.  Sub-chunks
-// multiply the tiles' cost, so short sequences in short chunks are cut where whole tiles would not be (3 tiles of 6
-// sequences, d = 64, chunks of 16: 24.4 us uncut, 18.7 cut; chunks of 64: 9.1 uncut).  A cut has to win by 2 us (backward: 1),
-// which its launches cost the host where nothing else keeps the device busy (a 256-token image: 19.2 us per block uncut, 22.6
-// cut, although the device is 0.6 us faster).  The cut chosen is within 19% of the best one, 0.3% off on average; a model of
-// rounds and tiles alone was 6% off on average and up to 2.2 times (5 tiles of 2 sequences, d = 72, chunks of 16: 53.6 us
-// uncut, 24.1 cut).
+// Segment length.  Cost of a pass in 0.1 us: launches, a fill per round of CTAs, tiles, and the scan.  An SM with one CTA works a
+// tile in two thirds of the time that two sharing it take.  Uncut sequences run the forward sweep alone; cut ones also the local
+// sweep and the scan; the backward pass needs the local sweep in either case.  Sub-chunks add to the tiles' cost, so short
+// sequences in chunks of 16 are cut where whole tiles would not be (3 tiles of 6 sequences, d = 64: 24.4 us uncut, 18.7 cut; chunks
+// of 64: 9.1 uncut).  A cut has to win by 2 us (backward: 1), which its launches cost the host where nothing else keeps the device
+// busy (a 256-token image: 19.2 us per block uncut, 22.6 cut, although the device is 0.6 us faster).
+// Against 3288 measured cuts of 2 to 768 sequences of 2 to 64 tiles, chunks of 16, 32 and 64, d = 64 and 72, gates of temperature
+// 16: the cut chosen is 0.1 to 0.6% off the best on average and at most 21% (300 sequences of 6 tiles, d = 72, backward).  The root
+// mean square of the cost's error is 5 to 12%; but forward passes in chunks of 32 are charged 190% for a tile that takes 117%
+// since two halves share a pass.  That is as close to the best (0.3%; 0.4% with 117), and with heads whose gates need shorter
+// sub-chunks it is the safer side: 80 sequences of 16 tiles, d = 72, tau = 2: 114 us, 171 with 117.  Backward passes have the 133 that
+// fits (with 170: 480 sequences of 16 tiles, d = 72, 696 us instead of 545).
 struct PassCost {
     int fixed[2], round[2], pair[2], alone[2];      // [cut]; pair: a tile on an SM with two CTAs, alone: with one
     int scan;                                       // per machine full of segments
     int chunk32, chunk16, d72;                      // factors of a tile's cost, per cent
 };
 constexpr PassCost kForward = {{21, 75}, {5, 8}, {32, 51}, {22, 37}, 35, 190, 310, 140};
-constexpr PassCost kBackward = {{14, 54}, {32, 23}, {88, 95}, {62, 73}, 67, 170, 280, 150};
+constexpr PassCost kBackward = {{14, 54}, {32, 23}, {88, 95}, {62, 73}, 67, 133, 280, 150};
 // Chunks above 64 tokens: forward plans stay within the scratch of dig_gla_fwd_static where uncut sequences do (the
 // same plan serves dig_gla_fwd, so that both give the same bits).  No other family's workspace is counted there that
 // would be larger anyway; with chunks of up to 64 the per-chunk states of the other families always are.
@@ -106,10 +108,13 @@ struct SumPlan {
 };
 // Where a sequence has too few tiles to fill the machine, orders of a forward pass side by side need fewer cuts or none, so no
 // local sweep and no scan; the results of a launch's orders then stand in buffers of their own, later launches add to them, and
-// one pass sums the buffers.  Costs as in make_plan, plus the buffers beyond the first, written and read at 0.6 MB per 0.1 us.
-// 768 tiles in 48 sequences, d = 64, four orders: 127 us one after the other, 82 side by side.  Backward passes keep one order
-// per launch: pairs took 180 instead of 198 us there, but their four tensors' buffers cost as much more in the sum.  Offsets of
-// the results have 31 bits.
+// one pass sums the buffers.  Costs as in make_plan, plus the buffers, written and read at 0.6 MB per 0.1 us, and the summing launch
+// (4 us).  bf16 results need the launch and one buffer in any case, fp32 results do not; both are charged half of it, since
+// one is to be the other rounded, and the bits depend on the cuts.  On 790 measured sums of 2 to 192 sequences of 1 to 64 tiles
+// the grouping is 0.5% off the best on average and 31% faster than one by one, 31 are slower by more than 2% (worst 20%, fp32
+// results of 32 sequences of 9 tiles).  768 tiles in 48 sequences, d = 64, four orders: 127 us one after the other, 82 side by side.
+// Backward passes keep one order per launch: pairs took 180 instead of 198 us there, but their four tensors' buffers cost as much
+// more in the sum.  Offsets of the results have 31 bits.
 class SumPlans {
     const Geom &g;
     const bool backward, narrow;
@@ -131,7 +136,8 @@ public:
             SumPlan p{1 << i, align256(elems * 4 << i), 0, launch[i]};
             p.buffers = backward ? (narrow ? 3 : 0) : (narrow || i > 0);
             if (n == 3 && i == 1 && launch[0] > launch[1]) p.launch = launch[0];          // the third order's launch
-            const long long c = cost[i] * ((n + p.k - 1) / p.k) + (long long)(100 * (p.k - 1) * 8 * elems / 600000);
+            long long c = cost[i] * (n / p.k) + (n % p.k ? cost[0] : 0);                  // three orders: a pair and one
+            if (i > 0) c += (long long)(100 * (2 * p.k - 1) * 4 * elems / 600000) + 2000;
             if (least < 0 || (c < least && p.bytes() <= limit)) {
                 least = c;
                 best = p;

@@ -12,7 +12,7 @@ def segment_bytes(segments: int, d: int) -> int:
 # per pass: launches, fill per round, a tile beside another CTA, a tile alone (each uncut, cut), scan; per cent for
 # chunks of 32 and 16 and for d = 72
 FORWARD = ((21, 75), (5, 8), (32, 51), (22, 37), 35, {32: 190, 16: 310}, 140)
-BACKWARD = ((14, 54), (32, 23), (88, 95), (62, 73), 67, {32: 170, 16: 280}, 150)
+BACKWARD = ((14, 54), (32, 23), (88, 95), (62, 73), 67, {32: 133, 16: 280}, 150)
 
 
 def costed_plan(sequences: int, ntile: int, backward: bool, chunk: int = 64, d: int = 64, limit: int | None = None) -> tuple[int, int, int]:
@@ -45,8 +45,11 @@ def sweep_plan(*args, **kw) -> tuple[int, int]:
 def orders_together(B: int, H: int, L: int, d: int, chunk: int, orders: int) -> int:
     """Scan orders that share a launch of a forward sum (chunks of up to 64)."""
     elems, best, k, j = B * L * H * d, None, 1, 1
+    launch = lambda n: costed_plan(B * H * n, -(-L // 64), False, chunk, d)[2] if n else 0
     while j <= orders and (j == 1 or elems * j < 1 << 31):
-        cost = costed_plan(B * H * j, -(-L // 64), False, chunk, d)[2] * -(-orders // j) + 100 * (j - 1) * 8 * elems // 600000
+        cost = launch(j) * (orders // j) + launch(orders % j)
+        if j > 1:
+            cost += 100 * (2 * j - 1) * 4 * elems // 600000 + 2000
         if best is None or cost < best:
             best, k = cost, j
         j *= 2

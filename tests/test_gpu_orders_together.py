@@ -33,8 +33,7 @@ def test_last_launch_needs_more_workspace_than_the_one_before(d, grid, B, H, dir
     from paper_2405_18428_b200 import dig
     from parity import TOL_BF16, oracle_threads, rel_err, to_dev
     L = grid[0] * grid[1]
-    k = orders_together(B, H, L, d, 64, 3)
-    assert k == 2 and launch_bytes(B, H, L, d, 64, 1) > launch_bytes(B, H, L, d, 64, 2)
+    assert orders_together(B, H, L, d, 64, 3) == 2 and launch_bytes(B, H, L, d, 64, 1) > launch_bytes(B, H, L, d, 64, 2)
     wl = Workload("orders", B=B, H=H, grid_h=grid[0], grid_w=grid[1], d_k=d, d_v=d, chunk=64, dtype="bf16", tau=(16.0, 4.0), seed=83)
     x = make_inputs(wl, conv=False)
     ref = oracle.gla_fwd_multi(x["q"], x["k"], x["v"], oracle.gate(x["g"], x["tau"]), *grid, dirs, threads=oracle_threads())
