@@ -5,6 +5,7 @@ import torch
 
 from paper_2405_18428_b200 import dig
 from paper_2405_18428_b200.inputs import Workload
+from sweep_plan import sweep_plan
 from test_gpu_state_io import _run
 
 pytestmark = pytest.mark.gpu
@@ -49,3 +50,28 @@ def test_a_nan_stays_in_its_half(d, direction):
     for n in ("q", "dO"):
         for got, want, name in zip(run(**{n: at + 10}), clean, ("out", "dq", "dk", "dv", "dgate")):
             assert torch.equal(got[:, behind], want[:, behind]), (n, name)
+
+
+@pytest.mark.parametrize("d,direction", [(64, 0), (72, 1)])
+@pytest.mark.parametrize("B,H,tiles", [(1, 6, 5), (10, 10, 3), (25, 8, 4), (10, 10, 5)])
+def test_one_pass_gives_the_bits_of_a_pass_per_half(B, H, tiles, d, direction):
+    """Gates under which every tile needs two halves, in chunks of 64 (a pass each in the backward sweep and in forward sweeps of up
+    to four tiles) and of 32 (one pass), the sequences cut alike."""
+    backward_too = sweep_plan(B * H, tiles, True, 64, d) == sweep_plan(B * H, tiles, True, 32, d)
+    assert sweep_plan(B * H, tiles, False, 64, d) == sweep_plan(B * H, tiles, False, 32, d) and (backward_too or d == 72)
+    L = 64 * tiles - 14
+    gen = torch.Generator(device="cuda").manual_seed(92)
+    normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda")
+    q, k, v, dO = (normal(B, L, H, d).to(torch.bfloat16) for _ in range(4))
+    gate = -0.4 - 0.01 * torch.rand((B, L, H, d), generator=gen, device="cuda")      # 32 rows: 18.5 to 18.9 of the limit's 23 (log2), 50 rows: 28.9
+    s_in, ds_out = normal(B, H, d, d), normal(B, H, d, d)
+
+    def run(chunk):
+        out = dig.dig_gla_fwd_state(q, k, v, gate, s_in, 1, L, chunk, direction)
+        return out, dig.dig_gla_bwd_state(q, k, v, gate, dO, s_in, ds_out, 1, L, chunk, direction)
+
+    (f64, b64), (f32, b32) = run(64), run(32)
+    assert all(torch.equal(x, y) for x, y in zip(f64, f32))
+    if backward_too:
+        assert all(torch.equal(x, y) for x, y in zip(b64, b32))
+    assert dig.dig_last_device_status() == dig.DIG_OK
