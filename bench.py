@@ -435,8 +435,8 @@ def sweep_entry(name, wl, torch, dig, peaks, local, flush, reps=20):
 
 
 def multi_direction_entry(wl, torch, dig, flush, reps=20):
-    """Sums over the four scan orders (Algorithm 3) of one workload: the library's entry points, which add
-    every order's fp32 results into one set of buffers, against four single-order calls plus torch adds."""
+    """Sums over the four scan orders (Algorithm 3) of one workload: the library's entry points, which form the
+    sums from fp32 buffers, against four single-order calls plus torch adds."""
     from paper_2405_18428_b200.inputs import make_inputs
     x = make_inputs(wl, conv=False)
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda().to(torch.bfloat16)
@@ -472,16 +472,18 @@ def multi_direction_entry(wl, torch, dig, flush, reps=20):
     d = wl.d_k
     # output bytes per (token, head) with d = d_k = d_v, bf16 results and an fp32 gate gradient:
     #   separate: 4 orders x 12d stored, then the adds read 4 x 12d and store 12d            -> 108 d
-    #   entry points: fp32 sums of out, dq, dk, dv (16d): stored once, read + stored 3 times, read once
-    #   more and rounded to 8d; the gate gradient (4d) stored once, read + stored 3 times      -> 164 d
+    #   entry points: out of four orders in one launch: four fp32 buffers (16d) stored, read, rounded to 2d -> 34 d;
+    #   dq, dk, dv: one set of fp32 buffers (12d) stored once, read + stored 3 times, read and rounded to 6d; the
+    #   gate gradient (4d) stored once, read + stored 3 times                                 -> 130 d
     sep_out, fus_out = th * 108 * d, th * 164 * d
     return {"workload": wl.name, "directions": list(dirs),
             "four_calls_plus_adds": median_single(separate, torch, reps, flush),
             "multi_entry_points": median_single(fused, torch, reps, flush),
             "output_bytes_model": {"four_calls_plus_adds": sep_out, "multi_entry_points": fus_out,
                                    "inputs_each": 4 * th * (fwd_b + bwd_b),
-                                   "note": "both read q, k, v, dO and the gates once per order; the entry points form the sums in fp32 "
-                                           "and round once, at the price of fp32 read-add-store traffic on the outputs"}}
+                                   "note": "both read q, k, v, dO and the gates once per order; the entry points form the sums in fp32 and "
+                                           "round once, at the price of fp32 traffic: a buffer of its own for the outputs of every order "
+                                           "that shares a launch, read-add-store per order for the gradients"}}
 
 
 def next_rows_entry(torch, dig, peaks, flush, reps=20):

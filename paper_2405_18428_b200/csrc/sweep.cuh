@@ -7,9 +7,9 @@
 // serving both operand orientations).  fp16's narrow exponent is handled by centring the in-chunk
 // decay: with Lam the cumulative gate inside a (sub-)chunk and c = Lam_end / 2 per channel, the
 // tiles hold q*exp(Lam - c) and k*exp(c - Lam), whose factors stay within exp(+-|Lam_end|/2).  A
-// tile whose gates sum to more than kSubLimit is worked in shorter sub-chunks (32, 16 or 8 rows of
-// the same tile, the other rows zero), each with its own centring; conversions saturate instead of
-// overflowing.
+// tile whose gates sum to more than kSubLimit is worked in shorter sub-chunks of 32, 16 or 8 rows,
+// each with its own centring: two of 32 in one pass over the tile where the kernel has the code for it,
+// otherwise a pass each with the other rows zero.  Conversions saturate instead of overflowing.
 //
 // Tile layout: no swizzle, "chunk-major": element (row, col) of a tile with R rows sits at
 //   (col / 8) * (16 R + 16) + 16 row + 2 (col % 8)
@@ -89,8 +89,8 @@ __device__ __forceinline__ void st8(float *p, const float (&f)[8])
 }
 // 8 results to global memory in the output storage type.  `add`: on top of what is there (fp32 outputs only;
 // used when several scan orders are summed into one buffer).  The addition is left to the L2 (a vector
-// reduction): every element gets one addition per scan order and the orders follow one another on the
-// stream, so the sum does not depend on scheduling, and nothing waits for the old values.
+// reduction): every element of a buffer gets one addition per launch and the launches follow one another on
+// the stream, so the sum does not depend on scheduling, and nothing waits for the old values.
 __device__ __forceinline__ void store_out8(float *p, const float (&f)[8], bool add = false)
 {
     if (add) {
